@@ -122,40 +122,45 @@ def _rotary_table(wl, device):
     return torch.stack([ang.cos(), ang.sin()], dim=-1).float().contiguous()
 
 
-def prepare(case, seed):
-    dev = "cuda"
-    actions, ratios = _lists(case)
-    state = {"case": case, "actions": actions, "ratios": ratios}
+def _inputs(case, seed, dev="cuda"):
+    """The tensors of a case by name, from the seed alone."""
     gen = torch.Generator(device=dev).manual_seed(seed)
     wl = _workload(case, seed)
     if case["kind"] == "cache":
         shape = (case["B"], wl.n_tokens, case["H"] * case["D"])
-        for key, scale in (("x", 3.0), ("o", 3.0), ("delta", 1.0)):
-            state[key] = torch.randn(shape, generator=gen, device=dev).mul_(scale).to(torch.bfloat16)
-        return state
+        return {key: torch.randn(shape, generator=gen, device=dev).mul_(scale).to(torch.bfloat16)
+                for key, scale in (("x", 3.0), ("o", 3.0), ("delta", 1.0))}
     q, k, v = inputs.make_qkv(wl, 0, device=dev)
-    out = torch.zeros_like(q)
+    if case["kind"] != "fused":
+        return {"q": q, "k": k, "v": v}
+    # raw projections: every token has a magnitude of its own, which the norm takes out again
+    mag = torch.exp(0.5 * torch.randn((case["B"], case["H"], wl.n_tokens, 1), generator=gen, device=dev))
+    t = {"q_raw": (q * mag).to(torch.bfloat16), "k_raw": (k * mag.flip(2)).to(torch.bfloat16), "v": v}
+    t["q_gain"], t["k_gain"] = (0.5 + torch.rand(case["D"], generator=gen, device=dev) for _ in range(2))
+    t["rot"] = _rotary_table(wl, dev)
+    return t
+
+
+def prepare(case, seed):
+    actions, ratios = _lists(case)
+    state = {"case": case, "actions": actions, "ratios": ratios, **_inputs(case, seed)}
+    if case["kind"] == "cache":
+        return state
+    state["out"] = torch.zeros_like(state["v"])
+    if case["kind"] == "fused":
+        state["q"], state["k"] = torch.zeros_like(state["q_raw"]), torch.zeros_like(state["k_raw"])
     strides = None
     if case["layout"] == "tokens":
-        q, k, v, out = (_token_major(t) for t in (q, k, v, out))
-        strides = q.stride()[:3]
-    state["ctx"] = binding.Context(case["B"], case["H"], case["D"], case["text"], wl.n_image, strides=strides)
-    state.update(q=q, k=k, v=v, out=out)
-    if case["kind"] == "fused":
-        # raw projections: every token has a magnitude of its own, which the norm takes out again
-        mag = torch.exp(0.5 * torch.randn((case["B"], case["H"], wl.n_tokens, 1), generator=gen, device=dev))
-        state["q_raw"], state["k_raw"] = (q * mag).to(torch.bfloat16), (k * mag.flip(2)).to(torch.bfloat16)
-        state["q"], state["k"] = torch.zeros_like(q), torch.zeros_like(k)
-        state["q_gain"], state["k_gain"] = (0.5 + torch.rand(case["D"], generator=gen, device=dev) for _ in range(2))
-        state["rot"] = _rotary_table(wl, dev)
-        if case["layout"] == "tokens":
-            for key in ("q_raw", "k_raw", "q", "k"):
+        for key in ("q", "k", "v", "out", "q_raw", "k_raw"):
+            if key in state:
                 state[key] = _token_major(state[key])
-    elif case["kind"] == "heads":
+        strides = state["q"].stride()[:3]
+    state["ctx"] = binding.Context(case["B"], case["H"], case["D"], case["text"], case["grid"] ** 2, strides=strides)
+    if case["kind"] == "heads":
         state["ratios"] = _head_ratios(case)
     elif case["kind"] == "device":
-        state["actions"] = torch.tensor(actions, dtype=torch.int32, device=dev)
-        state["ratios"] = torch.tensor(ratios, dtype=torch.float32, device=dev)
+        state["actions"] = torch.tensor(actions, dtype=torch.int32, device="cuda")
+        state["ratios"] = torch.tensor(ratios, dtype=torch.float32, device="cuda")
     elif case["kind"] == "mass":
         state["mass_scale"] = MASS_TEMPERATURE * case["D"] ** -0.5
     return state
@@ -226,3 +231,95 @@ def tolerance(case):
     # P is rounded to bf16 in front of P V and the result once more: against the same attention in 64 bits on the same
     # masks 1.7e-3 in the 2-norm and 7.6e-3 at most were seen; the masks themselves are whole values and do not differ
     return {"rel": 7e-3, "max": 3e-2, "differ": 0.0}
+
+
+def _f32(x):
+    """A float as the C interface hands it on: rounded to single precision."""
+    return torch.tensor(x, dtype=torch.float32).double().item()
+
+
+def _block_scores(q, k):
+    """[H, N, D] in 64 bits -> dot products of the 64-token block means, [H, nb, nb]."""
+    def means(t):
+        n_blocks = -(-t.shape[1] // 64)
+        padded = torch.nn.functional.pad(t, (0, 0, 0, 64 * n_blocks - t.shape[1])).unflatten(1, (n_blocks, 64)).sum(2)
+        count = torch.full((n_blocks, 1), 64.0, device=t.device, dtype=t.dtype)
+        count[-1] = t.shape[1] - 64 * (n_blocks - 1)
+        return padded / count
+    return means(q) @ means(k).transpose(1, 2)
+
+
+def _kept(case, scores, ratios):
+    """Boolean [H, nb, nb]: text blocks and the diagonal, and of the others the best (equal scores: the lower index)."""
+    H, nb, _ = scores.shape
+    ntb = -(-case["text"] // 64)
+    n_free = max(nb - ntb - 1, 0)
+    at = torch.arange(nb, device=scores.device)
+    forced = (at[:, None] < ntb) | (at[None, :] < ntb) | (at[:, None] == at[None, :])
+    s = scores.float().double().masked_fill(forced, -math.inf)         # the decision is made on single-precision scores
+    best, order = s.sort(dim=2, descending=True, stable=True)
+    if case["kind"] == "mass" and ratios[0] < 1.0:
+        temperature = _f32(MASS_TEMPERATURE * case["D"] ** -0.5)
+        w = torch.exp(temperature * (best - best[:, :, :1])).nan_to_num(0.0)     # rows without candidates: nan
+        before = w.cumsum(2) - w                                       # mass of the better candidates
+        take = before < _f32(ratios[0]) * w.sum(2, keepdim=True)
+    else:
+        count = torch.tensor([min(n_free, max(0, math.ceil(_f32(r) * n_free - 1e-6))) for r in ratios], device=scores.device)
+        take = at[None, None, :] < count[:, None, None]
+    take = take & (best > -math.inf)
+    return forced | torch.zeros_like(take).scatter(2, order, take)
+
+
+def _attention(q, k, v, kept):
+    """Softmax attention of [H, N, D] in 64 bits over the kept blocks; head by head, 2048 query rows at a time."""
+    out = torch.empty_like(v)
+    block = torch.arange(q.shape[1], device=q.device) // 64
+    for h in range(q.shape[0]):
+        for r in range(0, q.shape[1], 2048):
+            logits = (q[h, r:r + 2048] @ k[h].T) * q.shape[2] ** -0.5
+            logits.masked_fill_(~kept[h][block[r:r + 2048]][:, block], -math.inf)
+            out[h, r:r + 2048] = logits.softmax(1) @ v[h]
+    return out
+
+
+def _produce(raw, gain, rot):
+    """Norm, gain and rotary embedding of [H, N, D] in 64 bits."""
+    x = raw * torch.rsqrt(raw.square().mean(2, keepdim=True) + _f32(1e-6)) * gain
+    a, b = x[..., 0::2], x[..., 1::2]
+    c, s = rot[..., 0], rot[..., 1]
+    return torch.stack((a * c - b * s, a * s + b * c), dim=-1).flatten(2)
+
+
+def exact(case, seed):
+    """What run() returns, in 64 bits.  Masks and lists are whole values, compared as they are: None here."""
+    actions, ratios = _lists(case)
+    t = _inputs(case, seed)
+    if case["kind"] == "cache":
+        x, o, delta = (t[key].double() for key in ("x", "o", "delta"))
+        for b, a in enumerate(actions):
+            if a == 1:
+                o[b] = x[b] + delta[b]
+            elif a == 2:
+                delta[b] = o[b] - x[b]
+        return o, delta
+    out = torch.zeros_like(t["v"], dtype=torch.float64)
+    produced = [torch.zeros_like(out), torch.zeros_like(out)] if case["kind"] == "fused" else []
+    all_scores = []
+    for b, a in enumerate(actions):
+        if a != 2:
+            continue
+        if produced:
+            for p, key in zip(produced, ("q", "k")):
+                p[b] = _produce(t[key + "_raw"][b].double(), t[key + "_gain"].double(), t["rot"].double())
+            q, k = (p[b].to(torch.bfloat16).double() for p in produced)    # the attention reads them as they are stored
+        else:
+            q, k = t["q"][b].double(), t["k"][b].double()
+        scores = _block_scores(q, k)
+        all_scores.append(scores)
+        share = _head_ratios(case)[b] if case["kind"] == "heads" else [ratios[b]] * case["H"]
+        out[b] = _attention(q, k, t["v"][b].double(), _kept(case, scores, share))
+    if case["kind"] == "fused":
+        return produced[0], produced[1], out
+    if case["kind"] == "staged":
+        return torch.stack(all_scores), None, None, None, out
+    return out
