@@ -150,13 +150,14 @@ int get_map(rapid3_ctx* c, const void* base, CUtensorMap* out) {
 int attn_launch(rapid3_ctx* c, const TensorGeom& g, const void* q, const void* k, const void* v, void* out,
                 const ImgList& l, const int32_t* kept_idx, const int32_t* kept_cnt, const uint64_t* bitmask, float scale,
                 cudaStream_t st, const DevPlan* plan = nullptr, int n_cap = 0, bool after_select = false) {
-    CUtensorMap tq, tk, tv, to;
+    CUtensorMap tq, tk, tv;
     int r;
-    if ((r = get_map(c, q, &tq)) || (r = get_map(c, k, &tk)) || (r = get_map(c, v, &tv)) || (r = get_map(c, out, &to)))
+    if ((r = get_map(c, q, &tq)) || (r = get_map(c, k, &tk)) || (r = get_map(c, v, &tv)))
         return r;
+    if (reinterpret_cast<uintptr_t>(out) % 16) return RAPID3_ERR_INVALID_ARG;
     {
         ProfScope ps(c, PROF_ATTN, st);
-        if (launch_attention(tq, tk, tv, to, g, l, kept_idx, kept_cnt, bitmask, scale, c->status, st, plan, n_cap, -1,
+        if (launch_attention(tq, tk, tv, out, g, l, kept_idx, kept_cnt, bitmask, scale, c->status, st, plan, n_cap, -1,
                              after_select) != cudaSuccess)
             return RAPID3_ERR_CUDA;
     }
@@ -641,11 +642,12 @@ int rapid3_debug_inject_timeout(rapid3_ctx* c, const void* q, const void* k, con
     l.batch[0] = 0;
     l.slot[0] = -1;                                       // dense: every CTA walks all nb key blocks
     l.k_free[0] = 0;
-    CUtensorMap tq, tk, tv, to;
+    CUtensorMap tq, tk, tv;
     int r;
-    if ((r = get_map(c, q, &tq)) || (r = get_map(c, k, &tk)) || (r = get_map(c, v, &tv)) || (r = get_map(c, out, &to)))
+    if ((r = get_map(c, q, &tq)) || (r = get_map(c, k, &tk)) || (r = get_map(c, v, &tv)))
         return r;
-    if (launch_attention(tq, tk, tv, to, c->g, l, nullptr, nullptr, nullptr, softmax_scale, c->status,
+    if (reinterpret_cast<uintptr_t>(out) % 16) return RAPID3_ERR_INVALID_ARG;
+    if (launch_attention(tq, tk, tv, out, c->g, l, nullptr, nullptr, nullptr, softmax_scale, c->status,
                          static_cast<cudaStream_t>(stream), nullptr, 0, stop_group) != cudaSuccess)
         return RAPID3_ERR_CUDA;
     c->launches += 1;

@@ -125,7 +125,7 @@ cudaError_t launch_plan(const int32_t* action_dev, const float* ratio_dev, int B
 // lists; when present the kernel reads it instead of walking the lists.  inject_stop_group >= 0
 // launches the failure-injection build of the kernel (see rapid3_debug_inject_timeout).
 cudaError_t launch_attention(const CUtensorMap& tmq, const CUtensorMap& tmk, const CUtensorMap& tmv,
-                             const CUtensorMap& tmo, const TensorGeom& g, const ImgList& imgs, const int32_t* kept_idx,
+                             void* out, const TensorGeom& g, const ImgList& imgs, const int32_t* kept_idx,
                              const int32_t* kept_cnt, const uint64_t* bitmask, float softmax_scale, int* status,
                              cudaStream_t s, const DevPlan* plan = nullptr, int n_cap = 0, int inject_stop_group = -1,
                              int pdl = 0);   // 1: after the selection kernel, whose masks only the sparse images' thread blocks read

@@ -1,29 +1,38 @@
 // K3: masked flash-style joint attention over the kept key tiles (sm_100a).
 //
-// One CTA per (image, head, four adjacent 64-token query blocks) = two 128-row Q tiles (the
-// native UMMA M), one CTA per SM.  The four query blocks' ascending kept lists are merged into
-// one union list; the producer streams each key block of the union once through shared memory
-// and both tiles use it, which nearly halves the L2 -> SM traffic per MMA and leaves room for
-// deep K / V rings.  A tile issues no MMA for a key block that neither of its query blocks
-// kept; inside a tile a 64x64 sub-tile whose key block is not in that query block's own list
-// gets P = 0, so each query block attends exactly its own kept set.
+// The unit of work is a quad: one image, one head, four 64-token query blocks = two 128-row Q tiles (the native UMMA
+// M).  The four query blocks' ascending kept lists are merged into one union list; the producer streams each key block
+// of the union once through shared memory and both tiles use it, which nearly halves the L2 -> SM traffic per MMA and
+// leaves room for deep K / V rings.  A tile issues no MMA for a key block that neither of its query blocks kept; inside
+// a tile a 64x64 sub-tile whose key block is not in that query block's own list gets P = 0, so each query block attends
+// exactly its own kept set.
 //
-// Roles (608 threads):
-//   warp 16     producer: TMA loads (cp.async.bulk.tensor, 128-byte swizzle) of Q once, then
-//               the gathered K and V blocks into two rings of shared-memory stages; K(g) and
-//               V(g - 1), which the MMA warps need together, complete one barrier
+// One thread block per SM works through quads until none is left: it starts with the quad of its own block index and
+// then takes over those of blocks that have not started yet (clusterlaunchcontrol.try_cancel: the hardware's own
+// scheduler hands them out, in index order, so nothing has to be kept or reset in memory).  The roles walk the quads
+// each at its own pace -- while the softmax warps write the result of one quad, the next one's list is built, its Q, K
+// and V are on their way and its first scores are computed.  With a thread block per quad, barrier set-up, TMEM
+// allocation, mask read, first loads and first scores in front and the epilogue behind cost 6 us a quad, 12 % of a
+// dense one at D = 128 and 4608 tokens (three such images, dense, against that kernel in the same run: 725 -> 663 us;
+// at ratios 1, .5, .25: 530 -> 486 us; two images of 4429 tokens at D = 64 and ratio .25: 171 -> 160 us).
+//
+// Roles (640 threads):
+//   warps 0-15  softmax, eight warps per tile and four per SM sub-partition: a warp owns 16 query rows, a
+//               thread a quarter of two rows (16x256b fragments; 32 scores per key block); fp32 online
+//               softmax with lazy rescale of O, P(n) written back over S(n) as bf16, final O / l store
+//   warp 16     producer: TMA loads (cp.async.bulk.tensor, 128-byte swizzle) of Q, then the gathered K and V
+//               blocks into two rings of shared-memory stages; K(g) and V(g - 1), which the MMA warps need
+//               together, complete one barrier
 //   warps 17,18 UMMA issue, one warp per tile (warp 17 also owns the TMEM allocation).  S of a
 //               tile has NBUF buffers in TMEM (64 fp32 columns each): S(n + NBUF - 1) = Q K^T is
 //               issued before O += P(n) V, so the tensor pipe works on the next scores while the
 //               softmax warps are busy with the current ones.  Both warps walk the same union
 //               list, K ahead of V; a stage is released when both have passed it
-//   warps 0-15  softmax, eight warps per tile and four per SM sub-partition: a warp owns 16 query rows, a
-//               thread a quarter of two rows (16x256b fragments; 32 scores per key block); fp32 online
-//               softmax with lazy rescale of O, P(n) written back over S(n) as bf16, final O / l store
+//   warp 19     the next quad: takes it over, reads its masks and builds its union list
 // TMEM: tile t owns columns [256 t, 256 t + 256): S(n) at 64 (n mod NBUF), O behind the NBUF score buffers
 // (two of them and O at 128 for D = 128; three and O at 192 for D = 64, where the columns allow it).
 // Every mbarrier wait is bounded; a wait that runs out records RAPID3_ERR_TIMEOUT in the status
-// word and the CTA drains its copies, releases its TMEM and exits normally.
+// word and the thread block drains its copies, releases its TMEM and exits normally.
 #include "common.cuh"
 #include "ptx.cuh"
 
@@ -34,14 +43,19 @@ using namespace ptx;
 namespace {
 
 constexpr int SOFTMAX_WARPS = 16;
-constexpr int PRODUCER_WARP = 16, MMA_WARP0 = 17;
-constexpr int NTHREADS = 32 * (SOFTMAX_WARPS + 3);
+constexpr int PRODUCER_WARP = 16, MMA_WARP0 = 17, LIST_WARP = 19;
+constexpr int NTHREADS = 32 * (SOFTMAX_WARPS + 4);
 constexpr int TMEM_COLS = 512;
 constexpr int TILE_COLS = 256;      // TMEM columns of one Q tile
 constexpr int BLK_BYTES = 8192;     // 64 rows x 128 bytes: one 64-channel half of a 64-token block
 constexpr int QHALF_BYTES = 16384;  // one 64-channel half of a 128-row Q tile
 constexpr float RESCALE_LOG2 = 8.0f;
 constexpr int MAX_STAGES = 8;
+// The next quad is taken over when the producer has this many key blocks of the current one left to load (it runs up
+// to a ring ahead of the MMAs): early enough to have its list built in time, late enough not to hold a quad that
+// another SM could have started.
+// (2, 4 and 10 measured the same.)
+constexpr int TAKE_AHEAD = 4;
 
 struct AttnParams {
     TensorGeom g;
@@ -69,19 +83,31 @@ struct Cfg {
     static constexpr int O_COL = 64 * NBUF;                 // O accumulator behind them: 64 NBUF + D <= 256 columns per tile
 };
 
+// One quad as the roles see it, written by the list warp.
+struct Quad {
+    int n_u;                            // entries of the union list; -1: no more quads
+    int b, h;                           // image, head (of the tensors)
+    int tok[4];                         // first token of the quad's query blocks (>= N: there is no such block); tile t: 2 t, 2 t + 1
+    int16_t blk[RAPID3_MAX_NB];
+    uint8_t flag[RAPID3_MAX_NB];        // bit a: query block a keeps this key block
+};
+
 struct __align__(16) Ctl {
-    unsigned long long q_full;
+    uint4 taken;                        // answer of the last try_cancel
+    unsigned long long taken_full, near_end;
+    unsigned long long quad_full[2], quad_empty[2];
+    unsigned long long q_full, q_empty;
     unsigned long long k_full[MAX_STAGES], k_empty[MAX_STAGES];   // k_full[g % KS]: group g = K(g) and V(g - 1) have landed
     unsigned long long v_empty[MAX_STAGES];
     unsigned long long s_full[2][3], p_full[2][3];
     unsigned long long pv_done[2][2], o_done[2], drain[2];
     uint32_t tmem_base;
-    int n_u;
+    int n_early;                        // groups of the first quad that the list warp has loaded
     volatile int abort_flag;
-    uint32_t bm[4][32];
-    int16_t u_blk[RAPID3_MAX_NB];
-    uint8_t u_flag[RAPID3_MAX_NB];      // bit a: query block a of the quad keeps this key block
+    uint32_t bm[4][32];                 // the list warp's scratch
+    Quad quad[2];
 };
+constexpr int QUAD_USERS = SOFTMAX_WARPS + 3;   // warps that read a quad
 
 template <int D>
 constexpr size_t attn_smem_bytes() { return (size_t)Cfg<D>::DATA_BYTES + sizeof(Ctl) + 1024; }
@@ -92,6 +118,16 @@ __device__ __forceinline__ float max3(float a, float b, float c) {
     return d;
 }
 
+// Lane c of a quad of lanes holds words 0..3 of column pairs (c, c + 4, c + 8, c + 12); afterwards it holds words
+// 4 c .. 4 c + 3: a 4 x 4 transpose, two exchanges.
+__device__ __forceinline__ uint4 quad_transpose(uint32_t w0, uint32_t w1, uint32_t w2, uint32_t w3, int c) {
+    const bool b0 = c & 1, b1 = c & 2;
+    const uint32_t x = __shfl_xor_sync(0xffffffffu, b0 ? w0 : w1, 1), y = __shfl_xor_sync(0xffffffffu, b0 ? w2 : w3, 1);
+    const uint32_t p0 = b0 ? x : w0, p1 = b0 ? w1 : x, q0 = b0 ? y : w2, q1 = b0 ? w3 : y;
+    const uint32_t r0 = __shfl_xor_sync(0xffffffffu, b1 ? p0 : q0, 2), r1 = __shfl_xor_sync(0xffffffffu, b1 ? p1 : q1, 2);
+    return b1 ? make_uint4(r0, r1, q0, q1) : make_uint4(p0, p1, r0, r1);
+}
+
 // INJECT = true is the failure-injection build behind rapid3_debug_inject_timeout: the producer
 // stops before group prm.stop_group and every wait gives up after 2^12 polls, so the waits of all
 // roles run out and the abort path (status word, drain of the copies in flight, UMMA drain, TMEM
@@ -99,7 +135,7 @@ __device__ __forceinline__ float max3(float a, float b, float c) {
 template <int D, bool INJECT = false>
 __global__ void __launch_bounds__(NTHREADS, 1)
 attn_kernel(const __grid_constant__ CUtensorMap tmq, const __grid_constant__ CUtensorMap tmk,
-            const __grid_constant__ CUtensorMap tmv, const __grid_constant__ CUtensorMap tmo, const AttnParams prm) {
+            const __grid_constant__ CUtensorMap tmv, uint16_t* __restrict__ out, const AttnParams prm) {
     using C = Cfg<D>;
     constexpr int DH = C::DH, KS = C::KS, VS = C::VS, NBUF = C::NBUF, O_COL = C::O_COL;
     extern __shared__ uint8_t smem_raw[];
@@ -115,60 +151,17 @@ attn_kernel(const __grid_constant__ CUtensorMap tmq, const __grid_constant__ CUt
     const int warp = __shfl_sync(0xffffffffu, tid / 32, 0);
     const TensorGeom& g = prm.g;
     const int nb = g.nb, N = g.N;
-    // Work order, longest first (CTAs start in block-index order as SMs free up, so this is
-    // longest-processing-time-first scheduling): every quad of the dense images and the quads of
-    // the sparse images that hold a text query block walk all nb key blocks; the other quads of the
-    // sparse images follow, image by image in the list's order (descending keep ratio).
-    int quad, h, p, b, slot;
-    {
-        const int nq = (nb + 3) >> 2, ntq = min(nq, (g.n_text_blocks + 3) >> 2);
-        const int n_all = prm.plan ? prm.plan->all.n : prm.imgs.n;
-        const int nd = prm.plan ? prm.plan->n_dense : prm.n_dense, ns = n_all - nd;
-        int L = blockIdx.x;
-        if (L >= nq * g.H * n_all) return;               // device-resident plan: fewer images than the grid covers
-        const int heavy_dense = nd * g.H * nq, heavy_sparse = ns * g.H * ntq;
-        if (L < heavy_dense) {
-            p = L / (g.H * nq); L -= p * g.H * nq;
-            h = L / nq; quad = L - h * nq;
-        } else if (L < heavy_dense + heavy_sparse) {
-            L -= heavy_dense;
-            p = L / (g.H * ntq); L -= p * g.H * ntq; p += nd;
-            h = L / ntq; quad = L - h * ntq;
-        } else {
-            L -= heavy_dense + heavy_sparse;
-            const int nl = nq - ntq;
-            p = L / (g.H * nl); L -= p * g.H * nl; p += nd;
-            h = L / nl; quad = ntq + (L - h * nl);
-        }
-        b = prm.plan ? prm.plan->all.batch[p] : prm.imgs.batch[p];
-        slot = prm.plan ? prm.plan->all.slot[p] : prm.imgs.slot[p];
-    }
-    const int i0 = 4 * quad;
-    // Which two of the quad's four query blocks form a 128-row tile: neighbours (a, a + 1), or, when
-    // a row of the image grid spans two blocks, vertical neighbours (a, a + 2), whose kept lists
-    // overlap far more (measured on the 128 x 128 grid at keep ratio 0.25: 90 % against 63 % of
-    // the tile's MMA work lands on kept 64 x 64 sub-tiles).
-    // pair_stride 3 goes further on that grid: the whole quad is one column of it -- members
-    // (b, b + 2, b + 4, b + 6), the left or the right halves of four consecutive grid rows -- so both
-    // tiles want nearly the same key blocks (union of the quad 98 instead of 134 blocks at keep ratio
-    // 0.25, both tiles busy on 68 % of them instead of 23 %).  qblk(a) is member a's query block.
-    const bool ps2 = g.pair_stride == 2;
-    const bool vq = g.pair_stride == 3;
-    auto qblk = [&](int a) -> int {
-        int i = i0 + a;
-        if (vq && i >= g.n_text_blocks) {
-            const int r = i - g.n_text_blocks, w = r & 7;
-            i = g.n_text_blocks + (r & ~7) + ((w & 3) << 1) + (w >> 2);
-        }
-        return i;
-    };
+    const int n_quads = ((nb + 3) >> 2) * g.H * (prm.plan ? prm.plan->all.n : prm.imgs.n);
+    if ((int)blockIdx.x >= n_quads) return;              // device-resident plan: fewer images than the grid covers
 
-    const uint32_t bQ = smem_u32(&ctl->q_full);
+    const uint32_t bQ = smem_u32(&ctl->q_full), bQE = smem_u32(&ctl->q_empty);
     const uint32_t bKF = smem_u32(&ctl->k_full[0]), bKE = smem_u32(&ctl->k_empty[0]);
     const uint32_t bVE = smem_u32(&ctl->v_empty[0]);
     const uint32_t bSF = smem_u32(&ctl->s_full[0][0]), bPF = smem_u32(&ctl->p_full[0][0]);   // [tile][buf]: + 24 t + 8 buf
     const uint32_t bPV = smem_u32(&ctl->pv_done[0][0]);                                      // [tile][block parity]: + 16 t + 8 (n & 1)
     const uint32_t bOD = smem_u32(&ctl->o_done[0]);                                          // [tile]: + 8 t
+    const uint32_t bUF = smem_u32(&ctl->quad_full[0]), bUE = smem_u32(&ctl->quad_empty[0]);  // quad i: + 8 (i & 1)
+    const uint32_t bNE = smem_u32(&ctl->near_end), bT = smem_u32(&ctl->taken_full);
 
     // ---------------------------------------------------------------- setup
     if (warp == 0) {                                    // one barrier group per lane
@@ -185,108 +178,30 @@ attn_kernel(const __grid_constant__ CUtensorMap tmq, const __grid_constant__ CUt
             mbar_init(bPV + 16 * t + 8, 1);
             mbar_init(bOD + 8 * t, 1);
             mbar_init(smem_u32(&ctl->drain[t]), 1);
+            mbar_init(bUF + 8 * t, 1);
+            mbar_init(bUE + 8 * t, QUAD_USERS);
         } else if (lane == MAX_STAGES + 8) {
             mbar_init(bQ, 1);
+            mbar_init(bQE, 2);
+            mbar_init(bNE, 1);
+            mbar_init(bT, 1);
             ctl->abort_flag = 0;
-            ctl->n_u = 0;
+            ctl->n_early = 0;
         } else if (lane == MAX_STAGES + 9) {
             prefetch_tmap(&tmq);
             prefetch_tmap(&tmk);
             prefetch_tmap(&tmv);
-            prefetch_tmap(&tmo);
         }
         fence_mbar_init();
     }
-    if (tid < 128) ctl->bm[tid / 32][tid % 32] = 0;
     if (warp == MMA_WARP0) {
         tmem_alloc(smem_u32(&ctl->tmem_base), TMEM_COLS);
         tmem_relinquish();
         tc_fence_before();
     }
     __syncthreads();
-
-    // Key blocks known before the mask is read: a dense image keeps every block, and a mask of the selection kernel
-    // keeps the text blocks in every row, so the union list starts 0, 1, ... -- their K (and V) loads can start now.
-    const int n_early = (!INJECT && (slot < 0 || prm.bitmask32 != nullptr)) ? min(min(slot < 0 ? nb : g.n_text_blocks, nb), KS) : 0;
-    // The Q tiles do not depend on the mask: start their loads before the union list is built.
-    if (warp == PRODUCER_WARP && lane == 0) {
-        mbar_arrive_expect_tx(bQ, 2 * C::QTILE_BYTES);
-#pragma unroll
-        for (int a = 0; a < 4; ++a)
-#pragma unroll
-            for (int dh = 0; dh < DH; ++dh)
-                tma_load_4d(sQ + (ps2 ? (a & 1) : (a >> 1)) * C::QTILE_BYTES + dh * QHALF_BYTES +
-                                (ps2 ? (a >> 1) : (a & 1)) * BLK_BYTES, &tmq, bQ,
-                            dh * 64, qblk(a) * 64, g.h0 + h, b);
-        // groups 0 .. n_early - 1 (group g = K(g) with V(g - 1)): first use of their stages, nothing to wait for
-        for (int gi = 0; gi < n_early; ++gi) {
-            mbar_arrive_expect_tx(bKF + 8 * gi, C::KV_BYTES + (gi > 0 ? C::KV_BYTES : 0));
-#pragma unroll
-            for (int dh = 0; dh < DH; ++dh)
-                tma_load_4d(sK + gi * C::KV_BYTES + dh * BLK_BYTES, &tmk, bKF + 8 * gi, dh * 64, gi * 64, g.h0 + h, b);
-            if (gi > 0) {
-#pragma unroll
-                for (int dh = 0; dh < DH; ++dh)
-                    tma_load_4d(sV + (gi - 1) * C::KV_BYTES + dh * BLK_BYTES, &tmv, bKF + 8 * gi, dh * 64, (gi - 1) * 64, g.h0 + h, b);
-            }
-        }
-    }
-
-    // ---------------------------------------------------------------- union of the four kept lists
-    // bm[a] = bit set of the key blocks query block a keeps: copied from the bitmask when the
-    // caller has one, else rebuilt from the kept list; every block is kept for a dense image.
-    const int nw = (nb + 31) >> 5;
-    // Launched as a dependent of the selection kernel, a thread block of a sparse image waits here for the masks; one of
-    // a dense image reads nothing of them and runs on (an idle lane of its producer warp waits instead, so that the
-    // grid as a whole still ends after the selection kernel).  The masks are read past the L1 (ld.global.cg): this thread block may have
-    // started before they were written, and an L1 line of an earlier step must not answer.
-    if (slot >= 0) grid_dependency_wait();
-    if (slot >= 0 && prm.bitmask32 != nullptr) {
-        if (tid < 4 * nw) {
-            const int a = tid / nw, w = tid - a * nw;
-            if (qblk(a) < nb)
-                ctl->bm[a][w] = __ldcg(prm.bitmask32 + (((long long)slot * g.H + h) * nb + qblk(a)) * prm.words32 + w);
-        }
-    } else if (slot >= 0 && prm.kept_idx != nullptr) {
-        for (int a = 0; a < 4 && qblk(a) < nb; ++a) {
-            const long long row = ((long long)slot * g.H + h) * nb + qblk(a);
-            const int cnt = min(max(__ldcg(prm.kept_cnt + row), 0), nb);
-            const int32_t* lst = prm.kept_idx + row * nb;
-            for (int e = tid; e < cnt; e += NTHREADS) {
-                const int j = __ldcg(lst + e);
-                if ((unsigned)j < (unsigned)nb) atomicOr(&ctl->bm[a][j >> 5], 1u << (j & 31));
-                else atomicExch(prm.status, RAPID3_ERR_BAD_LIST);
-            }
-        }
-    } else if (tid < 32) {
-        const int n = min(max(nb - tid * 32, 0), 32);
-        const uint32_t val = n == 32 ? 0xffffffffu : ((1u << n) - 1u);
-        for (int a = 0; a < 4; ++a) ctl->bm[a][tid] = (qblk(a) < nb) ? val : 0u;
-    }
-    __syncthreads();
-    // one thread per key block: its position in the ascending union list is the number of union
-    // bits below it
-    for (int j = tid; j < nb; j += NTHREADS) {
-        const int w = j >> 5, bit = j & 31;
-        const uint32_t m0 = ctl->bm[0][w], m1 = ctl->bm[1][w], m2 = ctl->bm[2][w], m3 = ctl->bm[3][w];
-        const uint32_t u = m0 | m1 | m2 | m3;
-        if ((u >> bit) & 1u) {
-            int pos = __popc(u & ((1u << bit) - 1u));
-            for (int x = 0; x < w; ++x) pos += __popc(ctl->bm[0][x] | ctl->bm[1][x] | ctl->bm[2][x] | ctl->bm[3][x]);
-            ctl->u_blk[pos] = (int16_t)j;
-            ctl->u_flag[pos] = (uint8_t)(((m0 >> bit) & 1u) | (((m1 >> bit) & 1u) << 1) | (((m2 >> bit) & 1u) << 2) |
-                                         (((m3 >> bit) & 1u) << 3));
-        }
-    }
-    if (tid == 0) {
-        int tot = 0;
-        for (int x = 0; x < nw; ++x) tot += __popc(ctl->bm[0][x] | ctl->bm[1][x] | ctl->bm[2][x] | ctl->bm[3][x]);
-        ctl->n_u = tot;
-    }
-    __syncthreads();
     tc_fence_after();
     const uint32_t tmem_base = ctl->tmem_base;
-    const int n_u = ctl->n_u;
 
     auto fail = [&]() {
         atomicExch(prm.status, RAPID3_ERR_TIMEOUT);
@@ -306,66 +221,247 @@ attn_kernel(const __grid_constant__ CUtensorMap tmq, const __grid_constant__ CUt
     auto wait_warp = [&](uint32_t bar, uint32_t parity) -> bool {
         return __all_sync(0xffffffffu, wait(bar, parity));
     };
+    // Q tiles of a quad, and groups of its K and V blocks: group gi = K block gi together with V block gi - 1, which the
+    // MMA warps need as a pair before they issue S(gi) = Q K(gi)^T and O += P(gi - 1) V(gi - 1), so that the pair
+    // completes ONE barrier and costs them one wait per key block instead of two.  Group 0 is K(0) alone, group n_u is
+    // V(n_u - 1) alone.  Groups and V blocks are numbered through all quads of the thread block: group gi of a quad has
+    // number G = G0 + gi (n_u + 1 of them, the last without a K block), V block j number W0 + j (n_u of them).
+    auto load_q = [&](const Quad& u) {
+        mbar_arrive_expect_tx(bQ, 2 * C::QTILE_BYTES);
+#pragma unroll
+        for (int a = 0; a < 4; ++a)
+#pragma unroll
+            for (int dh = 0; dh < DH; ++dh)
+                tma_load_4d(sQ + (a >> 1) * C::QTILE_BYTES + dh * QHALF_BYTES + (a & 1) * BLK_BYTES, &tmq, bQ, dh * 64,
+                            u.tok[a], u.h, u.b);
+    };
+    auto issue_group = [&](const Quad& u, uint32_t G, int kb, uint32_t W, int vb) {   // key blocks, -1: none
+        const uint32_t bar = bKF + 8 * (G % KS);
+        mbar_arrive_expect_tx(bar, (kb >= 0 ? C::KV_BYTES : 0) + (vb >= 0 ? C::KV_BYTES : 0));
+        if (kb >= 0) {
+#pragma unroll
+            for (int dh = 0; dh < DH; ++dh)
+                tma_load_4d(sK + (G % KS) * C::KV_BYTES + dh * BLK_BYTES, &tmk, bar, dh * 64, kb * 64, u.h, u.b);
+        }
+        if (vb >= 0) {
+#pragma unroll
+            for (int dh = 0; dh < DH; ++dh)
+                tma_load_4d(sV + (W % VS) * C::KV_BYTES + dh * BLK_BYTES, &tmv, bar, dh * 64, vb * 64, u.h, u.b);
+        }
+    };
 
-    if (warp == PRODUCER_WARP) {
-        // ------------------------------------------------------------ producer
-        if (slot < 0 && lane == 1) grid_dependency_wait();   // see above; off every critical path
-        if (lane == 0) {
-            // Group g = K block g together with V block g - 1: the MMA warps need exactly that pair before they
-            // issue S(g) = Q K(g)^T and O += P(g-1) V(g-1), so the pair completes ONE barrier (g_full[g % KS]) and
-            // costs them one wait per key block instead of two.  Group 0 is K(0) alone, group n_u is V(n_u - 1)
-            // alone.  A group is armed once both ring stages it fills have been released.
-            int g_issued = n_early;
-            auto load_group = [&](int gi) -> bool {
-                const int s = gi % KS;
-                const bool has_k = gi < n_u, has_v = gi > 0;
-                // the K stage's release also tells that both MMA warps are past their wait on this barrier's
-                // previous phase (group gi - KS), so it is awaited even when group n_u brings no K block
-                if (!wait(bKE + 8 * s, ((gi / KS) & 1) ^ 1)) return false;
-                const int jv = gi - 1, sv = has_v ? jv % VS : 0;
-                if (has_v && !wait(bVE + 8 * sv, ((jv / VS) & 1) ^ 1)) return false;
-                mbar_arrive_expect_tx(bKF + 8 * s, (has_k ? C::KV_BYTES : 0) + (has_v ? C::KV_BYTES : 0));
-                if (has_k) {
-                    const int blk = ctl->u_blk[gi];
-#pragma unroll
-                    for (int dh = 0; dh < DH; ++dh)
-                        tma_load_4d(sK + s * C::KV_BYTES + dh * BLK_BYTES, &tmk, bKF + 8 * s, dh * 64, blk * 64, g.h0 + h, b);
+    if (warp == LIST_WARP) {
+        // ------------------------------------------------------------ quads and their union lists
+        // one lane polls: these waits are long, and the other lanes' polls would only take issue slots
+        auto wait_lane0 = [&](uint32_t bar, uint32_t parity) -> bool {
+            return __shfl_sync(0xffffffffu, (int)(lane != 0 || wait(bar, parity)), 0);
+        };
+        int L = blockIdx.x;
+        bool waited = false;                             // for the selection kernel, see below
+        for (uint32_t i = 0;; ++i) {
+            Quad& u = ctl->quad[i & 1];
+            if (!wait_lane0(bUE + 8 * (i & 1), ((i >> 1) & 1) ^ 1)) break;
+            if (L < 0) {
+                if (lane == 0) {
+                    u.n_u = -1;
+                    mbar_arrive(bUF + 8 * (i & 1));
                 }
-                if (has_v) {
-                    const int blk = ctl->u_blk[jv];
-#pragma unroll
-                    for (int dh = 0; dh < DH; ++dh)
-                        tma_load_4d(sV + sv * C::KV_BYTES + dh * BLK_BYTES, &tmv, bKF + 8 * s, dh * 64, blk * 64, g.h0 + h, b);
+                break;
+            }
+            // Work order, longest first (quads are handed out in index order, so this is longest-processing-time-first
+            // scheduling): every quad of the dense images and the quads of the sparse images that hold a text query
+            // block walk all nb key blocks; the other quads of the sparse images follow, image by image in the list's
+            // order (descending keep ratio).
+            int quad, h, p;
+            {
+                const int nq = (nb + 3) >> 2, ntq = min(nq, (g.n_text_blocks + 3) >> 2);
+                const int n_all = prm.plan ? prm.plan->all.n : prm.imgs.n;
+                const int nd = prm.plan ? prm.plan->n_dense : prm.n_dense, ns = n_all - nd;
+                const int heavy_dense = nd * g.H * nq, heavy_sparse = ns * g.H * ntq;
+                if (L < heavy_dense) {
+                    p = L / (g.H * nq); L -= p * g.H * nq;
+                    h = L / nq; quad = L - h * nq;
+                } else if (L < heavy_dense + heavy_sparse) {
+                    L -= heavy_dense;
+                    p = L / (g.H * ntq); L -= p * g.H * ntq; p += nd;
+                    h = L / ntq; quad = L - h * ntq;
+                } else {
+                    L -= heavy_dense + heavy_sparse;
+                    const int nl = nq - ntq;
+                    p = L / (g.H * nl); L -= p * g.H * nl; p += nd;
+                    h = L / nl; quad = ntq + (L - h * nl);
                 }
-                g_issued = gi + 1;
-                return true;
+            }
+            const int b = prm.plan ? prm.plan->all.batch[p] : prm.imgs.batch[p];
+            const int slot = prm.plan ? prm.plan->all.slot[p] : prm.imgs.slot[p];
+            // Which two of the quad's four query blocks form a 128-row tile: neighbours, or, when a row of the image
+            // grid spans two blocks (pair_stride 2), vertical neighbours (i, i + 2), whose kept lists overlap far more
+            // (measured on the 128 x 128 grid at keep ratio 0.25: 90 % against 63 % of the tile's MMA work lands on
+            // kept 64 x 64 sub-tiles).  pair_stride 3 goes further on that grid: the whole quad is one column of it --
+            // members (i, i + 2, i + 4, i + 6), the left or the right halves of four consecutive grid rows -- so both
+            // tiles want nearly the same key blocks (union of the quad 98 instead of 134 blocks at keep ratio 0.25,
+            // both tiles busy on 68 % of them instead of 23 %).  qblk(a) is member a's query block.
+            auto qblk = [&](int a) -> int {
+                int q = 4 * quad + (g.pair_stride == 2 ? ((a & 1) << 1) + (a >> 1) : a);
+                if (g.pair_stride == 3 && q >= g.n_text_blocks) {
+                    const int r = q - g.n_text_blocks, w = r & 7;
+                    q = g.n_text_blocks + (r & ~7) + ((w & 3) << 1) + (w >> 2);
+                }
+                return q;
             };
+            if (lane == 0) {
+                u.b = b;
+                u.h = g.h0 + h;
+#pragma unroll
+                for (int a = 0; a < 4; ++a) u.tok[a] = qblk(a) * 64;
+                if (i == 0) {
+                    // The first quad's Q tiles do not depend on the mask, nor do key blocks known before it is read: a
+                    // dense image keeps every block, and a mask of the selection kernel keeps the text blocks in every
+                    // row, so the union list starts 0, 1, ....  First use of their stages, nothing to wait for.
+                    load_q(u);
+                    const int n_early = (!INJECT && (slot < 0 || prm.bitmask32 != nullptr)) ? min(min(slot < 0 ? nb : g.n_text_blocks, nb), KS) : 0;
+                    for (int gi = 0; gi < n_early; ++gi) issue_group(u, gi, gi, gi - 1, gi - 1);
+                    ctl->n_early = n_early;
+                }
+            }
+            // m[a] = 32 bits of the set of key blocks that member a keeps: from the bitmask when the caller has one,
+            // else rebuilt from the kept list; every block for a dense image.
+            const int nw = (nb + 31) >> 5;
+            uint32_t m[4];
+            if (slot < 0) {
+                const int n = min(max(nb - lane * 32, 0), 32);
+                const uint32_t val = n == 32 ? 0xffffffffu : ((1u << n) - 1u);
+#pragma unroll
+                for (int a = 0; a < 4; ++a) m[a] = qblk(a) < nb ? val : 0u;
+            } else {
+                // Launched as a dependent of the selection kernel, the masks have to be waited for once.  They are read
+                // past the L1 (ld.global.cg): this thread block may have started before they were written, and an L1
+                // line of an earlier step must not answer.
+                if (!waited) grid_dependency_wait();
+                waited = true;
+                if (prm.bitmask32 != nullptr) {
+#pragma unroll
+                    for (int a = 0; a < 4; ++a)
+                        m[a] = (qblk(a) < nb && lane < nw)
+                                   ? __ldcg(prm.bitmask32 + (((long long)slot * g.H + h) * nb + qblk(a)) * prm.words32 + lane) : 0u;
+                } else {
+#pragma unroll
+                    for (int a = 0; a < 4; ++a) ctl->bm[a][lane] = 0u;
+                    __syncwarp();
+                    for (int a = 0; a < 4; ++a) {
+                        if (qblk(a) >= nb) continue;
+                        const long long row = ((long long)slot * g.H + h) * nb + qblk(a);
+                        const int cnt = min(max(__ldcg(prm.kept_cnt + row), 0), nb);
+                        const int32_t* lst = prm.kept_idx + row * nb;
+                        for (int e = lane; e < cnt; e += 32) {
+                            const int j = __ldcg(lst + e);
+                            if ((unsigned)j < (unsigned)nb) atomicOr(&ctl->bm[a][j >> 5], 1u << (j & 31));
+                            else atomicExch(prm.status, RAPID3_ERR_BAD_LIST);
+                        }
+                    }
+                    __syncwarp();
+#pragma unroll
+                    for (int a = 0; a < 4; ++a) m[a] = ctl->bm[a][lane];
+                }
+            }
+            // the position of a key block in the ascending union list is the number of union bits below it
+            const uint32_t un = m[0] | m[1] | m[2] | m[3];
+            int below = __popc(un);
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const int v = __shfl_up_sync(0xffffffffu, below, o);
+                if (lane >= o) below += v;
+            }
+            const int n_u = __shfl_sync(0xffffffffu, below, 31);
+            below -= __popc(un);
+            for (int w = 0; w < nw; ++w) {
+                const uint32_t uw = __shfl_sync(0xffffffffu, un, w);
+                const int pos = __shfl_sync(0xffffffffu, below, w) + __popc(uw & ((1u << lane) - 1u));
+                uint32_t f = 0u;
+#pragma unroll
+                for (int a = 0; a < 4; ++a) f |= ((__shfl_sync(0xffffffffu, m[a], w) >> lane) & 1u) << a;
+                if (f) {
+                    u.blk[pos] = (int16_t)(32 * w + lane);
+                    u.flag[pos] = (uint8_t)f;
+                }
+            }
+            if (lane == 0) u.n_u = n_u;
+            __syncwarp();
+            if (lane == 0) mbar_arrive(bUF + 8 * (i & 1));
+            // the next quad, when this one is nearly through
+            if (!wait_lane0(bNE, i & 1)) break;
+            if (lane == 0) {
+                mbar_arrive_expect_tx(bT, 16);
+                clc_try_cancel(smem_u32(&ctl->taken), bT);
+            }
+            __syncwarp();
+            // no way out before the answer is here: it is written into this thread block's shared memory
+            if (!__all_sync(0xffffffffu, mbar_wait(bT, i & 1))) {
+                if (lane == 0) fail();
+                break;
+            }
+            L = clc_taken(smem_u32(&ctl->taken));
+            if (L >= n_quads) L = -1;                    // none of the blocks behind it has work either
+        }
+        // A thread block that read no mask still ends after the selection kernel, so that the grid as a whole does.
+        if (!waited) grid_dependency_wait();
+    } else if (warp == PRODUCER_WARP) {
+        // ------------------------------------------------------------ producer
+        if (lane == 0) {
+            uint32_t G = 0, W0 = 0, n_q = 1;             // group to be issued next, the quad's first V block, Q loads so far
             bool ok = true;
-            for (int gi = n_early; ok && n_u > 0 && gi <= n_u; ++gi) {
-                if (INJECT && gi == prm.stop_group) break;
-                ok = load_group(gi);
+            uint32_t i = 0;
+            for (; ok; ++i) {
+                const Quad& u = ctl->quad[i & 1];
+                if (!(ok = wait(bUF + 8 * (i & 1), (i >> 1) & 1))) break;
+                const int n_u = u.n_u;
+                if (n_u < 0) break;
+                const int n_early = i == 0 ? ctl->n_early : 0;
+                G += n_early;
+                if (n_early > max(n_u - TAKE_AHEAD, 0)) mbar_arrive(bNE);
+                for (int gi = n_early; gi <= n_u; ++gi) {
+                    if (INJECT && gi == prm.stop_group) { ok = false; break; }
+                    if (gi == max(n_u - TAKE_AHEAD, 0)) mbar_arrive(bNE);
+                    // A group is issued once both ring stages it fills have been released.  The K stage's release also
+                    // tells that both MMA warps are past their wait on this barrier's previous phase (group G - KS),
+                    // so it is awaited even when the group brings no K block.
+                    if (!(ok = wait(bKE + 8 * (G % KS), ((G / KS) & 1) ^ 1))) break;
+                    const uint32_t W = W0 + gi - 1;
+                    if (gi > 0 && !(ok = wait(bVE + 8 * (W % VS), ((W / VS) & 1) ^ 1))) break;
+                    issue_group(u, G, gi < n_u ? u.blk[gi] : -1, W, gi > 0 ? u.blk[gi - 1] : -1);
+                    ++G;
+                    if (gi == 0 && i > 0) {              // the quad before has computed its last scores: its Q can go
+                        if (!(ok = wait(bQE, (i - 1) & 1))) break;
+                        load_q(u);
+                        ++n_q;
+                    }
+                }
+                if (!ok) break;
+                W0 += n_u;
+                mbar_arrive(bUE + 8 * (i & 1));
             }
             if (INJECT || ctl->abort_flag) {
                 // drain: do not leave the CTA while bulk copies may still land in its shared memory
-                mbar_wait(bQ, 0, 1u << 20);
-                for (int gi = max(0, g_issued - KS); gi < g_issued; ++gi)
-                    mbar_wait(bKF + 8 * (gi % KS), (gi / KS) & 1, 1u << 20);
+                mbar_wait(bQ, (n_q - 1) & 1, 1u << 20);
+                G = max(G, (uint32_t)ctl->n_early);
+                for (uint32_t x = G > KS ? G - KS : 0; x < G; ++x)
+                    mbar_wait(bKF + 8 * (x % KS), (x / KS) & 1, 1u << 20);
             }
         }
         __syncwarp();
     } else if (warp >= MMA_WARP0) {
         // ------------------------------------------------------------ UMMA issue, one warp per tile
-        // At D = 128 the whole warp runs the loop converged (addresses and descriptors stay warp-uniform) and
-        // one elected lane issues the tcgen05 instructions; at D = 64, where the time between a barrier's
-        // completion and the next issue shows in the launch time, the elected lane runs the loop alone, without
-        // the votes and warp barriers that convergence costs (measured: 1.8 % faster at D = 64, 0.4 % slower at
-        // D = 128).  Both warps pass over every block of
+        // At D = 64 the whole warp runs the loop converged and one elected lane issues the tcgen05 instructions; at
+        // D = 128, with one block's scores fewer to bridge the time between a barrier's completion and the next issue,
+        // the elected lane runs the loop alone, without the votes and warp barriers that convergence costs (attention
+        // of three 1024^2 images at ratios 1, .5, .25: 497 against 505 us; a 2048^2 one: 1054 against 1081 us; at
+        // D = 64 it is the other way round, 263 against 265 us).  Both warps pass over every block of
         // the union list, K one block ahead of V, also over blocks their tile does not use: the
         // stage barriers then see every phase in order and a stage is refilled only after both
         // tiles are past it.
         const int t = warp - MMA_WARP0;
-        const uint32_t tile_bits = ps2 ? (5u << t) : (3u << (2 * t));
-        constexpr bool SOLO = (D == 64);
+        const uint32_t tile_bits = 3u << (2 * t);
+        constexpr bool SOLO = (D == 128);
         const bool leader = elect_one();
         auto mma_wait = [&](uint32_t bar, uint32_t parity) -> bool {
             if constexpr (SOLO) return wait(bar, parity);
@@ -378,66 +474,93 @@ attn_kernel(const __grid_constant__ CUtensorMap tmq, const __grid_constant__ CUt
             const uint32_t bSFt = bSF + 24 * t, bPFt = bPF + 24 * t;
             constexpr uint32_t idesc_qk = idesc_bf16(128, 64, 0, 0);
             constexpr uint32_t idesc_pv = idesc_bf16(128, D, 0, 1);
-            int n_qk = 0, n_pv = 0;                        // blocks of this tile issued so far
-            // waits for group gi (K(gi) and V(gi - 1), see the producer), then issues S = Q K(gi)^T
-            auto k_step = [&](int j) -> bool {
-                const int s = j % KS;
-                if (!(mma_wait(bKF + 8 * s, (j / KS) & 1))) return false;
-                if (j >= n_u) return true;                 // the last group holds V(n_u - 1) only
-                const bool use = ctl->u_flag[j] & tile_bits;
-                if (use) {
-                    tc_fence_after();
-                    const uint32_t tS = tbase + 64 * (n_qk % NBUF);
-                    const uint32_t kb = sK + s * C::KV_BYTES;
-                    if (leader) {
-    #pragma unroll
-                        for (int ks = 0; ks < D / 16; ++ks)
-                            mma_ss(tS, smem_desc_sw128(qb + (ks / 4) * QHALF_BYTES + (ks % 4) * 32, 16, 1024),
-                                   smem_desc_sw128(kb + (ks / 4) * BLK_BYTES + (ks % 4) * 32, 16, 1024), idesc_qk, ks > 0);
-                        tc_commit(bKE + 8 * s);
-                        tc_commit(bSFt + 8 * (n_qk % NBUF));
+            int n_qk = 0, n_pv = 0;                        // blocks of this tile issued so far, in all quads
+            uint32_t G0 = 0, W0 = 0;
+            bool ok = true;
+            for (uint32_t i = 0; ok; ++i) {
+                const Quad& u = ctl->quad[i & 1];
+                if (!(ok = mma_wait(bUF + 8 * (i & 1), (i >> 1) & 1))) break;
+                const int n_u = u.n_u;
+                if (n_u < 0) break;
+                const int n_pv0 = n_pv;
+                // waits for group j (K(j) and V(j - 1), see the producer), then issues S = Q K(j)^T
+                auto k_step = [&](int j) -> bool {
+                    const uint32_t s = (G0 + j) % KS;
+                    if (!(mma_wait(bKF + 8 * s, ((G0 + j) / KS) & 1))) return false;
+                    if (j >= n_u) {                        // the last group holds V(n_u - 1) only
+                        if (leader) {
+                            mbar_arrive(bKE + 8 * s);
+                            if (n_u == 0) tc_commit(bQE);
+                        }
+                        return true;
                     }
-                    ++n_qk;
-                } else if (leader) {
-                    mbar_arrive(bKE + 8 * s);
+                    const bool use = u.flag[j] & tile_bits;
+                    if (use) {
+                        tc_fence_after();
+                        const uint32_t tS = tbase + 64 * (n_qk % NBUF);
+                        const uint32_t kb = sK + s * C::KV_BYTES;
+                        if (leader) {
+    #pragma unroll
+                            for (int ks = 0; ks < D / 16; ++ks)
+                                mma_ss(tS, smem_desc_sw128(qb + (ks / 4) * QHALF_BYTES + (ks % 4) * 32, 16, 1024),
+                                       smem_desc_sw128(kb + (ks / 4) * BLK_BYTES + (ks % 4) * 32, 16, 1024), idesc_qk, ks > 0);
+                            tc_commit(bKE + 8 * s);
+                            tc_commit(bSFt + 8 * (n_qk % NBUF));
+                        }
+                        ++n_qk;
+                    } else if (leader) {
+                        mbar_arrive(bKE + 8 * s);
+                    }
+                    if (leader && j == n_u - 1) tc_commit(bQE);
+                    if (!SOLO) __syncwarp();
+                    return true;
+                };
+                if (!(ok = mma_wait(bQ, i & 1))) break;
+                // the scores run NBUF - 1 key blocks ahead of the P V products
+                for (int j = 0; ok && j < NBUF - 1 && j <= n_u; ++j) ok = k_step(j);
+                for (int j = 0; ok && j < n_u; ++j) {
+                    // S(n + NBUF - 1) reuses the buffer of P(n - 1); the MMAs of the issuing thread execute in issue
+                    // order, so it is written only after P(n - 1) V has read it
+                    if (j + NBUF - 1 <= n_u && !(ok = k_step(j + NBUF - 1))) break;          // group j + 1 brings V(j)
+                    const uint32_t s = (W0 + j) % VS;
+                    const bool use = u.flag[j] & tile_bits;
+                    if (use && !(ok = (mma_wait(bPFt + 8 * (n_pv % NBUF), (n_pv / NBUF) & 1)))) break;
+                    if (use) {
+                        tc_fence_after();
+                        const uint32_t tP = tbase + 64 * (n_pv % NBUF);
+                        const uint32_t vb = sV + s * C::KV_BYTES;
+                        if (leader) {
+                            // the first product of a quad overwrites O: that its P is there tells that every softmax
+                            // warp of the tile has read the O of the quad before
+    #pragma unroll
+                            for (int ks = 0; ks < 4; ++ks)
+                                mma_ts(tO, tP + ks * 8, smem_desc_sw128(vb + ks * 2048, BLK_BYTES, 1024), idesc_pv,
+                                       (n_pv > n_pv0 || ks > 0) ? 1u : 0u);
+                            tc_commit(bVE + 8 * s);
+                            // pv_done: two barriers per tile, for the even and the odd blocks.  The softmax warps run up
+                            // to NBUF - 1 <= 2 blocks ahead of these products, and the parity of one barrier taking every
+                            // block could not tell "block n - 1 is done" from "block n - 3 is done"; with two, the one the
+                            // rescale path waits on (block n - 1's) can only be one phase behind, because S(n) exists only
+                            // once the product of block n - NBUF is over.  The epilogue may lag, so it has its own barrier.
+                            tc_commit(bPV + 16 * t + 8 * (n_pv & 1));
+                        }
+                        ++n_pv;
+                    } else if (leader) {
+                        mbar_arrive(bVE + 8 * s);
+                    }
+                    if (!SOLO) __syncwarp();
+                }
+                if (!ok) break;
+                if (leader) {
+                    // only where the tile has blocks: the next phase then needs the softmax warps' P, and they have
+                    // waited for this one by that time (a tile with nothing to do could complete two phases at once)
+                    if (n_pv > n_pv0) tc_commit(bOD + 8 * t);
+                    mbar_arrive(bUE + 8 * (i & 1));
                 }
                 if (!SOLO) __syncwarp();
-                return true;
-            };
-            bool ok = (mma_wait(bQ, 0));
-            // the scores run NBUF - 1 key blocks ahead of the P V products
-            for (int j = 0; ok && j < NBUF - 1 && j <= n_u && n_u > 0; ++j) ok = k_step(j);
-            for (int j = 0; ok && j < n_u; ++j) {
-                // S(n + NBUF - 1) reuses the buffer of P(n - 1); the MMAs of the issuing thread execute in issue
-                // order, so it is written only after P(n - 1) V has read it
-                if (j + NBUF - 1 <= n_u && !(ok = k_step(j + NBUF - 1))) break;          // group j + 1 brings V(j)
-                const int s = j % VS;
-                const bool use = ctl->u_flag[j] & tile_bits;
-                if (use && !(ok = (mma_wait(bPFt + 8 * (n_pv % NBUF), (n_pv / NBUF) & 1)))) break;
-                if (use) {
-                    tc_fence_after();
-                    const uint32_t tP = tbase + 64 * (n_pv % NBUF);
-                    const uint32_t vb = sV + s * C::KV_BYTES;
-                    if (leader) {
-    #pragma unroll
-                        for (int ks = 0; ks < 4; ++ks)
-                            mma_ts(tO, tP + ks * 8, smem_desc_sw128(vb + ks * 2048, BLK_BYTES, 1024), idesc_pv,
-                                   (n_pv > 0 || ks > 0) ? 1u : 0u);
-                        tc_commit(bVE + 8 * s);
-                        // pv_done: two barriers per tile, for the even and the odd blocks.  The softmax warps run up
-                        // to NBUF - 1 <= 2 blocks ahead of these products, and the parity of one barrier taking every
-                        // block could not tell "block n - 1 is done" from "block n - 3 is done"; with two, the one the
-                        // rescale path waits on (block n - 1's) can only be one phase behind, because S(n) exists only
-                        // once the product of block n - NBUF is over.  The epilogue may lag, so it has its own barrier.
-                        tc_commit(bPV + 16 * t + 8 * (n_pv & 1));
-                    }
-                    ++n_pv;
-                } else if (leader) {
-                    mbar_arrive(bVE + 8 * s);
-                }
-                if (!SOLO) __syncwarp();
+                G0 += n_u + 1;
+                W0 += n_u;
             }
-            if (ok && leader && n_pv > 0) tc_commit(bOD + 8 * t);
         }
         __syncwarp();
     } else {
@@ -449,8 +572,8 @@ attn_kernel(const __grid_constant__ CUtensorMap tmq, const __grid_constant__ CUt
         // 2 (lane % 4), + 1 -- 32 scores per key block.  The four threads of a quad share their rows' maximum
         // with two shuffles, and only when some row of the warp may have grown.
         const int t = (warp >> 2) & 1, wl = warp & 3, hf = warp >> 3;
-        const int a = ps2 ? 2 * (wl >> 1) + t : 2 * t + (wl >> 1);   // query block of the quad
-        const uint32_t tile_bits = ps2 ? (5u << t) : (3u << (2 * t));
+        const int a = 2 * t + (wl >> 1);               // query block of the quad
+        const uint32_t tile_bits = 3u << (2 * t);
         const int cg = lane & 3;                        // column pair within a group of eight
         const int row_lo = wl * 32 + hf * 16 + (lane >> 2);          // row of the 128-row tile; the second row is + 8
         const uint32_t lane_addr = tmem_base + ((uint32_t)(wl * 32 + hf * 16) << 16) + t * TILE_COLS;
@@ -458,16 +581,23 @@ attn_kernel(const __grid_constant__ CUtensorMap tmq, const __grid_constant__ CUt
         const uint32_t bSFt = bSF + 24 * t, bPFt = bPF + 24 * t, bPVt = bPV + 16 * t;
         const float c2 = prm.scale_log2;
         const int tail_valid = N - (nb - 1) * 64;      // valid tokens of the last block (1..64)
+        int n = 0;                                     // blocks of this tile so far, in all quads
+        uint32_t n_o = 0;                              // quads so far in which the tile had blocks
+        bool ok = true;
+        for (uint32_t i = 0;; ++i) {
+        const Quad& u = ctl->quad[i & 1];
+        if (!(ok = wait_warp(bUF + 8 * (i & 1), (i >> 1) & 1))) break;
+        const int n_u = u.n_u;
+        if (n_u < 0) break;
         float m_lo = -INFINITY, m_hi = -INFINITY;      // reference maxima of the two rows
         float l0 = 0.f, l1 = 0.f, l2 = 0.f, l3 = 0.f;  // partial row sums: (l0, l1) first row, (l2, l3) second row
-        bool ok = true;
         uint32_t r[32];
-        int n = 0;                                     // blocks of this tile so far
+        const int n0 = n;
         bool seeded = false;                           // the rows' reference maxima have been set (warp-uniform: a warp's rows share a query block)
         for (int j = 0; j < n_u; ++j) {
-            const uint32_t f = ctl->u_flag[j];
+            const uint32_t f = u.flag[j];
             if (!(f & tile_bits)) continue;            // neither query block of the tile kept it
-            const int blk = ctl->u_blk[j];
+            const int blk = u.blk[j];
             const bool act = (f >> a) & 1u;
             const int valid = (blk == nb - 1) ? tail_valid : 64;
             const int buf = n % NBUF;
@@ -572,11 +702,9 @@ attn_kernel(const __grid_constant__ CUtensorMap tmq, const __grid_constant__ CUt
             if (lane == 0) mbar_arrive(bPFt + 8 * buf);
             ++n;
         }
-        // epilogue: O / l -> bf16 -> the tile's (now unused) Q buffer in the 128-byte swizzled layout
-        // of the tensor map -> TMA stores, one per (query block, 64-channel half); rows past the
-        // end of the sequence are clipped by the store
-        if (ok && n > 0) ok = wait_warp(bOD + 8 * t, 0);
-        if (ok) {
+        if (!ok || (n > n0 && !(ok = wait_warp(bOD + 8 * t, n_o++ & 1)))) break;
+        // epilogue: O / l -> bf16 -> 16 bytes a lane, four lanes a 64-byte piece of a row
+        {
             tc_fence_after();
             float s_lo = l0 + l1, s_hi = l2 + l3;      // the quad's four partial sums make the row sum
             s_lo += __shfl_xor_sync(0xffffffffu, s_lo, 1);
@@ -584,54 +712,47 @@ attn_kernel(const __grid_constant__ CUtensorMap tmq, const __grid_constant__ CUt
             s_lo += __shfl_xor_sync(0xffffffffu, s_lo, 2);
             s_hi += __shfl_xor_sync(0xffffffffu, s_hi, 2);
             const float inv_lo = s_lo > 0.f ? 1.f / s_lo : 0.f, inv_hi = s_hi > 0.f ? 1.f / s_hi : 0.f;
-            uint8_t* so_lo = smem + t * C::QTILE_BYTES + row_lo * 128;
-            uint8_t* so_hi = so_lo + 8 * 128;
-            const int sw_lo = row_lo & 7, sw_hi = (row_lo + 8) & 7;
+            const int tok_lo = u.tok[a] + (row_lo & 63), tok_hi = tok_lo + 8;
+            uint16_t* o_lo = out + (long long)u.b * g.stride_b + (long long)u.h * g.stride_h + (long long)tok_lo * g.stride_n + 8 * cg;
+            uint16_t* o_hi = o_lo + 8 * g.stride_n;
             uint32_t o[16];
 #pragma unroll
             for (int ch = 0; ch < D / 32; ++ch) {
-                if (n > 0) {
+                if (n > n0) {
                     tmem_ld16x256_x4(tO + ch * 32, o);
                     tc_wait_ld();
                 } else {
 #pragma unroll
                     for (int e = 0; e < 16; ++e) o[e] = 0u;
                 }
+                uint32_t w_lo[4], w_hi[4];
 #pragma unroll
-                for (int k = 0; k < 4; ++k) {
-                    // channels 32 ch + 8 k + 2 cg, + 1: 16-byte chunk (4 (ch & 1) + k) of the 128-byte half row
-                    const int chunk = (ch & 1) * 4 + k;
-                    const uint32_t w_lo = pack_bf16(__uint_as_float(o[4 * k]) * inv_lo, __uint_as_float(o[4 * k + 1]) * inv_lo);
-                    const uint32_t w_hi = pack_bf16(__uint_as_float(o[4 * k + 2]) * inv_hi, __uint_as_float(o[4 * k + 3]) * inv_hi);
-                    *reinterpret_cast<uint32_t*>(so_lo + (ch >> 1) * QHALF_BYTES + ((chunk ^ sw_lo) << 4) + 4 * cg) = w_lo;
-                    *reinterpret_cast<uint32_t*>(so_hi + (ch >> 1) * QHALF_BYTES + ((chunk ^ sw_hi) << 4) + 4 * cg) = w_hi;
+                for (int k = 0; k < 4; ++k) {          // channels 32 ch + 8 k + 2 cg, + 1
+                    w_lo[k] = pack_bf16(__uint_as_float(o[4 * k]) * inv_lo, __uint_as_float(o[4 * k + 1]) * inv_lo);
+                    w_hi[k] = pack_bf16(__uint_as_float(o[4 * k + 2]) * inv_hi, __uint_as_float(o[4 * k + 3]) * inv_hi);
                 }
+                const uint4 v_lo = quad_transpose(w_lo[0], w_lo[1], w_lo[2], w_lo[3], cg);
+                const uint4 v_hi = quad_transpose(w_hi[0], w_hi[1], w_hi[2], w_hi[3], cg);
+                if (tok_lo < N) *reinterpret_cast<uint4*>(o_lo + 32 * ch) = v_lo;
+                if (tok_hi < N) *reinterpret_cast<uint4*>(o_hi + 32 * ch) = v_hi;
             }
-            fence_proxy_async_smem();
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(bUE + 8 * (i & 1));
         }
-        // the four warps of a query block meet, then one lane stores the block
-        const int qb_id = a;
-        named_barrier_sync(1 + qb_id, 128);
-        if (ok && (wl & 1) == 0 && hf == 0 && lane == 0 && qblk(qb_id) * 64 < N) {
-#pragma unroll
-            for (int dh = 0; dh < DH; ++dh)
-                tma_store_4d(&tmo, sQ + t * C::QTILE_BYTES + dh * QHALF_BYTES + (wl >> 1) * BLK_BYTES, dh * 64,
-                             qblk(qb_id) * 64, g.h0 + h, b);
-            bulk_commit_group();
-            bulk_wait_read_all();
         }
     }
 
     // ---------------------------------------------------------------- teardown
     tc_fence_before();
     __syncthreads();
-    if (warp >= MMA_WARP0) {
+    if (warp >= MMA_WARP0 && warp < MMA_WARP0 + 2) {
         if (ctl->abort_flag) {
             // make sure no UMMA of this warp is still in flight before the TMEM columns are released
-            const uint32_t bT = smem_u32(&ctl->drain[warp - MMA_WARP0]);
+            const uint32_t bD = smem_u32(&ctl->drain[warp - MMA_WARP0]);
             if (elect_one()) {
-                tc_commit(bT);
-                mbar_wait(bT, 0, 1u << 20);
+                tc_commit(bD);
+                mbar_wait(bD, 0, 1u << 20);
             }
             __syncwarp();
         }
@@ -664,7 +785,7 @@ cudaError_t attention_static_init() {
 }
 
 cudaError_t launch_attention(const CUtensorMap& tmq, const CUtensorMap& tmk, const CUtensorMap& tmv,
-                             const CUtensorMap& tmo,
+                             void* out,
                              const TensorGeom& g, const ImgList& imgs, const int32_t* kept_idx,
                              const int32_t* kept_cnt, const uint64_t* bitmask, float softmax_scale, int* status,
                              cudaStream_t s, const DevPlan* plan, int n_cap, int inject_stop_group, int pdl) {
@@ -689,13 +810,13 @@ cudaError_t launch_attention(const CUtensorMap& tmq, const CUtensorMap& tmk, con
     dim3 grid(((g.nb + 3) / 4) * g.H * (plan ? n_cap : imgs.n), 1, 1);
     if (inject_stop_group >= 0) {
         if (g.D == 128)
-            attn_kernel<128, true><<<grid, NTHREADS, attn_smem_bytes<128>(), s>>>(tmq, tmk, tmv, tmo, prm);
+            attn_kernel<128, true><<<grid, NTHREADS, attn_smem_bytes<128>(), s>>>(tmq, tmk, tmv, static_cast<uint16_t*>(out), prm);
         else
-            attn_kernel<64, true><<<grid, NTHREADS, attn_smem_bytes<64>(), s>>>(tmq, tmk, tmv, tmo, prm);
+            attn_kernel<64, true><<<grid, NTHREADS, attn_smem_bytes<64>(), s>>>(tmq, tmk, tmv, static_cast<uint16_t*>(out), prm);
     } else if (g.D == 128) {
-        return launch_kernel(attn_kernel<128>, grid, dim3(NTHREADS), attn_smem_bytes<128>(), s, pdl != 0, tmq, tmk, tmv, tmo, prm);
+        return launch_kernel(attn_kernel<128>, grid, dim3(NTHREADS), attn_smem_bytes<128>(), s, pdl != 0, tmq, tmk, tmv, static_cast<uint16_t*>(out), prm);
     } else {
-        return launch_kernel(attn_kernel<64>, grid, dim3(NTHREADS), attn_smem_bytes<64>(), s, pdl != 0, tmq, tmk, tmv, tmo, prm);
+        return launch_kernel(attn_kernel<64>, grid, dim3(NTHREADS), attn_smem_bytes<64>(), s, pdl != 0, tmq, tmk, tmv, static_cast<uint16_t*>(out), prm);
     }
     return cudaGetLastError();
 }
