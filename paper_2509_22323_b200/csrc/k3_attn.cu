@@ -49,7 +49,9 @@ constexpr int TMEM_COLS = 512;
 constexpr int TILE_COLS = 256;      // TMEM columns of one Q tile
 constexpr int BLK_BYTES = 8192;     // 64 rows x 128 bytes: one 64-channel half of a 64-token block
 constexpr int QHALF_BYTES = 16384;  // one 64-channel half of a 128-row Q tile
-constexpr float RESCALE_LOG2 = 8.0f;
+// A row's reference maximum moves when a partial sum of eight P exceeds 2^16, in the rows that grew by more than 2^12.
+// (How far P may exceed 1 costs no precision: P, O and l are floating point throughout.)
+constexpr float GROWN_SUM = 65536.0f, GROWN_LOG2 = 12.0f;
 constexpr int MAX_STAGES = 8;
 // The next quad is taken over when the producer has this many key blocks of the current one left to load (it runs up
 // to a ring ahead of the MMAs): early enough to have its list built in time, late enough not to hold a quad that
@@ -88,8 +90,7 @@ struct Quad {
     int n_u;                            // entries of the union list; -1: no more quads
     int b, h;                           // image, head (of the tensors)
     int tok[4];                         // first token of the quad's query blocks (>= N: there is no such block); tile t: 2 t, 2 t + 1
-    int16_t blk[RAPID3_MAX_NB];
-    uint8_t flag[RAPID3_MAX_NB];        // bit a: query block a keeps this key block
+    uint32_t ent[RAPID3_MAX_NB];        // ascending key blocks: ENT_BLK up; bit a: query block a keeps it; ENT_TAIL
 };
 
 struct __align__(16) Ctl {
@@ -107,6 +108,8 @@ struct __align__(16) Ctl {
     uint32_t bm[4][32];                 // the list warp's scratch
     Quad quad[2];
 };
+constexpr uint32_t ENT_TAIL = 16u;      // the sequence ends inside this key block
+constexpr int ENT_BLK = 8;              // the block's number from this bit on
 constexpr int QUAD_USERS = SOFTMAX_WARPS + 3;   // warps that read a quad
 
 template <int D>
@@ -126,6 +129,20 @@ __device__ __forceinline__ uint4 quad_transpose(uint32_t w0, uint32_t w1, uint32
     const uint32_t p0 = b0 ? x : w0, p1 = b0 ? w1 : x, q0 = b0 ? y : w2, q1 = b0 ? w3 : y;
     const uint32_t r0 = __shfl_xor_sync(0xffffffffu, b1 ? p0 : q0, 2), r1 = __shfl_xor_sync(0xffffffffu, b1 ? p1 : q1, 2);
     return b1 ? make_uint4(r0, r1, q0, q1) : make_uint4(p0, p1, r0, r1);
+}
+
+// Maxima of a quad's two rows over one key block, from the four threads' 16x256b fragments.
+__device__ __forceinline__ void row_maxima(const uint32_t (&r)[32], float& lo, float& hi) {
+    lo = hi = -INFINITY;
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+        lo = max3(lo, __uint_as_float(r[4 * k]), __uint_as_float(r[4 * k + 1]));
+        hi = max3(hi, __uint_as_float(r[4 * k + 2]), __uint_as_float(r[4 * k + 3]));
+    }
+    lo = fmaxf(lo, __shfl_xor_sync(0xffffffffu, lo, 1));
+    hi = fmaxf(hi, __shfl_xor_sync(0xffffffffu, hi, 1));
+    lo = fmaxf(lo, __shfl_xor_sync(0xffffffffu, lo, 2));
+    hi = fmaxf(hi, __shfl_xor_sync(0xffffffffu, hi, 2));
 }
 
 // INJECT = true is the failure-injection build behind rapid3_debug_inject_timeout: the producer
@@ -381,8 +398,8 @@ attn_kernel(const __grid_constant__ CUtensorMap tmq, const __grid_constant__ CUt
 #pragma unroll
                 for (int a = 0; a < 4; ++a) f |= ((__shfl_sync(0xffffffffu, m[a], w) >> lane) & 1u) << a;
                 if (f) {
-                    u.blk[pos] = (int16_t)(32 * w + lane);
-                    u.flag[pos] = (uint8_t)f;
+                    const int j = 32 * w + lane;
+                    u.ent[pos] = f | ((j + 1) * 64 > N ? ENT_TAIL : 0u) | ((uint32_t)j << ENT_BLK);
                 }
             }
             if (lane == 0) u.n_u = n_u;
@@ -428,7 +445,7 @@ attn_kernel(const __grid_constant__ CUtensorMap tmq, const __grid_constant__ CUt
                     if (!(ok = wait(bKE + 8 * (G % KS), ((G / KS) & 1) ^ 1))) break;
                     const uint32_t W = W0 + gi - 1;
                     if (gi > 0 && !(ok = wait(bVE + 8 * (W % VS), ((W / VS) & 1) ^ 1))) break;
-                    issue_group(u, G, gi < n_u ? u.blk[gi] : -1, W, gi > 0 ? u.blk[gi - 1] : -1);
+                    issue_group(u, G, gi < n_u ? (int)(u.ent[gi] >> ENT_BLK) : -1, W, gi > 0 ? (int)(u.ent[gi - 1] >> ENT_BLK) : -1);
                     ++G;
                     if (gi == 0 && i > 0) {              // the quad before has computed its last scores: its Q can go
                         if (!(ok = wait(bQE, (i - 1) & 1))) break;
@@ -494,7 +511,7 @@ attn_kernel(const __grid_constant__ CUtensorMap tmq, const __grid_constant__ CUt
                         }
                         return true;
                     }
-                    const bool use = u.flag[j] & tile_bits;
+                    const bool use = u.ent[j] & tile_bits;
                     if (use) {
                         tc_fence_after();
                         const uint32_t tS = tbase + 64 * (n_qk % NBUF);
@@ -523,7 +540,7 @@ attn_kernel(const __grid_constant__ CUtensorMap tmq, const __grid_constant__ CUt
                     // order, so it is written only after P(n - 1) V has read it
                     if (j + NBUF - 1 <= n_u && !(ok = k_step(j + NBUF - 1))) break;          // group j + 1 brings V(j)
                     const uint32_t s = (W0 + j) % VS;
-                    const bool use = u.flag[j] & tile_bits;
+                    const bool use = u.ent[j] & tile_bits;
                     if (use && !(ok = (mma_wait(bPFt + 8 * (n_pv % NBUF), (n_pv / NBUF) & 1)))) break;
                     if (use) {
                         tc_fence_after();
@@ -573,9 +590,9 @@ attn_kernel(const __grid_constant__ CUtensorMap tmq, const __grid_constant__ CUt
         // with two shuffles, and only when some row of the warp may have grown.
         const int t = (warp >> 2) & 1, wl = warp & 3, hf = warp >> 3;
         const int a = 2 * t + (wl >> 1);               // query block of the quad
-        const uint32_t tile_bits = 3u << (2 * t);
+        const uint32_t tile_bits = 3u << (2 * t), act_bit = 1u << a;
         const int cg = lane & 3;                        // column pair within a group of eight
-        const int row_lo = wl * 32 + hf * 16 + (lane >> 2);          // row of the 128-row tile; the second row is + 8
+        const int row_lo = wl * 32 + hf * 16 + (lane >> 2);
         const uint32_t lane_addr = tmem_base + ((uint32_t)(wl * 32 + hf * 16) << 16) + t * TILE_COLS;
         const uint32_t tO = lane_addr + O_COL;
         const uint32_t bSFt = bSF + 24 * t, bPFt = bPF + 24 * t, bPVt = bPV + 16 * t;
@@ -589,90 +606,85 @@ attn_kernel(const __grid_constant__ CUtensorMap tmq, const __grid_constant__ CUt
         if (!(ok = wait_warp(bUF + 8 * (i & 1), (i >> 1) & 1))) break;
         const int n_u = u.n_u;
         if (n_u < 0) break;
-        float m_lo = -INFINITY, m_hi = -INFINITY;      // reference maxima of the two rows
+        float nm_lo = INFINITY, nm_hi = INFINITY;      // reference maxima of the two rows, times -c2
         float l0 = 0.f, l1 = 0.f, l2 = 0.f, l3 = 0.f;  // partial row sums: (l0, l1) first row, (l2, l3) second row
         uint32_t r[32];
         const int n0 = n;
         bool seeded = false;                           // the rows' reference maxima have been set (warp-uniform: a warp's rows share a query block)
         for (int j = 0; j < n_u; ++j) {
-            const uint32_t f = u.flag[j];
-            if (!(f & tile_bits)) continue;            // neither query block of the tile kept it
-            const int blk = u.blk[j];
-            const bool act = (f >> a) & 1u;
-            const int valid = (blk == nb - 1) ? tail_valid : 64;
+            const uint32_t e = u.ent[j];
+            if (!(e & tile_bits)) continue;            // neither query block of the tile kept it
+            const bool act = e & act_bit;
             const int buf = n % NBUF;
             const uint32_t tS = lane_addr + 64 * buf;
-            if (!(ok = wait_warp(bSFt + 8 * buf, (n / NBUF) & 1))) break;
+            // A wait that runs out sets the abort flag, and the quad is gone through over whatever is there: nothing up
+            // to its end depends on a wait's result, so no vote is taken on the way.
+            wait(bSFt + 8 * buf, (n / NBUF) & 1);
+            __syncwarp();
             tc_fence_after();
             uint32_t pk[16];
             if (act) {
                 tmem_ld16x256_x8(tS, r);
                 tc_wait_ld();
-                if (valid != 64) {
+                if (e & ENT_TAIL) {
 #pragma unroll
                     for (int k = 0; k < 8; ++k)
 #pragma unroll
-                        for (int e = 0; e < 2; ++e)
-                            if (8 * k + 2 * cg + e >= valid) {       // -inf: outside the sequence
-                                r[4 * k + e] = 0xff800000u;
-                                r[4 * k + 2 + e] = 0xff800000u;
+                        for (int x = 0; x < 2; ++x)
+                            if (8 * k + 2 * cg + x >= tail_valid) {       // -inf: outside the sequence
+                                r[4 * k + x] = 0xff800000u;
+                                r[4 * k + 2 + x] = 0xff800000u;
                             }
                 }
-                // One pass over the 32 scores gives P = 2^(S c2 - m c2) (packed to bf16), the block's partial
-                // row sums and the thread's share of the block's row maxima.  The pass runs with the reference
-                // maxima as they stand, so the exponentials do not wait for this block's maximum; only when a
-                // row's maximum has grown by more than 2^8 (rare after the first blocks) O and l are rescaled
-                // and the pass is repeated.
+                // One pass over the 32 scores gives P = 2^(S c2 - m c2) (packed to bf16) and the block's partial row
+                // sums.  The pass runs with the reference maxima as they stand, so the exponentials do not wait for
+                // this block's maximum, and it takes no maximum at all: a P above 2^16 shows in the partial sum that it
+                // is part of (eight terms, none negative).  Only when a partial sum exceeds 2^16 (rare after a query
+                // block's first key block) the rows' maxima are taken, O and l are rescaled and the pass is repeated.
+                // Bound by issue slots and the exponential unit: against maxima in the pass, packed products, votes on
+                // the waits and P stored after the vote below, dense attention of two images of 4429 tokens at D = 64
+                // went from 325 to 303 us, three of 4608 at D = 128 from 596 to 585 us (bursts at full clocks).
                 float b0, b1, b2, b3;
                 bool redo;
                 if (!seeded) {
                     // the first block this query block keeps: take the rows' maxima before the pass instead of running
                     // the pass twice (from -inf every row "grows")
-                    float mx_lo = -INFINITY, mx_hi = -INFINITY;
-#pragma unroll
-                    for (int k = 0; k < 8; ++k) {
-                        mx_lo = max3(mx_lo, __uint_as_float(r[4 * k]), __uint_as_float(r[4 * k + 1]));
-                        mx_hi = max3(mx_hi, __uint_as_float(r[4 * k + 2]), __uint_as_float(r[4 * k + 3]));
-                    }
-                    mx_lo = fmaxf(mx_lo, __shfl_xor_sync(0xffffffffu, mx_lo, 1));
-                    mx_hi = fmaxf(mx_hi, __shfl_xor_sync(0xffffffffu, mx_hi, 1));
-                    m_lo = fmaxf(mx_lo, __shfl_xor_sync(0xffffffffu, mx_lo, 2));
-                    m_hi = fmaxf(mx_hi, __shfl_xor_sync(0xffffffffu, mx_hi, 2));
+                    row_maxima(r, nm_lo, nm_hi);
+                    nm_lo *= -c2; nm_hi *= -c2;
                     seeded = true;
                 }
                 do {
-                    const float ms_lo = m_lo * c2, ms_hi = m_hi * c2;
-                    float mx_lo = -INFINITY, mx_hi = -INFINITY;
                     b0 = b1 = b2 = b3 = 0.f;
 #pragma unroll
                     for (int k = 0; k < 8; ++k) {
                         float x0, x1, x2, x3;
-                        fma2(x0, x1, __uint_as_float(r[4 * k]), __uint_as_float(r[4 * k + 1]), c2, -ms_lo);
-                        fma2(x2, x3, __uint_as_float(r[4 * k + 2]), __uint_as_float(r[4 * k + 3]), c2, -ms_hi);
+                        x0 = fmaf(__uint_as_float(r[4 * k]), c2, nm_lo); x1 = fmaf(__uint_as_float(r[4 * k + 1]), c2, nm_lo);
+                        x2 = fmaf(__uint_as_float(r[4 * k + 2]), c2, nm_hi); x3 = fmaf(__uint_as_float(r[4 * k + 3]), c2, nm_hi);
                         x0 = ex2(x0); x1 = ex2(x1); x2 = ex2(x2); x3 = ex2(x3);
                         add2(b0, b1, x0, x1);
                         add2(b2, b3, x2, x3);
                         pk[2 * k] = pack_bf16(x0, x1);
                         pk[2 * k + 1] = pack_bf16(x2, x3);
-                        mx_lo = max3(mx_lo, __uint_as_float(r[4 * k]), __uint_as_float(r[4 * k + 1]));
-                        mx_hi = max3(mx_hi, __uint_as_float(r[4 * k + 2]), __uint_as_float(r[4 * k + 3]));
                     }
-                    // a thread sees a quarter of each row: if any thread of the warp sees growth, the quads
-                    // combine their maxima and decide row by row
-                    redo = __any_sync(0xffffffffu, (mx_lo - m_lo) * c2 > RESCALE_LOG2 || (mx_hi - m_hi) * c2 > RESCALE_LOG2);
+                    // P goes out before the vote on it is in, so that the two overlap; a repeated pass stores again before
+                    // anything is told that P is there
+                    tmem_st16x128_x8(tS, pk);
+                    // if any thread of the warp sees growth, the quads combine their maxima and decide row by row
+                    redo = __any_sync(0xffffffffu, max3(b0, b1, fmaxf(b2, b3)) > GROWN_SUM);
                     if (redo) {
-                        mx_lo = fmaxf(mx_lo, __shfl_xor_sync(0xffffffffu, mx_lo, 1));
-                        mx_hi = fmaxf(mx_hi, __shfl_xor_sync(0xffffffffu, mx_hi, 1));
-                        mx_lo = fmaxf(mx_lo, __shfl_xor_sync(0xffffffffu, mx_lo, 2));
-                        mx_hi = fmaxf(mx_hi, __shfl_xor_sync(0xffffffffu, mx_hi, 2));
-                        const bool g_lo = (mx_lo - m_lo) * c2 > RESCALE_LOG2, g_hi = (mx_hi - m_hi) * c2 > RESCALE_LOG2;   // true from -inf
-                        const bool f_lo = g_lo && m_lo != -INFINITY, f_hi = g_hi && m_hi != -INFINITY;   // O holds something to rescale
+                        float mx_lo, mx_hi;
+                        row_maxima(r, mx_lo, mx_hi);
+                        // a sum of eight above 2^16 has a term above 2^13 - 1: the row that asked for it always moves
+                        mx_lo *= -c2; mx_hi *= -c2;
+                        const bool g_lo = nm_lo - mx_lo > GROWN_LOG2, g_hi = nm_hi - mx_hi > GROWN_LOG2;
+                        const bool f_lo = g_lo && nm_lo != INFINITY, f_hi = g_hi && nm_hi != INFINITY;   // O holds something to rescale
                         if (__any_sync(0xffffffffu, f_lo || f_hi)) {
                             // O must be at rest: wait for P(n-1) V, which by the issue order of the products also
                             // tells that every earlier one is done
-                            if (!(ok = wait_warp(bPVt + 8 * ((n - 1) & 1), ((n - 1) >> 1) & 1))) break;
+                            wait(bPVt + 8 * ((n - 1) & 1), ((n - 1) >> 1) & 1);
+                            __syncwarp();
                             tc_fence_after();
-                            const float a_lo = f_lo ? ex2((m_lo - mx_lo) * c2) : 1.f, a_hi = f_hi ? ex2((m_hi - mx_hi) * c2) : 1.f;
+                            const float a_lo = f_lo ? ex2(mx_lo - nm_lo) : 1.f, a_hi = f_hi ? ex2(mx_hi - nm_hi) : 1.f;
                             l0 *= a_lo; l1 *= a_lo; l2 *= a_hi; l3 *= a_hi;
                             uint32_t o[16];
 #pragma unroll
@@ -685,24 +697,24 @@ attn_kernel(const __grid_constant__ CUtensorMap tmq, const __grid_constant__ CUt
                                 tmem_st16x256_x4(tO + ch * 32, o);
                             }
                         }
-                        if (g_lo) m_lo = mx_lo;
-                        if (g_hi) m_hi = mx_hi;
+                        if (g_lo) nm_lo = mx_lo;
+                        if (g_hi) nm_hi = mx_hi;
                     }
                 } while (redo);
-                if (!ok) break;
                 l0 += b0; l1 += b1; l2 += b2; l3 += b3;
             } else {
 #pragma unroll
                 for (int e = 0; e < 16; ++e) pk[e] = 0u;
+                tmem_st16x128_x8(tS, pk);
             }
-            tmem_st16x128_x8(tS, pk);
             tc_wait_st();
             tc_fence_before();
             __syncwarp();
             if (lane == 0) mbar_arrive(bPFt + 8 * buf);
             ++n;
         }
-        if (!ok || (n > n0 && !(ok = wait_warp(bOD + 8 * t, n_o++ & 1)))) break;
+        if (n > n0) wait(bOD + 8 * t, n_o++ & 1);
+        if (!(ok = __all_sync(0xffffffffu, !ctl->abort_flag))) break;
         // epilogue: O / l -> bf16 -> 16 bytes a lane, four lanes a 64-byte piece of a row
         {
             tc_fence_after();

@@ -199,15 +199,7 @@ __host__ __device__ constexpr uint32_t idesc_bf16(int M, int N, int a_mn_major, 
            (static_cast<uint32_t>(M >> 4) << 24);
 }
 
-// Packed fp32 pairs (one instruction for two lanes of work).
-__device__ __forceinline__ void fma2(float& d0, float& d1, float a0, float a1, float b, float c) {
-    uint64_t a, bb, cc, d;
-    asm("mov.b64 %0, {%1, %2};" : "=l"(a) : "f"(a0), "f"(a1));
-    asm("mov.b64 %0, {%1, %1};" : "=l"(bb) : "f"(b));
-    asm("mov.b64 %0, {%1, %1};" : "=l"(cc) : "f"(c));
-    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(bb), "l"(cc));
-    asm("mov.b64 {%0, %1}, %2;" : "=f"(d0), "=f"(d1) : "l"(d));
-}
+// Packed fp32 pairs (one instruction for two additions).
 __device__ __forceinline__ void add2(float& d0, float& d1, float a0, float a1) {
     uint64_t a, d;
     asm("mov.b64 %0, {%1, %2};" : "=l"(d) : "f"(d0), "f"(d1));

@@ -1,0 +1,35 @@
+"""The rule by which a row's reference maximum moves: a partial sum of eight P above 2^16.  Scores that rise from key
+block to key block by steps below, around and far above what the rule lets pass, in few keys of a block or in all."""
+import math
+
+import pytest
+import torch
+
+from paper_2509_22323_b200 import binding
+
+pytestmark = pytest.mark.gpu
+DEV = "cuda"
+
+
+@pytest.mark.parametrize("D", [64, 128])
+@pytest.mark.parametrize("step", [4.0, 12.9, 13.1, 15.9, 16.1, 19.0, 200.0])
+@pytest.mark.parametrize("every", [1, 64])
+def test_scores_rising_by_steps(D, step, every):
+    H, N = 2, 640 + 21
+    gen = torch.Generator(device=DEV).manual_seed(int(10 * step) + D + every)
+    q, k, v = (torch.randn((1, H, N, D), generator=gen, device=DEV) for _ in range(3))
+    at = torch.arange(N, device=DEV)
+    # channel 0 alone decides: step (in powers of two) per key block, in every `every`-th key; the others stay at 0
+    rise = torch.where(at % every == 0, step * (at // 64), 0.0)
+    q[..., 0], q[..., 1:] = 8.0, 0.1 * q[..., 1:]
+    k[..., 0], k[..., 1:] = rise * math.log(2.0) * D ** 0.5 / 8.0, 0.1 * k[..., 1:]
+    q, k, v = (t.to(torch.bfloat16) for t in (q, k, v))
+    ctx = binding.Context(1, H, D, 0, N)
+    out = torch.full_like(q, float("nan"))
+    ctx.rapid3_gated_step(q, k, v, out, [2], [1.0])
+    torch.cuda.synchronize()
+    assert ctx.last_status() == 0
+    ref = (q[0].double() @ k[0].double().transpose(1, 2) * D ** -0.5).softmax(-1) @ v[0].double()
+    # P and the result are rounded to bf16 (2^-9 each, relative to the values' range); scores up to 2000 in powers of
+    # two are 32-bit products, 2^-24 x 2000 x ln 2 relative in P
+    assert float((out[0].double() - ref).abs().max()) <= 2 ** -7 * float(v.abs().max())
