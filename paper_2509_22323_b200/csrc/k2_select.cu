@@ -1,159 +1,133 @@
 // K2: per (image, head, query-block row) forced + top-k block selection.
-// One warp per row.  The row of fp32 scores is staged in shared memory as order-preserving
-// 32-bit keys.  The k-th largest free candidate is found by a radix select over the key bits
-// (the bits all candidates share are skipped, the others go eight at a time through a 256-bin
-// histogram and a scan from the top; rows with at most 32 candidates rank each candidate by
-// counting the 64-bit (key, index) composites that beat it instead); a free
-// candidate is kept when its key is above that threshold, or equal to it and among the first
-// (lowest block index) of the equal ones still needed -- the order "score descending, index
-// ascending".  The bitmask is assembled with warp ballots and the ascending kept list with ballot
-// prefix counts, so the row is written in one pass.
+// One warp per row, the row's scores in registers as order-preserving 32-bit keys (IPL of them a lane, key block
+// 32 x + lane in register x).  The k-th largest free candidate is found by a radix search over the key bits, two at a
+// time from the highest bit in which two candidates differ: the candidates at or above each of the three trial
+// prefixes are counted in ten-bit fields of one word (there are at most 1023), which one warp-wide addition combines.
+// The search ends early when exactly k candidates are at or above the prefix.  A free candidate is kept when its key is
+// above that threshold, or equal to it and among the first (lowest block index) of the equal ones still needed -- the
+// order "score descending, index ascending".  The bitmask is assembled with warp ballots and the ascending kept list
+// with ballot prefix counts, so the row is written in one pass.
+// Bound by the latency of that chain: a warp has a row to itself and every row's warp is resident.  Keys in shared
+// memory and histograms of eight bits a round, which this replaces, took 7.3 us for two images of 24 heads x 70 rows
+// (now 4.8), 9.5 us for three of 72 (6.4) and 17.7 us for one of 264 (13.6).
+#include <type_traits>
+
 #include "common.cuh"
 
 namespace {
 
 constexpr int WARPS = 4;
 
+// Order-preserving key of a score: unsigned integers with the same order as the floats (-0 and +0 made equal), at least
+// 2^23 for any finite one.  Forced blocks and padding get key 0, below every trial prefix.
+__device__ __forceinline__ uint32_t score_key(float x) {
+    uint32_t u = __float_as_uint(x);
+    if (u == 0x80000000u) u = 0u;
+    return u ^ ((u >> 31) ? 0xffffffffu : 0x80000000u);
+}
+
+// Bits of the candidates' keys (non-zero ones): the number of low bits in which two of them differ, and what the bits
+// above are in all of them.
+template <int IPL>
+__device__ __forceinline__ int differing_bits(const uint32_t (&u)[IPL], uint32_t& common) {
+    uint32_t k_and = 0xffffffffu, k_or = 0u;
+#pragma unroll
+    for (int x = 0; x < IPL; ++x)
+        if (u[x]) { k_and &= u[x]; k_or |= u[x]; }
+    k_and = __reduce_and_sync(0xffffffffu, k_and);
+    k_or = __reduce_or_sync(0xffffffffu, k_or);
+    const uint32_t diff = k_and ^ k_or;
+    const int top = diff ? 32 - __clz(diff) : 0;
+    common = top >= 32 ? 0u : (k_or & ~((1u << top) - 1u));
+    return top;
+}
+
 // HK = NoHeadKeep: one keep count per image.  HK = HeadKeep: one per (image, head), passed by value.
 // HK = RowKeep: one per row, read from device memory.
-template <typename HK>
+template <typename HK, int IPL>
 __global__ void __launch_bounds__(WARPS * 32) select_kernel(const float* scores, TensorGeom g,
                                                             ImgList imgs, uint32_t* __restrict__ bitmask32,
                                                             int32_t* __restrict__ kept_idx,
                                                             int32_t* __restrict__ kept_cnt, int words32,
                                                             const DevPlan* __restrict__ plan, const HK hk) {
-    extern __shared__ unsigned long long srow[];          // [WARPS][nb_pad] 64-bit slots, then [WARPS][256] histogram bins
     const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
     const int nb = g.nb, ntb = g.n_text_blocks;
-    const int nb_pad = (nb + 31) & ~31;
-    const long long row = (long long)blockIdx.x * WARPS + warp;        // (p * H + h) * nb + i
+    const int ph = blockIdx.y, p = ph / g.H;            // p * H + h
+    const int i = blockIdx.x * WARPS + warp;
+    const int row = ph * nb + i;                        // at most 65535 x 1024
     grid_dependency_launch();
     grid_dependency_wait();                             // the scores come from the kernel before, which may still be running
-    const long long n_rows = (long long)(plan ? plan->sparse.n : imgs.n) * g.H * nb;
-    if (row >= n_rows) return;
-    const int i = (int)(row % nb);
-    const int p = (int)(row / ((long long)nb * g.H));
+    if (i >= nb || (plan && p >= plan->sparse.n)) return;
     // free candidates kept in this row: one count per image, or per (image, head) when the policy
     // sets a ratio for every head
     int k;
-    if constexpr (HK::mode == 1) k = hk.k[p * g.H + (int)((row / nb) % g.H)];
-    else if constexpr (HK::mode == 2) k = hk.k[row];
+    if constexpr (HK::mode == 1) k = hk.k[ph];
+    else if constexpr (HK::mode == 2) k = __ldcg(hk.k + row);
     else k = plan ? plan->sparse.k_free[p] : imgs.k_free[p];
-    // long rows keep 32-bit keys in the slots' memory, short rows 64-bit (key, index) composites
-    unsigned long long* c64 = srow + warp * nb_pad;
-    uint32_t* s = reinterpret_cast<uint32_t*>(c64);
-    const float* src = scores + row * nb;
+    const float* src = scores + (long long)row * nb;
     const bool text_row = i < ntb;
     const int n_free = max(nb - ntb - ((i >= ntb) ? 1 : 0), 0);
     const bool select = !text_row && k > 0 && k < n_free;
-    const bool radix = n_free > 32;                     // short rows: ranking by counting is cheaper (measured: 63 candidates already favour the histogram)
-    // key: unsigned integer with the same order as the float (-0 and +0 made equal), at least 2^23 for
-    // any finite score.  Forced blocks and padding get key 0: they match no radix prefix (every trial
-    // prefix has a bit set) and beat no candidate, so the loops below need no index tests.
-    for (int j = lane; j < nb_pad; j += 32) {
-        uint32_t u = 0u;
-        if (j < nb && j >= ntb && j != i) {
-            u = __float_as_uint(__ldcg(src + j));              // past the L1: see the wait above
-            if (u == 0x80000000u) u = 0u;
-            u ^= (u >> 31) ? 0xffffffffu : 0x80000000u;
-        }
-        // composite: equal scores rank by ascending block index, so no two candidates compare equal
-        if (radix) s[j] = u;
-        else c64[j] = u ? (((unsigned long long)u << 32) | (uint32_t)(0xffffffffu - (uint32_t)j)) : 0ull;
+    uint32_t u[IPL];
+#pragma unroll
+    for (int x = 0; x < IPL; ++x) {
+        const int j = 32 * x + lane;
+        u[x] = 0u;
+        if (select && j < nb && j >= ntb && j != i) u[x] = score_key(__ldcg(src + j));   // past the L1: see the wait above
     }
-    __syncwarp();
-    // radix select of the k-th largest key among the free candidates: the bits all candidates share are skipped,
-    // the rest is taken eight bits at a time, each round a 256-bin histogram of the candidates that still match
-    // the prefix (shared-memory atomics) and a scan over the bins from the top
     uint32_t prefix = 0u;
-    int want = k;                                       // rank still looked for inside the prefix group
-    if (select && radix) {
-        uint32_t* hist = reinterpret_cast<uint32_t*>(srow + WARPS * nb_pad) + warp * 256;
-        uint32_t k_and = 0xffffffffu, k_or = 0u;
-        for (int j = lane; j < nb_pad; j += 32) {
-            const uint32_t u = s[j];
-            if (u) { k_and &= u; k_or |= u; }
+    int want = 0;                                       // of the keys that equal `prefix`, how many are kept
+    if (select) {
+        int hi = differing_bits(u, prefix);             // the candidates that decide equal `prefix` from bit `hi` up
+        int at_least = n_free, above = 0;               // candidates at or above `prefix`, and above those that decide
+        while (hi > 0 && at_least > k) {
+            const int lo = max(hi - 2, 0);
+            const uint32_t d = 1u << lo, t1 = prefix + d, t2 = t1 + d, t3 = t2 + d;
+            uint32_t c = 0u;                            // candidates at or above the three trials
+            if (hi - lo == 2) {
+#pragma unroll
+                for (int x = 0; x < IPL; ++x) c += (u[x] >= t1 ? 1u : 0u) + (u[x] >= t2 ? 1u << 10 : 0u) + (u[x] >= t3 ? 1u << 20 : 0u);
+                c = __reduce_add_sync(0xffffffffu, c);
+            } else {
+#pragma unroll
+                for (int x = 0; x < IPL; ++x) c += u[x] >= t1 ? 1u : 0u;
+                c = __reduce_add_sync(0xffffffffu, c) | ((uint32_t)above << 10) | ((uint32_t)above << 20);   // no digit 2 or 3
+            }
+            const int c1 = c & 1023u, c2 = (c >> 10) & 1023u, c3 = c >> 20;
+            // the digit is the largest with k candidates or more at or above it
+            if (c3 >= k) { prefix = t3; at_least = c3; }
+            else if (c2 >= k) { prefix = t2; at_least = c2; above = c3; }
+            else if (c1 >= k) { prefix = t1; at_least = c1; above = c2; }
+            else above = c1;
+            hi = lo;
         }
-        k_and = __reduce_and_sync(0xffffffffu, k_and);
-        k_or = __reduce_or_sync(0xffffffffu, k_or);
-        const uint32_t diff = k_and ^ k_or;             // bits in which two candidates differ
-        const int top = diff ? 32 - __clz(diff) : 0;    // only bits below `top` can differ
-        prefix = top >= 32 ? 0u : (k_or & ~((1u << top) - 1u));
-        for (int hi = top; hi > 0; hi -= 8) {           // digit = bits [lo, hi)
-            const int lo = max(hi - 8, 0);
-            const uint32_t dmask = (1u << (hi - lo)) - 1u;
-#pragma unroll
-            for (int b = 0; b < 8; ++b) hist[8 * lane + b] = 0u;
-            __syncwarp();
-            for (int j = lane; j < nb_pad; j += 32) {
-                const uint32_t u = s[j];
-                if (u && (hi >= 32 || (u >> hi) == (prefix >> hi))) atomicAdd(&hist[(u >> lo) & dmask], 1u);
-            }
-            __syncwarp();
-            // lane l owns bins 8 l .. 8 l + 7; S = candidates in its bins and all higher ones
-            uint32_t hloc[8], T = 0u;
-#pragma unroll
-            for (int b = 0; b < 8; ++b) {
-                hloc[b] = hist[8 * lane + b];
-                T += hloc[b];
-            }
-            uint32_t S = T;
-#pragma unroll
-            for (int o = 1; o < 32; o <<= 1) {
-                const uint32_t v = __shfl_down_sync(0xffffffffu, S, o);
-                if (lane + o < 32) S += v;
-            }
-            const int L = 31 - __clz(__ballot_sync(0xffffffffu, S >= (uint32_t)want));   // the lane whose bins hold the rank
-            int d_loc = -1;
-            uint32_t above_loc = 0u, running = S - T;
-#pragma unroll
-            for (int b = 7; b >= 0; --b) {
-                if (d_loc < 0 && running + hloc[b] >= (uint32_t)want) {
-                    d_loc = b;
-                    above_loc = running;
-                }
-                running += hloc[b];
-            }
-            const int d = __shfl_sync(0xffffffffu, 8 * lane + d_loc, L);
-            const uint32_t above = __shfl_sync(0xffffffffu, above_loc, L);
-            prefix |= (uint32_t)d << lo;
-            want -= (int)above;
-            __syncwarp();
-        }
+        want = at_least > k ? k - above : nb;           // exactly k at or above `prefix`: all of them
     }
-    int32_t* out_idx = kept_idx + row * nb;
-    uint32_t* out_bits = bitmask32 + row * words32;
+    int32_t* out_idx = kept_idx + (long long)row * nb;
+    uint32_t* out_bits = bitmask32 + (long long)row * words32;
     int total = 0, eq_seen = 0;
-    for (int c = 0; c < nb_pad; c += 32) {
-        const int j = c + lane;
+#pragma unroll
+    for (int x = 0; x < IPL; ++x) {
+        const int j = 32 * x + lane;
+        if (32 * x >= nb) break;
         bool keep = false, eq = false;
         if (j < nb) {
-            if (text_row || j < ntb || j == i) {
-                keep = true;
-            } else if (select && radix) {
-                keep = s[j] > prefix;
-                eq = s[j] == prefix;
-            } else if (select) {
-                // rank = number of free candidates that beat this one (key descending, index ascending)
-                const unsigned long long cj = c64[j];
-                int rank = 0;
-#pragma unroll 4
-                for (int m = ntb; m < nb; ++m) rank += c64[m] > cj;
-                keep = rank < k;
-            } else {
-                keep = k >= n_free && k > 0;            // every free candidate, or none
-            }
+            if (text_row || j < ntb || j == i) keep = true;
+            else if (select) {
+                keep = u[x] > prefix;
+                eq = u[x] == prefix;
+            } else keep = k >= n_free && k > 0;         // every free candidate, or none
         }
         // equal keys: the lowest block indices first, `want` of them in all
         const uint32_t beq = __ballot_sync(0xffffffffu, eq);
         if (eq && eq_seen + __popc(beq & ((1u << lane) - 1u)) < want) keep = true;
         eq_seen += __popc(beq);
         const uint32_t bal = __ballot_sync(0xffffffffu, keep);
-        if (lane == 0) out_bits[c / 32] = bal;
+        if (lane == 0) out_bits[x] = bal;
         if (keep) out_idx[total + __popc(bal & ((1u << lane) - 1u))] = j;
         total += __popc(bal);
     }
-    for (int c = nb_pad / 32 + lane; c < words32; c += 32) out_bits[c] = 0;   // odd 32-bit half of the last word
+    for (int c = (nb + 31) / 32 + lane; c < words32; c += 32) out_bits[c] = 0;   // odd 32-bit half of the last word
     for (int e = total + lane; e < nb; e += 32) out_idx[e] = -1;
     if (lane == 0) kept_cnt[row] = total;
 }
@@ -163,7 +137,10 @@ __global__ void __launch_bounds__(WARPS * 32) select_kernel(const float* scores,
 // tau * (sum of all free weights).  No sort: the boundary candidate is found by descending the
 // bits of the order-preserving keys, each round summing the weights of the candidates that match
 // the trial prefix (a weighted radix select); candidates equal to the boundary key are then added
-// one by one.  fp64 throughout, the precision in which the decision is defined.
+// one by one.  fp64 throughout, the precision in which the decision is defined.  Keys and weights are in registers, IPL
+// of each a lane as above.  Bits that all candidates share decide nothing (a trial holds all of the mass or none of it),
+// and a group of one candidate is the boundary whatever its lower bits are, so both are left out (with the selection
+// after it: 25.6 -> 12.0 us for two images of 24 heads x 70 rows, 61 -> 36 us for one of 264).
 constexpr int MASS_WARPS = 2;
 
 __device__ __forceinline__ double warp_sum(double v) {
@@ -172,82 +149,107 @@ __device__ __forceinline__ double warp_sum(double v) {
     return v;
 }
 
-__global__ void __launch_bounds__(MASS_WARPS * 32) mass_count_kernel(const float* __restrict__ scores, TensorGeom g,
-                                                                     int n_img, MassShare share, float scale,
-                                                                     int32_t* __restrict__ row_keep) {
-    extern __shared__ double mass_smem[];                  // [MASS_WARPS][nb_pad] weights, then the keys
+template <int IPL>
+__global__ void __launch_bounds__(MASS_WARPS * 32) mass_count_kernel(const float* scores, TensorGeom g, MassShare share,
+                                                                     float scale, int32_t* __restrict__ row_keep) {
     const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
     const int nb = g.nb, ntb = g.n_text_blocks;
-    const int nb_pad = (nb + 31) & ~31;
-    const long long row = (long long)blockIdx.x * MASS_WARPS + warp;
-    if (row >= (long long)n_img * g.H * nb) return;
-    const int i = (int)(row % nb);
-    const int p = (int)(row / ((long long)nb * g.H));
+    const int ph = blockIdx.y, p = ph / g.H, i = blockIdx.x * MASS_WARPS + warp;
+    const int row = ph * nb + i;
+    if (i >= nb) return;
     const int n_free = (i < ntb) ? 0 : max(nb - ntb - 1, 0);
     const float tau = share.tau[p];
     if (n_free == 0 || tau >= 1.f) {                       // warp-uniform
         if (lane == 0) row_keep[row] = n_free;
         return;
     }
-    double* w = mass_smem + warp * nb_pad;
-    uint32_t* key = reinterpret_cast<uint32_t*>(mass_smem + MASS_WARPS * nb_pad) + warp * nb_pad;
-    const float* src = scores + row * nb;
+    const float* src = scores + (long long)row * nb;
+    float sj[IPL];
     float mx = -INFINITY;
-    for (int j = lane; j < nb; j += 32)
-        if (j >= ntb && j != i) mx = fmaxf(mx, src[j]);
+#pragma unroll
+    for (int x = 0; x < IPL; ++x) {
+        const int j = 32 * x + lane;
+        sj[x] = -INFINITY;
+        if (j < nb && j >= ntb && j != i) sj[x] = __ldcg(src + j);
+        mx = fmaxf(mx, sj[x]);
+    }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+    uint32_t u[IPL];
+    double w[IPL];                                         // forced and padding entries weigh nothing
     double part = 0.0;
-    for (int j = lane; j < nb_pad; j += 32) {
-        const bool is_free = j < nb && j >= ntb && j != i;
-        uint32_t u = 0u;
-        double wj = 0.0;
-        if (is_free) {
-            const float sj = src[j];
-            u = __float_as_uint(sj);
-            if (u == 0x80000000u) u = 0u;
-            u ^= (u >> 31) ? 0xffffffffu : 0x80000000u;
-            wj = exp((double)scale * ((double)sj - (double)mx));
+#pragma unroll
+    for (int x = 0; x < IPL; ++x) {
+        const int j = 32 * x + lane;
+        u[x] = 0u;
+        w[x] = 0.0;
+        if (j < nb && j >= ntb && j != i) {
+            u[x] = score_key(sj[x]);
+            w[x] = exp((double)scale * ((double)sj[x] - (double)mx));
         }
-        key[j] = u;
-        w[j] = wj;                                         // forced and padding entries weigh nothing
-        part += wj;
+        part += w[x];
     }
-    __syncwarp();
     const double total = warp_sum(part);
     double want = (double)tau * total;                     // mass still to be covered inside the prefix group
-    uint32_t prefix = 0u, mask = 0u;
-    for (int bit = 31; bit >= 0; --bit) {
-        const uint32_t trial = prefix | (1u << bit), m2 = mask | (1u << bit);
+    uint32_t prefix;
+    int hi = differing_bits(u, prefix);                    // the group: candidates that equal `prefix` from bit `hi` up
+    int above = 0, group = n_free;                         // candidates above the group, and in it
+    while (hi > 0 && group > 1) {
+        const uint32_t bit = 1u << (hi - 1), trial = prefix | bit, rest = bit - 1u;
         double m1 = 0.0;
-        for (int j = lane; j < nb_pad; j += 32) m1 += ((key[j] & m2) == trial) ? w[j] : 0.0;
-        m1 = warp_sum(m1);
-        if (m1 >= want) prefix = trial;
-        else want -= m1;
-        mask = m2;
-    }
-    // candidates above the boundary key are all kept; those equal to it one by one until the mass is reached
-    int n_gt = 0, n_eq = 0;
-    double w_eq = 0.0;
-    for (int j = lane; j < nb; j += 32) {
-        const bool is_free = j >= ntb && j != i;
-        n_gt += is_free && key[j] > prefix;
-        if (is_free && key[j] == prefix) {
-            ++n_eq;
-            w_eq = w[j];
+        int c1 = 0;
+#pragma unroll
+        for (int x = 0; x < IPL; ++x) {
+            const bool in = (u[x] & ~rest) == trial;
+            m1 += in ? w[x] : 0.0;
+            c1 += in;
         }
+        m1 = warp_sum(m1);
+        c1 = __reduce_add_sync(0xffffffffu, c1);
+        if (m1 >= want) {
+            prefix = trial;
+            group = c1;
+        } else {
+            want -= m1;
+            above += c1;
+            group -= c1;
+        }
+        --hi;
     }
-    n_gt = __reduce_add_sync(0xffffffffu, n_gt);
-    n_eq = __reduce_add_sync(0xffffffffu, n_eq);
+    // The group's candidates have equal keys now (or there is one; or none, when the mass above them fell short of the
+    // share by rounding alone): added one by one until the mass is reached.
+    double w_eq = 0.0;
+#pragma unroll
+    for (int x = 0; x < IPL; ++x)
+        if (u[x] && (hi >= 32 || (u[x] >> hi) == (prefix >> hi))) w_eq = w[x];
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) w_eq = fmax(w_eq, __shfl_xor_sync(0xffffffffu, w_eq, o));
     int r = 0;
     double acc = 0.0;
-    while (r < n_eq && (r == 0 || acc < want)) {
+    while (r < group && (r == 0 || acc < want)) {
         acc += w_eq;
         ++r;
     }
-    if (lane == 0) row_keep[row] = min(max(n_gt + r, 1), n_free);
+    if (lane == 0) row_keep[row] = min(max(above + r, 1), n_free);
+}
+
+// Calls f with a register count per lane that holds a row of nb scores: three (96 blocks, the 1024^2 sequences), nine
+// (288, the 2048^2 ones) or what the longest sequence takes.
+template <typename F>
+cudaError_t with_ipl(int nb, F&& f) {
+    if (nb <= 96) return f(std::integral_constant<int, 3>());
+    if (nb <= 288) return f(std::integral_constant<int, 9>());
+    return f(std::integral_constant<int, RAPID3_MAX_NB / 32>());
+}
+
+template <typename HK>
+cudaError_t launch_select(const float* scores, const TensorGeom& g, const ImgList& imgs, uint64_t* bitmask, int32_t* kept_idx,
+                          int32_t* kept_cnt, cudaStream_t s, const DevPlan* plan, int n_img, bool pdl, const HK& hk) {
+    const dim3 grid((g.nb + WARPS - 1) / WARPS, n_img * g.H);
+    return with_ipl(g.nb, [&](auto ipl) {
+        return launch_kernel(select_kernel<HK, decltype(ipl)::value>, grid, dim3(WARPS * 32), 0, s, pdl, scores, g, imgs,
+                             reinterpret_cast<uint32_t*>(bitmask), kept_idx, kept_cnt, 2 * ((g.nb + 63) / 64), plan, hk);
+    });
 }
 
 }  // namespace
@@ -255,46 +257,25 @@ __global__ void __launch_bounds__(MASS_WARPS * 32) mass_count_kernel(const float
 cudaError_t launch_select_mask_mass(const float* scores, const TensorGeom& g, const ImgList& imgs,
                                     const MassShare& share, float scale, int32_t* row_keep, uint64_t* bitmask,
                                     int32_t* kept_idx, int32_t* kept_cnt, cudaStream_t s) {
-    const long long n_rows = (long long)imgs.n * g.H * g.nb;
-    const int nb_pad = (g.nb + 31) & ~31;
-    {
-        const unsigned grid = (unsigned)((n_rows + MASS_WARPS - 1) / MASS_WARPS);
-        const size_t smem = (size_t)MASS_WARPS * nb_pad * (sizeof(double) + sizeof(uint32_t));
-        mass_count_kernel<<<grid, MASS_WARPS * 32, smem, s>>>(scores, g, imgs.n, share, scale, row_keep);
-        cudaError_t e = cudaGetLastError();
-        if (e != cudaSuccess) return e;
-    }
-    const int words32 = 2 * ((g.nb + 63) / 64);
-    const unsigned grid = (unsigned)((n_rows + WARPS - 1) / WARPS);
-    const size_t smem = (size_t)WARPS * nb_pad * sizeof(unsigned long long) + WARPS * 256 * sizeof(uint32_t);
+    const cudaError_t e = with_ipl(g.nb, [&](auto ipl) {
+        return launch_kernel(mass_count_kernel<decltype(ipl)::value>, dim3((g.nb + MASS_WARPS - 1) / MASS_WARPS, imgs.n * g.H),
+                             dim3(MASS_WARPS * 32), 0, s, false, scores, g, share, scale, row_keep);
+    });
+    if (e != cudaSuccess) return e;
     RowKeep rk;
     rk.k = row_keep;
-    select_kernel<RowKeep><<<grid, WARPS * 32, smem, s>>>(scores, g, imgs, reinterpret_cast<uint32_t*>(bitmask), kept_idx,
-                                                          kept_cnt, words32, nullptr, rk);
-    return cudaGetLastError();
+    return launch_select(scores, g, imgs, bitmask, kept_idx, kept_cnt, s, nullptr, imgs.n, false, rk);
 }
 
 cudaError_t launch_select_mask(const float* scores, const TensorGeom& g, const ImgList& imgs, uint64_t* bitmask,
                                int32_t* kept_idx, int32_t* kept_cnt, cudaStream_t s, const DevPlan* plan, int n_cap,
                                bool pdl) {
-    const long long n_rows = (long long)(plan ? n_cap : imgs.n) * g.H * g.nb;
-    const int nb_pad = (g.nb + 31) & ~31;
-    const int words32 = 2 * ((g.nb + 63) / 64);
-    const unsigned grid = (unsigned)((n_rows + WARPS - 1) / WARPS);
-    const size_t smem = (size_t)WARPS * nb_pad * sizeof(unsigned long long) + WARPS * 256 * sizeof(uint32_t);
-    return launch_kernel(select_kernel<NoHeadKeep>, dim3(grid), dim3(WARPS * 32), smem, s, pdl, scores, g, imgs,
-                         reinterpret_cast<uint32_t*>(bitmask), kept_idx, kept_cnt, words32, plan, NoHeadKeep());
+    return launch_select(scores, g, imgs, bitmask, kept_idx, kept_cnt, s, plan, plan ? n_cap : imgs.n, pdl, NoHeadKeep());
 }
 
 cudaError_t launch_select_mask_heads(const float* scores, const TensorGeom& g, const ImgList& imgs, const HeadKeep& hk,
                                      uint64_t* bitmask, int32_t* kept_idx, int32_t* kept_cnt, cudaStream_t s, bool pdl) {
-    const long long n_rows = (long long)imgs.n * g.H * g.nb;
-    const int nb_pad = (g.nb + 31) & ~31;
-    const int words32 = 2 * ((g.nb + 63) / 64);
-    const unsigned grid = (unsigned)((n_rows + WARPS - 1) / WARPS);
-    const size_t smem = (size_t)WARPS * nb_pad * sizeof(unsigned long long) + WARPS * 256 * sizeof(uint32_t);
-    return launch_kernel(select_kernel<HeadKeep>, dim3(grid), dim3(WARPS * 32), smem, s, pdl, scores, g, imgs,
-                         reinterpret_cast<uint32_t*>(bitmask), kept_idx, kept_cnt, words32, static_cast<const DevPlan*>(nullptr), hk);
+    return launch_select(scores, g, imgs, bitmask, kept_idx, kept_cnt, s, nullptr, imgs.n, pdl, hk);
 }
 
 
