@@ -454,7 +454,7 @@ static int gated_step_impl(rapid3_ctx* c, const void* q, const void* k, const vo
             ProfScope ps(c, PROF_SELECT, st);
             const cudaError_t e =
                 mass_scale ? launch_select_mask_mass(c->scores, g, sparse, share, *mass_scale, c->row_keep, c->bitmask,
-                                                     c->kept_idx, c->kept_cnt, st)
+                                                     c->kept_idx, c->kept_cnt, st, true)
                 : per_head ? launch_select_mask_heads(c->scores, g, sparse, hk, c->bitmask, c->kept_idx, c->kept_cnt, st, true)
                            : launch_select_mask(c->scores, g, sparse, c->bitmask, c->kept_idx, c->kept_cnt, st, nullptr, 0, true);
             if (e != cudaSuccess) return RAPID3_ERR_CUDA;
@@ -462,7 +462,7 @@ static int gated_step_impl(rapid3_ctx* c, const void* q, const void* k, const vo
         c->launches += mass_scale ? 3 : 2;
     }
     return attn_launch(c, g, q, k, v, out, all, sparse.n ? c->kept_idx : nullptr, sparse.n ? c->kept_cnt : nullptr,
-                       sparse.n ? c->bitmask : nullptr, softmax_scale, st, nullptr, 0, sparse.n > 0 && !mass_scale);
+                       sparse.n ? c->bitmask : nullptr, softmax_scale, st, nullptr, 0, sparse.n > 0);
 }
 
 int rapid3_gated_step(rapid3_ctx* c, const void* q, const void* k, const void* v, void* out,
@@ -523,15 +523,15 @@ int rapid3_gated_step_device(rapid3_ctx* c, const void* q, const void* k, const 
     }
     {
         ProfScope ps(c, PROF_SCORES, st);
-        if (launch_block_scores(c->pooled, c->g, B, c->scores, st, c->plan) != cudaSuccess) return RAPID3_ERR_CUDA;
+        if (launch_block_scores(c->pooled, c->g, B, c->scores, st, c->plan, true) != cudaSuccess) return RAPID3_ERR_CUDA;
     }
     {
         ProfScope ps(c, PROF_SELECT, st);
-        if (launch_select_mask(c->scores, c->g, none, c->bitmask, c->kept_idx, c->kept_cnt, st, c->plan, B) != cudaSuccess)
+        if (launch_select_mask(c->scores, c->g, none, c->bitmask, c->kept_idx, c->kept_cnt, st, c->plan, B, true) != cudaSuccess)
             return RAPID3_ERR_CUDA;
     }
     c->launches += 4;
-    return attn_launch(c, c->g, q, k, v, out, none, c->kept_idx, c->kept_cnt, c->bitmask, softmax_scale, st, c->plan, B);
+    return attn_launch(c, c->g, q, k, v, out, none, c->kept_idx, c->kept_cnt, c->bitmask, softmax_scale, st, c->plan, B, true);
 }
 
 int rapid3_gated_step_host(rapid3_ctx* c, const void* q_host, const void* k_host, const void* v_host, void* out_host,

@@ -59,8 +59,11 @@ struct TensorGeom {
 };
 
 // Programmatic dependent launch: a kernel launched with `pdl` set may start while the kernel before it in the stream
-// is still running, and must call grid_dependency_wait() before it touches anything that kernel writes; the kernel
-// before it calls grid_dependency_launch() to let it start.  Both are no-ops in an ordinary launch.
+// is still running, and must call grid_dependency_wait() before it touches anything that kernel writes (and read it past
+// the L1, whose lines the wait is not known to refresh); the kernel before it calls grid_dependency_launch() to let it
+// start.  Both are no-ops in an ordinary launch.  Every kernel here waits before it lets the next one start: when a kernel
+// runs, all kernels but the one right before it have ended -- so the attention kernel's thread blocks that need nothing
+// of the selection may run beside it, and find Q, K and V of whatever kernel came before the call.
 #ifdef __CUDACC__
 __device__ __forceinline__ void grid_dependency_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void grid_dependency_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
@@ -103,7 +106,7 @@ cudaError_t launch_select_mask_heads(const float* scores, const TensorGeom& g, c
 // at that count.
 cudaError_t launch_select_mask_mass(const float* scores, const TensorGeom& g, const ImgList& imgs,
                                     const MassShare& share, float scale, int32_t* row_keep, uint64_t* bitmask,
-                                    int32_t* kept_idx, int32_t* kept_cnt, cudaStream_t s);
+                                    int32_t* kept_idx, int32_t* kept_cnt, cudaStream_t s, bool pdl = false);   // after the scores kernel
 // K5: Q/K producer (RMS norm + gain + rotary embedding -> bf16) that also writes the block means of
 // the images with a workspace slot.  pooled is [2][n_sparse][H][nb][D].
 struct PrepArgs {

@@ -17,20 +17,21 @@ __device__ __forceinline__ float bf16_hi(uint32_t w) { return __uint_as_float(w 
 // one another: that keeps the kernel under 85 registers, six thread blocks per SM (measured 29 against 40 us on the
 // FLUX 1024^2 shapes, where 125 registers left four).
 template <int D>
-__global__ void __launch_bounds__(128, 6) pool_kernel(const uint16_t* __restrict__ q, const uint16_t* __restrict__ k,
+__global__ void __launch_bounds__(128, 6) pool_kernel(const uint16_t* q, const uint16_t* k,
                                                    TensorGeom g, ImgList imgs, double* __restrict__ pooled,
-                                                   const DevPlan* __restrict__ plan, int n_cap) {
+                                                   const DevPlan* plan, int n_cap) {
     constexpr int TPR = D / 8;          // lanes per token row (8 channels = 16 bytes each)
     constexpr int RPL = 32 / TPR;       // rows per warp-wide load
     constexpr int ITERS = 64 / RPL;     // loads per lane
     const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
     const int blk = blockIdx.x * 4 + warp, h = blockIdx.y;
-    grid_dependency_launch();                         // the scores kernel may be staged; it waits for this grid's end itself
+    grid_dependency_wait();                           // first kernel of a call: what comes before it may still be running
+    grid_dependency_launch();
     if (blk >= g.nb) return;
     const int which = blockIdx.z / n_cap;             // 0 = Q, 1 = K
     const int p = blockIdx.z - which * n_cap;
-    if (plan && p >= plan->sparse.n) return;          // device-resident plan: fewer images than the grid covers
-    const int batch = plan ? plan->sparse.batch[p] : imgs.batch[p];
+    if (plan && p >= __ldcg(&plan->sparse.n)) return;  // device-resident plan: fewer images than the grid covers
+    const int batch = plan ? __ldcg(&plan->sparse.batch[p]) : imgs.batch[p];
     const uint16_t* base = (which ? k : q) + (long long)batch * g.stride_b + (long long)(g.h0 + h) * g.stride_h;
     const int c = lane % TPR, r0 = lane / TPR;
     const int n0 = blk * 64;
@@ -47,7 +48,7 @@ __global__ void __launch_bounds__(128, 6) pool_kernel(const uint16_t* __restrict
             const int row = (it0 + u) * RPL + r0;
             v[u] = make_uint4(0, 0, 0, 0);
             if (row < valid)
-                v[u] = __ldg(reinterpret_cast<const uint4*>(base + (long long)(n0 + row) * g.stride_n + c * 8));
+                v[u] = __ldcg(reinterpret_cast<const uint4*>(base + (long long)(n0 + row) * g.stride_n + c * 8));
         }
 #pragma unroll
         for (int u = 0; u < 8; ++u) {
@@ -94,11 +95,9 @@ __global__ void __launch_bounds__(256) scores_kernel(const double* pooled, Tenso
     __shared__ double sq[T][LDS];
     __shared__ double sk[T][LDS];
     const int ph = blockIdx.z;                       // p * H + h
-    grid_dependency_launch();
-    // The block means come from the kernel before, which may still be running when this one starts: wait for its end,
-    // and read them past the L1 (ld.global.cg), whose lines no such wait is known to refresh.
     grid_dependency_wait();
-    if (plan && ph >= plan->sparse.n * g.H) return;
+    grid_dependency_launch();
+    if (plan && ph >= __ldcg(&plan->sparse.n) * g.H) return;
     const int i0 = blockIdx.y * T, j0 = blockIdx.x * T;
     const double* pq = pooled + (long long)ph * g.nb * g.D;
     const double* pk = pooled + ((long long)n_img * g.H + ph) * g.nb * g.D;
@@ -160,11 +159,8 @@ cudaError_t launch_block_pool(const void* q, const void* k, const TensorGeom& g,
                               double* pooled, cudaStream_t s, const DevPlan* plan, int n_cap) {
     if (!plan) n_cap = imgs.n;
     dim3 grid((g.nb + 3) / 4, g.H, 2 * n_cap);
-    if (g.D == 128)
-        pool_kernel<128><<<grid, 128, 0, s>>>((const uint16_t*)q, (const uint16_t*)k, g, imgs, pooled, plan, n_cap);
-    else
-        pool_kernel<64><<<grid, 128, 0, s>>>((const uint16_t*)q, (const uint16_t*)k, g, imgs, pooled, plan, n_cap);
-    return cudaGetLastError();
+    return launch_kernel(g.D == 128 ? pool_kernel<128> : pool_kernel<64>, grid, dim3(128), 0, s, true,
+                         static_cast<const uint16_t*>(q), static_cast<const uint16_t*>(k), g, imgs, pooled, plan, n_cap);
 }
 
 cudaError_t launch_block_scores(const double* pooled, const TensorGeom& g, int n_img, float* scores,

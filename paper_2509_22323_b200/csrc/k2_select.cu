@@ -49,21 +49,21 @@ __global__ void __launch_bounds__(WARPS * 32) select_kernel(const float* scores,
                                                             ImgList imgs, uint32_t* __restrict__ bitmask32,
                                                             int32_t* __restrict__ kept_idx,
                                                             int32_t* __restrict__ kept_cnt, int words32,
-                                                            const DevPlan* __restrict__ plan, const HK hk) {
+                                                            const DevPlan* plan, const HK hk) {
     const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
     const int nb = g.nb, ntb = g.n_text_blocks;
     const int ph = blockIdx.y, p = ph / g.H;            // p * H + h
     const int i = blockIdx.x * WARPS + warp;
     const int row = ph * nb + i;                        // at most 65535 x 1024
-    grid_dependency_launch();
     grid_dependency_wait();                             // the scores come from the kernel before, which may still be running
-    if (i >= nb || (plan && p >= plan->sparse.n)) return;
+    grid_dependency_launch();
+    if (i >= nb || (plan && p >= __ldcg(&plan->sparse.n))) return;
     // free candidates kept in this row: one count per image, or per (image, head) when the policy
     // sets a ratio for every head
     int k;
     if constexpr (HK::mode == 1) k = hk.k[ph];
     else if constexpr (HK::mode == 2) k = __ldcg(hk.k + row);
-    else k = plan ? plan->sparse.k_free[p] : imgs.k_free[p];
+    else k = plan ? __ldcg(&plan->sparse.k_free[p]) : imgs.k_free[p];
     const float* src = scores + (long long)row * nb;
     const bool text_row = i < ntb;
     const int n_free = max(nb - ntb - ((i >= ntb) ? 1 : 0), 0);
@@ -156,6 +156,8 @@ __global__ void __launch_bounds__(MASS_WARPS * 32) mass_count_kernel(const float
     const int nb = g.nb, ntb = g.n_text_blocks;
     const int ph = blockIdx.y, p = ph / g.H, i = blockIdx.x * MASS_WARPS + warp;
     const int row = ph * nb + i;
+    grid_dependency_wait();                                // for the scores
+    grid_dependency_launch();
     if (i >= nb) return;
     const int n_free = (i < ntb) ? 0 : max(nb - ntb - 1, 0);
     const float tau = share.tau[p];
@@ -256,15 +258,15 @@ cudaError_t launch_select(const float* scores, const TensorGeom& g, const ImgLis
 
 cudaError_t launch_select_mask_mass(const float* scores, const TensorGeom& g, const ImgList& imgs,
                                     const MassShare& share, float scale, int32_t* row_keep, uint64_t* bitmask,
-                                    int32_t* kept_idx, int32_t* kept_cnt, cudaStream_t s) {
+                                    int32_t* kept_idx, int32_t* kept_cnt, cudaStream_t s, bool pdl) {
     const cudaError_t e = with_ipl(g.nb, [&](auto ipl) {
         return launch_kernel(mass_count_kernel<decltype(ipl)::value>, dim3((g.nb + MASS_WARPS - 1) / MASS_WARPS, imgs.n * g.H),
-                             dim3(MASS_WARPS * 32), 0, s, false, scores, g, share, scale, row_keep);
+                             dim3(MASS_WARPS * 32), 0, s, pdl, scores, g, share, scale, row_keep);
     });
     if (e != cudaSuccess) return e;
     RowKeep rk;
     rk.k = row_keep;
-    return launch_select(scores, g, imgs, bitmask, kept_idx, kept_cnt, s, nullptr, imgs.n, false, rk);
+    return launch_select(scores, g, imgs, bitmask, kept_idx, kept_cnt, s, nullptr, imgs.n, true, rk);
 }
 
 cudaError_t launch_select_mask(const float* scores, const TensorGeom& g, const ImgList& imgs, uint64_t* bitmask,
@@ -284,8 +286,10 @@ cudaError_t launch_select_mask_heads(const float* scores, const TensorGeom& g, c
 // entry point does on the CPU, for callers whose sampled actions never leave the GPU.
 namespace {
 
-__global__ void plan_kernel(const int32_t* __restrict__ action, const float* __restrict__ ratio, int B, int n_free_img,
+__global__ void plan_kernel(const int32_t* action, const float* ratio, int B, int n_free_img,
                             DevPlan* __restrict__ plan, int* __restrict__ status) {
+    grid_dependency_wait();                           // first kernel of a call
+    grid_dependency_launch();
     if (threadIdx.x != 0 || blockIdx.x != 0) return;
     ImgList& sp = plan->sparse;
     ImgList& al = plan->all;
@@ -294,13 +298,13 @@ __global__ void plan_kernel(const int32_t* __restrict__ action, const float* __r
     int n_dense = 0;
     float ratio_of[RAPID3_MAX_IMG];
     for (int b = 0; b < B; ++b) {
-        const int a = action[b];
+        const int a = __ldcg(action + b);
         if (a != RAPID3_ACT_SKIP && a != RAPID3_ACT_REUSE && a != RAPID3_ACT_ATTEND) {
             atomicExch(status, RAPID3_ERR_INVALID_ARG);       // unknown action: treated as a skip
             continue;
         }
         if (a != RAPID3_ACT_ATTEND) continue;
-        const float r = ratio[b];
+        const float r = __ldcg(ratio + b);
         if (!(r > 0.f) || !(r <= 1.f)) {
             atomicExch(status, RAPID3_ERR_INVALID_ARG);       // ratio outside (0, 1]: image not processed
             continue;
@@ -336,6 +340,6 @@ __global__ void plan_kernel(const int32_t* __restrict__ action, const float* __r
 cudaError_t launch_plan(const int32_t* action_dev, const float* ratio_dev, int B, const TensorGeom& g, DevPlan* plan,
                         int* status, cudaStream_t s) {
     const int n_free_img = g.nb - g.n_text_blocks - 1;
-    plan_kernel<<<1, 32, 0, s>>>(action_dev, ratio_dev, B, n_free_img > 0 ? n_free_img : 0, plan, status);
-    return cudaGetLastError();
+    return launch_kernel(plan_kernel, dim3(1), dim3(32), 0, s, true, action_dev, ratio_dev, B, n_free_img > 0 ? n_free_img : 0,
+                         plan, status);
 }

@@ -168,7 +168,7 @@ attn_kernel(const __grid_constant__ CUtensorMap tmq, const __grid_constant__ CUt
     const int warp = __shfl_sync(0xffffffffu, tid / 32, 0);
     const TensorGeom& g = prm.g;
     const int nb = g.nb, N = g.N;
-    const int n_quads = ((nb + 3) >> 2) * g.H * (prm.plan ? prm.plan->all.n : prm.imgs.n);
+    const int n_quads = ((nb + 3) >> 2) * g.H * (prm.plan ? __ldcg(&prm.plan->all.n) : prm.imgs.n);
     if ((int)blockIdx.x >= n_quads) return;              // device-resident plan: fewer images than the grid covers
 
     const uint32_t bQ = smem_u32(&ctl->q_full), bQE = smem_u32(&ctl->q_empty);
@@ -292,8 +292,8 @@ attn_kernel(const __grid_constant__ CUtensorMap tmq, const __grid_constant__ CUt
             int quad, h, p;
             {
                 const int nq = (nb + 3) >> 2, ntq = min(nq, (g.n_text_blocks + 3) >> 2);
-                const int n_all = prm.plan ? prm.plan->all.n : prm.imgs.n;
-                const int nd = prm.plan ? prm.plan->n_dense : prm.n_dense, ns = n_all - nd;
+                const int n_all = prm.plan ? __ldcg(&prm.plan->all.n) : prm.imgs.n;
+                const int nd = prm.plan ? __ldcg(&prm.plan->n_dense) : prm.n_dense, ns = n_all - nd;
                 const int heavy_dense = nd * g.H * nq, heavy_sparse = ns * g.H * ntq;
                 if (L < heavy_dense) {
                     p = L / (g.H * nq); L -= p * g.H * nq;
@@ -309,8 +309,8 @@ attn_kernel(const __grid_constant__ CUtensorMap tmq, const __grid_constant__ CUt
                     h = L / nl; quad = ntq + (L - h * nl);
                 }
             }
-            const int b = prm.plan ? prm.plan->all.batch[p] : prm.imgs.batch[p];
-            const int slot = prm.plan ? prm.plan->all.slot[p] : prm.imgs.slot[p];
+            const int b = prm.plan ? __ldcg(&prm.plan->all.batch[p]) : prm.imgs.batch[p];
+            const int slot = prm.plan ? __ldcg(&prm.plan->all.slot[p]) : prm.imgs.slot[p];
             // Which two of the quad's four query blocks form a 128-row tile: neighbours, or, when a row of the image
             // grid spans two blocks (pair_stride 2), vertical neighbours (i, i + 2), whose kept lists overlap far more
             // (measured on the 128 x 128 grid at keep ratio 0.25: 90 % against 63 % of the tile's MMA work lands on

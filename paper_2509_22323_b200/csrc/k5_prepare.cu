@@ -28,11 +28,10 @@ __device__ __forceinline__ uint32_t pack2(float lo, float hi) {
 }
 
 template <int D>
-__global__ void __launch_bounds__(128, PREP_MINB) prepare_kernel(const uint16_t* __restrict__ q_raw,
-                                                      const uint16_t* __restrict__ k_raw, uint16_t* q_out,
-                                                      uint16_t* k_out, const float* __restrict__ q_gain,
-                                                      const float* __restrict__ k_gain,
-                                                      const float* __restrict__ rot, float eps, TensorGeom g,
+__global__ void __launch_bounds__(128, PREP_MINB) prepare_kernel(const uint16_t* q_raw,
+                                                      const uint16_t* k_raw, uint16_t* q_out,
+                                                      uint16_t* k_out, const float* q_gain,
+                                                      const float* k_gain, const float* rot, float eps, TensorGeom g,
                                                       ImgList imgs, int n_sparse, double* __restrict__ pooled) {
     constexpr int TPR = D / 8;          // lanes per token row (8 channels = 16 bytes each)
     constexpr int RPL = 32 / TPR;       // rows per warp-wide load
@@ -40,6 +39,8 @@ __global__ void __launch_bounds__(128, PREP_MINB) prepare_kernel(const uint16_t*
     constexpr int INFL = PREP_INFL;     // rows in flight per lane
     const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
     const int blk = blockIdx.x * 4 + warp, h = blockIdx.y;
+    grid_dependency_wait();                           // first kernel of a call: what comes before it may still be running
+    grid_dependency_launch();
     if (blk >= g.nb) return;
     const int which = blockIdx.z / imgs.n;            // 0 = Q, 1 = K
     const int p = blockIdx.z - which * imgs.n;
@@ -54,8 +55,8 @@ __global__ void __launch_bounds__(128, PREP_MINB) prepare_kernel(const uint16_t*
 
     float gn[8];
     {
-        const float4 g0 = __ldg(reinterpret_cast<const float4*>(gain + c * 8));
-        const float4 g1 = __ldg(reinterpret_cast<const float4*>(gain + c * 8 + 4));
+        const float4 g0 = __ldcg(reinterpret_cast<const float4*>(gain + c * 8));
+        const float4 g1 = __ldcg(reinterpret_cast<const float4*>(gain + c * 8 + 4));
         gn[0] = g0.x; gn[1] = g0.y; gn[2] = g0.z; gn[3] = g0.w;
         gn[4] = g1.x; gn[5] = g1.y; gn[6] = g1.z; gn[7] = g1.w;
     }
@@ -73,11 +74,11 @@ __global__ void __launch_bounds__(128, PREP_MINB) prepare_kernel(const uint16_t*
             cs[u][0] = make_float4(1.f, 0.f, 1.f, 0.f);
             cs[u][1] = make_float4(1.f, 0.f, 1.f, 0.f);
             if (row < valid) {
-                v[u] = __ldg(reinterpret_cast<const uint4*>(src + (long long)(n0 + row) * g.stride_n + c * 8));
+                v[u] = __ldcg(reinterpret_cast<const uint4*>(src + (long long)(n0 + row) * g.stride_n + c * 8));
                 if (rot) {
                     const float4* rp = reinterpret_cast<const float4*>(rot + ((long long)(n0 + row) * (D / 2) + c * 4) * 2);
-                    cs[u][0] = __ldg(rp);
-                    cs[u][1] = __ldg(rp + 1);
+                    cs[u][0] = __ldcg(rp);
+                    cs[u][1] = __ldcg(rp + 1);
                 }
             }
         }
@@ -138,9 +139,6 @@ cudaError_t launch_prepare(const PrepArgs& a, const TensorGeom& g, const ImgList
     const uint16_t* kr = static_cast<const uint16_t*>(a.k_raw);
     uint16_t* qo = static_cast<uint16_t*>(a.q_out);
     uint16_t* ko = static_cast<uint16_t*>(a.k_out);
-    if (g.D == 128)
-        prepare_kernel<128><<<grid, 128, 0, s>>>(qr, kr, qo, ko, a.q_gain, a.k_gain, a.rot, a.eps, g, imgs, n_sparse, pooled);
-    else
-        prepare_kernel<64><<<grid, 128, 0, s>>>(qr, kr, qo, ko, a.q_gain, a.k_gain, a.rot, a.eps, g, imgs, n_sparse, pooled);
-    return cudaGetLastError();
+    return launch_kernel(g.D == 128 ? prepare_kernel<128> : prepare_kernel<64>, grid, dim3(128), 0, s, true, qr, kr, qo, ko, a.q_gain,
+                         a.k_gain, a.rot, a.eps, g, imgs, n_sparse, pooled);
 }
