@@ -68,20 +68,32 @@ struct TensorGeom {
 __device__ __forceinline__ void grid_dependency_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void grid_dependency_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
+// `carveout`: percentage of the SM's first-level memory that the launch prefers as shared memory, -1 for the default.
 template <typename... KArgs, typename... Args>
-inline cudaError_t launch_kernel(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, bool pdl,
-                                 Args&&... args) {
+inline cudaError_t launch_kernel_carveout(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, bool pdl,
+                                          int carveout, Args&&... args) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = grid;
     cfg.blockDim = block;
     cfg.dynamicSmemBytes = smem;
     cfg.stream = s;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchAttribute attr[2];
     cfg.attrs = attr;
-    cfg.numAttrs = pdl ? 1 : 0;
+    cfg.numAttrs = 0;
+    if (pdl) {
+        attr[cfg.numAttrs].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        attr[cfg.numAttrs++].val.programmaticStreamSerializationAllowed = 1;
+    }
+    if (carveout >= 0) {
+        attr[cfg.numAttrs].id = cudaLaunchAttributePreferredSharedMemoryCarveout;
+        attr[cfg.numAttrs++].val.sharedMemCarveout = (unsigned)carveout;
+    }
     return cudaLaunchKernelEx(&cfg, kernel, static_cast<KArgs>(args)...);
+}
+template <typename... KArgs, typename... Args>
+inline cudaError_t launch_kernel(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, bool pdl,
+                                 Args&&... args) {
+    return launch_kernel_carveout(kernel, grid, block, smem, s, pdl, -1, static_cast<Args&&>(args)...);
 }
 #endif
 
@@ -132,4 +144,6 @@ cudaError_t launch_attention(const CUtensorMap& tmq, const CUtensorMap& tmk, con
                              const int32_t* kept_cnt, const uint64_t* bitmask, float softmax_scale, int* status,
                              cudaStream_t s, const DevPlan* plan = nullptr, int n_cap = 0, int inject_stop_group = -1,
                              int pdl = 0);   // 1: after the selection kernel, whose masks only the sparse images' thread blocks read
+// Kernel attributes on the current device; set when a context is created (scoring: also by the context-free entry).
 cudaError_t attention_static_init();
+cudaError_t scoring_static_init();

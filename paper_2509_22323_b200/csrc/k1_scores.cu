@@ -81,77 +81,73 @@ __device__ __forceinline__ void dmma_8x8x4(double& c0, double& c1, double a, dou
                  : "d"(a), "d"(b));
 }
 
-// T x T tile of S per CTA (T = 32; a multiple of 32), eight warps; a warp owns (T / 32) x (T / 16) fragments of 8 x 8 outputs.
-// D goes through shared memory in chunks of 32 channels (row stride 36 doubles: the fragment loads then touch every
-// bank pair twice, the minimum for 32 eight-byte lanes); the next chunk is fetched into registers while the
-// current one is multiplied.  Every output accumulates its products in ascending order of the four-channel groups.
-template <int T>
+__device__ __forceinline__ void copy16_async(double* dst, const double* src, bool valid) {   // past the L1; zeros if not valid
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;"
+                 ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src), "r"(valid ? 16 : 0)
+                 : "memory");
+}
+
+// 32 x 32 tile of S per thread block, eight warps; a warp owns two fragments of 8 x 8 outputs side by side.  The two
+// operands (32 block means each) are copied to shared memory as a whole, the first half of the channels as one group of
+// asynchronous copies and the second as another: a thread block has little else to do than to wait for them, and one
+// round trip is what that costs (chunks of 32 channels through registers cost one each: 28.6 -> 24 us at 264 blocks).
+// Rows are padded to D + 4 doubles: the fragment loads then touch every bank pair twice, the minimum for 32 eight-byte
+// lanes.  Every output accumulates its products in ascending order of the four-channel groups.
+template <int D>
 __global__ void __launch_bounds__(256) scores_kernel(const double* pooled, TensorGeom g, int n_img,
-                                                     float* __restrict__ scores, const DevPlan* __restrict__ plan) {
-    constexpr int NI = T / 32;           // 8-row fragments per warp
-    constexpr int NJ = T / 16;           // 8-column fragments per warp
-    constexpr int LD = T * 32 / 256;     // values a thread stages per operand and chunk
-    constexpr int LDS = 36;              // row stride of the staged chunks in doubles
-    __shared__ double sq[T][LDS];
-    __shared__ double sk[T][LDS];
+                                                     float* __restrict__ scores, const DevPlan* plan) {
+    constexpr int T = 32, LDS = D + 4;
+    extern __shared__ __align__(16) double tiles[];
+    double* sq = tiles;
+    double* sk = tiles + T * LDS;
     const int ph = blockIdx.z;                       // p * H + h
+    // The block means come from the kernel before, which may still be running when this one starts: wait for its end,
+    // and read them past the L1, whose lines no such wait is known to refresh.
     grid_dependency_wait();
     grid_dependency_launch();
     if (plan && ph >= __ldcg(&plan->sparse.n) * g.H) return;
     const int i0 = blockIdx.y * T, j0 = blockIdx.x * T;
-    const double* pq = pooled + (long long)ph * g.nb * g.D;
-    const double* pk = pooled + ((long long)n_img * g.H + ph) * g.nb * g.D;
+    const double* pq = pooled + ((long long)ph * g.nb + i0) * D;
+    const double* pk = pooled + (((long long)n_img * g.H + ph) * g.nb + j0) * D;
+#pragma unroll
+    for (int half = 0; half < 2; ++half) {
+#pragma unroll
+        for (int x = 0; x < T * D / 4 / 256; ++x) {
+            const int e = threadIdx.x + 256 * x, r = e / (D / 4), c = half * (D / 2) + 2 * (e % (D / 4));
+            const bool vq = i0 + r < g.nb, vk = j0 + r < g.nb;
+            copy16_async(sq + r * LDS + c, vq ? pq + r * D + c : pooled, vq);
+            copy16_async(sk + r * LDS + c, vk ? pk + r * D + c : pooled, vk);
+        }
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    }
     const int warp = threadIdx.x / 32, lane = threadIdx.x % 32, gr = lane >> 2, c = lane & 3;
-    const int ri = (warp >> 1) * (8 * NI), cj = (warp & 1) * (8 * NJ);   // the warp's corner inside the tile
-    double acc[NI][NJ][2];
+    const int ri = (warp >> 1) * 8, cj = (warp & 1) * 16;                // the warp's corner inside the tile
+    const double* aq = sq + (ri + gr) * LDS + c;
+    const double* bk = sk + (cj + gr) * LDS + c;
+    double acc[2][2] = {{0.0, 0.0}, {0.0, 0.0}};
 #pragma unroll
-    for (int a = 0; a < NI; ++a)
-#pragma unroll
-        for (int b = 0; b < NJ; ++b) acc[a][b][0] = acc[a][b][1] = 0.0;
-    double rq[LD], rk[LD];
-    auto fetch = [&](int d0) {
-#pragma unroll
-        for (int u = 0; u < LD; ++u) {
-            const int e = threadIdx.x + u * 256, r = e / 32, cc = e % 32;
-            rq[u] = (i0 + r < g.nb) ? __ldcg(pq + (long long)(i0 + r) * g.D + d0 + cc) : 0.0;
-            rk[u] = (j0 + r < g.nb) ? __ldcg(pk + (long long)(j0 + r) * g.D + d0 + cc) : 0.0;
-        }
-    };
-    fetch(0);
-    for (int d0 = 0; d0 < g.D; d0 += 32) {
-#pragma unroll
-        for (int u = 0; u < LD; ++u) {
-            const int e = threadIdx.x + u * 256, r = e / 32, cc = e % 32;
-            sq[r][cc] = rq[u];
-            sk[r][cc] = rk[u];
-        }
+    for (int half = 0; half < 2; ++half) {
+        if (half == 0) asm volatile("cp.async.wait_group 1;" ::: "memory");
+        else asm volatile("cp.async.wait_group 0;" ::: "memory");
         __syncthreads();
-        if (d0 + 32 < g.D) fetch(d0 + 32);
-#pragma unroll
-        for (int d = 0; d < 32; d += 4) {
-            double qa[NI], kb[NJ];
-#pragma unroll
-            for (int a = 0; a < NI; ++a) qa[a] = sq[ri + 8 * a + gr][d + c];
-#pragma unroll
-            for (int b = 0; b < NJ; ++b) kb[b] = sk[cj + 8 * b + gr][d + c];
-#pragma unroll
-            for (int a = 0; a < NI; ++a)
-#pragma unroll
-                for (int b = 0; b < NJ; ++b) dmma_8x8x4(acc[a][b][0], acc[a][b][1], qa[a], kb[b]);
+#pragma unroll 8
+        for (int d = half * (D / 2); d < (half + 1) * (D / 2); d += 4) {
+            const double a = aq[d];
+            dmma_8x8x4(acc[0][0], acc[0][1], a, bk[d]);
+            dmma_8x8x4(acc[1][0], acc[1][1], a, bk[8 * LDS + d]);
         }
-        __syncthreads();
     }
     float* so = scores + (long long)ph * g.nb * g.nb;
 #pragma unroll
-    for (int a = 0; a < NI; ++a)
+    for (int b = 0; b < 2; ++b)
 #pragma unroll
-        for (int b = 0; b < NJ; ++b)
-#pragma unroll
-            for (int e = 0; e < 2; ++e) {
-                const int i = i0 + ri + 8 * a + gr, j = j0 + cj + 8 * b + 2 * c + e;
-                if (i < g.nb && j < g.nb) so[(long long)i * g.nb + j] = (float)acc[a][b][e];
-            }
+        for (int e = 0; e < 2; ++e) {
+            const int i = i0 + ri + gr, j = j0 + cj + 8 * b + 2 * c + e;
+            if (i < g.nb && j < g.nb) so[(long long)i * g.nb + j] = (float)acc[b][e];
+        }
 }
+
+constexpr int scores_smem_bytes(int D) { return 2 * 32 * (D + 4) * (int)sizeof(double); }
 
 }  // namespace
 
@@ -159,16 +155,29 @@ cudaError_t launch_block_pool(const void* q, const void* k, const TensorGeom& g,
                               double* pooled, cudaStream_t s, const DevPlan* plan, int n_cap) {
     if (!plan) n_cap = imgs.n;
     dim3 grid((g.nb + 3) / 4, g.H, 2 * n_cap);
-    return launch_kernel(g.D == 128 ? pool_kernel<128> : pool_kernel<64>, grid, dim3(128), 0, s, true,
-                         static_cast<const uint16_t*>(q), static_cast<const uint16_t*>(k), g, imgs, pooled, plan, n_cap);
+    // Small inputs ask for the shared-memory split that the attention kernel needs, so that the SMs need not be drained and
+    // split anew between the kernels of the step; that takes the loads' L1 away, which costs large inputs more (17 MB:
+    // 47.3 -> 44.3 us a step; 27 MB: 265.0 -> 265.8, 54 MB: 204.3 -> 205.8, 208 MB: 999 -> 1003).
+    const long long bytes = 4ll * n_cap * g.H * g.N * g.D;
+    const int carveout = bytes <= (20ll << 20) ? (int)cudaSharedmemCarveoutMaxShared : -1;
+    return launch_kernel_carveout(g.D == 128 ? pool_kernel<128> : pool_kernel<64>, grid, dim3(128), 0, s, true, carveout,
+                                  static_cast<const uint16_t*>(q), static_cast<const uint16_t*>(k), g, imgs, pooled, plan,
+                                  n_cap);
 }
 
 cudaError_t launch_block_scores(const double* pooled, const TensorGeom& g, int n_img, float* scores,
                                 cudaStream_t s, const DevPlan* plan, bool pdl) {
     // with a plan n_img is the capacity.  32 x 32 tiles at every length: against 64 x 64 tiles they waste less of
     // the ragged edge and fill the SMs more evenly (30 against 35 us at 264 blocks, where 64 x 64 pads 264 to 320)
-    dim3 grid((g.nb + 31) / 32, (g.nb + 31) / 32, n_img * g.H);
-    return launch_kernel(scores_kernel<32>, grid, dim3(256), 0, s, pdl, pooled, g, n_img, scores, plan);
+    const dim3 grid((g.nb + 31) / 32, (g.nb + 31) / 32, n_img * g.H);
+    return launch_kernel(g.D == 128 ? scores_kernel<128> : scores_kernel<64>, grid, dim3(256), scores_smem_bytes(g.D), s, pdl,
+                         pooled, g, n_img, scores, plan);
+}
+
+cudaError_t scoring_static_init() {
+    const cudaError_t e = cudaFuncSetAttribute(scores_kernel<128>, cudaFuncAttributeMaxDynamicSharedMemorySize, scores_smem_bytes(128));
+    if (e != cudaSuccess) return e;
+    return cudaFuncSetAttribute(scores_kernel<64>, cudaFuncAttributeMaxDynamicSharedMemorySize, scores_smem_bytes(64));
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -253,6 +262,7 @@ extern "C" int rapid3_block_scores_static(const rapid3_shape* s, const void* q, 
     double* scratch = nullptr;
     const int r = static_scratch(&scratch);
     if (r != RAPID3_OK) return r;
+    if (scoring_static_init() != cudaSuccess) return RAPID3_ERR_CUDA;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     // every element of the used part of the scratch is written by the pooling kernel before the
     // scoring kernel reads it, so nothing has to be cleared between calls
