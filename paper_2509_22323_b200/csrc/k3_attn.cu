@@ -645,7 +645,6 @@ attn_kernel(const __grid_constant__ CUtensorMap tmq, const __grid_constant__ CUt
                 // the waits and P stored after the vote below, dense attention of two images of 4429 tokens at D = 64
                 // went from 325 to 303 us, three of 4608 at D = 128 from 596 to 585 us (bursts at full clocks).
                 float b0, b1, b2, b3;
-                bool redo;
                 if (!seeded) {
                     // the first block this query block keeps: take the rows' maxima before the pass instead of running
                     // the pass twice (from -inf every row "grows")
@@ -653,7 +652,7 @@ attn_kernel(const __grid_constant__ CUtensorMap tmq, const __grid_constant__ CUt
                     nm_lo *= -c2; nm_hi *= -c2;
                     seeded = true;
                 }
-                do {
+                for (;;) {
                     b0 = b1 = b2 = b3 = 0.f;
 #pragma unroll
                     for (int k = 0; k < 8; ++k) {
@@ -670,13 +669,16 @@ attn_kernel(const __grid_constant__ CUtensorMap tmq, const __grid_constant__ CUt
                     // anything is told that P is there
                     tmem_st16x128_x8(tS, pk);
                     // if any thread of the warp sees growth, the quads combine their maxima and decide row by row
-                    redo = __any_sync(0xffffffffu, max3(b0, b1, fmaxf(b2, b3)) > GROWN_SUM);
-                    if (redo) {
+                    if (!__any_sync(0xffffffffu, max3(b0, b1, fmaxf(b2, b3)) > GROWN_SUM)) break;
+                    {
                         float mx_lo, mx_hi;
                         row_maxima(r, mx_lo, mx_hi);
                         // a sum of eight above 2^16 has a term above 2^13 - 1: the row that asked for it always moves
                         mx_lo *= -c2; mx_hi *= -c2;
                         const bool g_lo = nm_lo - mx_lo > GROWN_LOG2, g_hi = nm_hi - mx_hi > GROWN_LOG2;
+                        // No row moves: done.  (Scores beyond 2^28 or so leave more than 2^16 of P to the rounding of their
+                        // product with c2, which no maximum takes away; a row moves at most once in a block.)
+                        if (!__any_sync(0xffffffffu, g_lo || g_hi)) break;
                         const bool f_lo = g_lo && nm_lo != INFINITY, f_hi = g_hi && nm_hi != INFINITY;   // O holds something to rescale
                         if (__any_sync(0xffffffffu, f_lo || f_hi)) {
                             // O must be at rest: wait for P(n-1) V, which by the issue order of the products also
@@ -700,7 +702,7 @@ attn_kernel(const __grid_constant__ CUtensorMap tmq, const __grid_constant__ CUt
                         if (g_lo) nm_lo = mx_lo;
                         if (g_hi) nm_hi = mx_hi;
                     }
-                } while (redo);
+                }
                 l0 += b0; l1 += b1; l2 += b2; l3 += b3;
             } else {
 #pragma unroll

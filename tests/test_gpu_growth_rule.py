@@ -33,3 +33,24 @@ def test_scores_rising_by_steps(D, step, every):
     # P and the result are rounded to bf16 (2^-9 each, relative to the values' range); scores up to 2000 in powers of
     # two are 32-bit products, 2^-24 x 2000 x ln 2 relative in P
     assert float((out[0].double() - ref).abs().max()) <= 2 ** -7 * float(v.abs().max())
+
+
+@pytest.mark.parametrize("D", [64, 128])
+@pytest.mark.parametrize("scale", [1e3, 1e5, 1e7, 1e12])
+def test_scores_whose_rounding_exceeds_the_rule(D, scale):
+    """Scores so large that the rounding of their scaled value alone is worth more than 2^16 in P: no maximum can bring
+    the partial sums under the rule, and the pass must end all the same."""
+    gen = torch.Generator(device=DEV).manual_seed(D)
+    q, k, v = (torch.randn((1, 2, 300, D), generator=gen, device=DEV) for _ in range(3))
+    q, k, v = (q * scale).to(torch.bfloat16), (k * scale).to(torch.bfloat16), v.to(torch.bfloat16)
+    ctx = binding.Context(1, 2, D, 0, 300)
+    out = torch.full_like(q, float("nan"))
+    ctx.rapid3_gated_step(q, k, v, out, [2], [1.0])
+    torch.cuda.synchronize()
+    assert ctx.last_status() == 0
+    if scale <= 1e3:                     # beyond, P itself may leave the range of 32-bit floats
+        s = q[0].double() @ k[0].double().transpose(1, 2) * D ** -0.5
+        ref = s.softmax(-1) @ v[0].double()
+        clear = (s.topk(2, dim=-1).values.diff(dim=-1).squeeze(-1) < -100.0)     # one key decides, in any arithmetic
+        assert bool(clear.any())
+        assert float((out[0].double() - ref).abs()[clear].max()) <= 2 ** -7 * float(v.abs().max())
