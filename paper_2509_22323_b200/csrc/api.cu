@@ -158,7 +158,7 @@ int attn_launch(rapid3_ctx* c, const TensorGeom& g, const void* q, const void* k
     {
         ProfScope ps(c, PROF_ATTN, st);
         if (launch_attention(tq, tk, tv, out, g, l, kept_idx, kept_cnt, bitmask, scale, c->status, st, plan, n_cap, -1,
-                             after_select) != cudaSuccess)
+                             !after_select) != cudaSuccess)
             return RAPID3_ERR_CUDA;
     }
     c->launches += 1;
@@ -286,7 +286,7 @@ int rapid3_block_scores(rapid3_ctx* c, const void* q, const void* k, const int32
     }
     {
         ProfScope ps(c, PROF_SCORES, st);
-        if (launch_block_scores(c->pooled, c->g, n_img, scores, st, nullptr, true) != cudaSuccess) return RAPID3_ERR_CUDA;
+        if (launch_block_scores(c->pooled, c->g, n_img, scores, st) != cudaSuccess) return RAPID3_ERR_CUDA;
     }
     c->launches += 2;
     return RAPID3_OK;
@@ -448,15 +448,15 @@ static int gated_step_impl(rapid3_ctx* c, const void* q, const void* k, const vo
         }
         {
             ProfScope ps(c, PROF_SCORES, st);
-            if (launch_block_scores(c->pooled, g, sparse.n, c->scores, st, nullptr, true) != cudaSuccess) return RAPID3_ERR_CUDA;
+            if (launch_block_scores(c->pooled, g, sparse.n, c->scores, st) != cudaSuccess) return RAPID3_ERR_CUDA;
         }
         {
             ProfScope ps(c, PROF_SELECT, st);
             const cudaError_t e =
                 mass_scale ? launch_select_mask_mass(c->scores, g, sparse, share, *mass_scale, c->row_keep, c->bitmask,
-                                                     c->kept_idx, c->kept_cnt, st, true)
-                : per_head ? launch_select_mask_heads(c->scores, g, sparse, hk, c->bitmask, c->kept_idx, c->kept_cnt, st, true)
-                           : launch_select_mask(c->scores, g, sparse, c->bitmask, c->kept_idx, c->kept_cnt, st, nullptr, 0, true);
+                                                     c->kept_idx, c->kept_cnt, st)
+                : per_head ? launch_select_mask_heads(c->scores, g, sparse, hk, c->bitmask, c->kept_idx, c->kept_cnt, st)
+                           : launch_select_mask(c->scores, g, sparse, c->bitmask, c->kept_idx, c->kept_cnt, st);
             if (e != cudaSuccess) return RAPID3_ERR_CUDA;
         }
         c->launches += mass_scale ? 3 : 2;
@@ -523,11 +523,11 @@ int rapid3_gated_step_device(rapid3_ctx* c, const void* q, const void* k, const 
     }
     {
         ProfScope ps(c, PROF_SCORES, st);
-        if (launch_block_scores(c->pooled, c->g, B, c->scores, st, c->plan, true) != cudaSuccess) return RAPID3_ERR_CUDA;
+        if (launch_block_scores(c->pooled, c->g, B, c->scores, st, c->plan) != cudaSuccess) return RAPID3_ERR_CUDA;
     }
     {
         ProfScope ps(c, PROF_SELECT, st);
-        if (launch_select_mask(c->scores, c->g, none, c->bitmask, c->kept_idx, c->kept_cnt, st, c->plan, B, true) != cudaSuccess)
+        if (launch_select_mask(c->scores, c->g, none, c->bitmask, c->kept_idx, c->kept_cnt, st, c->plan, B) != cudaSuccess)
             return RAPID3_ERR_CUDA;
     }
     c->launches += 4;

@@ -58,10 +58,10 @@ struct TensorGeom {
     long long stride_b, stride_h, stride_n;   // elements
 };
 
-// Programmatic dependent launch: a kernel launched with `pdl` set may start while the kernel before it in the stream
+// Programmatic dependent launch: every kernel of a step is launched so that it may start while the kernel before it in the stream
 // is still running, and must call grid_dependency_wait() before it touches anything that kernel writes (and read it past
 // the L1, whose lines the wait is not known to refresh); the kernel before it calls grid_dependency_launch() to let it
-// start.  Both are no-ops in an ordinary launch.  Every kernel here waits before it lets the next one start: when a kernel
+// start.  Every kernel here waits before it lets the next one start: when a kernel
 // runs, all kernels but the one right before it have ended -- so the attention kernel's thread blocks that need nothing
 // of the selection may run beside it, and find Q, K and V of whatever kernel came before the call.
 #ifdef __CUDACC__
@@ -70,7 +70,7 @@ __device__ __forceinline__ void grid_dependency_launch() { asm volatile("griddep
 
 // `carveout`: percentage of the SM's first-level memory that the launch prefers as shared memory, -1 for the default.
 template <typename... KArgs, typename... Args>
-inline cudaError_t launch_kernel_carveout(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, bool pdl,
+inline cudaError_t launch_kernel_carveout(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t s,
                                           int carveout, Args&&... args) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = grid;
@@ -79,21 +79,17 @@ inline cudaError_t launch_kernel_carveout(void (*kernel)(KArgs...), dim3 grid, d
     cfg.stream = s;
     cudaLaunchAttribute attr[2];
     cfg.attrs = attr;
-    cfg.numAttrs = 0;
-    if (pdl) {
-        attr[cfg.numAttrs].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-        attr[cfg.numAttrs++].val.programmaticStreamSerializationAllowed = 1;
-    }
-    if (carveout >= 0) {
-        attr[cfg.numAttrs].id = cudaLaunchAttributePreferredSharedMemoryCarveout;
-        attr[cfg.numAttrs++].val.sharedMemCarveout = (unsigned)carveout;
-    }
+    cfg.numAttrs = carveout >= 0 ? 2 : 1;
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    attr[1].id = cudaLaunchAttributePreferredSharedMemoryCarveout;
+    attr[1].val.sharedMemCarveout = (unsigned)carveout;
     return cudaLaunchKernelEx(&cfg, kernel, static_cast<KArgs>(args)...);
 }
 template <typename... KArgs, typename... Args>
-inline cudaError_t launch_kernel(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, bool pdl,
+inline cudaError_t launch_kernel(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t s,
                                  Args&&... args) {
-    return launch_kernel_carveout(kernel, grid, block, smem, s, pdl, -1, static_cast<Args&&>(args)...);
+    return launch_kernel_carveout(kernel, grid, block, smem, s, -1, static_cast<Args&&>(args)...);
 }
 #endif
 
@@ -102,23 +98,21 @@ inline cudaError_t launch_kernel(void (*kernel)(KArgs...), dim3 grid, dim3 block
 // for `n_cap` images; CTAs beyond the planned count return at once.  pooled is [2][n_cap][H][nb][D].
 cudaError_t launch_block_pool(const void* q, const void* k, const TensorGeom& g, const ImgList& imgs,
                               double* pooled, cudaStream_t s, const DevPlan* plan = nullptr, int n_cap = 0);
-// `pdl`: the kernel before it in the stream is this library's pooling kernel (same for the launchers below: the
-// kernel named in their comment), so the launch may be a programmatic dependent one.
 cudaError_t launch_block_scores(const double* pooled, const TensorGeom& g, int n_img, float* scores,
-                                cudaStream_t s, const DevPlan* plan = nullptr, bool pdl = false);
+                                cudaStream_t s, const DevPlan* plan = nullptr);
 // K2: forced + top-k selection.
 cudaError_t launch_select_mask(const float* scores, const TensorGeom& g, const ImgList& imgs,
                                uint64_t* bitmask, int32_t* kept_idx, int32_t* kept_cnt, cudaStream_t s,
-                               const DevPlan* plan = nullptr, int n_cap = 0, bool pdl = false);   // after the scores kernel
+                               const DevPlan* plan = nullptr, int n_cap = 0);
 cudaError_t launch_select_mask_heads(const float* scores, const TensorGeom& g, const ImgList& imgs,
                                      const HeadKeep& hk, uint64_t* bitmask, int32_t* kept_idx, int32_t* kept_cnt,
-                                     cudaStream_t s, bool pdl = false);                           // after the scores kernel
+                                     cudaStream_t s);
 // K2, cumulative-mass variant: row_keep[row] = smallest count of best free candidates holding a share
 // tau of the row's softmax mass (weights exp(scale * (S - row max)), fp64), then the top-k selection
 // at that count.
 cudaError_t launch_select_mask_mass(const float* scores, const TensorGeom& g, const ImgList& imgs,
                                     const MassShare& share, float scale, int32_t* row_keep, uint64_t* bitmask,
-                                    int32_t* kept_idx, int32_t* kept_cnt, cudaStream_t s, bool pdl = false);   // after the scores kernel
+                                    int32_t* kept_idx, int32_t* kept_cnt, cudaStream_t s);
 // K5: Q/K producer (RMS norm + gain + rotary embedding -> bf16) that also writes the block means of
 // the images with a workspace slot.  pooled is [2][n_sparse][H][nb][D].
 struct PrepArgs {
@@ -143,7 +137,7 @@ cudaError_t launch_attention(const CUtensorMap& tmq, const CUtensorMap& tmk, con
                              void* out, const TensorGeom& g, const ImgList& imgs, const int32_t* kept_idx,
                              const int32_t* kept_cnt, const uint64_t* bitmask, float softmax_scale, int* status,
                              cudaStream_t s, const DevPlan* plan = nullptr, int n_cap = 0, int inject_stop_group = -1,
-                             int pdl = 0);   // 1: after the selection kernel, whose masks only the sparse images' thread blocks read
+                             bool wait_first = true);   // false: after the selection kernel, for whose masks the quads of sparse images wait themselves
 // Kernel attributes on the current device; set when a context is created (scoring: also by the context-free entry).
 cudaError_t attention_static_init();
 cudaError_t scoring_static_init();

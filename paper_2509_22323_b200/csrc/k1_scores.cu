@@ -160,17 +160,17 @@ cudaError_t launch_block_pool(const void* q, const void* k, const TensorGeom& g,
     // 47.3 -> 44.3 us a step; 27 MB: 265.0 -> 265.8, 54 MB: 204.3 -> 205.8, 208 MB: 999 -> 1003).
     const long long bytes = 4ll * n_cap * g.H * g.N * g.D;
     const int carveout = bytes <= (20ll << 20) ? (int)cudaSharedmemCarveoutMaxShared : -1;
-    return launch_kernel_carveout(g.D == 128 ? pool_kernel<128> : pool_kernel<64>, grid, dim3(128), 0, s, true, carveout,
+    return launch_kernel_carveout(g.D == 128 ? pool_kernel<128> : pool_kernel<64>, grid, dim3(128), 0, s, carveout,
                                   static_cast<const uint16_t*>(q), static_cast<const uint16_t*>(k), g, imgs, pooled, plan,
                                   n_cap);
 }
 
 cudaError_t launch_block_scores(const double* pooled, const TensorGeom& g, int n_img, float* scores,
-                                cudaStream_t s, const DevPlan* plan, bool pdl) {
+                                cudaStream_t s, const DevPlan* plan) {
     // with a plan n_img is the capacity.  32 x 32 tiles at every length: against 64 x 64 tiles they waste less of
     // the ragged edge and fill the SMs more evenly (30 against 35 us at 264 blocks, where 64 x 64 pads 264 to 320)
     const dim3 grid((g.nb + 31) / 32, (g.nb + 31) / 32, n_img * g.H);
-    return launch_kernel(g.D == 128 ? scores_kernel<128> : scores_kernel<64>, grid, dim3(256), scores_smem_bytes(g.D), s, pdl,
+    return launch_kernel(g.D == 128 ? scores_kernel<128> : scores_kernel<64>, grid, dim3(256), scores_smem_bytes(g.D), s,
                          pooled, g, n_img, scores, plan);
 }
 
@@ -267,7 +267,7 @@ extern "C" int rapid3_block_scores_static(const rapid3_shape* s, const void* q, 
     // every element of the used part of the scratch is written by the pooling kernel before the
     // scoring kernel reads it, so nothing has to be cleared between calls
     if (launch_block_pool(q, k, g, l, scratch, st) != cudaSuccess) return RAPID3_ERR_CUDA;
-    if (launch_block_scores(scratch, g, n_img, scores, st, nullptr, true) != cudaSuccess) return RAPID3_ERR_CUDA;
+    if (launch_block_scores(scratch, g, n_img, scores, st) != cudaSuccess) return RAPID3_ERR_CUDA;
     return RAPID3_OK;
 }
 

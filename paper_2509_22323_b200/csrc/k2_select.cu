@@ -246,10 +246,10 @@ cudaError_t with_ipl(int nb, F&& f) {
 
 template <typename HK>
 cudaError_t launch_select(const float* scores, const TensorGeom& g, const ImgList& imgs, uint64_t* bitmask, int32_t* kept_idx,
-                          int32_t* kept_cnt, cudaStream_t s, const DevPlan* plan, int n_img, bool pdl, const HK& hk) {
+                          int32_t* kept_cnt, cudaStream_t s, const DevPlan* plan, int n_img, const HK& hk) {
     const dim3 grid((g.nb + WARPS - 1) / WARPS, n_img * g.H);
     return with_ipl(g.nb, [&](auto ipl) {
-        return launch_kernel(select_kernel<HK, decltype(ipl)::value>, grid, dim3(WARPS * 32), 0, s, pdl, scores, g, imgs,
+        return launch_kernel(select_kernel<HK, decltype(ipl)::value>, grid, dim3(WARPS * 32), 0, s, scores, g, imgs,
                              reinterpret_cast<uint32_t*>(bitmask), kept_idx, kept_cnt, 2 * ((g.nb + 63) / 64), plan, hk);
     });
 }
@@ -258,26 +258,25 @@ cudaError_t launch_select(const float* scores, const TensorGeom& g, const ImgLis
 
 cudaError_t launch_select_mask_mass(const float* scores, const TensorGeom& g, const ImgList& imgs,
                                     const MassShare& share, float scale, int32_t* row_keep, uint64_t* bitmask,
-                                    int32_t* kept_idx, int32_t* kept_cnt, cudaStream_t s, bool pdl) {
+                                    int32_t* kept_idx, int32_t* kept_cnt, cudaStream_t s) {
     const cudaError_t e = with_ipl(g.nb, [&](auto ipl) {
         return launch_kernel(mass_count_kernel<decltype(ipl)::value>, dim3((g.nb + MASS_WARPS - 1) / MASS_WARPS, imgs.n * g.H),
-                             dim3(MASS_WARPS * 32), 0, s, pdl, scores, g, share, scale, row_keep);
+                             dim3(MASS_WARPS * 32), 0, s, scores, g, share, scale, row_keep);
     });
     if (e != cudaSuccess) return e;
     RowKeep rk;
     rk.k = row_keep;
-    return launch_select(scores, g, imgs, bitmask, kept_idx, kept_cnt, s, nullptr, imgs.n, true, rk);
+    return launch_select(scores, g, imgs, bitmask, kept_idx, kept_cnt, s, nullptr, imgs.n, rk);
 }
 
 cudaError_t launch_select_mask(const float* scores, const TensorGeom& g, const ImgList& imgs, uint64_t* bitmask,
-                               int32_t* kept_idx, int32_t* kept_cnt, cudaStream_t s, const DevPlan* plan, int n_cap,
-                               bool pdl) {
-    return launch_select(scores, g, imgs, bitmask, kept_idx, kept_cnt, s, plan, plan ? n_cap : imgs.n, pdl, NoHeadKeep());
+                               int32_t* kept_idx, int32_t* kept_cnt, cudaStream_t s, const DevPlan* plan, int n_cap) {
+    return launch_select(scores, g, imgs, bitmask, kept_idx, kept_cnt, s, plan, plan ? n_cap : imgs.n, NoHeadKeep());
 }
 
 cudaError_t launch_select_mask_heads(const float* scores, const TensorGeom& g, const ImgList& imgs, const HeadKeep& hk,
-                                     uint64_t* bitmask, int32_t* kept_idx, int32_t* kept_cnt, cudaStream_t s, bool pdl) {
-    return launch_select(scores, g, imgs, bitmask, kept_idx, kept_cnt, s, nullptr, imgs.n, pdl, hk);
+                                     uint64_t* bitmask, int32_t* kept_idx, int32_t* kept_cnt, cudaStream_t s) {
+    return launch_select(scores, g, imgs, bitmask, kept_idx, kept_cnt, s, nullptr, imgs.n, hk);
 }
 
 
@@ -340,6 +339,6 @@ __global__ void plan_kernel(const int32_t* action, const float* ratio, int B, in
 cudaError_t launch_plan(const int32_t* action_dev, const float* ratio_dev, int B, const TensorGeom& g, DevPlan* plan,
                         int* status, cudaStream_t s) {
     const int n_free_img = g.nb - g.n_text_blocks - 1;
-    return launch_kernel(plan_kernel, dim3(1), dim3(32), 0, s, true, action_dev, ratio_dev, B, n_free_img > 0 ? n_free_img : 0,
+    return launch_kernel(plan_kernel, dim3(1), dim3(32), 0, s, action_dev, ratio_dev, B, n_free_img > 0 ? n_free_img : 0,
                          plan, status);
 }

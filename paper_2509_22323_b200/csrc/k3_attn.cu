@@ -70,6 +70,7 @@ struct AttnParams {
     const DevPlan* plan;           // optional: image list and n_dense from device memory (grid sized for n_cap images)
     int* status;
     float scale_log2;
+    bool wait_first;               // nothing is read before the kernel in front has ended
     int stop_group;                // failure-injection build of the kernel only: the producer stops before this group
 };
 
@@ -216,6 +217,7 @@ attn_kernel(const __grid_constant__ CUtensorMap tmq, const __grid_constant__ CUt
         tmem_relinquish();
         tc_fence_before();
     }
+    if (prm.wait_first) grid_dependency_wait();
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem_base = ctl->tmem_base;
@@ -802,7 +804,7 @@ cudaError_t launch_attention(const CUtensorMap& tmq, const CUtensorMap& tmk, con
                              void* out,
                              const TensorGeom& g, const ImgList& imgs, const int32_t* kept_idx,
                              const int32_t* kept_cnt, const uint64_t* bitmask, float softmax_scale, int* status,
-                             cudaStream_t s, const DevPlan* plan, int n_cap, int inject_stop_group, int pdl) {
+                             cudaStream_t s, const DevPlan* plan, int n_cap, int inject_stop_group, bool wait_first) {
     if (!g_attr_set) {
         cudaError_t e = attention_static_init();
         if (e != cudaSuccess) return e;
@@ -820,6 +822,7 @@ cudaError_t launch_attention(const CUtensorMap& tmq, const CUtensorMap& tmk, con
     while (n_dense < imgs.n && (imgs.slot[n_dense] < 0 || kept_idx == nullptr)) ++n_dense;
     prm.n_dense = n_dense;
     prm.plan = plan;
+    prm.wait_first = wait_first;
     prm.stop_group = inject_stop_group;
     dim3 grid(((g.nb + 3) / 4) * g.H * (plan ? n_cap : imgs.n), 1, 1);
     if (inject_stop_group >= 0) {
@@ -828,9 +831,9 @@ cudaError_t launch_attention(const CUtensorMap& tmq, const CUtensorMap& tmk, con
         else
             attn_kernel<64, true><<<grid, NTHREADS, attn_smem_bytes<64>(), s>>>(tmq, tmk, tmv, static_cast<uint16_t*>(out), prm);
     } else if (g.D == 128) {
-        return launch_kernel(attn_kernel<128>, grid, dim3(NTHREADS), attn_smem_bytes<128>(), s, pdl != 0, tmq, tmk, tmv, static_cast<uint16_t*>(out), prm);
+        return launch_kernel(attn_kernel<128>, grid, dim3(NTHREADS), attn_smem_bytes<128>(), s, tmq, tmk, tmv, static_cast<uint16_t*>(out), prm);
     } else {
-        return launch_kernel(attn_kernel<64>, grid, dim3(NTHREADS), attn_smem_bytes<64>(), s, pdl != 0, tmq, tmk, tmv, static_cast<uint16_t*>(out), prm);
+        return launch_kernel(attn_kernel<64>, grid, dim3(NTHREADS), attn_smem_bytes<64>(), s, tmq, tmk, tmv, static_cast<uint16_t*>(out), prm);
     }
     return cudaGetLastError();
 }

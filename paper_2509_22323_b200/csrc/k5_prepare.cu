@@ -139,6 +139,6 @@ cudaError_t launch_prepare(const PrepArgs& a, const TensorGeom& g, const ImgList
     const uint16_t* kr = static_cast<const uint16_t*>(a.k_raw);
     uint16_t* qo = static_cast<uint16_t*>(a.q_out);
     uint16_t* ko = static_cast<uint16_t*>(a.k_out);
-    return launch_kernel(g.D == 128 ? prepare_kernel<128> : prepare_kernel<64>, grid, dim3(128), 0, s, true, qr, kr, qo, ko, a.q_gain,
+    return launch_kernel(g.D == 128 ? prepare_kernel<128> : prepare_kernel<64>, grid, dim3(128), 0, s, qr, kr, qo, ko, a.q_gain,
                          a.k_gain, a.rot, a.eps, g, imgs, n_sparse, pooled);
 }
