@@ -46,6 +46,7 @@ constexpr int SOFTMAX_WARPS = 16;
 constexpr int PRODUCER_WARP = 16, MMA_WARP0 = 17, LIST_WARP = 19;
 constexpr int NTHREADS = 32 * (SOFTMAX_WARPS + 4);
 constexpr int TMEM_COLS = 512;
+constexpr int SM_COUNT = 148;       // of a B200
 constexpr int TILE_COLS = 256;      // TMEM columns of one Q tile
 constexpr int BLK_BYTES = 8192;     // 64 rows x 128 bytes: one 64-channel half of a 64-token block
 constexpr int QHALF_BYTES = 16384;  // one 64-channel half of a 128-row Q tile
@@ -70,6 +71,7 @@ struct AttnParams {
     const DevPlan* plan;           // optional: image list and n_dense from device memory (grid sized for n_cap images)
     int* status;
     float scale_log2;
+    int halves;                    // 1: a unit of work is one tile of a quad, the other tile of its thread block idles
     bool wait_first;               // nothing is read before the kernel in front has ended
     int stop_group;                // failure-injection build of the kernel only: the producer stops before this group
 };
@@ -169,7 +171,7 @@ attn_kernel(const __grid_constant__ CUtensorMap tmq, const __grid_constant__ CUt
     const int warp = __shfl_sync(0xffffffffu, tid / 32, 0);
     const TensorGeom& g = prm.g;
     const int nb = g.nb, N = g.N;
-    const int n_quads = ((nb + 3) >> 2) * g.H * (prm.plan ? __ldcg(&prm.plan->all.n) : prm.imgs.n);
+    const int n_quads = (((nb + 3) >> 2) * g.H * (prm.plan ? __ldcg(&prm.plan->all.n) : prm.imgs.n)) << prm.halves;
     if ((int)blockIdx.x >= n_quads) return;              // device-resident plan: fewer images than the grid covers
 
     const uint32_t bQ = smem_u32(&ctl->q_full), bQE = smem_u32(&ctl->q_empty);
@@ -292,6 +294,8 @@ attn_kernel(const __grid_constant__ CUtensorMap tmq, const __grid_constant__ CUt
             // block walk all nb key blocks; the other quads of the sparse images follow, image by image in the list's
             // order (descending keep ratio).
             int quad, h, p;
+            const int half = prm.halves ? L & 1 : -1;    // the tile to work on, or both
+            L >>= prm.halves;
             {
                 const int nq = (nb + 3) >> 2, ntq = min(nq, (g.n_text_blocks + 3) >> 2);
                 const int n_all = prm.plan ? __ldcg(&prm.plan->all.n) : prm.imgs.n;
@@ -321,6 +325,7 @@ attn_kernel(const __grid_constant__ CUtensorMap tmq, const __grid_constant__ CUt
             // tiles want nearly the same key blocks (union of the quad 98 instead of 134 blocks at keep ratio 0.25,
             // both tiles busy on 68 % of them instead of 23 %).  qblk(a) is member a's query block.
             auto qblk = [&](int a) -> int {
+                if (half >= 0 && (a >> 1) != half) return nb;           // not of this unit: like a block past the end
                 int q = 4 * quad + (g.pair_stride == 2 ? ((a & 1) << 1) + (a >> 1) : a);
                 if (g.pair_stride == 3 && q >= g.n_text_blocks) {
                     const int r = q - g.n_text_blocks, w = r & 7;
@@ -338,7 +343,8 @@ attn_kernel(const __grid_constant__ CUtensorMap tmq, const __grid_constant__ CUt
                     // dense image keeps every block, and a mask of the selection kernel keeps the text blocks in every
                     // row, so the union list starts 0, 1, ....  First use of their stages, nothing to wait for.
                     load_q(u);
-                    const int n_early = (!INJECT && (slot < 0 || prm.bitmask32 != nullptr)) ? min(min(slot < 0 ? nb : g.n_text_blocks, nb), KS) : 0;
+                    const bool none = min(min(qblk(0), qblk(1)), min(qblk(2), qblk(3))) >= nb;   // the second half of a ragged last quad
+                    const int n_early = (!INJECT && !none && (slot < 0 || prm.bitmask32 != nullptr)) ? min(min(slot < 0 ? nb : g.n_text_blocks, nb), KS) : 0;
                     for (int gi = 0; gi < n_early; ++gi) issue_group(u, gi, gi, gi - 1, gi - 1);
                     ctl->n_early = n_early;
                 }
@@ -824,7 +830,13 @@ cudaError_t launch_attention(const CUtensorMap& tmq, const CUtensorMap& tmk, con
     prm.plan = plan;
     prm.wait_first = wait_first;
     prm.stop_group = inject_stop_group;
-    dim3 grid(((g.nb + 3) / 4) * g.H * (plan ? n_cap : imgs.n), 1, 1);
+    // Where the two tiles of every quad find an SM each, they go to two thread blocks: a tile that has the SM to itself goes
+    // through its key blocks in about 0.63 of the time of two that share it (whole steps of one image, us: 2 heads x 72
+    // blocks at D = 128 70.7 -> 62.1, 6 heads x 11 blocks 16.4 -> 13.8, 2 heads x 22 blocks at D = 64 26.3 -> 23.8; with
+    // more tiles than SMs the shared K and V stream wins).
+    const int quads = ((g.nb + 3) / 4) * g.H * (plan ? n_cap : imgs.n);
+    prm.halves = 2 * quads <= SM_COUNT ? 1 : 0;
+    dim3 grid(quads << prm.halves, 1, 1);
     if (inject_stop_group >= 0) {
         if (g.D == 128)
             attn_kernel<128, true><<<grid, NTHREADS, attn_smem_bytes<128>(), s>>>(tmq, tmk, tmv, static_cast<uint16_t*>(out), prm);

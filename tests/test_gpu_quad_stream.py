@@ -1,7 +1,7 @@
 """A thread block of the attention kernel works through many quads of query blocks, each role at its own pace.  What
 an image gets must not depend on what else the launch holds: every image of a large batch, whose kept lists mix full,
-short and empty rows, equals the same image run alone (one or two quads per thread block) bit for bit, and rows that
-keep nothing are zero."""
+short and empty rows, equals the same image run alone (a quad or half of one per thread block) bit for bit, and rows
+that keep nothing are zero."""
 import pytest
 import torch
 
