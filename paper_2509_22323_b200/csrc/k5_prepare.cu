@@ -40,7 +40,6 @@ __global__ void __launch_bounds__(128, PREP_MINB) prepare_kernel(const uint16_t*
     const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
     const int blk = blockIdx.x * 4 + warp, h = blockIdx.y;
     grid_dependency_wait();                           // first kernel of a call: what comes before it may still be running
-    grid_dependency_launch();
     if (blk >= g.nb) return;
     const int which = blockIdx.z / imgs.n;            // 0 = Q, 1 = K
     const int p = blockIdx.z - which * imgs.n;
@@ -117,6 +116,9 @@ __global__ void __launch_bounds__(128, PREP_MINB) prepare_kernel(const uint16_t*
             }
         }
     }
+    // Only now may the scores kernel's thread blocks come in: let in at the top, they cost a small launch more than their
+    // early start saves (steps of 144 and 28 quads from raw projections 25.5 -> 22.3 and 30.5 -> 27.4 us).
+    grid_dependency_launch();
     if (slot < 0) return;                             // a dense image is not scored (warp-uniform)
 #pragma unroll
     for (int o = TPR; o < 32; o <<= 1)
