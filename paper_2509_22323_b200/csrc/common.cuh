@@ -127,7 +127,7 @@ struct PrepArgs {
 };
 cudaError_t launch_prepare(const PrepArgs& a, const TensorGeom& g, const ImgList& imgs, int n_sparse, double* pooled,
                            cudaStream_t s);
-// Builds the plan from device-resident actions and keep ratios (one thread; B <= RAPID3_MAX_IMG).
+// Builds the plan from device-resident actions and keep ratios (one thread block; B <= RAPID3_MAX_IMG).
 cudaError_t launch_plan(const int32_t* action_dev, const float* ratio_dev, int B, const TensorGeom& g,
                         DevPlan* plan, int* status, cudaStream_t s);
 // K3: attention over kept tiles.  `bitmask` (optional) is the select kernel's bitmask of the same

@@ -285,53 +285,64 @@ cudaError_t launch_select_mask_heads(const float* scores, const TensorGeom& g, c
 // entry point does on the CPU, for callers whose sampled actions never leave the GPU.
 namespace {
 
-__global__ void plan_kernel(const int32_t* action, const float* ratio, int B, int n_free_img,
-                            DevPlan* __restrict__ plan, int* __restrict__ status) {
+// One thread decides; the loads, which would cost it a round trip each, and the stores are the whole block's.
+__global__ void __launch_bounds__(RAPID3_MAX_IMG) plan_kernel(const int32_t* action, const float* ratio, int B, int n_free_img,
+                                                              DevPlan* __restrict__ plan, int* __restrict__ status) {
+    __shared__ DevPlan out;
+    __shared__ int act[RAPID3_MAX_IMG];
+    __shared__ float rat[RAPID3_MAX_IMG], ratio_of[RAPID3_MAX_IMG];
+    constexpr int WORDS = sizeof(DevPlan) / sizeof(int);
+    static_assert(sizeof(DevPlan) % sizeof(int) == 0, "copied word by word");
     grid_dependency_wait();                           // first kernel of a call
     grid_dependency_launch();
-    if (threadIdx.x != 0 || blockIdx.x != 0) return;
-    ImgList& sp = plan->sparse;
-    ImgList& al = plan->all;
-    sp.n = 0;
-    al.n = 0;
-    int n_dense = 0;
-    float ratio_of[RAPID3_MAX_IMG];
-    for (int b = 0; b < B; ++b) {
-        const int a = __ldcg(action + b);
-        if (a != RAPID3_ACT_SKIP && a != RAPID3_ACT_REUSE && a != RAPID3_ACT_ATTEND) {
-            atomicExch(status, RAPID3_ERR_INVALID_ARG);       // unknown action: treated as a skip
-            continue;
-        }
-        if (a != RAPID3_ACT_ATTEND) continue;
-        const float r = __ldcg(ratio + b);
-        if (!(r > 0.f) || !(r <= 1.f)) {
-            atomicExch(status, RAPID3_ERR_INVALID_ARG);       // ratio outside (0, 1]: image not processed
-            continue;
-        }
-        int slot = -1;
-        if (r < 1.f) {
-            slot = sp.n++;
-            sp.batch[slot] = b;
-            sp.slot[slot] = slot;
-            double x = ceil((double)r * (double)n_free_img - 1e-6);
-            x = x < 0.0 ? 0.0 : (x > (double)n_free_img ? (double)n_free_img : x);
-            sp.k_free[slot] = (int)x;
-        } else {
-            ++n_dense;
-        }
-        int pos = al.n++;
-        while (pos > 0 && ratio_of[pos - 1] < r) {            // insertion sort, descending ratio, stable
-            al.batch[pos] = al.batch[pos - 1];
-            al.slot[pos] = al.slot[pos - 1];
-            ratio_of[pos] = ratio_of[pos - 1];
-            --pos;
-        }
-        al.batch[pos] = b;
-        al.slot[pos] = slot;
-        al.k_free[pos] = 0;
-        ratio_of[pos] = r;
+    for (int x = threadIdx.x; x < WORDS; x += RAPID3_MAX_IMG) reinterpret_cast<int*>(&out)[x] = 0;
+    if (threadIdx.x < B) {
+        act[threadIdx.x] = __ldcg(action + threadIdx.x);
+        rat[threadIdx.x] = __ldcg(ratio + threadIdx.x);
     }
-    plan->n_dense = n_dense;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        ImgList& sp = out.sparse;
+        ImgList& al = out.all;
+        int n_dense = 0;
+        for (int b = 0; b < B; ++b) {
+            const int a = act[b];
+            if (a != RAPID3_ACT_SKIP && a != RAPID3_ACT_REUSE && a != RAPID3_ACT_ATTEND) {
+                atomicExch(status, RAPID3_ERR_INVALID_ARG);   // unknown action: treated as a skip
+                continue;
+            }
+            if (a != RAPID3_ACT_ATTEND) continue;
+            const float r = rat[b];
+            if (!(r > 0.f) || !(r <= 1.f)) {
+                atomicExch(status, RAPID3_ERR_INVALID_ARG);   // ratio outside (0, 1]: image not processed
+                continue;
+            }
+            int slot = -1;
+            if (r < 1.f) {
+                slot = sp.n++;
+                sp.batch[slot] = b;
+                sp.slot[slot] = slot;
+                double x = ceil((double)r * (double)n_free_img - 1e-6);
+                x = x < 0.0 ? 0.0 : (x > (double)n_free_img ? (double)n_free_img : x);
+                sp.k_free[slot] = (int)x;
+            } else {
+                ++n_dense;
+            }
+            int pos = al.n++;
+            while (pos > 0 && ratio_of[pos - 1] < r) {        // insertion sort, descending ratio, stable
+                al.batch[pos] = al.batch[pos - 1];
+                al.slot[pos] = al.slot[pos - 1];
+                ratio_of[pos] = ratio_of[pos - 1];
+                --pos;
+            }
+            al.batch[pos] = b;
+            al.slot[pos] = slot;
+            ratio_of[pos] = r;
+        }
+        out.n_dense = n_dense;
+    }
+    __syncthreads();
+    for (int x = threadIdx.x; x < WORDS; x += RAPID3_MAX_IMG) reinterpret_cast<int*>(plan)[x] = reinterpret_cast<const int*>(&out)[x];
 }
 
 }  // namespace
@@ -339,6 +350,6 @@ __global__ void plan_kernel(const int32_t* action, const float* ratio, int B, in
 cudaError_t launch_plan(const int32_t* action_dev, const float* ratio_dev, int B, const TensorGeom& g, DevPlan* plan,
                         int* status, cudaStream_t s) {
     const int n_free_img = g.nb - g.n_text_blocks - 1;
-    return launch_kernel(plan_kernel, dim3(1), dim3(32), 0, s, action_dev, ratio_dev, B, n_free_img > 0 ? n_free_img : 0,
+    return launch_kernel(plan_kernel, dim3(1), dim3(RAPID3_MAX_IMG), 0, s, action_dev, ratio_dev, B, n_free_img > 0 ? n_free_img : 0,
                          plan, status);
 }
