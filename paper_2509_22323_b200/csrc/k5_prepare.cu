@@ -62,23 +62,34 @@ __global__ void __launch_bounds__(128, PREP_MINB) prepare_kernel(const uint16_t*
     double acc[8];
 #pragma unroll
     for (int e = 0; e < 8; ++e) acc[e] = 0.0;
+    auto load_raw = [&](int it, uint4 (&v)[INFL]) {
+#pragma unroll
+        for (int u = 0; u < INFL; ++u) {
+            const int row = (it + u) * RPL + r0;
+            v[u] = make_uint4(0, 0, 0, 0);
+            if (row < valid) v[u] = __ldcg(reinterpret_cast<const uint4*>(src + (long long)(n0 + row) * g.stride_n + c * 8));
+        }
+    };
+    // The next rows are on their way while these are worked on (a lane reads them before it writes them, should the
+    // output lie over the input): one 4608-token image of 24 heads 33.3 -> 32.2 us.
+    uint4 next[INFL];
+    load_raw(0, next);
 #pragma unroll 1
     for (int it0 = 0; it0 < ITERS; it0 += INFL) {
         uint4 v[INFL];
         float4 cs[INFL][2];
 #pragma unroll
+        for (int u = 0; u < INFL; ++u) v[u] = next[u];
+        if (it0 + INFL < ITERS) load_raw(it0 + INFL, next);
+#pragma unroll
         for (int u = 0; u < INFL; ++u) {
             const int row = (it0 + u) * RPL + r0;
-            v[u] = make_uint4(0, 0, 0, 0);
             cs[u][0] = make_float4(1.f, 0.f, 1.f, 0.f);
             cs[u][1] = make_float4(1.f, 0.f, 1.f, 0.f);
-            if (row < valid) {
-                v[u] = __ldcg(reinterpret_cast<const uint4*>(src + (long long)(n0 + row) * g.stride_n + c * 8));
-                if (rot) {
-                    const float4* rp = reinterpret_cast<const float4*>(rot + ((long long)(n0 + row) * (D / 2) + c * 4) * 2);
-                    cs[u][0] = __ldcg(rp);
-                    cs[u][1] = __ldcg(rp + 1);
-                }
+            if (rot && row < valid) {
+                const float4* rp = reinterpret_cast<const float4*>(rot + ((long long)(n0 + row) * (D / 2) + c * 4) * 2);
+                cs[u][0] = __ldcg(rp);
+                cs[u][1] = __ldcg(rp + 1);
             }
         }
 #pragma unroll
