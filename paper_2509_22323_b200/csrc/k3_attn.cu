@@ -50,9 +50,12 @@ constexpr int SM_COUNT = 148;       // of a B200
 constexpr int TILE_COLS = 256;      // TMEM columns of one Q tile
 constexpr int BLK_BYTES = 8192;     // 64 rows x 128 bytes: one 64-channel half of a 64-token block
 constexpr int QHALF_BYTES = 16384;  // one 64-channel half of a 128-row Q tile
-// A row's reference maximum moves when a partial sum of eight P exceeds 2^16, in the rows that grew by more than 2^12.
-// (How far P may exceed 1 costs no precision: P, O and l are floating point throughout.)
-constexpr float GROWN_SUM = 65536.0f, GROWN_LOG2 = 12.0f;
+// A row's reference maximum moves when a P of it exceeds 2^8; the partial sum of eight that it is part of then does too.
+// How far P may exceed 1 costs no precision (P, O and l are floating point throughout), but it costs range: O holds up to
+// the row's sum of P times a value.  With sums of 2^16 and growth of 2^12 as the rule, values from 2^112 on overflowed,
+// with this one from 2^118 on, and it takes as long (dense attention of three images of 4608 tokens at D = 128: 581.7 and
+// 581.7 us; two of 4429 at D = 64: 310.6 and 310.1; bursts).
+constexpr float GROWN_SUM = 256.0f, GROWN_LOG2 = 8.0f;
 constexpr int MAX_STAGES = 8;
 // The next quad is taken over when the producer has this many key blocks of the current one left to load (it runs up
 // to a ring ahead of the MMAs): early enough to have its list built in time, late enough not to hold a quad that
@@ -646,8 +649,8 @@ attn_kernel(const __grid_constant__ CUtensorMap tmq, const __grid_constant__ CUt
                 }
                 // One pass over the 32 scores gives P = 2^(S c2 - m c2) (packed to bf16) and the block's partial row
                 // sums.  The pass runs with the reference maxima as they stand, so the exponentials do not wait for
-                // this block's maximum, and it takes no maximum at all: a P above 2^16 shows in the partial sum that it
-                // is part of (eight terms, none negative).  Only when a partial sum exceeds 2^16 (rare after a query
+                // this block's maximum, and it takes no maximum at all: a P above 2^8 shows in the partial sum that it
+                // is part of (eight terms, none negative).  Only when a partial sum exceeds 2^8 (rare after a query
                 // block's first key block) the rows' maxima are taken, O and l are rescaled and the pass is repeated.
                 // Bound by issue slots and the exponential unit: against maxima in the pass, packed products, votes on
                 // the waits and P stored after the vote below, dense attention of two images of 4429 tokens at D = 64
@@ -681,11 +684,11 @@ attn_kernel(const __grid_constant__ CUtensorMap tmq, const __grid_constant__ CUt
                     {
                         float mx_lo, mx_hi;
                         row_maxima(r, mx_lo, mx_hi);
-                        // a sum of eight above 2^16 has a term above 2^13 - 1: the row that asked for it always moves
                         mx_lo *= -c2; mx_hi *= -c2;
                         const bool g_lo = nm_lo - mx_lo > GROWN_LOG2, g_hi = nm_hi - mx_hi > GROWN_LOG2;
-                        // No row moves: done.  (Scores beyond 2^28 or so leave more than 2^16 of P to the rounding of their
-                        // product with c2, which no maximum takes away; a row moves at most once in a block.)
+                        // No row moves: done.  (Eight smaller P made the sum; or scores beyond 2^27 or so leave more than
+                        // 2^8 of P to the rounding of their product with c2, which no maximum takes away.  A row moves at
+                        // most once in a block.)
                         if (!__any_sync(0xffffffffu, g_lo || g_hi)) break;
                         const bool f_lo = g_lo && nm_lo != INFINITY, f_hi = g_hi && nm_hi != INFINITY;   // O holds something to rescale
                         if (__any_sync(0xffffffffu, f_lo || f_hi)) {
