@@ -61,8 +61,9 @@ struct TensorGeom {
 // Programmatic dependent launch: every kernel of a step is launched so that it may start while the kernel before it in the stream
 // is still running, and must call grid_dependency_wait() before it touches anything that kernel writes (and read it past
 // the L1, whose lines the wait is not known to refresh); the kernel before it calls grid_dependency_launch() to let it
-// start.  Every kernel here waits before it lets the next one start: when a kernel
-// runs, all kernels but the one right before it have ended -- so the attention kernel's thread blocks that need nothing
+// start.  Every kernel here waits before it lets the next one start (the attention kernel, which signals nothing, before it
+// ends; a thread block without work may leave at once where another waits): when a kernel runs, all kernels but the one
+// right before it have ended -- so the attention kernel's thread blocks that need nothing
 // of the selection may run beside it, and find Q, K and V of whatever kernel came before the call.
 #ifdef __CUDACC__
 __device__ __forceinline__ void grid_dependency_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }

@@ -175,7 +175,12 @@ attn_kernel(const __grid_constant__ CUtensorMap tmq, const __grid_constant__ CUt
     const TensorGeom& g = prm.g;
     const int nb = g.nb, N = g.N;
     const int n_quads = (((nb + 3) >> 2) * g.H * (prm.plan ? __ldcg(&prm.plan->all.n) : prm.imgs.n)) << prm.halves;
-    if ((int)blockIdx.x >= n_quads) return;              // device-resident plan: fewer images than the grid covers
+    if ((int)blockIdx.x >= n_quads) {                    // device-resident plan: fewer images than the grid covers
+        // When none attends, no other thread block waits for the selection kernel: the grid must not end before that does
+        // (it may still have the plan to read, which the next call rewrites).
+        if (n_quads == 0) grid_dependency_wait();
+        return;
+    }
 
     const uint32_t bQ = smem_u32(&ctl->q_full), bQE = smem_u32(&ctl->q_empty);
     const uint32_t bKF = smem_u32(&ctl->k_full[0]), bKE = smem_u32(&ctl->k_empty[0]);

@@ -121,3 +121,44 @@ def test_queued_steps_of_the_other_entry_points(name, variant):
     assert ctx.last_status() == 0
     for s in range(n_sets):
         assert torch.equal(outs[s].view(torch.int16), alone[s].view(torch.int16)), f"{name} {variant}: input set {s}"
+
+
+def test_queued_device_steps_whose_decisions_change():
+    """Device-action steps, each with a plan of its own -- several sparse images, one, dense ones only, none that attends --
+    queued behind one another: every output and the masks of the last step equal those of the step run alone, whichever
+    comes last and whatever the one before it planned."""
+    wl = inputs.Workload("dev_queue", 6, 2, 128, 77, 24, 2.0, (0.5,) * 6, rope=True, seed=57)
+    q, k, v = inputs.make_qkv(wl, 0, device=DEV)
+    plans = [([2, 0, 2, 2, 1, 2], [0.5, 1.0, 1.0, 0.25, 0.5, 0.5]), ([0, 1, 0, 1, 0, 1], [0.5] * 6),
+             ([2] * 6, [0.3, 0.25, 0.75, 0.3, 0.9, 0.1]), ([2, 2, 0, 0, 2, 1], [1.0] * 6),
+             ([1, 0, 0, 0, 0, 0], [0.25] * 6), ([0, 0, 0, 0, 2, 0], [0.5] * 6)]
+    dev = [(torch.tensor(a, dtype=torch.int32, device=DEV), torch.tensor(r, dtype=torch.float32, device=DEV)) for a, r in plans]
+
+    def step(ctx, i, out):
+        ctx.rapid3_gated_step_device(q, k, v, out, *dev[i], wl.softmax_scale)
+
+    def state(ctx, i):
+        n = count_sparse(*plans[i])
+        return [w.clone() for w in ctx.workspace(n)] if n else []
+
+    alone = []
+    for i in range(len(plans)):
+        ctx = binding.Context(wl.batch, wl.heads, wl.head_dim, wl.n_text, wl.n_image)
+        out = torch.zeros_like(q)
+        step(ctx, i, out)
+        torch.cuda.synchronize()
+        assert ctx.last_status() == 0
+        alone.append((out, state(ctx, i)))
+    for stride in (1, 5):                                       # both orders of neighbours
+        ctx = binding.Context(wl.batch, wl.heads, wl.head_dim, wl.n_text, wl.n_image)
+        outs = [torch.zeros_like(q) for _ in plans]
+        for last in range(len(plans)):
+            torch.cuda.synchronize()
+            for n in range(4 * len(plans) + 1):                 # no synchronisation inside this loop
+                step(ctx, (last + stride * n) % len(plans), outs[(last + stride * n) % len(plans)])
+            torch.cuda.synchronize()
+            assert ctx.last_status() == 0
+            for got, (want, _) in zip(outs, alone):
+                assert torch.equal(got.view(torch.int16), want.view(torch.int16))
+            for got, want in zip(state(ctx, last), alone[last][1]):
+                assert torch.equal(got, want)
