@@ -695,6 +695,7 @@ attn_kernel(const __grid_constant__ CUtensorMap tmq, const __grid_constant__ CUt
                         // 2^8 of P to the rounding of their product with c2, which no maximum takes away.  A row moves at
                         // most once in a block.)
                         if (!__any_sync(0xffffffffu, g_lo || g_hi)) break;
+                        tc_wait_st();                     // nothing else orders the repeated pass's store of P behind this one's
                         const bool f_lo = g_lo && nm_lo != INFINITY, f_hi = g_hi && nm_hi != INFINITY;   // O holds something to rescale
                         if (__any_sync(0xffffffffu, f_lo || f_hi)) {
                             // O must be at rest: wait for P(n-1) V, which by the issue order of the products also
