@@ -62,6 +62,9 @@ constexpr int MAX_STAGES = 8;
 // another SM could have started.
 // (2, 4 and 10 measured the same.)
 constexpr int TAKE_AHEAD = 4;
+// After a wait has run out the softmax warps go on for up to this many key blocks, each a wait of 16 polls of about 8 us.
+// (Over the whole of a quad, with 256 polls a block, that was 2.06 s at two heads of 1024 key blocks; now 4.7 ms.)
+constexpr int ABORT_EVERY = 32;
 
 struct AttnParams {
     TensorGeom g;
@@ -241,7 +244,7 @@ attn_kernel(const __grid_constant__ CUtensorMap tmq, const __grid_constant__ CUt
         constexpr uint32_t limit = INJECT ? (1u << 12) : (1u << 22);
         for (uint32_t it = 0; it < limit; ++it) {
             if (mbar_try_wait(bar, parity)) return true;
-            if ((it & 255u) == 255u && ctl->abort_flag) return false;
+            if ((it & 15u) == 15u && ctl->abort_flag) return false;
         }
         fail();
         return false;
@@ -627,14 +630,17 @@ attn_kernel(const __grid_constant__ CUtensorMap tmq, const __grid_constant__ CUt
         uint32_t r[32];
         const int n0 = n;
         bool seeded = false;                           // the rows' reference maxima have been set (warp-uniform: a warp's rows share a query block)
-        for (int j = 0; j < n_u; ++j) {
+        // A wait that runs out sets the abort flag; nothing up to the end of a quad depends on a wait's result, so no vote is
+        // taken on the way, and the flag is looked at every ABORT_EVERY key blocks only.
+        for (int j0 = 0; j0 < n_u; j0 += ABORT_EVERY) {
+        if (__any_sync(0xffffffffu, ctl->abort_flag)) break;
+        const int j1 = min(j0 + ABORT_EVERY, n_u);
+        for (int j = j0; j < j1; ++j) {
             const uint32_t e = u.ent[j];
             if (!(e & tile_bits)) continue;            // neither query block of the tile kept it
             const bool act = e & act_bit;
             const int buf = n % NBUF;
             const uint32_t tS = lane_addr + 64 * buf;
-            // A wait that runs out sets the abort flag, and the quad is gone through over whatever is there: nothing up
-            // to its end depends on a wait's result, so no vote is taken on the way.
             wait(bSFt + 8 * buf, (n / NBUF) & 1);
             __syncwarp();
             tc_fence_after();
@@ -731,6 +737,7 @@ attn_kernel(const __grid_constant__ CUtensorMap tmq, const __grid_constant__ CUt
             __syncwarp();
             if (lane == 0) mbar_arrive(bPFt + 8 * buf);
             ++n;
+        }
         }
         if (n > n0) wait(bOD + 8 * t, n_o++ & 1);
         if (!(ok = __all_sync(0xffffffffu, !ctl->abort_flag))) break;

@@ -5,6 +5,8 @@
   RAPID3_ERR_TIMEOUT through the status word, and leave the context usable.
 * The tensor-map cache of a context: one context fed more distinct buffers than it has cache
   slots must keep computing with the right tensors."""
+import time
+
 import numpy as np
 import pytest
 import torch
@@ -50,6 +52,24 @@ def test_wait_that_runs_out_sets_the_status_and_returns(D, stop_group):
     ref = oracle.gated_step(Q.cpu(), K.cpu(), V.cpu(), acts, ratios, wl.n_text, wl.softmax_scale)
     for b in range(2):
         parity.compare_outputs(out[b], ref[b]["out"], f"after a timeout, img {b}")
+
+
+@pytest.mark.parametrize("D", [64, 128])
+def test_a_wait_that_ran_out_does_not_delay_the_end_by_the_sequence(D):
+    """512 key blocks: 256 thread blocks, two rounds of them, each over after 4096 polls and 16 more for each of the next 32
+    key blocks at most, under 10 us a poll: 92 ms.  (256 polls at every key block that was left took 0.5 s.)"""
+    q = torch.randn((1, 2, 512 * 64, D), device=DEV).to(torch.bfloat16)
+    out = torch.zeros_like(q)
+    ctx = binding.Context(1, 2, D, 0, 512 * 64)
+    took = []
+    for _ in range(3):
+        torch.cuda.synchronize()
+        t0 = time.perf_counter()
+        ctx.rapid3_debug_inject_timeout(q, q, q, out, 1)
+        torch.cuda.synchronize()
+        took.append(time.perf_counter() - t0)
+        assert ctx.last_status() == ERR_TIMEOUT
+    assert min(took) < 0.2, took
 
 
 def test_injection_entry_refuses_bad_arguments():
