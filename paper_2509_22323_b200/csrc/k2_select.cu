@@ -192,6 +192,16 @@ __global__ void __launch_bounds__(MASS_WARPS * 32) mass_count_kernel(const float
         part += w[x];
     }
     const double total = warp_sum(part);
+    if (total != total) {
+        // A weight is not a number (a NaN among the scores, an infinite maximum): no share compares with it, and every
+        // candidate is kept -- those of key 0, which only a NaN with all bits set has, as one.
+        int c = 0;
+#pragma unroll
+        for (int x = 0; x < IPL; ++x) c += u[x] != 0u;
+        c = __reduce_add_sync(0xffffffffu, c);
+        if (lane == 0) row_keep[row] = min(c + 1, n_free);
+        return;
+    }
     double want = (double)tau * total;                     // mass still to be covered inside the prefix group
     uint32_t prefix;
     int hi = differing_bits(u, prefix);                    // the group: candidates that equal `prefix` from bit `hi` up

@@ -119,3 +119,28 @@ def test_gated_step_with_mass_selection():
     parity.compare_outputs(out[2], ref, "mass gate dense img 2")
     with pytest.raises(binding.Rapid3Error):
         ctx.rapid3_gated_step_mass(Q, K, V, out, acts, [0.6, 0.5, 1.0, 0.0, 0.5], scale)
+
+
+@pytest.mark.parametrize("nb", [5, 72, 264, 400])
+@pytest.mark.parametrize("what", ["nan", "minus_inf", "inf", "nan_beside_equal_scores", "minus_inf_at_scale_0"])
+def test_weights_that_are_not_numbers_keep_every_candidate(nb, what):
+    """A row whose weights' sum is not a number compares with no share: all of it is kept, whatever scores are equal."""
+    ctx = binding.Context(1, 2, 64, 64, 64 * (nb - 1))
+    S = torch.randn((1, 2, nb, nb), generator=torch.Generator().manual_seed(nb))
+    scale = 0.0 if what == "minus_inf_at_scale_0" else 1.0
+    if what == "nan":
+        S.fill_(float("nan"))
+    elif what == "nan_beside_equal_scores":
+        S.fill_(-2.0)
+        S[..., 2] = float("nan")                    # in every row but its own a candidate
+    elif what == "inf":
+        S.fill_(float("inf"))
+    else:
+        S.fill_(float("-inf"))
+    keep, bitmask, idx, cnt = ctx.rapid3_select_mask_mass(S.to(DEV), [0.5], scale)
+    torch.cuda.synchronize()
+    n_free = nb - 2                                  # of the rows past the text block
+    rows = [i for i in range(1, nb) if not (what == "nan_beside_equal_scores" and i == 2)]
+    assert (keep[:, :, rows] == n_free).all()
+    assert (cnt[:, :, rows] == nb).all()
+    parity.check_lists(idx, cnt, binding.bitmask_to_dense(bitmask, nb).numpy())
