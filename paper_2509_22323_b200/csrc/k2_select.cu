@@ -245,12 +245,18 @@ __global__ void __launch_bounds__(MASS_WARPS * 32) mass_count_kernel(const float
     if (lane == 0) row_keep[row] = min(max(above + r, 1), n_free);
 }
 
-// Calls f with a register count per lane that holds a row of nb scores: three (96 blocks, the 1024^2 sequences), nine
-// (288, the 2048^2 ones) or what the longest sequence takes.
+// Calls f with a register count per lane that holds a row of nb scores.  A kernel takes the time that its count takes, not
+// the row, so the counts lie no further apart than by a half.  One image of 24 heads, us, with the counts 3, 9 and 32 alone /
+// as it is / the histograms in shared memory that this replaces.  Top-k: 150 blocks 11.9 / 7.8 / 11.5, 200 13.2 / 13.1 / 14.7,
+// 289 30.8 / 19.6 / 22.2, 400 42.7 / 27.6 / 32.9, 512 55.2 / 35.7 / 47.8, 600 67.0 / 55.3 / 64.4, 1024 145 / 144 / 262.
+// Cumulative mass with its selection: 150 28.2 / 19.1 / 36.1, 289 86.5 / 52.9 / 72.5, 512 157 / 95.9 / 158, 1024 385 / 384 / 748.
 template <typename F>
 cudaError_t with_ipl(int nb, F&& f) {
     if (nb <= 96) return f(std::integral_constant<int, 3>());
+    if (nb <= 192) return f(std::integral_constant<int, 6>());
     if (nb <= 288) return f(std::integral_constant<int, 9>());
+    if (nb <= 512) return f(std::integral_constant<int, 16>());
+    if (nb <= 768) return f(std::integral_constant<int, 24>());
     return f(std::integral_constant<int, RAPID3_MAX_NB / 32>());
 }
 
