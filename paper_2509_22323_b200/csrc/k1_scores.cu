@@ -262,7 +262,10 @@ extern "C" int rapid3_block_scores_static(const rapid3_shape* s, const void* q, 
     double* scratch = nullptr;
     const int r = static_scratch(&scratch);
     if (r != RAPID3_OK) return r;
-    if (scoring_static_init() != cudaSuccess) return RAPID3_ERR_CUDA;
+    if (scoring_static_init() != cudaSuccess) {
+        cudaGetLastError();
+        return RAPID3_ERR_CUDA;
+    }
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     // every element of the used part of the scratch is written by the pooling kernel before the
     // scoring kernel reads it, so nothing has to be cleared between calls

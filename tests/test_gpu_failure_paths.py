@@ -4,7 +4,9 @@
   (its producer stops early, its waits give up after 4096 polls) must return, report
   RAPID3_ERR_TIMEOUT through the status word, and leave the context usable.
 * The tensor-map cache of a context: one context fed more distinct buffers than it has cache
-  slots must keep computing with the right tensors."""
+  slots must keep computing with the right tensors.
+* A call whose launch is refused reports it once: the next call starts without it."""
+import ctypes
 import time
 
 import numpy as np
@@ -18,7 +20,7 @@ from tests import parity
 pytestmark = pytest.mark.gpu
 DEV = "cuda"
 POISON = 0x7FC1
-ERR_TIMEOUT = -5
+ERR_CUDA, ERR_TIMEOUT = -4, -5
 
 
 def poison_like(t):
@@ -113,3 +115,33 @@ def test_one_context_many_distinct_buffers():
     ref = oracle.gated_step(Q.cpu(), K.cpu(), V.cpu(), acts, ratios, wl.n_text, wl.softmax_scale)
     for b in range(2):
         parity.compare_outputs(outs[-1][b], ref[b]["out"], f"many buffers img {b}")
+
+
+def test_a_refused_launch_is_reported_once():
+    """A call on a stream whose capture has been invalidated is refused by the runtime; the call after it, on a sound
+    stream, is not."""
+    wl = inputs.Workload("refused", 1, 2, 64, 64, 8, 2.0, (0.5,), seed=95)
+    Q, K, V = inputs.make_qkv(wl, 0, device=DEV)
+    out = torch.zeros_like(Q)
+    ctx = binding.Context(wl.batch, wl.heads, wl.head_dim, wl.n_text, wl.n_image)
+    ctx.rapid3_gated_step(Q, K, V, out, [2], [0.5], wl.softmax_scale)
+    torch.cuda.synchronize()
+    want = out.clone()
+    delta = V.clone()
+    cudart = ctypes.CDLL("libcudart.so.12")                  # torch's own, already loaded
+    stream = torch.cuda.Stream()
+    handle, graph = ctypes.c_void_p(stream.cuda_stream), ctypes.c_void_p()
+    for ratio in (0.5, 1.0):                                 # the pooling kernel is the first to be refused, then the attention
+        assert cudart.cudaStreamBeginCapture(handle, 1) == 0     # thread-local mode
+        assert cudart.cudaStreamSynchronize(handle) != 0         # not permitted: the capture is invalid from here on
+        with torch.cuda.stream(stream), pytest.raises(binding.Rapid3Error) as e:
+            ctx.rapid3_gated_step(Q, K, V, out, [2], [ratio], wl.softmax_scale)
+        assert e.value.code == ERR_CUDA
+        assert cudart.cudaStreamEndCapture(handle, ctypes.byref(graph)) != 0
+        cudart.cudaGetLastError()
+        binding.rapid3_cache_step(Q, out, delta, [2])        # judged by the last error of the library's own runtime
+    out.zero_()
+    ctx.rapid3_gated_step(Q, K, V, out, [2], [0.5], wl.softmax_scale)
+    torch.cuda.synchronize()
+    assert ctx.last_status() == 0
+    assert torch.equal(out.view(torch.int16), want.view(torch.int16))
