@@ -511,7 +511,7 @@ int rapid3_gated_step_device(rapid3_ctx* c, const void* q, const void* k, const 
     if (!(softmax_scale > 0.f) || !isfinite(softmax_scale)) return RAPID3_ERR_INVALID_ARG;
     if ((reinterpret_cast<uintptr_t>(q) % 16) || (reinterpret_cast<uintptr_t>(k) % 16)) return RAPID3_ERR_INVALID_ARG;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    // The host never sees the actions: a one-thread kernel does the gate and compaction into the
+    // The host never sees the actions: a kernel of one thread block does the gate and compaction into the
     // context's device-resident plan, and every following kernel is launched with a grid that covers
     // all B images and takes its image list from the plan; the surplus CTAs return at once.
     if (launch_plan(action_dev, keep_ratio_dev, B, c->g, c->plan, c->status, st) != cudaSuccess) return RAPID3_ERR_CUDA;

@@ -702,7 +702,7 @@ attn_kernel(const __grid_constant__ CUtensorMap tmq, const __grid_constant__ CUt
                         // most once in a block.)
                         if (!__any_sync(0xffffffffu, g_lo || g_hi)) break;
                         tc_wait_st();                     // nothing else orders the repeated pass's store of P behind this one's
-                        const bool f_lo = g_lo && nm_lo != INFINITY, f_hi = g_hi && nm_hi != INFINITY;   // O holds something to rescale
+                        const bool f_lo = g_lo && nm_lo != INFINITY, f_hi = g_hi && nm_hi != INFINITY;   // not so where -inf was all it had
                         if (__any_sync(0xffffffffu, f_lo || f_hi)) {
                             // O must be at rest: wait for P(n-1) V, which by the issue order of the products also
                             // tells that every earlier one is done
