@@ -39,6 +39,7 @@ struct rapid3_ctx {
     int32_t* kept_cnt = nullptr;  // [B_max][H][nb]
     int32_t* row_keep = nullptr;  // [B_max][H][nb]: per-row counts of the cumulative-mass selection
     int* status = nullptr;
+    AttnParts parts;              // how the attention of a small context is cut, and its workspace
     DevPlan* plan = nullptr;      // device-resident plan of rapid3_gated_step_device
     // host-tensor staging of rapid3_gated_step_host (created on first use)
     void* stage[4] = {nullptr, nullptr, nullptr, nullptr};
@@ -158,7 +159,7 @@ int attn_launch(rapid3_ctx* c, const TensorGeom& g, const void* q, const void* k
     {
         ProfScope ps(c, PROF_ATTN, st);
         if (launch_attention(tq, tk, tv, out, g, l, kept_idx, kept_cnt, bitmask, scale, c->status, st, plan, n_cap, -1,
-                             !after_select) != cudaSuccess)
+                             !after_select, &c->parts, &c->launches) != cudaSuccess)
             return RAPID3_ERR_CUDA;
     }
     c->launches += 1;
@@ -226,6 +227,7 @@ int rapid3_create(rapid3_ctx** out, const rapid3_shape* shape) {
     c->encode = reinterpret_cast<EncodeTiledFn>(fn);
 
     const size_t B = shape->B_max, H = g.H, nb = g.nb;
+    c->parts = attention_parts(g, shape->B_max);
     bool ok = cudaMalloc(&c->pooled, 2 * B * H * nb * g.D * sizeof(double)) == cudaSuccess &&
               cudaMalloc(&c->scores, B * H * nb * nb * sizeof(float)) == cudaSuccess &&
               cudaMalloc(&c->bitmask, B * H * nb * c->words * sizeof(uint64_t)) == cudaSuccess &&
@@ -236,6 +238,7 @@ int rapid3_create(rapid3_ctx** out, const rapid3_shape* shape) {
               cudaMemset(c->status, 0, sizeof(int)) == cudaSuccess &&
               cudaMalloc(&c->plan, sizeof(DevPlan)) == cudaSuccess &&
               cudaMemset(c->plan, 0, sizeof(DevPlan)) == cudaSuccess;
+    if (ok && c->parts.any()) ok = cudaMalloc(&c->parts.partial, attention_partial_bytes(g, shape->B_max, c->parts)) == cudaSuccess;
     if (!ok) {
         cudaGetLastError();
         rapid3_destroy(c);
@@ -260,6 +263,7 @@ int rapid3_destroy(rapid3_ctx* c) {
     cudaFree(c->row_keep);
     cudaFree(c->status);
     cudaFree(c->plan);
+    cudaFree(c->parts.partial);
     for (void* s : c->stage) cudaFree(s);
     if (c->up_s) cudaStreamDestroy(c->up_s);
     if (c->down_s) cudaStreamDestroy(c->down_s);

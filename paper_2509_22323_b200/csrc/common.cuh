@@ -58,6 +58,19 @@ struct TensorGeom {
     long long stride_b, stride_h, stride_n;   // elements
 };
 
+// Into how many parts the attention cuts the list of a quad of query blocks: of a dense image, of a sparse image's quads with
+// text rows, of its other quads; and where the parts leave their results.
+struct AttnParts {
+    int dense = 1, text = 1, light = 1;
+    float4* partial = nullptr;       // attention_partial_bytes()
+    __host__ __device__ bool any() const { return dense > 1 || text > 1 || light > 1; }
+};
+// Units of work of an attention launch over n_img images, n_dense of them dense.
+__host__ __device__ inline int attention_units(const TensorGeom& g, const AttnParts& parts, int n_img, int n_dense) {
+    const int nq = (g.nb + 3) / 4, t = (g.n_text_blocks + 3) / 4, ntq = t < nq ? t : nq;
+    return g.H * (n_dense * nq * parts.dense + (n_img - n_dense) * (ntq * parts.text + (nq - ntq) * parts.light));
+}
+
 // Programmatic dependent launch: every kernel of a step is launched so that it may start while the kernel before it in the stream
 // is still running, and must call grid_dependency_wait() before it touches anything that kernel writes (and read it past
 // the L1, whose lines the wait is not known to refresh); the kernel before it calls grid_dependency_launch() to let it
@@ -140,7 +153,11 @@ cudaError_t launch_attention(const CUtensorMap& tmq, const CUtensorMap& tmk, con
                              void* out, const TensorGeom& g, const ImgList& imgs, const int32_t* kept_idx,
                              const int32_t* kept_cnt, const uint64_t* bitmask, float softmax_scale, int* status,
                              cudaStream_t s, const DevPlan* plan = nullptr, int n_cap = 0, int inject_stop_group = -1,
-                             bool wait_first = true);   // false: after the selection kernel, for whose masks the quads of sparse images wait themselves
+                             bool wait_first = true,
+                             // with `parts` lists may be worked on in parts, in one launch more (added to *launches)
+                             const AttnParts* parts = nullptr, int64_t* launches = nullptr);   // false: after the selection kernel, for whose masks the quads of sparse images wait themselves
+AttnParts attention_parts(const TensorGeom& g, int n_img);     // without its pointers
+size_t attention_partial_bytes(const TensorGeom& g, int n_img, const AttnParts& parts);
 // Kernel attributes on the current device; set when a context is created (scoring: also by the context-free entry).
 cudaError_t attention_static_init();
 cudaError_t scoring_static_init();

@@ -33,6 +33,8 @@
 // (two of them and O at 128 for D = 128; three and O at 192 for D = 64, where the columns allow it).
 // Every mbarrier wait is bounded; a wait that runs out records RAPID3_ERR_TIMEOUT in the status
 // word and the thread block drains its copies, releases its TMEM and exits normally.
+#include <algorithm>
+
 #include "common.cuh"
 #include "ptx.cuh"
 
@@ -62,6 +64,9 @@ constexpr int MAX_STAGES = 8;
 // another SM could have started.
 // (2, 4 and 10 measured the same.)
 constexpr int TAKE_AHEAD = 4;
+// Parts of a list; units of work whose results lie in memory between the attention kernel and add_parts_kernel (62 MB at
+// D = 128); the shortest rows, in key blocks, and the most quads with which attention_parts() looks for a cut at all.
+constexpr int MAX_PARTS = 8, MAX_LEFT = 444, MIN_CUT = 24, MAX_CUT = 600;
 // After a wait has run out the softmax warps go on for up to this many key blocks, each a wait of 16 polls of about 8 us.
 // (Over the whole of a quad, with 256 polls a block, that was 2.06 s at two heads of 1024 key blocks; now 4.7 ms.)
 constexpr int ABORT_EVERY = 32;
@@ -77,7 +82,7 @@ struct AttnParams {
     const DevPlan* plan;           // optional: image list and n_dense from device memory (grid sized for n_cap images)
     int* status;
     float scale_log2;
-    int halves;                    // 1: a unit of work is one tile of a quad, the other tile of its thread block idles
+    AttnParts parts;               // SPLIT build: how many units of work the union list of a quad goes to
     bool wait_first;               // nothing is read before the kernel in front has ended
     int stop_group;                // failure-injection build of the kernel only: the producer stops before this group
 };
@@ -99,6 +104,7 @@ struct Quad {
     int n_u;                            // entries of the union list; -1: no more quads
     int b, h;                           // image, head (of the tensors)
     int tok[4];                         // first token of the quad's query blocks (>= N: there is no such block); tile t: 2 t, 2 t + 1
+    int part, parts, store;             // SPLIT build: this unit's part of the quad's list, of how many; where part 0 leaves its results
     uint32_t ent[RAPID3_MAX_NB];        // ascending key blocks: ENT_BLK up; bit a: query block a keeps it; ENT_TAIL
 };
 
@@ -115,9 +121,12 @@ struct __align__(16) Ctl {
     int n_early;                        // groups of the first quad that the list warp has loaded
     volatile int abort_flag;
     uint32_t bm[4][32];                 // the list warp's scratch
+    float nm[SOFTMAX_WARPS][16];        // SPLIT build: the reference maxima of a warp's rows, times -c2, as they last moved
     Quad quad[2];
 };
 constexpr uint32_t ENT_TAIL = 16u;      // the sequence ends inside this key block
+template <int D>
+constexpr int PARTIAL_F4 = D / 8 + 1;   // float4 that a lane leaves of a part: its share of O; reference maxima and sums of its two rows
 constexpr int ENT_BLK = 8;              // the block's number from this bit on
 constexpr int QUAD_USERS = SOFTMAX_WARPS + 3;   // warps that read a quad
 
@@ -128,6 +137,22 @@ __device__ __forceinline__ float max3(float a, float b, float c) {
     float d;
     asm("max.f32 %0, %1, %2, %3;" : "=f"(d) : "f"(a), "f"(b), "f"(c));
     return d;
+}
+
+// Which two of the quad's four query blocks form a 128-row tile: neighbours, or, when a row of the image
+// grid spans two blocks (pair_stride 2), vertical neighbours (i, i + 2), whose kept lists overlap far more
+// (measured on the 128 x 128 grid at keep ratio 0.25: 90 % against 63 % of the tile's MMA work lands on
+// kept 64 x 64 sub-tiles).  pair_stride 3 goes further on that grid: the whole quad is one column of it --
+// members (i, i + 2, i + 4, i + 6), the left or the right halves of four consecutive grid rows -- so both
+// tiles want nearly the same key blocks (union of the quad 98 instead of 134 blocks at keep ratio 0.25,
+// both tiles busy on 68 % of them instead of 23 %).
+__device__ __forceinline__ int quad_block(const TensorGeom& g, int quad, int a) {
+    int q = 4 * quad + (g.pair_stride == 2 ? ((a & 1) << 1) + (a >> 1) : a);
+    if (g.pair_stride == 3 && q >= g.n_text_blocks) {
+        const int r = q - g.n_text_blocks, w = r & 7;
+        q = g.n_text_blocks + (r & ~7) + ((w & 3) << 1) + (w >> 2);
+    }
+    return q;
 }
 
 // Lane c of a quad of lanes holds words 0..3 of column pairs (c, c + 4, c + 8, c + 12); afterwards it holds words
@@ -158,10 +183,15 @@ __device__ __forceinline__ void row_maxima(const uint32_t (&r)[32], float& lo, f
 // stops before group prm.stop_group and every wait gives up after 2^12 polls, so the waits of all
 // roles run out and the abort path (status word, drain of the copies in flight, UMMA drain, TMEM
 // release) is what runs.  The product launches only use INJECT = false.
-template <int D, bool INJECT = false>
+//
+// SPLIT = true is the build for contexts whose quads leave SMs without work: the union list of a quad is cut into
+// parts of equal length, each a unit of work (attention_parts() says how many).  A softmax warp leaves its rows of a part -- O,
+// not divided by the row sums, the sums and the reference maxima -- in global memory, and add_parts_kernel makes the result
+// of them.  (Added up by the last part of a quad to arrive, in this kernel, they cost its main loop 12 to 14 %: registers.)
+template <int D, bool INJECT = false, bool SPLIT = false>
 __global__ void __launch_bounds__(NTHREADS, 1)
 attn_kernel(const __grid_constant__ CUtensorMap tmq, const __grid_constant__ CUtensorMap tmk,
-            const __grid_constant__ CUtensorMap tmv, uint16_t* __restrict__ out, const AttnParams prm) {
+            const __grid_constant__ CUtensorMap tmv, uint16_t* __restrict__ out, const __grid_constant__ AttnParams prm) {
     using C = Cfg<D>;
     constexpr int DH = C::DH, KS = C::KS, VS = C::VS, NBUF = C::NBUF, O_COL = C::O_COL;
     extern __shared__ uint8_t smem_raw[];
@@ -177,7 +207,15 @@ attn_kernel(const __grid_constant__ CUtensorMap tmq, const __grid_constant__ CUt
     const int warp = __shfl_sync(0xffffffffu, tid / 32, 0);
     const TensorGeom& g = prm.g;
     const int nb = g.nb, N = g.N;
-    const int n_quads = (((nb + 3) >> 2) * g.H * (prm.plan ? __ldcg(&prm.plan->all.n) : prm.imgs.n)) << prm.halves;
+    const int n_images = prm.plan ? __ldcg(&prm.plan->all.n) : prm.imgs.n;
+    int n_quads = ((nb + 3) >> 2) * g.H * n_images;      // units of work: quads, ...
+    if constexpr (SPLIT) n_quads = attention_units(g, prm.parts, n_images, prm.plan ? __ldcg(&prm.plan->n_dense) : prm.n_dense);   // ... parts, ...
+    // ... or halves of either: where the two tiles of every unit find an SM each, they go to two thread blocks.  A tile that
+    // has the SM to itself goes through its key blocks in 0.66 and 0.56 us (D = 128, 64), where two that share it take 0.84 and
+    // 0.72 (whole steps of one image: 6 heads x 11 blocks 16.4 -> 13.8 us, 2 heads x 22 blocks at D = 64 26.3 -> 23.8; with more
+    // tiles than SMs the shared K and V stream wins).
+    const int halves = 2 * n_quads <= SM_COUNT ? 1 : 0;
+    n_quads <<= halves;
     if ((int)blockIdx.x >= n_quads) {                    // device-resident plan: fewer images than the grid covers
         // When none attends, no other thread block waits for the selection kernel: the grid must not end before that does
         // (it may still have the plan to read, which the next call rewrites).
@@ -282,6 +320,8 @@ attn_kernel(const __grid_constant__ CUtensorMap tmq, const __grid_constant__ CUt
         }
     };
 
+    // the pool is the launch's 640 x 96: 512 x 104 + 128 x 64
+    if (SPLIT && warp >= SOFTMAX_WARPS) reg_dec<64>();
     if (warp == LIST_WARP) {
         // ------------------------------------------------------------ quads and their union lists
         // one lane polls: these waits are long, and the other lanes' polls would only take issue slots
@@ -305,13 +345,39 @@ attn_kernel(const __grid_constant__ CUtensorMap tmq, const __grid_constant__ CUt
             // block walk all nb key blocks; the other quads of the sparse images follow, image by image in the list's
             // order (descending keep ratio).
             int quad, h, p;
-            const int half = prm.halves ? L & 1 : -1;    // the tile to work on, or both
-            L >>= prm.halves;
+            const int half = halves ? L & 1 : -1;    // the tile to work on, or both
+            L >>= halves;
+            int part = 0, parts = 1;
             {
                 const int nq = (nb + 3) >> 2, ntq = min(nq, (g.n_text_blocks + 3) >> 2);
                 const int n_all = prm.plan ? __ldcg(&prm.plan->all.n) : prm.imgs.n;
                 const int nd = prm.plan ? __ldcg(&prm.plan->n_dense) : prm.n_dense, ns = n_all - nd;
                 const int heavy_dense = nd * g.H * nq, heavy_sparse = ns * g.H * ntq;
+                if constexpr (SPLIT) {                   // in units first: the parts of a quad follow one another
+                    const AttnParts& ap = prm.parts;
+                    const int ud = heavy_dense * ap.dense, ut = heavy_sparse * ap.text;
+                    int store = 0, quads = 0;            // units before these that leave results; quads before these
+                    if (L < ud) {
+                        parts = ap.dense;
+                    } else if (L < ud + ut) {
+                        L -= ud;
+                        parts = ap.text;
+                        store = ap.dense > 1 ? ud : 0;
+                        quads = heavy_dense;
+                    } else {
+                        L -= ud + ut;
+                        parts = ap.light;
+                        store = (ap.dense > 1 ? ud : 0) + (ap.text > 1 ? ut : 0);
+                        quads = heavy_dense + heavy_sparse;
+                    }
+                    part = L % parts;
+                    if (lane == 0) u.store = store + L - part;
+                    L = quads + L / parts;
+                    if (lane == 0) {
+                        u.part = part;
+                        u.parts = parts;
+                    }
+                }
                 if (L < heavy_dense) {
                     p = L / (g.H * nq); L -= p * g.H * nq;
                     h = L / nq; quad = L - h * nq;
@@ -328,22 +394,12 @@ attn_kernel(const __grid_constant__ CUtensorMap tmq, const __grid_constant__ CUt
             }
             const int b = prm.plan ? __ldcg(&prm.plan->all.batch[p]) : prm.imgs.batch[p];
             const int slot = prm.plan ? __ldcg(&prm.plan->all.slot[p]) : prm.imgs.slot[p];
-            // Which two of the quad's four query blocks form a 128-row tile: neighbours, or, when a row of the image
-            // grid spans two blocks (pair_stride 2), vertical neighbours (i, i + 2), whose kept lists overlap far more
-            // (measured on the 128 x 128 grid at keep ratio 0.25: 90 % against 63 % of the tile's MMA work lands on
-            // kept 64 x 64 sub-tiles).  pair_stride 3 goes further on that grid: the whole quad is one column of it --
-            // members (i, i + 2, i + 4, i + 6), the left or the right halves of four consecutive grid rows -- so both
-            // tiles want nearly the same key blocks (union of the quad 98 instead of 134 blocks at keep ratio 0.25,
-            // both tiles busy on 68 % of them instead of 23 %).  qblk(a) is member a's query block.
-            auto qblk = [&](int a) -> int {
+            auto qblk = [&](int a) -> int {              // member a's query block
                 if (half >= 0 && (a >> 1) != half) return nb;           // not of this unit: like a block past the end
-                int q = 4 * quad + (g.pair_stride == 2 ? ((a & 1) << 1) + (a >> 1) : a);
-                if (g.pair_stride == 3 && q >= g.n_text_blocks) {
-                    const int r = q - g.n_text_blocks, w = r & 7;
-                    q = g.n_text_blocks + (r & ~7) + ((w & 3) << 1) + (w >> 2);
-                }
-                return q;
+                return quad_block(g, quad, a);
             };
+            // the query block whose kept blocks m[a] below holds: where a list is cut into parts depends on the whole quad
+            auto mblk = [&](int a) -> int { return SPLIT && parts > 1 ? quad_block(g, quad, a) : qblk(a); };
             if (lane == 0) {
                 u.b = b;
                 u.h = g.h0 + h;
@@ -355,7 +411,8 @@ attn_kernel(const __grid_constant__ CUtensorMap tmq, const __grid_constant__ CUt
                     // row, so the union list starts 0, 1, ....  First use of their stages, nothing to wait for.
                     load_q(u);
                     const bool none = min(min(qblk(0), qblk(1)), min(qblk(2), qblk(3))) >= nb;   // the second half of a ragged last quad
-                    const int n_early = (!INJECT && !none && (slot < 0 || prm.bitmask32 != nullptr)) ? min(min(slot < 0 ? nb : g.n_text_blocks, nb), KS) : 0;
+                    int n_early = (!INJECT && !none && (slot < 0 || prm.bitmask32 != nullptr)) ? min(min(slot < 0 ? nb : g.n_text_blocks, nb), KS) : 0;
+                    if (SPLIT && parts > 1) n_early = part == 0 ? min(n_early, (slot < 0 ? nb : g.n_text_blocks) / parts) : 0;   // its part of the list is no shorter
                     for (int gi = 0; gi < n_early; ++gi) issue_group(u, gi, gi, gi - 1, gi - 1);
                     ctl->n_early = n_early;
                 }
@@ -368,7 +425,7 @@ attn_kernel(const __grid_constant__ CUtensorMap tmq, const __grid_constant__ CUt
                 const int n = min(max(nb - lane * 32, 0), 32);
                 const uint32_t val = n == 32 ? 0xffffffffu : ((1u << n) - 1u);
 #pragma unroll
-                for (int a = 0; a < 4; ++a) m[a] = qblk(a) < nb ? val : 0u;
+                for (int a = 0; a < 4; ++a) m[a] = mblk(a) < nb ? val : 0u;
             } else {
                 // Launched as a dependent of the selection kernel, the masks have to be waited for once.  They are read
                 // past the L1 (ld.global.cg): this thread block may have started before they were written, and an L1
@@ -378,15 +435,15 @@ attn_kernel(const __grid_constant__ CUtensorMap tmq, const __grid_constant__ CUt
                 if (prm.bitmask32 != nullptr) {
 #pragma unroll
                     for (int a = 0; a < 4; ++a)
-                        m[a] = (qblk(a) < nb && lane < nw)
-                                   ? __ldcg(prm.bitmask32 + (((long long)slot * g.H + h) * nb + qblk(a)) * prm.words32 + lane) : 0u;
+                        m[a] = (mblk(a) < nb && lane < nw)
+                                   ? __ldcg(prm.bitmask32 + (((long long)slot * g.H + h) * nb + mblk(a)) * prm.words32 + lane) : 0u;
                 } else {
 #pragma unroll
                     for (int a = 0; a < 4; ++a) ctl->bm[a][lane] = 0u;
                     __syncwarp();
                     for (int a = 0; a < 4; ++a) {
-                        if (qblk(a) >= nb) continue;
-                        const long long row = ((long long)slot * g.H + h) * nb + qblk(a);
+                        if (mblk(a) >= nb) continue;
+                        const long long row = ((long long)slot * g.H + h) * nb + mblk(a);
                         const int cnt = min(max(__ldcg(prm.kept_cnt + row), 0), nb);
                         const int32_t* lst = prm.kept_idx + row * nb;
                         for (int e = lane; e < cnt; e += 32) {
@@ -401,15 +458,27 @@ attn_kernel(const __grid_constant__ CUtensorMap tmq, const __grid_constant__ CUt
                 }
             }
             // the position of a key block in the ascending union list is the number of union bits below it
-            const uint32_t un = m[0] | m[1] | m[2] | m[3];
-            int below = __popc(un);
+            auto union_bits_below = [&](uint32_t bits, int& all) -> int {
+                int x = __popc(bits);
 #pragma unroll
-            for (int o = 1; o < 32; o <<= 1) {
-                const int v = __shfl_up_sync(0xffffffffu, below, o);
-                if (lane >= o) below += v;
+                for (int o = 1; o < 32; o <<= 1) {
+                    const int v = __shfl_up_sync(0xffffffffu, x, o);
+                    if (lane >= o) x += v;
+                }
+                all = __shfl_sync(0xffffffffu, x, 31);
+                return x - __popc(bits);
+            };
+            int n_u;
+            if (SPLIT && parts > 1) {                    // of the quad's union, the blocks from `first` up to `last` are this part's
+                uint32_t from = m[0] | m[1] | m[2] | m[3], to = from;
+                const int at = union_bits_below(from, n_u), first = n_u * part / parts, last = n_u * (part + 1) / parts;
+                for (int x = min(max(first - at, 0), 32); x > 0; --x) from &= from - 1u;
+                for (int x = min(max(last - at, 0), 32); x > 0; --x) to &= to - 1u;
+#pragma unroll
+                for (int a = 0; a < 4; ++a) m[a] &= qblk(a) < nb ? from & ~to : 0u;
             }
-            const int n_u = __shfl_sync(0xffffffffu, below, 31);
-            below -= __popc(un);
+            const uint32_t un = m[0] | m[1] | m[2] | m[3];
+            const int below = union_bits_below(un, n_u);
             for (int w = 0; w < nw; ++w) {
                 const uint32_t uw = __shfl_sync(0xffffffffu, un, w);
                 const int pos = __shfl_sync(0xffffffffu, below, w) + __popc(uw & ((1u << lane) - 1u));
@@ -607,6 +676,7 @@ attn_kernel(const __grid_constant__ CUtensorMap tmq, const __grid_constant__ CUt
         // (r_lo = lane / 4 and r_lo + 8 of the sixteen) and, of every group of eight score columns, the pair
         // 2 (lane % 4), + 1 -- 32 scores per key block.  The four threads of a quad share their rows' maximum
         // with two shuffles, and only when some row of the warp may have grown.
+        if (SPLIT) reg_inc<104>();
         const int t = (warp >> 2) & 1, wl = warp & 3, hf = warp >> 3;
         const int a = 2 * t + (wl >> 1);               // query block of the quad
         const uint32_t tile_bits = 3u << (2 * t), act_bit = 1u << a;
@@ -616,6 +686,7 @@ attn_kernel(const __grid_constant__ CUtensorMap tmq, const __grid_constant__ CUt
         const uint32_t tO = lane_addr + O_COL;
         const uint32_t bSFt = bSF + 24 * t, bPFt = bPF + 24 * t, bPVt = bPV + 16 * t;
         const float c2 = prm.scale_log2;
+        float* const ref = &ctl->nm[warp][lane >> 2];  // of the thread's rows: a thread of each quad writes it, all of them read it
         const int tail_valid = N - (nb - 1) * 64;      // valid tokens of the last block (1..64)
         int n = 0;                                     // blocks of this tile so far, in all quads
         uint32_t n_o = 0;                              // quads so far in which the tile had blocks
@@ -629,6 +700,7 @@ attn_kernel(const __grid_constant__ CUtensorMap tmq, const __grid_constant__ CUt
         float l0 = 0.f, l1 = 0.f, l2 = 0.f, l3 = 0.f;  // partial row sums: (l0, l1) first row, (l2, l3) second row
         uint32_t r[32];
         const int n0 = n;
+        if (SPLIT && cg == 0) ref[0] = ref[8] = INFINITY;
         bool seeded = false;                           // the rows' reference maxima have been set (warp-uniform: a warp's rows share a query block)
         // A wait that runs out sets the abort flag; nothing up to the end of a quad depends on a wait's result, so no vote is
         // taken on the way, and the flag is looked at every ABORT_EVERY key blocks only.
@@ -673,6 +745,7 @@ attn_kernel(const __grid_constant__ CUtensorMap tmq, const __grid_constant__ CUt
                     row_maxima(r, nm_lo, nm_hi);
                     nm_lo *= -c2; nm_hi *= -c2;
                     seeded = true;
+                    if (SPLIT && cg == 0) { ref[0] = nm_lo; ref[8] = nm_hi; }
                 }
                 for (;;) {
                     b0 = b1 = b2 = b3 = 0.f;
@@ -724,6 +797,7 @@ attn_kernel(const __grid_constant__ CUtensorMap tmq, const __grid_constant__ CUt
                         }
                         if (g_lo) nm_lo = mx_lo;
                         if (g_hi) nm_hi = mx_hi;
+                        if (SPLIT && cg == 0) { ref[0] = nm_lo; ref[8] = nm_hi; }
                     }
                 }
                 l0 += b0; l1 += b1; l2 += b2; l3 += b3;
@@ -742,7 +816,39 @@ attn_kernel(const __grid_constant__ CUtensorMap tmq, const __grid_constant__ CUt
         if (n > n0) wait(bOD + 8 * t, n_o++ & 1);
         if (!(ok = __all_sync(0xffffffffu, !ctl->abort_flag))) break;
         // epilogue: O / l -> bf16 -> 16 bytes a lane, four lanes a 64-byte piece of a row
-        {
+        if (SPLIT && u.parts > 1) {
+            // a part of the list: O as it is, the row sums and the reference maxima go to memory
+            tc_fence_after();
+            if (u.tok[a] < N) {                        // the same in every part of the quad
+                uint32_t at = warp * (PARTIAL_F4<D> * 32) + lane;
+                float4* mine = prm.parts.partial + (size_t)(u.store + u.part) * (SOFTMAX_WARPS * PARTIAL_F4<D> * 32) + at;
+                uint32_t o[16];
+#pragma unroll 1
+                for (int ch = 0; ch < D / 32; ++ch) {
+                    if (n > n0) {
+                        tmem_ld16x256_x4(tO + ch * 32, o);
+                        tc_wait_ld();
+                    } else {
+#pragma unroll
+                        for (int e = 0; e < 16; ++e) o[e] = 0u;
+                    }
+#pragma unroll
+                    for (int k = 0; k < 4; ++k)
+                        __stcg(mine + 32 * (4 * ch + k), make_float4(__uint_as_float(o[4 * k]), __uint_as_float(o[4 * k + 1]),
+                                                                     __uint_as_float(o[4 * k + 2]), __uint_as_float(o[4 * k + 3])));
+                }
+                __syncwarp();                          // for `ref`
+                float s_lo = l0 + l1, s_hi = l2 + l3;
+                s_lo += __shfl_xor_sync(0xffffffffu, s_lo, 1);
+                s_hi += __shfl_xor_sync(0xffffffffu, s_hi, 1);
+                s_lo += __shfl_xor_sync(0xffffffffu, s_lo, 2);
+                s_hi += __shfl_xor_sync(0xffffffffu, s_hi, 2);
+                __stcg(mine + 32 * (PARTIAL_F4<D> - 1), make_float4(ref[0], ref[8], s_lo, s_hi));
+            }
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(bUE + 8 * (i & 1));
+        } else {
             tc_fence_after();
             float s_lo = l0 + l1, s_hi = l2 + l3;      // the quad's four partial sums make the row sum
             s_lo += __shfl_xor_sync(0xffffffffu, s_lo, 1);
@@ -802,6 +908,89 @@ attn_kernel(const __grid_constant__ CUtensorMap tmq, const __grid_constant__ CUt
     }
 }
 
+// The results of the quads whose lists were worked on in parts: what the parts have left, added up in the order of the list.
+// A warp does a softmax warp's sixteen rows, 32 channels of them, with every part's loads in flight at once: bound by two round
+// trips to the L2.  The lanes hold what the attention kernel's lanes held.
+template <int D>
+__global__ void __launch_bounds__(128) add_parts_kernel(uint16_t* __restrict__ out, const TensorGeom g, const __grid_constant__ ImgList imgs,
+                                                        int n_dense, const DevPlan* plan, const AttnParts ap) {
+    constexpr int CH = D / 32;
+    constexpr size_t part_f4 = (size_t)SOFTMAX_WARPS * PARTIAL_F4<D> * 32;
+    const int lane = threadIdx.x % 32, cg = lane & 3;
+    grid_dependency_wait();
+    grid_dependency_launch();
+    const int item = blockIdx.x * 4 + threadIdx.x / 32, warp = item / CH % SOFTMAX_WARPS, ch = item % CH;
+    const int nq = (g.nb + 3) >> 2, ntq = min(nq, (g.n_text_blocks + 3) >> 2), nl = nq - ntq;
+    const int nd = plan ? __ldcg(&plan->n_dense) : n_dense, ns = (plan ? __ldcg(&plan->all.n) : imgs.n) - nd;
+    const int qd = ap.dense > 1 ? nd * g.H * nq : 0, qt = ap.text > 1 ? ns * g.H * ntq : 0, ql = ap.light > 1 ? ns * g.H * nl : 0;
+    int x = item / CH / SOFTMAX_WARPS, p, h, quad, parts, store;
+    if (x < qd) {
+        parts = ap.dense; store = x * parts;
+        p = x / (g.H * nq); x -= p * g.H * nq;
+        h = x / nq; quad = x - h * nq;
+    } else if (x < qd + qt) {
+        x -= qd;
+        parts = ap.text; store = qd * ap.dense + x * parts;
+        p = x / (g.H * ntq); x -= p * g.H * ntq; p += nd;
+        h = x / ntq; quad = x - h * ntq;
+    } else {
+        x -= qd + qt;
+        if (x >= ql) return;
+        parts = ap.light; store = qd * ap.dense + qt * ap.text + x * parts;
+        p = x / (g.H * nl); x -= p * g.H * nl; p += nd;
+        h = x / nl; quad = ntq + x - h * nl;
+    }
+    const int tok_lo = 64 * quad_block(g, quad, 2 * ((warp >> 2) & 1) + ((warp & 3) >> 1)) + (warp & 1) * 32 + (warp >> 3) * 16 + (lane >> 2);
+    const int tok_hi = tok_lo + 8;
+    if (tok_lo - (lane >> 2) >= g.N) return;             // nothing was left for rows past the end
+    const int b = plan ? __ldcg(&plan->all.batch[p]) : imgs.batch[p];
+    const float4* base = ap.partial + (size_t)store * part_f4 + (size_t)warp * PARTIAL_F4<D> * 32 + lane;
+    float4 v[MAX_PARTS], x4[MAX_PARTS][4];
+#pragma unroll
+    for (int i = 0; i < MAX_PARTS; ++i) {
+        v[i] = make_float4(INFINITY, INFINITY, 0.f, 0.f);
+        if (i < parts) {
+            v[i] = __ldcg(base + i * part_f4 + 32 * (PARTIAL_F4<D> - 1));
+#pragma unroll
+            for (int k = 0; k < 4; ++k) x4[i][k] = __ldcg(base + i * part_f4 + 32 * (4 * ch + k));
+        }
+    }
+    float m_lo = INFINITY, m_hi = INFINITY, s_lo = 0.f, s_hi = 0.f;      // maxima times -c2
+#pragma unroll
+    for (int i = 0; i < MAX_PARTS; ++i) {
+        m_lo = fminf(m_lo, v[i].x);
+        m_hi = fminf(m_hi, v[i].y);
+    }
+    float f[16];
+#pragma unroll
+    for (int e = 0; e < 16; ++e) f[e] = 0.f;
+#pragma unroll
+    for (int i = 0; i < MAX_PARTS; ++i)
+        if (i < parts) {
+            // a part in which a row kept nothing (no maximum) counts for nothing
+            const float w_lo = v[i].x == INFINITY ? 0.f : ex2(m_lo - v[i].x), w_hi = v[i].y == INFINITY ? 0.f : ex2(m_hi - v[i].y);
+            s_lo = fmaf(w_lo, v[i].z, s_lo);
+            s_hi = fmaf(w_hi, v[i].w, s_hi);
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                f[4 * k] = fmaf(w_lo, x4[i][k].x, f[4 * k]); f[4 * k + 1] = fmaf(w_lo, x4[i][k].y, f[4 * k + 1]);
+                f[4 * k + 2] = fmaf(w_hi, x4[i][k].z, f[4 * k + 2]); f[4 * k + 3] = fmaf(w_hi, x4[i][k].w, f[4 * k + 3]);
+            }
+        }
+    const float inv_lo = s_lo > 0.f ? 1.f / s_lo : 0.f, inv_hi = s_hi > 0.f ? 1.f / s_hi : 0.f;
+    uint32_t a_lo[4], a_hi[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        a_lo[k] = pack_bf16(f[4 * k] * inv_lo, f[4 * k + 1] * inv_lo);
+        a_hi[k] = pack_bf16(f[4 * k + 2] * inv_hi, f[4 * k + 3] * inv_hi);
+    }
+    const uint4 o_lo = quad_transpose(a_lo[0], a_lo[1], a_lo[2], a_lo[3], cg);
+    const uint4 o_hi = quad_transpose(a_hi[0], a_hi[1], a_hi[2], a_hi[3], cg);
+    uint16_t* o = out + (long long)b * g.stride_b + (long long)(g.h0 + h) * g.stride_h + (long long)tok_lo * g.stride_n + 8 * cg + 32 * ch;
+    if (tok_lo < g.N) *reinterpret_cast<uint4*>(o) = o_lo;
+    if (tok_hi < g.N) *reinterpret_cast<uint4*>(o + 8 * g.stride_n) = o_hi;
+}
+
 bool g_attr_set = false;
 
 }  // namespace
@@ -811,6 +1000,12 @@ cudaError_t attention_static_init() {
                                          (int)attn_smem_bytes<128>());
     if (e != cudaSuccess) return e;
     e = cudaFuncSetAttribute(attn_kernel<64>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)attn_smem_bytes<64>());
+    if (e != cudaSuccess) return e;
+    e = cudaFuncSetAttribute(attn_kernel<128, false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             (int)attn_smem_bytes<128>());
+    if (e != cudaSuccess) return e;
+    e = cudaFuncSetAttribute(attn_kernel<64, false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             (int)attn_smem_bytes<64>());
     if (e != cudaSuccess) return e;
     e = cudaFuncSetAttribute(attn_kernel<128, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              (int)attn_smem_bytes<128>());
@@ -822,11 +1017,106 @@ cudaError_t attention_static_init() {
     return cudaSuccess;
 }
 
+// When the last SM is through with the units of work of three classes, n[i] of t[i] us, handed out in this order as SMs are free.
+static double units_time(const int (&n)[3], const double (&t)[3]) {
+    struct Group { double at; int sms; } group[5] = {{0.0, SM_COUNT}};   // SMs by when they are free
+    int groups = 1;
+    double end = 0.0;
+    for (int i = 0; i < 3; ++i)
+        for (int left = n[i]; left > 0;) {
+            int g = 0;
+            for (int j = 1; j < groups; ++j)
+                if (group[j].at < group[g].at) g = j;
+            if (left < group[g].sms) {                   // some of the group's SMs stay free
+                group[groups++] = {group[g].at, group[g].sms - left};
+                group[g].sms = left;
+            }
+            left -= group[g].sms;
+            group[g].at += t[i];
+            end = std::max(end, group[g].at);
+        }
+    return end;
+}
+
+// Units of work whose results are left in memory, at most, in a launch of such a context.
+static size_t left_units(const TensorGeom& g, int n_img, const AttnParts& parts) {
+    const int nq = (g.nb + 3) / 4, ntq = std::min(nq, (g.n_text_blocks + 3) / 4);
+    const int d = parts.dense > 1 ? nq * parts.dense : 0;
+    const int s = (parts.text > 1 ? ntq * parts.text : 0) + (parts.light > 1 ? (nq - ntq) * parts.light : 0);
+    return (size_t)std::max(d, s) * g.H * n_img;
+}
+
+// Into how many parts the attention of a context of up to n_img images cuts the lists of its quads.  What an image gets must
+// not depend on the launch it is in, so this is the context's and the image's own: quads of a dense image, of a sparse one's
+// text rows (which keep every block), and the others.  Of all cuts, the one with the best times over these launches: every image
+// dense; all sparse, the other quads' unions holding 0.3, 0.6 or 0.9 of the blocks; half of them dense; half of them
+// attending at all.  It must be 10 % better than whole lists in the mean and in none of them worse by more than 2 %.  The
+// times: 0.72 and 0.84 us a key block (D = 64, 128), 0.56 and 0.66 us where a tile has its SM to itself, 1 us a unit; a
+// part's write 1 and 2 us, add_parts_kernel 3.5 us and what was left at 4.5 TB/s (1.5 us where it finds nothing).  Short rows
+// (MIN_CUT) are left whole: their calls wait for the host, whom one more launch costs 2 us.
+// Attention alone, us, whole lists / parts: 18 quads of 72 blocks 46.8 / 16.7 (D = 64, eight parts), 54.1 / 20.9 (D = 128);
+// 36 quads of 72 47.3 / 23.2, 55.0 / 30.0 (four); 18 of 33 24.9 / 13.6 (eight), 28.6 / 16.2 (four); 72 of 72 48.6 / 36.7,
+// 56.3 / 47.1 (two); 60 of 12 13.7 / 15.7, 15.5 / 21.0 (two).  Steps: 46 quads of 92 blocks at ratio 0.25, D = 64 61.6 / 31.8
+// (text rows in five, the others in three); 132 of 264 at ratio 0.2, D = 128 231 / 135 (text rows in four); 198 of 262 at ratios
+// 1, 0.5 and 0.2, D = 64 359, 289 and 196 / 289, 237 and 148 (in two, text rows in three).
+AttnParts attention_parts(const TensorGeom& g, int n_img) {
+    AttnParts best;
+    const int nq = (g.nb + 3) / 4, ntq = std::min(nq, (g.n_text_blocks + 3) / 4);
+    if (g.nb < MIN_CUT || (long long)nq * g.H * n_img > MAX_CUT) return best;
+    const bool wide = g.D == 128;
+    auto time = [&](int dense, int sparse, double held, const AttnParts& p) {
+        const int quads[3] = {nq * g.H * dense, ntq * g.H * sparse, (nq - ntq) * g.H * sparse}, parts[3] = {p.dense, p.text, p.light};
+        const double blocks[3] = {(double)g.nb, (double)g.nb, held * g.nb};
+        int n[3], units = 0, left = 0;
+        for (int i = 0; i < 3; ++i) {
+            units += n[i] = quads[i] * parts[i];
+            if (parts[i] > 1) left += n[i];
+        }
+        const bool one = 2 * units <= SM_COUNT;
+        double t[3];
+        for (int i = 0; i < 3; ++i) {
+            if (one) n[i] *= 2;
+            t[i] = blocks[i] / parts[i] * (wide ? (one ? 0.66 : 0.84) : (one ? 0.56 : 0.72)) + 1.0 + (parts[i] > 1 ? g.D / 64 : 0);
+        }
+        return units_time(n, t) + 5.0 + (left > 0 ? 3.5 + left * (1.1e-3 * g.D / 4.5) : p.any() ? 1.5 : 0.0);
+    };
+    const int half = n_img / 2;
+    const struct { int dense, sparse; double held; } launches[] = {
+        {n_img, 0, 1.0}, {0, n_img, 0.3}, {0, n_img, 0.6}, {0, n_img, 0.9}, {half, n_img - half, 0.3}, {half, n_img - half, 0.6},
+        {n_img - half, 0, 1.0}, {0, n_img - half, 0.6}};
+    constexpr int N = sizeof launches / sizeof launches[0];
+    double whole[N], least = 0.9 * N;
+    for (int i = 0; i < N; ++i) whole[i] = time(launches[i].dense, launches[i].sparse, launches[i].held, AttnParts());
+    for (int pd = 1; pd <= MAX_PARTS; ++pd)
+        for (int pl = 1; pl <= MAX_PARTS; ++pl)
+            for (int pt = ntq ? pl : 1; pt <= (ntq ? MAX_PARTS : 1); ++pt) {
+                AttnParts p;
+                p.dense = pd;
+                p.text = pt;
+                p.light = pl;
+                if (!p.any() || left_units(g, n_img, p) > MAX_LEFT) continue;
+                double sum = 0.0, most = 0.0;
+                for (int i = 0; i < N && most <= 1.02 && sum < least; ++i) {
+                    const double x = time(launches[i].dense, launches[i].sparse, launches[i].held, p) / whole[i];
+                    sum += x;
+                    most = std::max(most, x);
+                }
+                if (sum < least && most <= 1.02) {
+                    least = sum;
+                    best = p;
+                }
+            }
+    return best;
+}
+size_t attention_partial_bytes(const TensorGeom& g, int n_img, const AttnParts& parts) {
+    return left_units(g, n_img, parts) * SOFTMAX_WARPS * 32 * sizeof(float4) * (g.D == 128 ? PARTIAL_F4<128> : PARTIAL_F4<64>);
+}
 cudaError_t launch_attention(const CUtensorMap& tmq, const CUtensorMap& tmk, const CUtensorMap& tmv,
                              void* out,
                              const TensorGeom& g, const ImgList& imgs, const int32_t* kept_idx,
                              const int32_t* kept_cnt, const uint64_t* bitmask, float softmax_scale, int* status,
-                             cudaStream_t s, const DevPlan* plan, int n_cap, int inject_stop_group, bool wait_first) {
+                             cudaStream_t s, const DevPlan* plan, int n_cap, int inject_stop_group, bool wait_first,
+                             const AttnParts* parts, int64_t* launches) {
     if (!g_attr_set) {
         cudaError_t e = attention_static_init();
         if (e != cudaSuccess) return e;
@@ -846,18 +1136,29 @@ cudaError_t launch_attention(const CUtensorMap& tmq, const CUtensorMap& tmk, con
     prm.plan = plan;
     prm.wait_first = wait_first;
     prm.stop_group = inject_stop_group;
-    // Where the two tiles of every quad find an SM each, they go to two thread blocks: a tile that has the SM to itself goes
-    // through its key blocks in about 0.63 of the time of two that share it (whole steps of one image, us: 2 heads x 72
-    // blocks at D = 128 70.7 -> 62.1, 6 heads x 11 blocks 16.4 -> 13.8, 2 heads x 22 blocks at D = 64 26.3 -> 23.8; with
-    // more tiles than SMs the shared K and V stream wins).
-    const int quads = ((g.nb + 3) / 4) * g.H * (plan ? n_cap : imgs.n);
-    prm.halves = 2 * quads <= SM_COUNT ? 1 : 0;
-    dim3 grid(quads << prm.halves, 1, 1);
+    const int n_img = plan ? n_cap : imgs.n, pairs = g.H * n_img, nq = (g.nb + 3) / 4, ntq = std::min(nq, (g.n_text_blocks + 3) / 4);
+    int left = 0;                              // quads whose lists are worked on in parts, at most
+    if (parts && inject_stop_group < 0) {
+        const int d = parts->dense > 1 ? nq : 0, t = (parts->text > 1 ? ntq : 0) + (parts->light > 1 ? nq - ntq : 0);
+        left = plan ? pairs * std::max(d, t) : g.H * (n_dense * d + (imgs.n - n_dense) * t);
+        if (left > 0) prm.parts = *parts;
+    }
+    const int units = plan ? std::max(attention_units(g, prm.parts, n_img, n_img), attention_units(g, prm.parts, n_img, 0))
+                           : attention_units(g, prm.parts, n_img, n_dense);
+    // halves: up to as many thread blocks as SMs.  Where a plan may hold fewer units than the largest launch, it may halve them.
+    dim3 grid(2 * units <= SM_COUNT ? 2 * units : plan ? std::max(units, SM_COUNT) : units, 1, 1);
     if (inject_stop_group >= 0) {
         if (g.D == 128)
             attn_kernel<128, true><<<grid, NTHREADS, attn_smem_bytes<128>(), s>>>(tmq, tmk, tmv, static_cast<uint16_t*>(out), prm);
         else
             attn_kernel<64, true><<<grid, NTHREADS, attn_smem_bytes<64>(), s>>>(tmq, tmk, tmv, static_cast<uint16_t*>(out), prm);
+    } else if (left > 0) {
+        cudaError_t e = launch_kernel(g.D == 128 ? attn_kernel<128, false, true> : attn_kernel<64, false, true>, grid, dim3(NTHREADS),
+                                      g.D == 128 ? attn_smem_bytes<128>() : attn_smem_bytes<64>(), s, tmq, tmk, tmv, static_cast<uint16_t*>(out), prm);
+        if (e != cudaSuccess) return e;
+        *launches += 1;
+        return launch_kernel(g.D == 128 ? add_parts_kernel<128> : add_parts_kernel<64>, dim3(left * SOFTMAX_WARPS * (g.D / 32) / 4), dim3(128), 0, s,
+                             static_cast<uint16_t*>(out), g, imgs, n_dense, plan, prm.parts);
     } else if (g.D == 128) {
         return launch_kernel(attn_kernel<128>, grid, dim3(NTHREADS), attn_smem_bytes<128>(), s, tmq, tmk, tmv, static_cast<uint16_t*>(out), prm);
     } else {

@@ -17,6 +17,12 @@ __device__ __forceinline__ uint32_t lane_id() {
     return l;
 }
 
+// Registers of this warp's group of four warps, given back to the thread block's pool or taken from it.
+template <int N>
+__device__ __forceinline__ void reg_dec() { asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(N)); }
+template <int N>
+__device__ __forceinline__ void reg_inc() { asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(N)); }
+
 // One lane of a converged warp (the same one for the whole kernel is not guaranteed).
 __device__ __forceinline__ bool elect_one() {
     uint32_t pred;
