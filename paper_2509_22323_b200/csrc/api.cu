@@ -40,6 +40,7 @@ struct rapid3_ctx {
     int32_t* row_keep = nullptr;  // [B_max][H][nb]: per-row counts of the cumulative-mass selection
     int* status = nullptr;
     AttnParts parts;              // how the attention of a small context is cut, and its workspace
+    QuadOrder order;              // the order of a step's quads, and its workspace
     DevPlan* plan = nullptr;      // device-resident plan of rapid3_gated_step_device
     // host-tensor staging of rapid3_gated_step_host (created on first use)
     void* stage[4] = {nullptr, nullptr, nullptr, nullptr};
@@ -147,10 +148,17 @@ int get_map(rapid3_ctx* c, const void* base, CUtensorMap* out) {
     return RAPID3_OK;
 }
 
+// Whether a step over n_img attending images hands its last quads out by their length, and where that is kept.
+QuadOrder step_order(const rapid3_ctx* c, const TensorGeom& g, int n_img) {
+    const int quads = attention_units(g, AttnParts(), n_img, 0);
+    return quads > ORDER_FROM && quads <= ORDER_TO ? c->order : QuadOrder();      // without pointers where the context has none
+}
+
 // `g` is the context's geometry or a copy of it narrowed to a range of heads.
 int attn_launch(rapid3_ctx* c, const TensorGeom& g, const void* q, const void* k, const void* v, void* out,
                 const ImgList& l, const int32_t* kept_idx, const int32_t* kept_cnt, const uint64_t* bitmask, float scale,
-                cudaStream_t st, const DevPlan* plan = nullptr, int n_cap = 0, bool after_select = false) {
+                cudaStream_t st, const DevPlan* plan = nullptr, int n_cap = 0, bool after_select = false,
+                const QuadOrder& order = QuadOrder()) {
     CUtensorMap tq, tk, tv;
     int r;
     if ((r = get_map(c, q, &tq)) || (r = get_map(c, k, &tk)) || (r = get_map(c, v, &tv)))
@@ -159,7 +167,7 @@ int attn_launch(rapid3_ctx* c, const TensorGeom& g, const void* q, const void* k
     {
         ProfScope ps(c, PROF_ATTN, st);
         if (launch_attention(tq, tk, tv, out, g, l, kept_idx, kept_cnt, bitmask, scale, c->status, st, plan, n_cap, -1,
-                             !after_select, &c->parts, &c->launches) != cudaSuccess)
+                             !after_select, &c->parts, &c->launches, order) != cudaSuccess)
             return RAPID3_ERR_CUDA;
     }
     c->launches += 1;
@@ -238,6 +246,10 @@ int rapid3_create(rapid3_ctx** out, const rapid3_shape* shape) {
               cudaMemset(c->status, 0, sizeof(int)) == cudaSuccess &&
               cudaMalloc(&c->plan, sizeof(DevPlan)) == cudaSuccess &&
               cudaMemset(c->plan, 0, sizeof(DevPlan)) == cudaSuccess;
+    if (ok && !c->parts.any() && attention_units(g, c->parts, (int)B, 0) > ORDER_FROM) {
+        ok = cudaMalloc(&c->order.count, (1 + ORDER_LAST) * ORDER_CLASSES * sizeof(uint32_t)) == cudaSuccess;
+        c->order.list = c->order.count + ORDER_CLASSES;
+    }
     if (ok && c->parts.any()) ok = cudaMalloc(&c->parts.partial, attention_partial_bytes(g, shape->B_max, c->parts)) == cudaSuccess;
     if (!ok) {
         cudaGetLastError();
@@ -264,6 +276,7 @@ int rapid3_destroy(rapid3_ctx* c) {
     cudaFree(c->status);
     cudaFree(c->plan);
     cudaFree(c->parts.partial);
+    cudaFree(c->order.count);
     for (void* s : c->stage) cudaFree(s);
     if (c->up_s) cudaStreamDestroy(c->up_s);
     if (c->down_s) cudaStreamDestroy(c->down_s);
@@ -443,6 +456,9 @@ static int gated_step_impl(rapid3_ctx* c, const void* q, const void* k, const vo
         if (launch_prepare(*prep, g, all, sparse.n, c->pooled, st) != cudaSuccess) return RAPID3_ERR_CUDA;
         c->launches += 1;
     }
+    const QuadOrder order = sparse.n > 0 ? step_order(c, g, all.n) : QuadOrder();
+    for (int p = 0; p < all.n; ++p)                       // for the selection kernel: place in the attention's list
+        if (all.slot[p] >= 0) sparse.slot[all.slot[p]] = p - (all.n - sparse.n);
     if (sparse.n > 0) {
         if ((reinterpret_cast<uintptr_t>(q) % 16) || (reinterpret_cast<uintptr_t>(k) % 16)) return RAPID3_ERR_INVALID_ARG;
         if (!prep) {
@@ -452,21 +468,21 @@ static int gated_step_impl(rapid3_ctx* c, const void* q, const void* k, const vo
         }
         {
             ProfScope ps(c, PROF_SCORES, st);
-            if (launch_block_scores(c->pooled, g, sparse.n, c->scores, st) != cudaSuccess) return RAPID3_ERR_CUDA;
+            if (launch_block_scores(c->pooled, g, sparse.n, c->scores, st, nullptr, order) != cudaSuccess) return RAPID3_ERR_CUDA;
         }
         {
             ProfScope ps(c, PROF_SELECT, st);
             const cudaError_t e =
                 mass_scale ? launch_select_mask_mass(c->scores, g, sparse, share, *mass_scale, c->row_keep, c->bitmask,
-                                                     c->kept_idx, c->kept_cnt, st)
-                : per_head ? launch_select_mask_heads(c->scores, g, sparse, hk, c->bitmask, c->kept_idx, c->kept_cnt, st)
-                           : launch_select_mask(c->scores, g, sparse, c->bitmask, c->kept_idx, c->kept_cnt, st);
+                                                     c->kept_idx, c->kept_cnt, st, order)
+                : per_head ? launch_select_mask_heads(c->scores, g, sparse, hk, c->bitmask, c->kept_idx, c->kept_cnt, st, order)
+                           : launch_select_mask(c->scores, g, sparse, c->bitmask, c->kept_idx, c->kept_cnt, st, nullptr, 0, order);
             if (e != cudaSuccess) return RAPID3_ERR_CUDA;
         }
         c->launches += mass_scale ? 3 : 2;
     }
     return attn_launch(c, g, q, k, v, out, all, sparse.n ? c->kept_idx : nullptr, sparse.n ? c->kept_cnt : nullptr,
-                       sparse.n ? c->bitmask : nullptr, softmax_scale, st, nullptr, 0, sparse.n > 0);
+                       sparse.n ? c->bitmask : nullptr, softmax_scale, st, nullptr, 0, sparse.n > 0, order);
 }
 
 int rapid3_gated_step(rapid3_ctx* c, const void* q, const void* k, const void* v, void* out,
@@ -521,21 +537,22 @@ int rapid3_gated_step_device(rapid3_ctx* c, const void* q, const void* k, const 
     if (launch_plan(action_dev, keep_ratio_dev, B, c->g, c->plan, c->status, st) != cudaSuccess) return RAPID3_ERR_CUDA;
     ImgList none;
     none.n = 0;
+    const QuadOrder order = step_order(c, c->g, B);
     {
         ProfScope ps(c, PROF_POOL, st);
         if (launch_block_pool(q, k, c->g, none, c->pooled, st, c->plan, B) != cudaSuccess) return RAPID3_ERR_CUDA;
     }
     {
         ProfScope ps(c, PROF_SCORES, st);
-        if (launch_block_scores(c->pooled, c->g, B, c->scores, st, c->plan) != cudaSuccess) return RAPID3_ERR_CUDA;
+        if (launch_block_scores(c->pooled, c->g, B, c->scores, st, c->plan, order) != cudaSuccess) return RAPID3_ERR_CUDA;
     }
     {
         ProfScope ps(c, PROF_SELECT, st);
-        if (launch_select_mask(c->scores, c->g, none, c->bitmask, c->kept_idx, c->kept_cnt, st, c->plan, B) != cudaSuccess)
+        if (launch_select_mask(c->scores, c->g, none, c->bitmask, c->kept_idx, c->kept_cnt, st, c->plan, B, order) != cudaSuccess)
             return RAPID3_ERR_CUDA;
     }
     c->launches += 4;
-    return attn_launch(c, c->g, q, k, v, out, none, c->kept_idx, c->kept_cnt, c->bitmask, softmax_scale, st, c->plan, B, true);
+    return attn_launch(c, c->g, q, k, v, out, none, c->kept_idx, c->kept_cnt, c->bitmask, softmax_scale, st, c->plan, B, true, order);
 }
 
 int rapid3_gated_step_host(rapid3_ctx* c, const void* q_host, const void* k_host, const void* v_host, void* out_host,

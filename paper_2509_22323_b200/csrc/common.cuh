@@ -71,6 +71,36 @@ __host__ __device__ inline int attention_units(const TensorGeom& g, const AttnPa
     return g.H * (n_dense * nq * parts.dense + (n_img - n_dense) * (ntq * parts.text + (nq - ntq) * parts.light));
 }
 
+// Which two of the quad's four query blocks form a 128-row tile: neighbours, or, when a row of the image
+// grid spans two blocks (pair_stride 2), vertical neighbours (i, i + 2), whose kept lists overlap far more
+// (measured on the 128 x 128 grid at keep ratio 0.25: 90 % against 63 % of the tile's MMA work lands on
+// kept 64 x 64 sub-tiles).  pair_stride 3 goes further on that grid: the whole quad is one column of it --
+// members (i, i + 2, i + 4, i + 6), the left or the right halves of four consecutive grid rows -- so both
+// tiles want nearly the same key blocks (union of the quad 98 instead of 134 blocks at keep ratio 0.25,
+// both tiles busy on 68 % of them instead of 23 %).
+__host__ __device__ inline int quad_block(const TensorGeom& g, int quad, int a) {
+    int q = 4 * quad + (g.pair_stride == 2 ? ((a & 1) << 1) + (a >> 1) : a);
+    if (g.pair_stride == 3 && q >= g.n_text_blocks) {
+        const int r = q - g.n_text_blocks, w = r & 7;
+        q = g.n_text_blocks + (r & ~7) + ((w & 3) << 1) + (w >> 2);
+    }
+    return q;
+}
+
+// The last ORDER_LAST quads of a launch (of sparse images, without text rows) by how long they take, longest first: the selection kernel, which
+// knows a quad's lists, puts it into one of ORDER_CLASSES classes of equal width, and the attention kernel hands them out
+// class by class.  In the order of images and heads the last quads of a launch may be long ones, for which the other SMs
+// wait; the quads before them stay in that order, in which the thread blocks at work share the K and V of a few heads.
+// For launches of more than ORDER_FROM quads (two for each SM) up to ORDER_TO: whole steps of 864 quads, us, two images with a ratio for every
+// head 197.5 -> 190.2, by cumulative mass 358.2 -> 346.3, a dense one and one at 0.5 (D = 64) 262.5 -> 257.3; one image of 432
+// quads at 0.5 from raw projections 190.5 -> 182.9.  Outside these bounds the idle SMs at the end cost less than the heads'
+// first reads at once and the longer selection do (192 quads 41.2 -> 42.1; 1632 quads at D = 64 303.5 -> 313.7).
+constexpr int ORDER_CLASSES = 32, ORDER_LAST = 444, ORDER_FROM = 296, ORDER_TO = 1000;
+struct QuadOrder {
+    uint32_t* count = nullptr;       // [ORDER_CLASSES] quads of the class; the scores kernel of a step sets them to zero
+    uint32_t* list = nullptr;        // [ORDER_CLASSES][ORDER_LAST] (place of the image * H + head) * quads + quad, in any order
+};
+
 // Programmatic dependent launch: every kernel of a step is launched so that it may start while the kernel before it in the stream
 // is still running, and must call grid_dependency_wait() before it touches anything that kernel writes (and read it past
 // the L1, whose lines the wait is not known to refresh); the kernel before it calls grid_dependency_launch() to let it
@@ -115,20 +145,20 @@ inline cudaError_t launch_kernel(void (*kernel)(KArgs...), dim3 grid, dim3 block
 cudaError_t launch_block_pool(const void* q, const void* k, const TensorGeom& g, const ImgList& imgs,
                               double* pooled, cudaStream_t s, const DevPlan* plan = nullptr, int n_cap = 0);
 cudaError_t launch_block_scores(const double* pooled, const TensorGeom& g, int n_img, float* scores,
-                                cudaStream_t s, const DevPlan* plan = nullptr);
+                                cudaStream_t s, const DevPlan* plan = nullptr, const QuadOrder& order = QuadOrder());
 // K2: forced + top-k selection.
 cudaError_t launch_select_mask(const float* scores, const TensorGeom& g, const ImgList& imgs,
                                uint64_t* bitmask, int32_t* kept_idx, int32_t* kept_cnt, cudaStream_t s,
-                               const DevPlan* plan = nullptr, int n_cap = 0);
+                               const DevPlan* plan = nullptr, int n_cap = 0, const QuadOrder& order = QuadOrder());
 cudaError_t launch_select_mask_heads(const float* scores, const TensorGeom& g, const ImgList& imgs,
                                      const HeadKeep& hk, uint64_t* bitmask, int32_t* kept_idx, int32_t* kept_cnt,
-                                     cudaStream_t s);
+                                     cudaStream_t s, const QuadOrder& order = QuadOrder());
 // K2, cumulative-mass variant: row_keep[row] = smallest count of best free candidates holding a share
 // tau of the row's softmax mass (weights exp(scale * (S - row max)), fp64), then the top-k selection
 // at that count.
 cudaError_t launch_select_mask_mass(const float* scores, const TensorGeom& g, const ImgList& imgs,
                                     const MassShare& share, float scale, int32_t* row_keep, uint64_t* bitmask,
-                                    int32_t* kept_idx, int32_t* kept_cnt, cudaStream_t s);
+                                    int32_t* kept_idx, int32_t* kept_cnt, cudaStream_t s, const QuadOrder& order = QuadOrder());
 // K5: Q/K producer (RMS norm + gain + rotary embedding -> bf16) that also writes the block means of
 // the images with a workspace slot.  pooled is [2][n_sparse][H][nb][D].
 struct PrepArgs {
@@ -155,7 +185,8 @@ cudaError_t launch_attention(const CUtensorMap& tmq, const CUtensorMap& tmk, con
                              cudaStream_t s, const DevPlan* plan = nullptr, int n_cap = 0, int inject_stop_group = -1,
                              bool wait_first = true,
                              // with `parts` lists may be worked on in parts, in one launch more (added to *launches)
-                             const AttnParts* parts = nullptr, int64_t* launches = nullptr);   // false: after the selection kernel, for whose masks the quads of sparse images wait themselves
+                             const AttnParts* parts = nullptr, int64_t* launches = nullptr,
+                             const QuadOrder& order = QuadOrder());   // false: after the selection kernel, for whose masks the quads of sparse images wait themselves
 AttnParts attention_parts(const TensorGeom& g, int n_img);     // without its pointers
 size_t attention_partial_bytes(const TensorGeom& g, int n_img, const AttnParts& parts);
 // Kernel attributes on the current device; set when a context is created (scoring: also by the context-free entry).

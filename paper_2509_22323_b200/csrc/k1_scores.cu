@@ -95,7 +95,7 @@ __device__ __forceinline__ void copy16_async(double* dst, const double* src, boo
 // lanes.  Every output accumulates its products in ascending order of the four-channel groups.
 template <int D>
 __global__ void __launch_bounds__(256) scores_kernel(const double* pooled, TensorGeom g, int n_img,
-                                                     float* __restrict__ scores, const DevPlan* plan) {
+                                                     float* __restrict__ scores, const DevPlan* plan, uint32_t* order_count) {
     constexpr int T = 32, LDS = D + 4;
     extern __shared__ __align__(16) double tiles[];
     double* sq = tiles;
@@ -105,6 +105,8 @@ __global__ void __launch_bounds__(256) scores_kernel(const double* pooled, Tenso
     // and read them past the L1, whose lines no such wait is known to refresh.
     grid_dependency_wait();
     grid_dependency_launch();
+    // the attention of the step before, which reads these, has ended: the kernel in front has waited for it
+    if (order_count && blockIdx.x + blockIdx.y + blockIdx.z == 0 && threadIdx.x < ORDER_CLASSES) order_count[threadIdx.x] = 0u;
     if (plan && ph >= __ldcg(&plan->sparse.n) * g.H) return;
     const int i0 = blockIdx.y * T, j0 = blockIdx.x * T;
     const double* pq = pooled + ((long long)ph * g.nb + i0) * D;
@@ -166,12 +168,12 @@ cudaError_t launch_block_pool(const void* q, const void* k, const TensorGeom& g,
 }
 
 cudaError_t launch_block_scores(const double* pooled, const TensorGeom& g, int n_img, float* scores,
-                                cudaStream_t s, const DevPlan* plan) {
+                                cudaStream_t s, const DevPlan* plan, const QuadOrder& order) {
     // with a plan n_img is the capacity.  32 x 32 tiles at every length: against 64 x 64 tiles they waste less of
     // the ragged edge and fill the SMs more evenly (30 against 35 us at 264 blocks, where 64 x 64 pads 264 to 320)
     const dim3 grid((g.nb + 31) / 32, (g.nb + 31) / 32, n_img * g.H);
     return launch_kernel(g.D == 128 ? scores_kernel<128> : scores_kernel<64>, grid, dim3(256), scores_smem_bytes(g.D), s,
-                         pooled, g, n_img, scores, plan);
+                         pooled, g, n_img, scores, plan, order.count);
 }
 
 cudaError_t scoring_static_init() {

@@ -44,92 +44,128 @@ __device__ __forceinline__ int differing_bits(const uint32_t (&u)[IPL], uint32_t
 
 // HK = NoHeadKeep: one keep count per image.  HK = HeadKeep: one per (image, head), passed by value.
 // HK = RowKeep: one per row, read from device memory.
-template <typename HK, int IPL>
+// ORDER: the quads' places in the attention's order come out too (see QuadOrder); imgs.slot then holds an image's place among the
+// sparse ones in the attention's list.
+template <typename HK, int IPL, bool ORDER>
 __global__ void __launch_bounds__(WARPS * 32) select_kernel(const float* scores, TensorGeom g,
                                                             ImgList imgs, uint32_t* __restrict__ bitmask32,
                                                             int32_t* __restrict__ kept_idx,
                                                             int32_t* __restrict__ kept_cnt, int words32,
-                                                            const DevPlan* plan, const HK hk) {
+                                                            const DevPlan* plan, const QuadOrder order, const HK hk) {
+    __shared__ uint32_t kept[ORDER ? WARPS : 1][ORDER ? IPL : 1];        // the thread block's rows: the four query blocks of a quad
     const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
     const int nb = g.nb, ntb = g.n_text_blocks;
     const int ph = blockIdx.y, p = ph / g.H;            // p * H + h
-    const int i = blockIdx.x * WARPS + warp;
+    const int i = quad_block(g, blockIdx.x, warp);
     const int row = ph * nb + i;                        // at most 65535 x 1024
     grid_dependency_wait();                             // the scores come from the kernel before, which may still be running
     grid_dependency_launch();
-    if (i >= nb || (plan && p >= __ldcg(&plan->sparse.n))) return;
-    // free candidates kept in this row: one count per image, or per (image, head) when the policy
-    // sets a ratio for every head
-    int k;
-    if constexpr (HK::mode == 1) k = hk.k[ph];
-    else if constexpr (HK::mode == 2) k = __ldcg(hk.k + row);
-    else k = plan ? __ldcg(&plan->sparse.k_free[p]) : imgs.k_free[p];
-    const float* src = scores + (long long)row * nb;
-    const bool text_row = i < ntb;
-    const int n_free = max(nb - ntb - ((i >= ntb) ? 1 : 0), 0);
-    const bool select = !text_row && k > 0 && k < n_free;
-    uint32_t u[IPL];
+    if (plan && p >= __ldcg(&plan->sparse.n)) return;
+    if (i < nb) {
+        // free candidates kept in this row: one count per image, or per (image, head) when the policy
+        // sets a ratio for every head
+        int k;
+        if constexpr (HK::mode == 1) k = hk.k[ph];
+        else if constexpr (HK::mode == 2) k = __ldcg(hk.k + row);
+        else k = plan ? __ldcg(&plan->sparse.k_free[p]) : imgs.k_free[p];
+        const float* src = scores + (long long)row * nb;
+        const bool text_row = i < ntb;
+        const int n_free = max(nb - ntb - ((i >= ntb) ? 1 : 0), 0);
+        const bool select = !text_row && k > 0 && k < n_free;
+        uint32_t u[IPL];
 #pragma unroll
-    for (int x = 0; x < IPL; ++x) {
-        const int j = 32 * x + lane;
-        u[x] = 0u;
-        if (select && j < nb && j >= ntb && j != i) u[x] = score_key(__ldcg(src + j));   // past the L1: see the wait above
-    }
-    uint32_t prefix = 0u;
-    int want = 0;                                       // of the keys that equal `prefix`, how many are kept
-    if (select) {
-        int hi = differing_bits(u, prefix);             // the candidates that decide equal `prefix` from bit `hi` up
-        int at_least = n_free, above = 0;               // candidates at or above `prefix`, and above those that decide
-        while (hi > 0 && at_least > k) {
-            const int lo = max(hi - 2, 0);
-            const uint32_t d = 1u << lo, t1 = prefix + d, t2 = t1 + d, t3 = t2 + d;
-            uint32_t c = 0u;                            // candidates at or above the three trials
-            if (hi - lo == 2) {
+        for (int x = 0; x < IPL; ++x) {
+            const int j = 32 * x + lane;
+            u[x] = 0u;
+            if (select && j < nb && j >= ntb && j != i) u[x] = score_key(__ldcg(src + j));   // past the L1: see the wait above
+        }
+        uint32_t prefix = 0u;
+        int want = 0;                                       // of the keys that equal `prefix`, how many are kept
+        if (select) {
+            int hi = differing_bits(u, prefix);             // the candidates that decide equal `prefix` from bit `hi` up
+            int at_least = n_free, above = 0;               // candidates at or above `prefix`, and above those that decide
+            while (hi > 0 && at_least > k) {
+                const int lo = max(hi - 2, 0);
+                const uint32_t d = 1u << lo, t1 = prefix + d, t2 = t1 + d, t3 = t2 + d;
+                uint32_t c = 0u;                            // candidates at or above the three trials
+                if (hi - lo == 2) {
 #pragma unroll
-                for (int x = 0; x < IPL; ++x) c += (u[x] >= t1 ? 1u : 0u) + (u[x] >= t2 ? 1u << 10 : 0u) + (u[x] >= t3 ? 1u << 20 : 0u);
-                c = __reduce_add_sync(0xffffffffu, c);
-            } else {
+                    for (int x = 0; x < IPL; ++x) c += (u[x] >= t1 ? 1u : 0u) + (u[x] >= t2 ? 1u << 10 : 0u) + (u[x] >= t3 ? 1u << 20 : 0u);
+                    c = __reduce_add_sync(0xffffffffu, c);
+                } else {
 #pragma unroll
-                for (int x = 0; x < IPL; ++x) c += u[x] >= t1 ? 1u : 0u;
-                c = __reduce_add_sync(0xffffffffu, c) | ((uint32_t)above << 10) | ((uint32_t)above << 20);   // no digit 2 or 3
+                    for (int x = 0; x < IPL; ++x) c += u[x] >= t1 ? 1u : 0u;
+                    c = __reduce_add_sync(0xffffffffu, c) | ((uint32_t)above << 10) | ((uint32_t)above << 20);   // no digit 2 or 3
+                }
+                const int c1 = c & 1023u, c2 = (c >> 10) & 1023u, c3 = c >> 20;
+                // the digit is the largest with k candidates or more at or above it
+                if (c3 >= k) { prefix = t3; at_least = c3; }
+                else if (c2 >= k) { prefix = t2; at_least = c2; above = c3; }
+                else if (c1 >= k) { prefix = t1; at_least = c1; above = c2; }
+                else above = c1;
+                hi = lo;
             }
-            const int c1 = c & 1023u, c2 = (c >> 10) & 1023u, c3 = c >> 20;
-            // the digit is the largest with k candidates or more at or above it
-            if (c3 >= k) { prefix = t3; at_least = c3; }
-            else if (c2 >= k) { prefix = t2; at_least = c2; above = c3; }
-            else if (c1 >= k) { prefix = t1; at_least = c1; above = c2; }
-            else above = c1;
-            hi = lo;
+            want = at_least > k ? k - above : nb;           // exactly k at or above `prefix`: all of them
         }
-        want = at_least > k ? k - above : nb;           // exactly k at or above `prefix`: all of them
-    }
-    int32_t* out_idx = kept_idx + (long long)row * nb;
-    uint32_t* out_bits = bitmask32 + (long long)row * words32;
-    int total = 0, eq_seen = 0;
+        int32_t* out_idx = kept_idx + (long long)row * nb;
+        uint32_t* out_bits = bitmask32 + (long long)row * words32;
+        int total = 0, eq_seen = 0;
 #pragma unroll
-    for (int x = 0; x < IPL; ++x) {
-        const int j = 32 * x + lane;
-        if (32 * x >= nb) break;
-        bool keep = false, eq = false;
-        if (j < nb) {
-            if (text_row || j < ntb || j == i) keep = true;
-            else if (select) {
-                keep = u[x] > prefix;
-                eq = u[x] == prefix;
-            } else keep = k >= n_free && k > 0;         // every free candidate, or none
+        for (int x = 0; x < IPL; ++x) {
+            const int j = 32 * x + lane;
+            if (32 * x >= nb) break;
+            bool keep = false, eq = false;
+            if (j < nb) {
+                if (text_row || j < ntb || j == i) keep = true;
+                else if (select) {
+                    keep = u[x] > prefix;
+                    eq = u[x] == prefix;
+                } else keep = k >= n_free && k > 0;         // every free candidate, or none
+            }
+            // equal keys: the lowest block indices first, `want` of them in all
+            const uint32_t beq = __ballot_sync(0xffffffffu, eq);
+            if (eq && eq_seen + __popc(beq & ((1u << lane) - 1u)) < want) keep = true;
+            eq_seen += __popc(beq);
+            const uint32_t bal = __ballot_sync(0xffffffffu, keep);
+            if (lane == 0) {
+                out_bits[x] = bal;
+                if constexpr (ORDER) kept[warp][x] = bal;
+            }
+            if (keep) out_idx[total + __popc(bal & ((1u << lane) - 1u))] = j;
+            total += __popc(bal);
         }
-        // equal keys: the lowest block indices first, `want` of them in all
-        const uint32_t beq = __ballot_sync(0xffffffffu, eq);
-        if (eq && eq_seen + __popc(beq & ((1u << lane) - 1u)) < want) keep = true;
-        eq_seen += __popc(beq);
-        const uint32_t bal = __ballot_sync(0xffffffffu, keep);
-        if (lane == 0) out_bits[x] = bal;
-        if (keep) out_idx[total + __popc(bal & ((1u << lane) - 1u))] = j;
-        total += __popc(bal);
+        for (int c = (nb + 31) / 32 + lane; c < words32; c += 32) out_bits[c] = 0;   // odd 32-bit half of the last word
+        for (int e = total + lane; e < nb; e += 32) out_idx[e] = -1;
+        if (lane == 0) kept_cnt[row] = total;
+    } else if (ORDER && lane < IPL) {
+        kept[ORDER ? warp : 0][ORDER ? lane : 0] = 0u;
     }
-    for (int c = (nb + 31) / 32 + lane; c < words32; c += 32) out_bits[c] = 0;   // odd 32-bit half of the last word
-    for (int e = total + lane; e < nb; e += 32) out_idx[e] = -1;
-    if (lane == 0) kept_cnt[row] = total;
+    if constexpr (ORDER) {
+        __syncthreads();
+        const int nq = (nb + 3) >> 2, ntq = (ntb + 3) >> 2, quad = blockIdx.x;
+        if (warp > 0 || quad < ntq) return;             // quads with text rows come earlier
+        int rank = imgs.slot[p], n_sparse = imgs.n;
+        if (plan) {
+            n_sparse = __ldcg(&plan->sparse.n);
+            const int n_all = __ldcg(&plan->all.n);
+            auto here = [&](int at) { return at < n_all && __ldcg(&plan->all.slot[at]) == p; };
+            const uint32_t lo = __ballot_sync(0xffffffffu, here(lane)), hi = __ballot_sync(0xffffffffu, here(32 + lane));
+            rank = (lo ? __ffs(lo) - 1 : 31 + __ffs(hi)) - __ldcg(&plan->n_dense);
+        }
+        const int nl = nq - ntq;
+        if ((rank * g.H + ph % g.H) * nl + quad - ntq < n_sparse * g.H * nl - ORDER_LAST) return;
+        // the quad's time, in quarters of a key block of two tiles: one that only one tile uses takes three quarters
+        int time = 0;
+        if (32 * lane < nb) {
+            const uint32_t t0 = kept[0][lane] | kept[1][lane], t1 = kept[2][lane] | kept[3][lane];
+            time = 2 * __popc(t0 | t1) + __popc(t0) + __popc(t1);
+        }
+        time = __reduce_add_sync(0xffffffffu, time);
+        if (lane == 0) {
+            const int c = ORDER_CLASSES - 1 - time * (ORDER_CLASSES - 1) / (4 * nb);
+            order.list[c * ORDER_LAST + atomicAdd(order.count + c, 1u)] = (rank * g.H + ph % g.H) * nq + quad;
+        }
+    }
 }
 
 // Cumulative-mass rule: one warp per row finds the smallest count k of best free candidates (score
@@ -262,11 +298,11 @@ cudaError_t with_ipl(int nb, F&& f) {
 
 template <typename HK>
 cudaError_t launch_select(const float* scores, const TensorGeom& g, const ImgList& imgs, uint64_t* bitmask, int32_t* kept_idx,
-                          int32_t* kept_cnt, cudaStream_t s, const DevPlan* plan, int n_img, const HK& hk) {
+                          int32_t* kept_cnt, cudaStream_t s, const DevPlan* plan, int n_img, const QuadOrder& order, const HK& hk) {
     const dim3 grid((g.nb + WARPS - 1) / WARPS, n_img * g.H);
     return with_ipl(g.nb, [&](auto ipl) {
-        return launch_kernel(select_kernel<HK, decltype(ipl)::value>, grid, dim3(WARPS * 32), 0, s, scores, g, imgs,
-                             reinterpret_cast<uint32_t*>(bitmask), kept_idx, kept_cnt, 2 * ((g.nb + 63) / 64), plan, hk);
+        return launch_kernel(order.count ? select_kernel<HK, decltype(ipl)::value, true> : select_kernel<HK, decltype(ipl)::value, false>, grid, dim3(WARPS * 32), 0, s, scores, g, imgs,
+                             reinterpret_cast<uint32_t*>(bitmask), kept_idx, kept_cnt, 2 * ((g.nb + 63) / 64), plan, order, hk);
     });
 }
 
@@ -274,7 +310,7 @@ cudaError_t launch_select(const float* scores, const TensorGeom& g, const ImgLis
 
 cudaError_t launch_select_mask_mass(const float* scores, const TensorGeom& g, const ImgList& imgs,
                                     const MassShare& share, float scale, int32_t* row_keep, uint64_t* bitmask,
-                                    int32_t* kept_idx, int32_t* kept_cnt, cudaStream_t s) {
+                                    int32_t* kept_idx, int32_t* kept_cnt, cudaStream_t s, const QuadOrder& order) {
     const cudaError_t e = with_ipl(g.nb, [&](auto ipl) {
         return launch_kernel(mass_count_kernel<decltype(ipl)::value>, dim3((g.nb + MASS_WARPS - 1) / MASS_WARPS, imgs.n * g.H),
                              dim3(MASS_WARPS * 32), 0, s, scores, g, share, scale, row_keep);
@@ -282,17 +318,18 @@ cudaError_t launch_select_mask_mass(const float* scores, const TensorGeom& g, co
     if (e != cudaSuccess) return e;
     RowKeep rk;
     rk.k = row_keep;
-    return launch_select(scores, g, imgs, bitmask, kept_idx, kept_cnt, s, nullptr, imgs.n, rk);
+    return launch_select(scores, g, imgs, bitmask, kept_idx, kept_cnt, s, nullptr, imgs.n, order, rk);
 }
 
 cudaError_t launch_select_mask(const float* scores, const TensorGeom& g, const ImgList& imgs, uint64_t* bitmask,
-                               int32_t* kept_idx, int32_t* kept_cnt, cudaStream_t s, const DevPlan* plan, int n_cap) {
-    return launch_select(scores, g, imgs, bitmask, kept_idx, kept_cnt, s, plan, plan ? n_cap : imgs.n, NoHeadKeep());
+                               int32_t* kept_idx, int32_t* kept_cnt, cudaStream_t s, const DevPlan* plan, int n_cap,
+                               const QuadOrder& order) {
+    return launch_select(scores, g, imgs, bitmask, kept_idx, kept_cnt, s, plan, plan ? n_cap : imgs.n, order, NoHeadKeep());
 }
 
 cudaError_t launch_select_mask_heads(const float* scores, const TensorGeom& g, const ImgList& imgs, const HeadKeep& hk,
-                                     uint64_t* bitmask, int32_t* kept_idx, int32_t* kept_cnt, cudaStream_t s) {
-    return launch_select(scores, g, imgs, bitmask, kept_idx, kept_cnt, s, nullptr, imgs.n, hk);
+                                     uint64_t* bitmask, int32_t* kept_idx, int32_t* kept_cnt, cudaStream_t s, const QuadOrder& order) {
+    return launch_select(scores, g, imgs, bitmask, kept_idx, kept_cnt, s, nullptr, imgs.n, order, hk);
 }
 
 

@@ -82,6 +82,7 @@ struct AttnParams {
     const DevPlan* plan;           // optional: image list and n_dense from device memory (grid sized for n_cap images)
     int* status;
     float scale_log2;
+    QuadOrder order;               // optional: the order of the sparse images' quads without text rows
     AttnParts parts;               // SPLIT build: how many units of work the union list of a quad goes to
     bool wait_first;               // nothing is read before the kernel in front has ended
     int stop_group;                // failure-injection build of the kernel only: the producer stops before this group
@@ -139,22 +140,6 @@ __device__ __forceinline__ float max3(float a, float b, float c) {
     return d;
 }
 
-// Which two of the quad's four query blocks form a 128-row tile: neighbours, or, when a row of the image
-// grid spans two blocks (pair_stride 2), vertical neighbours (i, i + 2), whose kept lists overlap far more
-// (measured on the 128 x 128 grid at keep ratio 0.25: 90 % against 63 % of the tile's MMA work lands on
-// kept 64 x 64 sub-tiles).  pair_stride 3 goes further on that grid: the whole quad is one column of it --
-// members (i, i + 2, i + 4, i + 6), the left or the right halves of four consecutive grid rows -- so both
-// tiles want nearly the same key blocks (union of the quad 98 instead of 134 blocks at keep ratio 0.25,
-// both tiles busy on 68 % of them instead of 23 %).
-__device__ __forceinline__ int quad_block(const TensorGeom& g, int quad, int a) {
-    int q = 4 * quad + (g.pair_stride == 2 ? ((a & 1) << 1) + (a >> 1) : a);
-    if (g.pair_stride == 3 && q >= g.n_text_blocks) {
-        const int r = q - g.n_text_blocks, w = r & 7;
-        q = g.n_text_blocks + (r & ~7) + ((w & 3) << 1) + (w >> 2);
-    }
-    return q;
-}
-
 // Lane c of a quad of lanes holds words 0..3 of column pairs (c, c + 4, c + 8, c + 12); afterwards it holds words
 // 4 c .. 4 c + 3: a 4 x 4 transpose, two exchanges.
 __device__ __forceinline__ uint4 quad_transpose(uint32_t w0, uint32_t w1, uint32_t w2, uint32_t w3, int c) {
@@ -188,12 +173,15 @@ __device__ __forceinline__ void row_maxima(const uint32_t (&r)[32], float& lo, f
 // parts of equal length, each a unit of work (attention_parts() says how many).  A softmax warp leaves its rows of a part -- O,
 // not divided by the row sums, the sums and the reference maxima -- in global memory, and add_parts_kernel makes the result
 // of them.  (Added up by the last part of a quad to arrive, in this kernel, they cost its main loop 12 to 14 %: registers.)
-template <int D, bool INJECT = false, bool SPLIT = false>
+//
+// ORDERED is the build for launches whose last quads are handed out by their length (QuadOrder).
+template <int D, bool INJECT = false, bool SPLIT = false, bool ORDERED = false>
 __global__ void __launch_bounds__(NTHREADS, 1)
 attn_kernel(const __grid_constant__ CUtensorMap tmq, const __grid_constant__ CUtensorMap tmk,
             const __grid_constant__ CUtensorMap tmv, uint16_t* __restrict__ out, const __grid_constant__ AttnParams prm) {
     using C = Cfg<D>;
     constexpr int DH = C::DH, KS = C::KS, VS = C::VS, NBUF = C::NBUF, O_COL = C::O_COL;
+    constexpr bool MORE_REGS = SPLIT || (ORDERED && D == 128);
     extern __shared__ uint8_t smem_raw[];
     const uint32_t raw = smem_u32(smem_raw);
     const uint32_t pad = ((raw + 1023u) & ~1023u) - raw;
@@ -320,8 +308,9 @@ attn_kernel(const __grid_constant__ CUtensorMap tmq, const __grid_constant__ CUt
         }
     };
 
-    // the pool is the launch's 640 x 96: 512 x 104 + 128 x 64
-    if (SPLIT && warp >= SOFTMAX_WARPS) reg_dec<64>();
+    // The pool is the launch's 640 x 96: 512 x 104 + 128 x 64.  Without it these builds keep five to ten words in local memory
+    // (step of 864 quads at D = 128 354.5 -> 353.0 us, of 432 204.5 -> 202.6; at D = 64 257.4 -> 258.4, not there).
+    if (MORE_REGS && warp >= SOFTMAX_WARPS) reg_dec<64>();
     if (warp == LIST_WARP) {
         // ------------------------------------------------------------ quads and their union lists
         // one lane polls: these waits are long, and the other lanes' polls would only take issue slots
@@ -330,6 +319,8 @@ attn_kernel(const __grid_constant__ CUtensorMap tmq, const __grid_constant__ CUt
         };
         int L = blockIdx.x;
         bool waited = false;                             // for the selection kernel, see below
+        uint32_t class_end = 0u;                         // quads of the classes up to the lane's, once `have_classes`
+        bool have_classes = false;
         for (uint32_t i = 0;; ++i) {
             Quad& u = ctl->quad[i & 1];
             if (!wait_lane0(bUE + 8 * (i & 1), ((i >> 1) & 1) ^ 1)) break;
@@ -387,9 +378,29 @@ attn_kernel(const __grid_constant__ CUtensorMap tmq, const __grid_constant__ CUt
                     h = L / ntq; quad = L - h * ntq;
                 } else {
                     L -= heavy_dense + heavy_sparse;
-                    const int nl = nq - ntq;
-                    p = L / (g.H * nl); L -= p * g.H * nl; p += nd;
-                    h = L / nl; quad = ntq + (L - h * nl);
+                    const int nl = nq - ntq, rest = L - max(ns * g.H * nl - ORDER_LAST, 0);
+                    if (ORDERED && rest >= 0) {
+                        // the quad at this place of the order that the selection kernel has found
+                        if (!have_classes) {
+                            if (!waited) grid_dependency_wait();
+                            waited = have_classes = true;
+                            class_end = __ldcg(prm.order.count + lane);
+#pragma unroll
+                            for (int o = 1; o < 32; o <<= 1) {
+                                const uint32_t v = __shfl_up_sync(0xffffffffu, class_end, o);
+                                if (lane >= o) class_end += v;
+                            }
+                        }
+                        const int c = min(__popc(__ballot_sync(0xffffffffu, class_end <= (uint32_t)rest)), ORDER_CLASSES - 1);
+                        const int before = __shfl_sync(0xffffffffu, (int)class_end, max(c - 1, 0));
+                        L = __ldcg(prm.order.list + c * ORDER_LAST + rest - (c > 0 ? before : 0));
+                        quad = L % nq; L /= nq;
+                        h = L % g.H;
+                        p = nd + L / g.H;
+                    } else {
+                        p = L / (g.H * nl); L -= p * g.H * nl; p += nd;
+                        h = L / nl; quad = ntq + (L - h * nl);
+                    }
                 }
             }
             const int b = prm.plan ? __ldcg(&prm.plan->all.batch[p]) : prm.imgs.batch[p];
@@ -676,7 +687,7 @@ attn_kernel(const __grid_constant__ CUtensorMap tmq, const __grid_constant__ CUt
         // (r_lo = lane / 4 and r_lo + 8 of the sixteen) and, of every group of eight score columns, the pair
         // 2 (lane % 4), + 1 -- 32 scores per key block.  The four threads of a quad share their rows' maximum
         // with two shuffles, and only when some row of the warp may have grown.
-        if (SPLIT) reg_inc<104>();
+        if (MORE_REGS) reg_inc<104>();
         const int t = (warp >> 2) & 1, wl = warp & 3, hf = warp >> 3;
         const int a = 2 * t + (wl >> 1);               // query block of the quad
         const uint32_t tile_bits = 3u << (2 * t), act_bit = 1u << a;
@@ -1007,6 +1018,12 @@ cudaError_t attention_static_init() {
     e = cudaFuncSetAttribute(attn_kernel<64, false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              (int)attn_smem_bytes<64>());
     if (e != cudaSuccess) return e;
+    e = cudaFuncSetAttribute(attn_kernel<128, false, false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             (int)attn_smem_bytes<128>());
+    if (e != cudaSuccess) return e;
+    e = cudaFuncSetAttribute(attn_kernel<64, false, false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             (int)attn_smem_bytes<64>());
+    if (e != cudaSuccess) return e;
     e = cudaFuncSetAttribute(attn_kernel<128, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              (int)attn_smem_bytes<128>());
     if (e != cudaSuccess) return e;
@@ -1116,7 +1133,7 @@ cudaError_t launch_attention(const CUtensorMap& tmq, const CUtensorMap& tmk, con
                              const TensorGeom& g, const ImgList& imgs, const int32_t* kept_idx,
                              const int32_t* kept_cnt, const uint64_t* bitmask, float softmax_scale, int* status,
                              cudaStream_t s, const DevPlan* plan, int n_cap, int inject_stop_group, bool wait_first,
-                             const AttnParts* parts, int64_t* launches) {
+                             const AttnParts* parts, int64_t* launches, const QuadOrder& order) {
     if (!g_attr_set) {
         cudaError_t e = attention_static_init();
         if (e != cudaSuccess) return e;
@@ -1134,6 +1151,7 @@ cudaError_t launch_attention(const CUtensorMap& tmq, const CUtensorMap& tmk, con
     while (n_dense < imgs.n && (imgs.slot[n_dense] < 0 || kept_idx == nullptr)) ++n_dense;
     prm.n_dense = n_dense;
     prm.plan = plan;
+    prm.order = order;
     prm.wait_first = wait_first;
     prm.stop_group = inject_stop_group;
     const int n_img = plan ? n_cap : imgs.n, pairs = g.H * n_img, nq = (g.nb + 3) / 4, ntq = std::min(nq, (g.n_text_blocks + 3) / 4);
@@ -1159,10 +1177,11 @@ cudaError_t launch_attention(const CUtensorMap& tmq, const CUtensorMap& tmk, con
         *launches += 1;
         return launch_kernel(g.D == 128 ? add_parts_kernel<128> : add_parts_kernel<64>, dim3(left * SOFTMAX_WARPS * (g.D / 32) / 4), dim3(128), 0, s,
                              static_cast<uint16_t*>(out), g, imgs, n_dense, plan, prm.parts);
-    } else if (g.D == 128) {
-        return launch_kernel(attn_kernel<128>, grid, dim3(NTHREADS), attn_smem_bytes<128>(), s, tmq, tmk, tmv, static_cast<uint16_t*>(out), prm);
     } else {
-        return launch_kernel(attn_kernel<64>, grid, dim3(NTHREADS), attn_smem_bytes<64>(), s, tmq, tmk, tmv, static_cast<uint16_t*>(out), prm);
+        return launch_kernel(order.count ? (g.D == 128 ? attn_kernel<128, false, false, true> : attn_kernel<64, false, false, true>)
+                                         : (g.D == 128 ? attn_kernel<128> : attn_kernel<64>),
+                             grid, dim3(NTHREADS), g.D == 128 ? attn_smem_bytes<128>() : attn_smem_bytes<64>(), s, tmq, tmk, tmv,
+                             static_cast<uint16_t*>(out), prm);
     }
     return cudaGetLastError();
 }

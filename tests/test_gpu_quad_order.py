@@ -1,0 +1,45 @@
+"""Launches of some hundred quads hand their last ones out by length.  In which order a quad is worked on does not touch its
+result: every image of such a step equals the same image alone, whose few quads come in order, bit for bit -- for
+every selection rule, for batches whose last quads are all, some and not any of the ordered ones, and for decisions on the GPU."""
+import pytest
+import torch
+
+from paper_2509_22323_b200 import binding
+
+pytestmark = pytest.mark.gpu
+DEV = "cuda"
+
+
+@pytest.mark.parametrize("D,n_text,n_image,H,B", [
+    (64, 77, 2400, 8, 4),        # 320 quads, all of those without text in the order; text and image rows in one quad
+    (128, 0, 9 * 64 + 5, 25, 4),  # 300 quads, ragged, no text
+    (128, 128, 1111, 16, 8),     # 640 quads: the first of those without text come as they are
+    (64, 64, 128 * 128, 4, 3),   # 780 quads of two-block grid rows
+    (64, 512, 128 * 128, 2, 4),  # 528 column quads
+])
+def test_ordered_quads_equal_quads_in_order(D, n_text, n_image, H, B):
+    N = n_text + n_image
+    gen = torch.Generator(device=DEV).manual_seed(N)
+    q, k, v = (torch.randn((B, H, N, D), generator=gen, device=DEV).to(torch.bfloat16) for _ in range(3))
+    ctx = binding.Context(B, H, D, n_text, n_image)
+    ratios = [(0.3, 1.0, 0.7, 0.15)[b % 4] for b in range(B)]
+    per_head = [[min(1.0, ratios[b] * (0.5, 1.0, 1.5)[h % 3]) for h in range(H)] for b in range(B)]
+    calls = {
+        "step": lambda out, acts: ctx.rapid3_gated_step(q, k, v, out, acts, ratios),
+        "heads": lambda out, acts: ctx.rapid3_gated_step_heads(q, k, v, out, acts, per_head),
+        "mass": lambda out, acts: ctx.rapid3_gated_step_mass(q, k, v, out, acts, ratios, 4 * D ** -0.5),
+        "device": lambda out, acts: ctx.rapid3_gated_step_device(q, k, v, out, torch.tensor(acts, dtype=torch.int32, device=DEV),
+                                                                 torch.tensor(ratios, device=DEV)),
+    }
+    for name, call in calls.items():
+        for acts in ([2] * B, [2] * (B - 1) + [1]):
+            out, alone = torch.full_like(q, float("nan")), torch.full_like(q, float("nan"))
+            for _ in range(2):                                     # the counts of the step before are gone
+                call(out, acts)
+            for b in range(B):
+                if acts[b] == 2:
+                    (calls["step"] if name == "device" else call)(alone, [2 if i == b else 0 for i in range(B)])
+            torch.cuda.synchronize()
+            assert ctx.last_status() == 0
+            assert torch.equal(out.view(torch.int16), alone.view(torch.int16)), (name, acts)
+            assert torch.isfinite(out[[a == 2 for a in acts]]).all()
