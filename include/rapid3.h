@@ -152,6 +152,8 @@ int rapid3_sparse_joint_attn(rapid3_ctx* ctx, const void* q, const void* k, cons
  * passes.  Skipped and reusing images launch no work and their rows of `out` stay untouched.
  * Scores, masks and kept lists of the sparse images live in the context's workspace
  * (see rapid3_workspace), compacted in ascending batch order of the sparse images.
+ * With a sparse image the call launches pool, scores, selection and attention, or, where there are many
+ * heads and enough attention for all SMs, one kernel for the whole scoring pass and the attention beside it.
  * The call only launches kernels (the tensor maps of a set of base pointers are encoded on the host at
  * their first use and cached), so after one plain call with the same tensors it can be captured
  * into a CUDA graph and replayed on buffers refilled in place; the actions and ratios are then
@@ -181,8 +183,7 @@ int rapid3_gated_step_heads(rapid3_ctx* ctx, const void* q, const void* k, const
  * top-k selection: mass_share_host[b] in (0, 1] is the share of attending image b (ignored for the
  * others); a share of exactly 1 makes the image dense (no scoring); mass_scale as in
  * rapid3_select_mask_mass.  Five launches with a sparse image (pool, scores, counts, selection,
- * attention).  The per-row counts stay in the context's workspace.  Everything else as in
- * rapid3_gated_step.
+ * attention), or two (see rapid3_gated_step).  Everything else as there.
  */
 int rapid3_gated_step_mass(rapid3_ctx* ctx, const void* q, const void* k, const void* v, void* out,
                            const int32_t* action_host, const float* mass_share_host, float mass_scale, int B,
@@ -198,7 +199,7 @@ int rapid3_gated_step_mass(rapid3_ctx* ctx, const void* q, const void* k, const 
  *     r = 1 / sqrt(mean(x^2) + eps);   y[d] = x[d] * r * gain[d];
  *     z[2i] = y[2i] cos - y[2i+1] sin,  z[2i+1] = y[2i] sin + y[2i+1] cos,  (cos, sin) = rot[n][i]
  * rounded once to bf16 (fp32 arithmetic).  Then scoring, selection and attention run on q, k, v
- * exactly as in rapid3_gated_step (4 launches with a sparse image, 2 without).
+ * exactly as in rapid3_gated_step (4 or 3 launches with a sparse image, 2 without).
  *   q_raw, k_raw, q, k : device, bf16, the context's [B, H, N, D] strides, 16-byte aligned;
  *                        q may equal q_raw and k may equal k_raw (in place);
  *   q_gain, k_gain     : device, fp32 [D], 16-byte aligned;
@@ -216,7 +217,7 @@ int rapid3_gated_step_fused(rapid3_ctx* ctx, const void* q_raw, const void* k_ra
  * actions on the device; reading them back would cost a host synchronisation per step and layer):
  * action_dev [B] int32 and keep_ratio_dev [B] float are DEVICE arrays, read by the kernels when
  * they run on `stream`, not at call time.  A kernel of one thread block builds the image lists, then the
- * four kernels of rapid3_gated_step are launched with grids sized for all B images; thread blocks
+ * kernels of rapid3_gated_step are launched with grids sized for all B images; thread blocks
  * of images that do not attend return at once.  Results (output, workspace contents) are those of
  * rapid3_gated_step with the same actions.  An action outside {SKIP, REUSE, ATTEND} or a ratio
  * outside (0, 1] cannot be rejected at call time: that image is not processed and the device status
@@ -270,7 +271,9 @@ int64_t rapid3_launch_count(rapid3_ctx* ctx);
  * pairs between reads); enable = 2 brackets the attention kernel only (an event pair costs a few
  * microseconds of stream time, which matters beside the short scoring kernels); 0 switches it off.  rapid3_profile_read waits for the recorded events, returns the summed device
  * time in milliseconds and the launch count per kernel kind
- * (0 block pool, 1 block scores, 2 mask select, 3 attention) and clears the record.
+ * (0 block pool, 1 block scores, 2 mask select, 3 attention) and clears the record.  Where one kernel does
+ * the whole scoring pass it counts as kind 0, or behind the producer of Q and K as kind 1.  An event
+ * pair also keeps the attention kernel from starting beside that pass.
  */
 int rapid3_profile(rapid3_ctx* ctx, int enable);
 int rapid3_profile_read(rapid3_ctx* ctx, double* ms /* [4] */, int64_t* launches /* [4] */);

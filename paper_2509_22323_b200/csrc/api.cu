@@ -154,6 +154,11 @@ QuadOrder step_order(const rapid3_ctx* c, const TensorGeom& g, int n_img) {
     return quads > ORDER_FROM && quads <= ORDER_TO ? c->order : QuadOrder();      // without pointers where the context has none
 }
 
+// SM time, in us, of a step's attention that needs no mask: quads of dense images, of text rows alone in sparse ones.
+double mask_free_us(const TensorGeom& g, int dense, int sparse) {
+    return (double)g.H * (dense * ((g.nb + 3) / 4) + sparse * (g.n_text_blocks / 4)) * g.nb * (g.D == 128 ? 0.84 : 0.72);
+}
+
 // `g` is the context's geometry or a copy of it narrowed to a range of heads.
 int attn_launch(rapid3_ctx* c, const TensorGeom& g, const void* q, const void* k, const void* v, void* out,
                 const ImgList& l, const int32_t* kept_idx, const int32_t* kept_cnt, const uint64_t* bitmask, float scale,
@@ -246,10 +251,8 @@ int rapid3_create(rapid3_ctx** out, const rapid3_shape* shape) {
               cudaMemset(c->status, 0, sizeof(int)) == cudaSuccess &&
               cudaMalloc(&c->plan, sizeof(DevPlan)) == cudaSuccess &&
               cudaMemset(c->plan, 0, sizeof(DevPlan)) == cudaSuccess;
-    if (ok && !c->parts.any() && attention_units(g, c->parts, (int)B, 0) > ORDER_FROM) {
-        ok = cudaMalloc(&c->order.count, (1 + ORDER_LAST) * ORDER_CLASSES * sizeof(uint32_t)) == cudaSuccess;
-        c->order.list = c->order.count + ORDER_CLASSES;
-    }
+    if (ok && !c->parts.any() && attention_units(g, c->parts, (int)B, 0) > ORDER_FROM)
+        ok = cudaMalloc(&c->order.cls, ORDER_LAST) == cudaSuccess;
     if (ok && c->parts.any()) ok = cudaMalloc(&c->parts.partial, attention_partial_bytes(g, shape->B_max, c->parts)) == cudaSuccess;
     if (!ok) {
         cudaGetLastError();
@@ -276,7 +279,7 @@ int rapid3_destroy(rapid3_ctx* c) {
     cudaFree(c->status);
     cudaFree(c->plan);
     cudaFree(c->parts.partial);
-    cudaFree(c->order.count);
+    cudaFree(c->order.cls);
     for (void* s : c->stage) cudaFree(s);
     if (c->up_s) cudaStreamDestroy(c->up_s);
     if (c->down_s) cudaStreamDestroy(c->down_s);
@@ -461,6 +464,16 @@ static int gated_step_impl(rapid3_ctx* c, const void* q, const void* k, const vo
         if (all.slot[p] >= 0) sparse.slot[all.slot[p]] = p - (all.n - sparse.n);
     if (sparse.n > 0) {
         if ((reinterpret_cast<uintptr_t>(q) % 16) || (reinterpret_cast<uintptr_t>(k) % 16)) return RAPID3_ERR_INVALID_ARG;
+    }
+    const int cluster = scoring_cluster(g, all.n, sparse.n * g.H, !prep, mass_scale != nullptr, mask_free_us(g, all.n - sparse.n, sparse.n));
+    if (sparse.n > 0 && cluster > 0) {
+        ProfScope ps(c, prep ? PROF_SCORES : PROF_POOL, st);
+        if (launch_scoring(q, k, g, sparse, c->pooled, c->scores, c->bitmask, c->kept_idx, c->kept_cnt, cluster, !prep,
+                           per_head ? &hk : nullptr, mass_scale ? &share : nullptr, mass_scale ? *mass_scale : 0.f, st, nullptr, 0,
+                           order) != cudaSuccess)
+            return RAPID3_ERR_CUDA;
+        c->launches += 1;
+    } else if (sparse.n > 0) {
         if (!prep) {
             ProfScope ps(c, PROF_POOL, st);
             if (launch_block_pool(q, k, g, sparse, c->pooled, st) != cudaSuccess) return RAPID3_ERR_CUDA;
@@ -468,7 +481,7 @@ static int gated_step_impl(rapid3_ctx* c, const void* q, const void* k, const vo
         }
         {
             ProfScope ps(c, PROF_SCORES, st);
-            if (launch_block_scores(c->pooled, g, sparse.n, c->scores, st, nullptr, order) != cudaSuccess) return RAPID3_ERR_CUDA;
+            if (launch_block_scores(c->pooled, g, sparse.n, c->scores, st) != cudaSuccess) return RAPID3_ERR_CUDA;
         }
         {
             ProfScope ps(c, PROF_SELECT, st);
@@ -538,13 +551,22 @@ int rapid3_gated_step_device(rapid3_ctx* c, const void* q, const void* k, const 
     ImgList none;
     none.n = 0;
     const QuadOrder order = step_order(c, c->g, B);
+    // chosen as for a batch of which every other image is dense
+    if (const int cluster = scoring_cluster(c->g, B, (B + 1) / 2 * c->g.H, true, false, mask_free_us(c->g, B / 2, (B + 1) / 2))) {
+        ProfScope ps(c, PROF_POOL, st);
+        if (launch_scoring(q, k, c->g, none, c->pooled, c->scores, c->bitmask, c->kept_idx, c->kept_cnt, cluster, true, nullptr, nullptr,
+                           0.f, st, c->plan, B, order) != cudaSuccess)
+            return RAPID3_ERR_CUDA;
+        c->launches += 2;
+        return attn_launch(c, c->g, q, k, v, out, none, c->kept_idx, c->kept_cnt, c->bitmask, softmax_scale, st, c->plan, B, true, order);
+    }
     {
         ProfScope ps(c, PROF_POOL, st);
         if (launch_block_pool(q, k, c->g, none, c->pooled, st, c->plan, B) != cudaSuccess) return RAPID3_ERR_CUDA;
     }
     {
         ProfScope ps(c, PROF_SCORES, st);
-        if (launch_block_scores(c->pooled, c->g, B, c->scores, st, c->plan, order) != cudaSuccess) return RAPID3_ERR_CUDA;
+        if (launch_block_scores(c->pooled, c->g, B, c->scores, st, c->plan) != cudaSuccess) return RAPID3_ERR_CUDA;
     }
     {
         ProfScope ps(c, PROF_SELECT, st);

@@ -12,6 +12,8 @@
 #define RAPID3_MAX_IMG 64     // images per launch (lists travel as kernel arguments)
 #define RAPID3_MAX_NB 1024    // key blocks per sequence (65536 tokens)
 
+constexpr int SM_COUNT = 148; // of a B200
+
 // Per-launch image list.  batch[p]: index into the B dimension of Q/K/V/O.
 // slot[p]: index into the compacted scores / mask / kept-list arrays, or -1 for a dense image.
 // k_free[p]: free candidates kept per image row (select kernel).
@@ -95,10 +97,9 @@ __host__ __device__ inline int quad_block(const TensorGeom& g, int quad, int a) 
 // head 197.5 -> 190.2, by cumulative mass 358.2 -> 346.3, a dense one and one at 0.5 (D = 64) 262.5 -> 257.3; one image of 432
 // quads at 0.5 from raw projections 190.5 -> 182.9.  Outside these bounds the idle SMs at the end cost less than the heads'
 // first reads at once and the longer selection do (192 quads 41.2 -> 42.1; 1632 quads at D = 64 303.5 -> 313.7).
-constexpr int ORDER_CLASSES = 32, ORDER_LAST = 444, ORDER_FROM = 296, ORDER_TO = 1000;
+constexpr int ORDER_CLASSES = 32, ORDER_LAST = 448, ORDER_FROM = 296, ORDER_TO = 1000;
 struct QuadOrder {
-    uint32_t* count = nullptr;       // [ORDER_CLASSES] quads of the class; the scores kernel of a step sets them to zero
-    uint32_t* list = nullptr;        // [ORDER_CLASSES][ORDER_LAST] (place of the image * H + head) * quads + quad, in any order
+    uint8_t* cls = nullptr;          // [ORDER_LAST] class of the quad at that place from the first of the last on; 16-byte aligned
 };
 
 // Programmatic dependent launch: every kernel of a step is launched so that it may start while the kernel before it in the stream
@@ -132,6 +133,27 @@ inline cudaError_t launch_kernel_carveout(void (*kernel)(KArgs...), dim3 grid, d
     if (e != cudaSuccess) cudaGetLastError();     // the caller has it: the next call must not find it again
     return e;
 }
+// The same for a kernel of clusters of that many thread blocks.
+template <typename... KArgs, typename... Args>
+inline cudaError_t launch_kernel_cluster(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, int cluster,
+                                         Args&&... args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cudaLaunchAttribute attr[2];
+    cfg.attrs = attr;
+    cfg.numAttrs = 2;
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    attr[1].id = cudaLaunchAttributeClusterDimension;
+    attr[1].val.clusterDim.x = (unsigned)cluster;
+    attr[1].val.clusterDim.y = attr[1].val.clusterDim.z = 1;
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, static_cast<KArgs>(args)...);
+    if (e != cudaSuccess) cudaGetLastError();
+    return e;
+}
 template <typename... KArgs, typename... Args>
 inline cudaError_t launch_kernel(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t s,
                                  Args&&... args) {
@@ -145,7 +167,7 @@ inline cudaError_t launch_kernel(void (*kernel)(KArgs...), dim3 grid, dim3 block
 cudaError_t launch_block_pool(const void* q, const void* k, const TensorGeom& g, const ImgList& imgs,
                               double* pooled, cudaStream_t s, const DevPlan* plan = nullptr, int n_cap = 0);
 cudaError_t launch_block_scores(const double* pooled, const TensorGeom& g, int n_img, float* scores,
-                                cudaStream_t s, const DevPlan* plan = nullptr, const QuadOrder& order = QuadOrder());
+                                cudaStream_t s, const DevPlan* plan = nullptr);
 // K2: forced + top-k selection.
 cudaError_t launch_select_mask(const float* scores, const TensorGeom& g, const ImgList& imgs,
                                uint64_t* bitmask, int32_t* kept_idx, int32_t* kept_cnt, cudaStream_t s,
@@ -159,6 +181,14 @@ cudaError_t launch_select_mask_heads(const float* scores, const TensorGeom& g, c
 cudaError_t launch_select_mask_mass(const float* scores, const TensorGeom& g, const ImgList& imgs,
                                     const MassShare& share, float scale, int32_t* row_keep, uint64_t* bitmask,
                                     int32_t* kept_idx, int32_t* kept_cnt, cudaStream_t s, const QuadOrder& order = QuadOrder());
+// K6: means (pool = true; else they are there), scores and selection in one launch of clusters of `cluster` thread blocks.  heads: a count per (image, head); share: the cumulative-mass rule; neither: imgs.k_free.
+cudaError_t launch_scoring(const void* q, const void* k, const TensorGeom& g, const ImgList& imgs, double* pooled, float* scores,
+                           uint64_t* bitmask, int32_t* kept_idx, int32_t* kept_cnt, int cluster, bool pool, const HeadKeep* heads,
+                           const MassShare* share, float mass_scale, cudaStream_t s, const DevPlan* plan = nullptr, int n_cap = 0,
+                           const QuadOrder& order = QuadOrder());
+// The cluster size for that many (image, head) pairs of a step with `images` attending, beside heavy_us of SM time of attention
+// that needs no mask; 0: not this way.
+int scoring_cluster(const TensorGeom& g, int images, int pairs, bool pool, bool mass, double heavy_us);
 // K5: Q/K producer (RMS norm + gain + rotary embedding -> bf16) that also writes the block means of
 // the images with a workspace slot.  pooled is [2][n_sparse][H][nb][D].
 struct PrepArgs {

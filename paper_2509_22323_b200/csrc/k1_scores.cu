@@ -3,26 +3,19 @@
 //                   fp64 accumulation, mean over the valid tokens of the block.
 //                   HBM-bound: reads Q and K exactly once.
 //   scores_kernel : S[i][j] = Qbar[i,:] . Kbar[j,:] in fp64 (fp64 mma.sync fragments), rounded once to fp32.
-#include "common.cuh"
+#include "scoring.cuh"
+
+using namespace scoring;
 
 namespace {
 
-__device__ __forceinline__ float bf16_lo(uint32_t w) { return __uint_as_float(w << 16); }
-__device__ __forceinline__ float bf16_hi(uint32_t w) { return __uint_as_float(w & 0xffff0000u); }
-
-// One warp per (Q|K, image, head, 64-token block).  A token row of D channels is D / 8 lanes of
-// 16 bytes, so one warp-wide load covers 32 / (D / 8) rows; every lane keeps fp64 sums of its 8
-// channels over the rows it sees (eight loads in flight per lane), and the lanes that hold the
-// same channels are then added with shuffles.  No shared memory.  The batches of eight loads are not unrolled into
+// One warp per (Q|K, image, head, 64-token block).  No shared memory.  The batches of eight loads are not unrolled into
 // one another: that keeps the kernel under 85 registers, six thread blocks per SM (measured 29 against 40 us on the
 // FLUX 1024^2 shapes, where 125 registers left four).
 template <int D>
 __global__ void __launch_bounds__(128, 6) pool_kernel(const uint16_t* q, const uint16_t* k,
                                                    TensorGeom g, ImgList imgs, double* __restrict__ pooled,
                                                    const DevPlan* plan, int n_cap) {
-    constexpr int TPR = D / 8;          // lanes per token row (8 channels = 16 bytes each)
-    constexpr int RPL = 32 / TPR;       // rows per warp-wide load
-    constexpr int ITERS = 64 / RPL;     // loads per lane
     const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
     const int blk = blockIdx.x * 4 + warp, h = blockIdx.y;
     grid_dependency_wait();                           // first kernel of a call: what comes before it may still be running
@@ -31,60 +24,10 @@ __global__ void __launch_bounds__(128, 6) pool_kernel(const uint16_t* q, const u
     const int p = blockIdx.z - which * n_cap;
     if (plan && p >= __ldcg(&plan->sparse.n)) return;  // device-resident plan: fewer images than the grid covers
     const int batch = plan ? __ldcg(&plan->sparse.batch[p]) : imgs.batch[p];
-    const uint16_t* base = (which ? k : q) + (long long)batch * g.stride_b + (long long)(g.h0 + h) * g.stride_h;
-    const int c = lane % TPR, r0 = lane / TPR;
-    const int n0 = blk * 64;
-    const int valid = min(64, g.N - n0);
-
-    double acc[8];
-#pragma unroll
-    for (int e = 0; e < 8; ++e) acc[e] = 0.0;
-#pragma unroll 1
-    for (int it0 = 0; it0 < ITERS; it0 += 8) {
-        uint4 v[8];
-#pragma unroll
-        for (int u = 0; u < 8; ++u) {
-            const int row = (it0 + u) * RPL + r0;
-            v[u] = make_uint4(0, 0, 0, 0);
-            if (row < valid)
-                v[u] = __ldcg(reinterpret_cast<const uint4*>(base + (long long)(n0 + row) * g.stride_n + c * 8));
-        }
-#pragma unroll
-        for (int u = 0; u < 8; ++u) {
-            acc[0] += (double)bf16_lo(v[u].x); acc[1] += (double)bf16_hi(v[u].x);
-            acc[2] += (double)bf16_lo(v[u].y); acc[3] += (double)bf16_hi(v[u].y);
-            acc[4] += (double)bf16_lo(v[u].z); acc[5] += (double)bf16_hi(v[u].z);
-            acc[6] += (double)bf16_lo(v[u].w); acc[7] += (double)bf16_hi(v[u].w);
-        }
-    }
-    grid_dependency_launch();                         // not before the loads are through (steps of 17 to 25 us: 1 to 2 %)
-#pragma unroll
-    for (int off = TPR; off < 32; off <<= 1)
-#pragma unroll
-        for (int e = 0; e < 8; ++e) acc[e] += __shfl_xor_sync(0xffffffffu, acc[e], off);
-    if (lane < TPR) {
-        double* o = pooled + ((((long long)which * n_cap + p) * g.H + h) * g.nb + blk) * D + c * 8;
-        const double inv = 1.0 / (double)valid;
-#pragma unroll
-        for (int e = 0; e < 8; e += 2) {
-            double2 w2 = make_double2(acc[e] * inv, acc[e + 1] * inv);
-            *reinterpret_cast<double2*>(o + e) = w2;
-        }
-    }
-}
-
-// D(8 x 8, fp64) += A(8 x 4, row) * B(4 x 8, col) on the fp64 tensor path (four times the rate of the fp64 FMA pipe
-// on this part).  Lane l holds a = A[l / 4][l % 4], b = B[l % 4][l / 4] and c0, c1 = D[l / 4][2 (l % 4) + {0, 1}].
-__device__ __forceinline__ void dmma_8x8x4(double& c0, double& c1, double a, double b) {
-    asm volatile("mma.sync.aligned.m8n8k4.row.col.f64.f64.f64.f64 {%0, %1}, {%2}, {%3}, {%0, %1};"
-                 : "+d"(c0), "+d"(c1)
-                 : "d"(a), "d"(b));
-}
-
-__device__ __forceinline__ void copy16_async(double* dst, const double* src, bool valid) {   // past the L1; zeros if not valid
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;"
-                 ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src), "r"(valid ? 16 : 0)
-                 : "memory");
+    const uint16_t* base = (which ? k : q) + (long long)batch * g.stride_b + (long long)(g.h0 + h) * g.stride_h + (long long)(blk * 64) * g.stride_n;
+    double* out = pooled + ((((long long)which * n_cap + p) * g.H + h) * g.nb + blk) * D;
+    // the next kernel's start: not before the loads are through (steps of 17 to 25 us: 1 to 2 %)
+    pool_block<D>(base, g.stride_n, min(64, g.N - blk * 64), out, lane, [] { grid_dependency_launch(); });
 }
 
 // 32 x 32 tile of S per thread block, eight warps; a warp owns two fragments of 8 x 8 outputs side by side.  The two
@@ -95,7 +38,7 @@ __device__ __forceinline__ void copy16_async(double* dst, const double* src, boo
 // lanes.  Every output accumulates its products in ascending order of the four-channel groups.
 template <int D>
 __global__ void __launch_bounds__(256) scores_kernel(const double* pooled, TensorGeom g, int n_img,
-                                                     float* __restrict__ scores, const DevPlan* plan, uint32_t* order_count) {
+                                                     float* __restrict__ scores, const DevPlan* plan) {
     constexpr int T = 32, LDS = D + 4;
     extern __shared__ __align__(16) double tiles[];
     double* sq = tiles;
@@ -105,8 +48,6 @@ __global__ void __launch_bounds__(256) scores_kernel(const double* pooled, Tenso
     // and read them past the L1, whose lines no such wait is known to refresh.
     grid_dependency_wait();
     grid_dependency_launch();
-    // the attention of the step before, which reads these, has ended: the kernel in front has waited for it
-    if (order_count && blockIdx.x + blockIdx.y + blockIdx.z == 0 && threadIdx.x < ORDER_CLASSES) order_count[threadIdx.x] = 0u;
     if (plan && ph >= __ldcg(&plan->sparse.n) * g.H) return;
     const int i0 = blockIdx.y * T, j0 = blockIdx.x * T;
     const double* pq = pooled + ((long long)ph * g.nb + i0) * D;
@@ -168,12 +109,12 @@ cudaError_t launch_block_pool(const void* q, const void* k, const TensorGeom& g,
 }
 
 cudaError_t launch_block_scores(const double* pooled, const TensorGeom& g, int n_img, float* scores,
-                                cudaStream_t s, const DevPlan* plan, const QuadOrder& order) {
+                                cudaStream_t s, const DevPlan* plan) {
     // with a plan n_img is the capacity.  32 x 32 tiles at every length: against 64 x 64 tiles they waste less of
     // the ragged edge and fill the SMs more evenly (30 against 35 us at 264 blocks, where 64 x 64 pads 264 to 320)
     const dim3 grid((g.nb + 31) / 32, (g.nb + 31) / 32, n_img * g.H);
     return launch_kernel(g.D == 128 ? scores_kernel<128> : scores_kernel<64>, grid, dim3(256), scores_smem_bytes(g.D), s,
-                         pooled, g, n_img, scores, plan, order.count);
+                         pooled, g, n_img, scores, plan);
 }
 
 cudaError_t scoring_static_init() {

@@ -48,7 +48,6 @@ constexpr int SOFTMAX_WARPS = 16;
 constexpr int PRODUCER_WARP = 16, MMA_WARP0 = 17, LIST_WARP = 19;
 constexpr int NTHREADS = 32 * (SOFTMAX_WARPS + 4);
 constexpr int TMEM_COLS = 512;
-constexpr int SM_COUNT = 148;       // of a B200
 constexpr int TILE_COLS = 256;      // TMEM columns of one Q tile
 constexpr int BLK_BYTES = 8192;     // 64 rows x 128 bytes: one 64-channel half of a 64-token block
 constexpr int QHALF_BYTES = 16384;  // one 64-channel half of a 128-row Q tile
@@ -148,6 +147,32 @@ __device__ __forceinline__ uint4 quad_transpose(uint32_t w0, uint32_t w1, uint32
     const uint32_t p0 = b0 ? x : w0, p1 = b0 ? w1 : x, q0 = b0 ? y : w2, q1 = b0 ? w3 : y;
     const uint32_t r0 = __shfl_xor_sync(0xffffffffu, b1 ? p0 : q0, 2), r1 = __shfl_xor_sync(0xffffffffu, b1 ? p1 : q1, 2);
     return b1 ? make_uint4(r0, r1, q0, q1) : make_uint4(p0, p1, r0, r1);
+}
+
+// Place of the `rest`-th quad in the order of the classes; a lane holds those of quads 16 lane .. 16 lane + 15, 0xff: no quad.
+__device__ __forceinline__ int order_find(const uint32_t (&cls)[4], int rest, int lane) {
+    auto below = [&](uint32_t c) {                       // of the lane's quads, those of a class below c
+        int n = 0;
+#pragma unroll
+        for (int x = 0; x < 4; ++x) n += __popc(__vcmpltu4(cls[x], c * 0x01010101u)) >> 3;
+        return n;
+    };
+    uint32_t c = 0u;                                     // the quad's class: the last with no more than `rest` quads below it
+#pragma unroll
+    for (uint32_t bit = ORDER_CLASSES / 2; bit > 0; bit >>= 1)
+        if ((int)__reduce_add_sync(0xffffffffu, (uint32_t)below(c | bit)) <= rest) c |= bit;
+    const int lower = below(c), own = below(c + 1u) - lower;
+    int before = own;                                    // quads of the class in the lanes below this one
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const int v = __shfl_up_sync(0xffffffffu, before, o);
+        if (lane >= o) before += v;
+    }
+    int skip = rest - (int)__reduce_add_sync(0xffffffffu, (uint32_t)lower) - (before - own), at = -1;
+#pragma unroll
+    for (int x = 0; x < 16; ++x)
+        if (((cls[x / 4] >> (8 * (x % 4))) & 0xffu) == c && skip-- == 0) at = 16 * lane + x;
+    return (int)__reduce_max_sync(0xffffffffu, at);      // the other lanes have -1
 }
 
 // Maxima of a quad's two rows over one key block, from the four threads' 16x256b fragments.
@@ -319,7 +344,7 @@ attn_kernel(const __grid_constant__ CUtensorMap tmq, const __grid_constant__ CUt
         };
         int L = blockIdx.x;
         bool waited = false;                             // for the selection kernel, see below
-        uint32_t class_end = 0u;                         // quads of the classes up to the lane's, once `have_classes`
+        uint32_t classes[4];                             // of sixteen quads in the order, once `have_classes`
         bool have_classes = false;
         for (uint32_t i = 0;; ++i) {
             Quad& u = ctl->quad[i & 1];
@@ -374,33 +399,32 @@ attn_kernel(const __grid_constant__ CUtensorMap tmq, const __grid_constant__ CUt
                     h = L / nq; quad = L - h * nq;
                 } else if (L < heavy_dense + heavy_sparse) {
                     L -= heavy_dense;
-                    p = L / (g.H * ntq); L -= p * g.H * ntq; p += nd;
-                    h = L / ntq; quad = L - h * ntq;
+                    // those of text rows alone first: they need no mask, which may not be there yet
+                    const int ntf = SPLIT ? ntq : g.n_text_blocks >> 2, n_full = ns * g.H * ntf;
+                    const bool full = L < n_full;
+                    const int first = full ? 0 : ntf, n = full ? ntf : ntq - ntf;       // quads of a head from `first` on
+                    if (!full) L -= n_full;
+                    p = L / (g.H * n); L -= p * g.H * n; p += nd;
+                    h = L / n; quad = first + L - h * n;
                 } else {
                     L -= heavy_dense + heavy_sparse;
-                    const int nl = nq - ntq, rest = L - max(ns * g.H * nl - ORDER_LAST, 0);
+                    const int nl = nq - ntq, in_order = max(ns * g.H * nl - ORDER_LAST, 0), rest = L - in_order;
                     if (ORDERED && rest >= 0) {
-                        // the quad at this place of the order that the selection kernel has found
+                        // the quad at place `rest` of the order that the selection kernel has found: of sixteen classes a lane
                         if (!have_classes) {
                             if (!waited) grid_dependency_wait();
                             waited = have_classes = true;
-                            class_end = __ldcg(prm.order.count + lane);
+                            const uint4 v = 16 * lane < ORDER_LAST ? __ldcg(reinterpret_cast<const uint4*>(prm.order.cls) + lane) : make_uint4(0, 0, 0, 0);
+                            classes[0] = v.x; classes[1] = v.y; classes[2] = v.z; classes[3] = v.w;
+                            const int n = ns * g.H * nl - in_order;      // quads in the order; the bytes behind them count for nothing
 #pragma unroll
-                            for (int o = 1; o < 32; o <<= 1) {
-                                const uint32_t v = __shfl_up_sync(0xffffffffu, class_end, o);
-                                if (lane >= o) class_end += v;
-                            }
+                            for (int x = 0; x < 16; ++x)
+                                if (16 * lane + x >= n) classes[x / 4] |= 0xffu << (8 * (x % 4));
                         }
-                        const int c = min(__popc(__ballot_sync(0xffffffffu, class_end <= (uint32_t)rest)), ORDER_CLASSES - 1);
-                        const int before = __shfl_sync(0xffffffffu, (int)class_end, max(c - 1, 0));
-                        L = __ldcg(prm.order.list + c * ORDER_LAST + rest - (c > 0 ? before : 0));
-                        quad = L % nq; L /= nq;
-                        h = L % g.H;
-                        p = nd + L / g.H;
-                    } else {
-                        p = L / (g.H * nl); L -= p * g.H * nl; p += nd;
-                        h = L / nl; quad = ntq + (L - h * nl);
+                        L = in_order + order_find(classes, rest, lane);
                     }
+                    p = L / (g.H * nl); L -= p * g.H * nl; p += nd;
+                    h = L / nl; quad = ntq + (L - h * nl);
                 }
             }
             const int b = prm.plan ? __ldcg(&prm.plan->all.batch[p]) : prm.imgs.batch[p];
@@ -409,6 +433,8 @@ attn_kernel(const __grid_constant__ CUtensorMap tmq, const __grid_constant__ CUt
                 if (half >= 0 && (a >> 1) != half) return nb;           // not of this unit: like a block past the end
                 return quad_block(g, quad, a);
             };
+            // a dense image's quad, or one of text rows in a mask of the selection kernel: every block is kept, no mask is read
+            const bool all_kept = slot < 0 || (prm.bitmask32 != nullptr && 4 * quad + 3 < g.n_text_blocks);
             // the query block whose kept blocks m[a] below holds: where a list is cut into parts depends on the whole quad
             auto mblk = [&](int a) -> int { return SPLIT && parts > 1 ? quad_block(g, quad, a) : qblk(a); };
             if (lane == 0) {
@@ -422,8 +448,8 @@ attn_kernel(const __grid_constant__ CUtensorMap tmq, const __grid_constant__ CUt
                     // row, so the union list starts 0, 1, ....  First use of their stages, nothing to wait for.
                     load_q(u);
                     const bool none = min(min(qblk(0), qblk(1)), min(qblk(2), qblk(3))) >= nb;   // the second half of a ragged last quad
-                    int n_early = (!INJECT && !none && (slot < 0 || prm.bitmask32 != nullptr)) ? min(min(slot < 0 ? nb : g.n_text_blocks, nb), KS) : 0;
-                    if (SPLIT && parts > 1) n_early = part == 0 ? min(n_early, (slot < 0 ? nb : g.n_text_blocks) / parts) : 0;   // its part of the list is no shorter
+                    int n_early = (!INJECT && !none && (all_kept || prm.bitmask32 != nullptr)) ? min(min(all_kept ? nb : g.n_text_blocks, nb), KS) : 0;
+                    if (SPLIT && parts > 1) n_early = part == 0 ? min(n_early, (all_kept ? nb : g.n_text_blocks) / parts) : 0;   // its part of the list is no shorter
                     for (int gi = 0; gi < n_early; ++gi) issue_group(u, gi, gi, gi - 1, gi - 1);
                     ctl->n_early = n_early;
                 }
@@ -432,7 +458,7 @@ attn_kernel(const __grid_constant__ CUtensorMap tmq, const __grid_constant__ CUt
             // else rebuilt from the kept list; every block for a dense image.
             const int nw = (nb + 31) >> 5;
             uint32_t m[4];
-            if (slot < 0) {
+            if (all_kept) {
                 const int n = min(max(nb - lane * 32, 0), 32);
                 const uint32_t val = n == 32 ? 0xffffffffu : ((1u << n) - 1u);
 #pragma unroll
@@ -1178,7 +1204,7 @@ cudaError_t launch_attention(const CUtensorMap& tmq, const CUtensorMap& tmk, con
         return launch_kernel(g.D == 128 ? add_parts_kernel<128> : add_parts_kernel<64>, dim3(left * SOFTMAX_WARPS * (g.D / 32) / 4), dim3(128), 0, s,
                              static_cast<uint16_t*>(out), g, imgs, n_dense, plan, prm.parts);
     } else {
-        return launch_kernel(order.count ? (g.D == 128 ? attn_kernel<128, false, false, true> : attn_kernel<64, false, false, true>)
+        return launch_kernel(order.cls ? (g.D == 128 ? attn_kernel<128, false, false, true> : attn_kernel<64, false, false, true>)
                                          : (g.D == 128 ? attn_kernel<128> : attn_kernel<64>),
                              grid, dim3(NTHREADS), g.D == 128 ? attn_smem_bytes<128>() : attn_smem_bytes<64>(), s, tmq, tmk, tmv,
                              static_cast<uint16_t*>(out), prm);
