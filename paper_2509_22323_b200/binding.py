@@ -106,7 +106,8 @@ def _f32(xs: Sequence[float]):
 
 
 def _stream() -> int:
-    return torch.cuda.current_stream().cuda_stream
+    # the handle of torch.cuda.current_stream() without the Stream object around it, which takes 3.2 us of a call to build (0.2 so)
+    return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
 
 
 def _ptr(t: Optional[torch.Tensor]):
