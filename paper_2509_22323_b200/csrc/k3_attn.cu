@@ -478,16 +478,36 @@ attn_kernel(const __grid_constant__ CUtensorMap tmq, const __grid_constant__ CUt
 #pragma unroll
                     for (int a = 0; a < 4; ++a) ctl->bm[a][lane] = 0u;
                     __syncwarp();
+                    // the counts and the first 64 entries of all four rows on their way at once, the entries before their counts are
+                    // known (324 quads of 10 to 33 blocks: whole staged calls 81.5 -> 80.3 us; 144 quads 40.9 -> 38.3)
+                    const int32_t* lst[4];
+                    int cnt[4], first[4], second[4];
+#pragma unroll
                     for (int a = 0; a < 4; ++a) {
-                        if (mblk(a) >= nb) continue;
-                        const long long row = ((long long)slot * g.H + h) * nb + mblk(a);
-                        const int cnt = min(max(__ldcg(prm.kept_cnt + row), 0), nb);
-                        const int32_t* lst = prm.kept_idx + row * nb;
-                        for (int e = lane; e < cnt; e += 32) {
-                            const int j = __ldcg(lst + e);
-                            if ((unsigned)j < (unsigned)nb) atomicOr(&ctl->bm[a][j >> 5], 1u << (j & 31));
-                            else atomicExch(prm.status, RAPID3_ERR_BAD_LIST);
-                        }
+                        const bool in = mblk(a) < nb;
+                        const long long row = ((long long)slot * g.H + h) * nb + (in ? mblk(a) : 0);
+                        lst[a] = prm.kept_idx + row * nb;
+                        cnt[a] = in ? __ldcg(prm.kept_cnt + row) : 0;
+                        first[a] = in && lane < nb ? __ldcg(lst[a] + lane) : 0;
+                        second[a] = in && 32 + lane < nb ? __ldcg(lst[a] + 32 + lane) : 0;
+                    }
+                    auto put = [&](int a, int e, int j) {
+                        if (e >= min(cnt[a], nb)) return;
+                        if ((unsigned)j < (unsigned)nb) atomicOr(&ctl->bm[a][j >> 5], 1u << (j & 31));
+                        else atomicExch(prm.status, RAPID3_ERR_BAD_LIST);
+                    };
+#pragma unroll
+                    for (int a = 0; a < 4; ++a) {
+                        put(a, lane, first[a]);
+                        put(a, 32 + lane, second[a]);
+                    }
+                    const int most = min(max(max(cnt[0], cnt[1]), max(cnt[2], cnt[3])), nb);
+                    for (int e = 64 + lane; e < most; e += 32) {
+                        int j[4];
+#pragma unroll
+                        for (int a = 0; a < 4; ++a) j[a] = e < min(cnt[a], nb) ? __ldcg(lst[a] + e) : 0;
+#pragma unroll
+                        for (int a = 0; a < 4; ++a) put(a, e, j[a]);
                     }
                     __syncwarp();
 #pragma unroll
