@@ -8,15 +8,6 @@
 // HBM-bound: reads the raw Q and K once, writes Q and K once.
 #include "common.cuh"
 
-// Measured on FLUX 1024^2 shapes: two rows in flight per lane at six CTAs per SM (74 registers) beat deeper
-// prefetch at lower occupancy; the kernel is bound by instruction issue and latency, not by the loads in flight.
-#ifndef PREP_INFL
-#define PREP_INFL 2
-#endif
-#ifndef PREP_MINB
-#define PREP_MINB 6
-#endif
-
 namespace {
 
 __device__ __forceinline__ float bf16_lo(uint32_t w) { return __uint_as_float(w << 16); }
@@ -27,8 +18,12 @@ __device__ __forceinline__ uint32_t pack2(float lo, float hi) {
     return d;
 }
 
-template <int D>
-__global__ void __launch_bounds__(128, PREP_MINB) prepare_kernel(const uint16_t* q_raw,
+// INFL rows in flight per lane.  Two at six thread blocks per SM beat deeper prefetch at lower occupancy on large launches, which are
+// bound by instruction issue and latency, not by the loads in flight; eight where the thread blocks have an SM to themselves or nearly
+// so and the time is the chain of their loads (steps of one image from raw projections: 2 heads x 36 blocks at D = 64
+// 26.6 -> 25.5 us, 12 heads x 10 blocks at D = 128 29.0 -> 27.4).
+template <int D, int INFL>
+__global__ void __launch_bounds__(128, INFL > 2 ? 2 : 6) prepare_kernel(const uint16_t* q_raw,
                                                       const uint16_t* k_raw, uint16_t* q_out,
                                                       uint16_t* k_out, const float* q_gain,
                                                       const float* k_gain, const float* rot, float eps, TensorGeom g,
@@ -36,7 +31,6 @@ __global__ void __launch_bounds__(128, PREP_MINB) prepare_kernel(const uint16_t*
     constexpr int TPR = D / 8;          // lanes per token row (8 channels = 16 bytes each)
     constexpr int RPL = 32 / TPR;       // rows per warp-wide load
     constexpr int ITERS = 64 / RPL;     // loads per lane
-    constexpr int INFL = PREP_INFL;     // rows in flight per lane
     const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
     const int blk = blockIdx.x * 4 + warp, h = blockIdx.y;
     grid_dependency_wait();                           // first kernel of a call: what comes before it may still be running
@@ -152,6 +146,8 @@ cudaError_t launch_prepare(const PrepArgs& a, const TensorGeom& g, const ImgList
     const uint16_t* kr = static_cast<const uint16_t*>(a.k_raw);
     uint16_t* qo = static_cast<uint16_t*>(a.q_out);
     uint16_t* ko = static_cast<uint16_t*>(a.k_out);
-    return launch_kernel(g.D == 128 ? prepare_kernel<128> : prepare_kernel<64>, grid, dim3(128), 0, s, qr, kr, qo, ko, a.q_gain,
+    const bool few = (long long)grid.x * grid.y * grid.z <= 2 * SM_COUNT;
+    return launch_kernel(few ? (g.D == 128 ? prepare_kernel<128, 8> : prepare_kernel<64, 8>)
+                             : (g.D == 128 ? prepare_kernel<128, 2> : prepare_kernel<64, 2>), grid, dim3(128), 0, s, qr, kr, qo, ko, a.q_gain,
                          a.k_gain, a.rot, a.eps, g, imgs, n_sparse, pooled);
 }

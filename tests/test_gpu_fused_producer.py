@@ -120,3 +120,32 @@ def test_fused_producer_all_dense_and_argument_checks():
     with pytest.raises(binding.Rapid3Error) as e:                  # misaligned gain pointer
         ctx.rapid3_gated_step_fused(Qr, Kr, V, torch.ones(65, device=DEV)[1:], k_gain, rot, EPS, q, k, out, [2, 2], [1.0, 1.0])
     assert e.value.code == -1
+
+
+@pytest.mark.parametrize("D,H,n_text,n_image,in_place", [(128, 8, 77, 36 * 64 - 76, True), (64, 9, 0, 32 * 64 + 1, False)])
+def test_producer_of_few_and_of_many_blocks(D, H, n_text, n_image, in_place):
+    """Two images in one launch (more than two thread blocks of the producer an SM) and one at a time (fewer; more rows in
+    flight): the same Q, K, block means' masks and outputs, bit for bit."""
+    N = n_text + n_image
+    gen = torch.Generator(device=DEV).manual_seed(D)
+    Qr, Kr, V = [torch.randn((2, H, N, D), generator=gen, device=DEV).to(torch.bfloat16) for _ in range(3)]
+    gain = [0.5 + torch.rand(D, generator=gen, device=DEV) for _ in range(2)]
+    ang = torch.rand((N, D // 2), generator=gen, device=DEV) * 6.283185
+    rot = torch.stack([torch.cos(ang), torch.sin(ang)], dim=-1).contiguous()
+
+    def step(b):
+        src = [t[b].clone() for t in (Qr, Kr)]
+        q, k = src if in_place else [poison_like(t) for t in src]
+        out = poison_like(q)
+        n = q.shape[0]
+        ctx = binding.Context(n, H, D, n_text, n_image)
+        ctx.rapid3_gated_step_fused(*src, V[b].clone(), *gain, rot, EPS, q, k, out, [2] * n, [0.5] * n)
+        torch.cuda.synchronize()
+        assert ctx.last_status() == 0
+        return [t.clone() for t in (q.view(torch.int16), k.view(torch.int16), out.view(torch.int16), *ctx.workspace(n)[:2])]
+
+    both = step(slice(0, 2))
+    for b in range(2):
+        for x, y in zip(both, step(slice(b, b + 1))):
+            assert torch.equal(x[b:b + 1], y)
+    check_produced(Qr[1], both[0][1].view(torch.bfloat16), gain[0], rot, "Q")
