@@ -110,7 +110,7 @@ struct Quad {
 
 struct __align__(16) Ctl {
     uint4 taken;                        // answer of the last try_cancel
-    unsigned long long taken_full, near_end;
+    unsigned long long taken_full, near_end, first_known;
     unsigned long long quad_full[2], quad_empty[2];
     unsigned long long q_full, q_empty;
     unsigned long long k_full[MAX_STAGES], k_empty[MAX_STAGES];   // k_full[g % KS]: group g = K(g) and V(g - 1) have landed
@@ -118,7 +118,7 @@ struct __align__(16) Ctl {
     unsigned long long s_full[2][3], p_full[2][3];
     unsigned long long pv_done[2][2], o_done[2], drain[2];
     uint32_t tmem_base;
-    int n_early;                        // groups of the first quad that the list warp has loaded
+    int n_early;                        // groups of the first quad that the producer loads before its list is there
     volatile int abort_flag;
     uint32_t bm[4][32];                 // the list warp's scratch
     float nm[SOFTMAX_WARPS][16];        // SPLIT build: the reference maxima of a warp's rows, times -c2, as they last moved
@@ -206,7 +206,6 @@ attn_kernel(const __grid_constant__ CUtensorMap tmq, const __grid_constant__ CUt
             const __grid_constant__ CUtensorMap tmv, uint16_t* __restrict__ out, const __grid_constant__ AttnParams prm) {
     using C = Cfg<D>;
     constexpr int DH = C::DH, KS = C::KS, VS = C::VS, NBUF = C::NBUF, O_COL = C::O_COL;
-    constexpr bool MORE_REGS = SPLIT || (ORDERED && D == 128);
     extern __shared__ uint8_t smem_raw[];
     const uint32_t raw = smem_u32(smem_raw);
     const uint32_t pad = ((raw + 1023u) & ~1023u) - raw;
@@ -243,7 +242,7 @@ attn_kernel(const __grid_constant__ CUtensorMap tmq, const __grid_constant__ CUt
     const uint32_t bPV = smem_u32(&ctl->pv_done[0][0]);                                      // [tile][block parity]: + 16 t + 8 (n & 1)
     const uint32_t bOD = smem_u32(&ctl->o_done[0]);                                          // [tile]: + 8 t
     const uint32_t bUF = smem_u32(&ctl->quad_full[0]), bUE = smem_u32(&ctl->quad_empty[0]);  // quad i: + 8 (i & 1)
-    const uint32_t bNE = smem_u32(&ctl->near_end), bT = smem_u32(&ctl->taken_full);
+    const uint32_t bNE = smem_u32(&ctl->near_end), bT = smem_u32(&ctl->taken_full), bFK = smem_u32(&ctl->first_known);
 
     // ---------------------------------------------------------------- setup
     if (warp == 0) {                                    // one barrier group per lane
@@ -267,8 +266,8 @@ attn_kernel(const __grid_constant__ CUtensorMap tmq, const __grid_constant__ CUt
             mbar_init(bQE, 2);
             mbar_init(bNE, 1);
             mbar_init(bT, 1);
+            mbar_init(bFK, 1);
             ctl->abort_flag = 0;
-            ctl->n_early = 0;
         } else if (lane == MAX_STAGES + 9) {
             prefetch_tmap(&tmq);
             prefetch_tmap(&tmk);
@@ -333,9 +332,9 @@ attn_kernel(const __grid_constant__ CUtensorMap tmq, const __grid_constant__ CUt
         }
     };
 
-    // The pool is the launch's 640 x 96: 512 x 104 + 128 x 64.  Without it these builds keep five to ten words in local memory
-    // (step of 864 quads at D = 128 354.5 -> 353.0 us, of 432 204.5 -> 202.6; at D = 64 257.4 -> 258.4, not there).
-    if (MORE_REGS && warp >= SOFTMAX_WARPS) reg_dec<64>();
+    // The pool is the launch's 640 x 96: 512 x 104 + 128 x 64.  Without it this build keeps ten words of the softmax warps in
+    // local memory; in the other builds it gains nothing (ordered, D = 128: fused step of 432 quads 197.0 us without, 199.8 with).
+    if (SPLIT && warp >= SOFTMAX_WARPS) reg_dec<64>();
     if (warp == LIST_WARP) {
         // ------------------------------------------------------------ quads and their union lists
         // one lane polls: these waits are long, and the other lanes' polls would only take issue slots
@@ -433,8 +432,9 @@ attn_kernel(const __grid_constant__ CUtensorMap tmq, const __grid_constant__ CUt
                 if (half >= 0 && (a >> 1) != half) return nb;           // not of this unit: like a block past the end
                 return quad_block(g, quad, a);
             };
+            const bool masks = ORDERED || prm.bitmask32 != nullptr;      // of the selection kernel (it finds the order), else lists of the caller's
             // a dense image's quad, or one of text rows in a mask of the selection kernel: every block is kept, no mask is read
-            const bool all_kept = slot < 0 || (prm.bitmask32 != nullptr && 4 * quad + 3 < g.n_text_blocks);
+            const bool all_kept = slot < 0 || (masks && 4 * quad + 3 < g.n_text_blocks);
             // the query block whose kept blocks m[a] below holds: where a list is cut into parts depends on the whole quad
             auto mblk = [&](int a) -> int { return SPLIT && parts > 1 ? quad_block(g, quad, a) : qblk(a); };
             if (lane == 0) {
@@ -445,13 +445,14 @@ attn_kernel(const __grid_constant__ CUtensorMap tmq, const __grid_constant__ CUt
                 if (i == 0) {
                     // The first quad's Q tiles do not depend on the mask, nor do key blocks known before it is read: a
                     // dense image keeps every block, and a mask of the selection kernel keeps the text blocks in every
-                    // row, so the union list starts 0, 1, ....  First use of their stages, nothing to wait for.
-                    load_q(u);
+                    // row, so the union list starts 0, 1, ....  The producer loads them while the list is built (by this
+                    // lane, ahead of the masks, they kept the first list back: steps of 288 quads at D = 64 41.6 -> 40.8 us,
+                    // of 24 at D = 128 23.9 -> 23.0, lists of the caller's for 324 quads 80.2 -> 78.9).
                     const bool none = min(min(qblk(0), qblk(1)), min(qblk(2), qblk(3))) >= nb;   // the second half of a ragged last quad
-                    int n_early = (!INJECT && !none && (all_kept || prm.bitmask32 != nullptr)) ? min(min(all_kept ? nb : g.n_text_blocks, nb), KS) : 0;
+                    int n_early = (!INJECT && !none && (all_kept || masks)) ? min(min(all_kept ? nb : g.n_text_blocks, nb), KS) : 0;
                     if (SPLIT && parts > 1) n_early = part == 0 ? min(n_early, (all_kept ? nb : g.n_text_blocks) / parts) : 0;   // its part of the list is no shorter
-                    for (int gi = 0; gi < n_early; ++gi) issue_group(u, gi, gi, gi - 1, gi - 1);
                     ctl->n_early = n_early;
+                    mbar_arrive(bFK);
                 }
             }
             // m[a] = 32 bits of the set of key blocks that member a keeps: from the bitmask when the caller has one,
@@ -469,7 +470,7 @@ attn_kernel(const __grid_constant__ CUtensorMap tmq, const __grid_constant__ CUt
                 // line of an earlier step must not answer.
                 if (!waited) grid_dependency_wait();
                 waited = true;
-                if (prm.bitmask32 != nullptr) {
+                if (masks) {
 #pragma unroll
                     for (int a = 0; a < 4; ++a)
                         m[a] = (mblk(a) < nb && lane < nw)
@@ -570,16 +571,21 @@ attn_kernel(const __grid_constant__ CUtensorMap tmq, const __grid_constant__ CUt
     } else if (warp == PRODUCER_WARP) {
         // ------------------------------------------------------------ producer
         if (lane == 0) {
-            uint32_t G = 0, W0 = 0, n_q = 1;             // group to be issued next, the quad's first V block, Q loads so far
-            bool ok = true;
+            uint32_t G = 0, W0 = 0, n_q = 0;             // group to be issued next, the quad's first V block, Q loads so far
+            bool ok = wait(bFK, 0);
             uint32_t i = 0;
+            if (ok) {                                    // first use of all stages, nothing to wait for
+                const int n_early = ctl->n_early;
+                load_q(ctl->quad[0]);
+                n_q = 1;
+                for (; (int)G < n_early; ++G) issue_group(ctl->quad[0], G, G, G - 1, (int)G - 1);
+            }
             for (; ok; ++i) {
                 const Quad& u = ctl->quad[i & 1];
                 if (!(ok = wait(bUF + 8 * (i & 1), (i >> 1) & 1))) break;
                 const int n_u = u.n_u;
                 if (n_u < 0) break;
                 const int n_early = i == 0 ? ctl->n_early : 0;
-                G += n_early;
                 if (n_early > max(n_u - TAKE_AHEAD, 0)) mbar_arrive(bNE);
                 for (int gi = n_early; gi <= n_u; ++gi) {
                     if (INJECT && gi == prm.stop_group) { ok = false; break; }
@@ -604,8 +610,7 @@ attn_kernel(const __grid_constant__ CUtensorMap tmq, const __grid_constant__ CUt
             }
             if (INJECT || ctl->abort_flag) {
                 // drain: do not leave the CTA while bulk copies may still land in its shared memory
-                mbar_wait(bQ, (n_q - 1) & 1, 1u << 20);
-                G = max(G, (uint32_t)ctl->n_early);
+                if (n_q > 0) mbar_wait(bQ, (n_q - 1) & 1, 1u << 20);
                 for (uint32_t x = G > KS ? G - KS : 0; x < G; ++x)
                     mbar_wait(bKF + 8 * (x % KS), (x / KS) & 1, 1u << 20);
             }
@@ -733,7 +738,7 @@ attn_kernel(const __grid_constant__ CUtensorMap tmq, const __grid_constant__ CUt
         // (r_lo = lane / 4 and r_lo + 8 of the sixteen) and, of every group of eight score columns, the pair
         // 2 (lane % 4), + 1 -- 32 scores per key block.  The four threads of a quad share their rows' maximum
         // with two shuffles, and only when some row of the warp may have grown.
-        if (MORE_REGS) reg_inc<104>();
+        if (SPLIT) reg_inc<104>();
         const int t = (warp >> 2) & 1, wl = warp & 3, hf = warp >> 3;
         const int a = 2 * t + (wl >> 1);               // query block of the quad
         const uint32_t tile_bits = 3u << (2 * t), act_bit = 1u << a;
