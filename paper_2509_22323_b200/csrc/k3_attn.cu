@@ -200,7 +200,11 @@ __device__ __forceinline__ void row_maxima(const uint32_t (&r)[32], float& lo, f
 // of them.  (Added up by the last part of a quad to arrive, in this kernel, they cost its main loop 12 to 14 %: registers.)
 //
 // ORDERED is the build for launches whose last quads are handed out by their length (QuadOrder).
-template <int D, bool INJECT = false, bool SPLIT = false, bool ORDERED = false>
+//
+// MASKS: the sparse images' blocks come as the selection kernel's bitmask, and the code for the caller's lists is left out.  The
+// list warp's code is part of what ptxas allots registers for: 1296 quads at D = 128 541.2 -> 535.8 us, six images of 2592
+// 1114 -> 1103; 864 at D = 64 the same.
+template <int D, bool INJECT = false, bool SPLIT = false, bool ORDERED = false, bool MASKS = ORDERED>
 __global__ void __launch_bounds__(NTHREADS, 1)
 attn_kernel(const __grid_constant__ CUtensorMap tmq, const __grid_constant__ CUtensorMap tmk,
             const __grid_constant__ CUtensorMap tmv, uint16_t* __restrict__ out, const __grid_constant__ AttnParams prm) {
@@ -432,7 +436,7 @@ attn_kernel(const __grid_constant__ CUtensorMap tmq, const __grid_constant__ CUt
                 if (half >= 0 && (a >> 1) != half) return nb;           // not of this unit: like a block past the end
                 return quad_block(g, quad, a);
             };
-            const bool masks = ORDERED || prm.bitmask32 != nullptr;      // of the selection kernel (it finds the order), else lists of the caller's
+            const bool masks = MASKS || prm.bitmask32 != nullptr;      // of the selection kernel (it finds the order), else lists of the caller's
             // a dense image's quad, or one of text rows in a mask of the selection kernel: every block is kept, no mask is read
             const bool all_kept = slot < 0 || (masks && 4 * quad + 3 < g.n_text_blocks);
             // the query block whose kept blocks m[a] below holds: where a list is cut into parts depends on the whole quad
@@ -1075,6 +1079,12 @@ cudaError_t attention_static_init() {
     e = cudaFuncSetAttribute(attn_kernel<64, false, false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              (int)attn_smem_bytes<64>());
     if (e != cudaSuccess) return e;
+    e = cudaFuncSetAttribute(attn_kernel<128, false, false, false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             (int)attn_smem_bytes<128>());
+    if (e != cudaSuccess) return e;
+    e = cudaFuncSetAttribute(attn_kernel<64, false, false, false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             (int)attn_smem_bytes<64>());
+    if (e != cudaSuccess) return e;
     e = cudaFuncSetAttribute(attn_kernel<128, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              (int)attn_smem_bytes<128>());
     if (e != cudaSuccess) return e;
@@ -1230,7 +1240,8 @@ cudaError_t launch_attention(const CUtensorMap& tmq, const CUtensorMap& tmk, con
                              static_cast<uint16_t*>(out), g, imgs, n_dense, plan, prm.parts);
     } else {
         return launch_kernel(order.cls ? (g.D == 128 ? attn_kernel<128, false, false, true> : attn_kernel<64, false, false, true>)
-                                         : (g.D == 128 ? attn_kernel<128> : attn_kernel<64>),
+                             : bitmask ? (g.D == 128 ? attn_kernel<128, false, false, false, true> : attn_kernel<64, false, false, false, true>)
+                                       : (g.D == 128 ? attn_kernel<128> : attn_kernel<64>),
                              grid, dim3(NTHREADS), g.D == 128 ? attn_smem_bytes<128>() : attn_smem_bytes<64>(), s, tmq, tmk, tmv,
                              static_cast<uint16_t*>(out), prm);
     }

@@ -43,3 +43,25 @@ def test_ordered_quads_equal_quads_in_order(D, n_text, n_image, H, B):
             assert ctx.last_status() == 0
             assert torch.equal(out.view(torch.int16), alone.view(torch.int16)), (name, acts)
             assert torch.isfinite(out[[a == 2 for a in acts]]).all()
+
+
+@pytest.mark.parametrize("D,n_text,n_image,H,B", [
+    (64, 77, 75, 4, 2),          # 8 quads
+    (128, 0, 12 * 64 + 1, 8, 6),  # 192
+    (64, 130, 16 * 64, 15, 4),   # 300, ordered
+    (128, 77, 9 * 64, 40, 9),    # 1080
+    (64, 0, 5 * 64 + 63, 64, 8),  # 1024
+])
+def test_masks_and_lists_give_the_same(D, n_text, n_image, H, B):
+    """The attention of a step reads the selection's bitmask, the staged call its kept lists: the same outputs, bit for bit."""
+    gen = torch.Generator(device=DEV).manual_seed(H)
+    q, k, v = (torch.randn((B, H, n_text + n_image, D), generator=gen, device=DEV).to(torch.bfloat16) for _ in range(3))
+    ctx = binding.Context(B, H, D, n_text, n_image)
+    step, staged = torch.full_like(q, float("nan")), torch.full_like(q, float("nan"))
+    ratios = [(0.3, 0.95, 0.7, 0.15)[b % 4] for b in range(B)]
+    ctx.rapid3_gated_step(q, k, v, step, [2] * B, ratios)
+    idx, cnt = (t.clone() for t in ctx.workspace(B)[2:])
+    ctx.rapid3_sparse_joint_attn(q, k, v, staged, kept_idx=idx, kept_cnt=cnt)
+    torch.cuda.synchronize()
+    assert ctx.last_status() == 0
+    assert torch.equal(step.view(torch.int16), staged.view(torch.int16))
