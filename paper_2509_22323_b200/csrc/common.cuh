@@ -1,5 +1,5 @@
 // Shared declarations of the rapid3 CUDA library: launch-argument structs and the internal
-// launcher prototypes.  Host API in api.cu; kernels in k1_scores.cu, k2_select.cu, k3_attn.cu.
+// launcher prototypes.  Host API in api.cu; kernels in k1_scores.cu to k6_scoring.cu.
 #pragma once
 
 #include <cuda.h>
