@@ -148,6 +148,15 @@ int get_map(rapid3_ctx* c, const void* base, CUtensorMap* out) {
     return RAPID3_OK;
 }
 
+// Whether the result lies apart from Q.  The attention reads a quad's Q before it writes there, so a step may run in place; but it
+// must not start beside a kernel that is still to read Q, which scoring_kernel without a producer in front of it is.
+bool apart(const rapid3_ctx* c, const void* q, const void* out) {
+    const TensorGeom& g = c->g;
+    const uintptr_t size = 2 * ((c->shape.B_max - 1) * g.stride_b + (c->shape.H - 1) * g.stride_h + (g.N - 1) * g.stride_n + g.D);
+    const uintptr_t a = reinterpret_cast<uintptr_t>(q), b = reinterpret_cast<uintptr_t>(out);
+    return a + size <= b || b + size <= a;
+}
+
 // Whether a step over n_img attending images hands its last quads out by their length, and where that is kept.
 QuadOrder step_order(const rapid3_ctx* c, const TensorGeom& g, int n_img) {
     const int quads = attention_units(g, AttnParts(), n_img, 0);
@@ -465,7 +474,8 @@ static int gated_step_impl(rapid3_ctx* c, const void* q, const void* k, const vo
     if (sparse.n > 0) {
         if ((reinterpret_cast<uintptr_t>(q) % 16) || (reinterpret_cast<uintptr_t>(k) % 16)) return RAPID3_ERR_INVALID_ARG;
     }
-    const int cluster = scoring_cluster(g, all.n, sparse.n * g.H, !prep, mass_scale != nullptr, mask_free_us(g, all.n - sparse.n, sparse.n));
+    const int cluster = !prep && !apart(c, q, out) ? 0
+                        : scoring_cluster(g, all.n, sparse.n * g.H, !prep, mass_scale != nullptr, mask_free_us(g, all.n - sparse.n, sparse.n));
     if (sparse.n > 0 && cluster > 0) {
         ProfScope ps(c, prep ? PROF_SCORES : PROF_POOL, st);
         if (launch_scoring(q, k, g, sparse, c->pooled, c->scores, c->bitmask, c->kept_idx, c->kept_cnt, cluster, !prep,
@@ -552,7 +562,8 @@ int rapid3_gated_step_device(rapid3_ctx* c, const void* q, const void* k, const 
     none.n = 0;
     const QuadOrder order = step_order(c, c->g, B);
     // chosen as for a batch of which every other image is dense
-    if (const int cluster = scoring_cluster(c->g, B, (B + 1) / 2 * c->g.H, true, false, mask_free_us(c->g, B / 2, (B + 1) / 2))) {
+    const int cluster = apart(c, q, out) ? scoring_cluster(c->g, B, (B + 1) / 2 * c->g.H, true, false, mask_free_us(c->g, B / 2, (B + 1) / 2)) : 0;
+    if (cluster > 0) {
         ProfScope ps(c, PROF_POOL, st);
         if (launch_scoring(q, k, c->g, none, c->pooled, c->scores, c->bitmask, c->kept_idx, c->kept_cnt, cluster, true, nullptr, nullptr,
                            0.f, st, c->plan, B, order) != cudaSuccess)

@@ -84,3 +84,42 @@ def test_means_of_numbers_that_are_not_finite():
         assert torch.equal(s[ok].isinf(), ref[ok].isinf())
         fin = ref.isfinite()
         assert float(((s - ref)[fin].abs() / (1e-6 * ref[fin].abs() + 1e-6 * ref[fin].abs().mean().clamp(max=1.0))).max()) <= 1.0
+
+
+@pytest.mark.parametrize("D,H,n_text,n_image,ratios,packed", [
+    (64, 24, 333, 1024, (0.3, 0.6), False),                        # whole text quads write while other rows' means are taken
+    (128, 24, 512, 1600, (1.0, 0.5, 0.25), False),                 # a dense image beside two sparse ones
+    (128, 24, 512, 1600, (1.0, 0.5, 0.25), True),                  # Q, K, V and the result in turn in one buffer
+])
+def test_steps_in_place(D, H, n_text, n_image, ratios, packed):
+    """The result may take Q's place, or lie between the tensors: the same scores, masks and results as in a buffer of its own."""
+    B, N = len(ratios), n_text + n_image
+    gen = torch.Generator(device=DEV).manual_seed(N)
+    if packed:
+        buf = torch.randn((B, N, 4, H, D), generator=gen, device=DEV).to(torch.bfloat16)
+        q, k, v, place = (buf[:, :, i].permute(0, 2, 1, 3) for i in range(4))
+        strides = q.stride()[:3]
+    else:
+        q, k, v = (torch.randn((B, H, N, D), generator=gen, device=DEV).to(torch.bfloat16) for _ in range(3))
+        place, strides = q, None
+    q0 = q.clone()
+    n_sparse = sum(r < 1.0 for r in ratios)
+    acts_dev, ratios_dev = torch.full((B,), 2, dtype=torch.int32, device=DEV), torch.tensor(ratios, device=DEV)
+    ctx = binding.Context(B, H, D, n_text, n_image, strides=strides) if strides else binding.Context(B, H, D, n_text, n_image)
+    calls = {
+        "step": lambda out: ctx.rapid3_gated_step(q, k, v, out, [2] * B, ratios),
+        "heads": lambda out: ctx.rapid3_gated_step_heads(q, k, v, out, [2] * B, [[r] * H for r in ratios]),
+        "mass": lambda out: ctx.rapid3_gated_step_mass(q, k, v, out, [2] * B, ratios, 4 * D ** -0.5),
+        "device": lambda out: ctx.rapid3_gated_step_device(q, k, v, out, acts_dev, ratios_dev),
+    }
+    for name, call in calls.items():
+        apart = torch.empty_like(buf)[:, :, 3].permute(0, 2, 1, 3) if packed else torch.empty_like(q)
+        call(apart)
+        torch.cuda.synchronize()
+        scores = ctx.workspace(n_sparse)[0].clone()
+        call(place)
+        torch.cuda.synchronize()
+        assert ctx.last_status() == 0
+        assert torch.equal(ctx.workspace(n_sparse)[0], scores), name
+        assert torch.equal(bits(place), bits(apart)), name
+        q.copy_(q0)
