@@ -216,8 +216,8 @@ int rapid3_gated_step_fused(rapid3_ctx* ctx, const void* q_raw, const void* k_ra
  * The same step with the policy's decisions left on the GPU (Sec. 3.3: the heads sample their
  * actions on the device; reading them back would cost a host synchronisation per step and layer):
  * action_dev [B] int32 and keep_ratio_dev [B] float are DEVICE arrays, read by the kernels when
- * they run on `stream`, not at call time.  A kernel of one thread block builds the image lists, then the
- * kernels of rapid3_gated_step are launched with grids sized for all B images; thread blocks
+ * they run on `stream`, not at call time.  A kernel of one thread block builds the image lists, then pool,
+ * scores, selection and attention are launched with grids sized for all B images; thread blocks
  * of images that do not attend return at once.  Results (output, workspace contents) are those of
  * rapid3_gated_step with the same actions.  An action outside {SKIP, REUSE, ATTEND} or a ratio
  * outside (0, 1] cannot be rejected at call time: that image is not processed and the device status

@@ -184,8 +184,7 @@ cudaError_t launch_select_mask_mass(const float* scores, const TensorGeom& g, co
 // K6: means (pool = true; else they are there), scores and selection in one launch of clusters of `cluster` thread blocks.  heads: a count per (image, head); share: the cumulative-mass rule; neither: imgs.k_free.
 cudaError_t launch_scoring(const void* q, const void* k, const TensorGeom& g, const ImgList& imgs, double* pooled, float* scores,
                            uint64_t* bitmask, int32_t* kept_idx, int32_t* kept_cnt, int cluster, bool pool, const HeadKeep* heads,
-                           const MassShare* share, float mass_scale, cudaStream_t s, const DevPlan* plan = nullptr, int n_cap = 0,
-                           const QuadOrder& order = QuadOrder());
+                           const MassShare* share, float mass_scale, cudaStream_t s, const QuadOrder& order = QuadOrder());
 // The cluster size for that many (image, head) pairs of a step with `images` attending, beside heavy_us of SM time of attention
 // that needs no mask; 0: not this way.
 int scoring_cluster(const TensorGeom& g, int images, int pairs, bool pool, bool mass, double heavy_us);

@@ -24,7 +24,7 @@ constexpr int WARPS = 24, KSTAGES = 2, KCOLS = 48;
 constexpr int SMEM_MAX = 225 * 1024;
 constexpr int SCORING_FROM = 222;
 
-// Which rule gives a row's count: one per image (host or plan), one per (image, head), the cumulative mass.
+// Which rule gives a row's count: one per image, one per (image, head), the cumulative mass.
 struct MassRule {
     static constexpr int mode = 3;
     MassShare share;
@@ -35,14 +35,12 @@ struct ScoreArgs {
     const uint16_t* k;
     TensorGeom g;
     ImgList imgs;                  // sparse images; slot: place among them in the attention's list
-    double* pooled;                // [2][n_cap][H][nb][D]
+    double* pooled;                // [2][imgs.n][H][nb][D]
     float* scores;
     uint32_t* bitmask32;
     int32_t* kept_idx;
     int32_t* kept_cnt;
     int words32;
-    const DevPlan* plan;
-    int n_cap;
     QuadOrder order;
     int cluster;                   // thread blocks of a cluster
     int rows;                      // of S that are in shared memory at a time
@@ -77,96 +75,93 @@ __global__ void __launch_bounds__(WARPS * 32, 1) scoring_kernel(const __grid_con
     const int nb = g.nb, nq = (nb + 3) >> 2, H = g.H;
     grid_dependency_wait();
     grid_dependency_launch();
-    const int n_sparse = a.plan ? __ldcg(&a.plan->sparse.n) : a.imgs.n;
     const int rank = a.cluster > 1 ? (int)cluster_rank() : 0;
     const int quads = (nq + a.cluster - 1) / a.cluster, q_first = rank * quads, q_end = min(nq, q_first + quads);   // this thread block's
     // row r of a panel that begins at quad q0 is this query block
     auto row_block = [&](int q0, int r) { return q0 + (r >> 2) < q_end ? quad_block(g, q0 + (r >> 2), r & 3) : nb; };
 
-    for (int ph = blockIdx.x / a.cluster; ph < n_sparse * H; ph += gridDim.x / a.cluster) {
-        const int p = ph / H, h = ph - p * H;
-        const double* mean_q = a.pooled + (long long)ph * nb * D;
-        const double* mean_k = a.pooled + ((long long)a.n_cap * H + ph) * nb * D;
-        if (a.pool) {
-            const int batch = a.plan ? __ldcg(&a.plan->sparse.batch[p]) : a.imgs.batch[p];
-            const long long at = (long long)batch * g.stride_b + (long long)(g.h0 + h) * g.stride_h;
-            for (int u = rank * WARPS + warp; u < 2 * nb; u += a.cluster * WARPS) {
-                const int which = u >= nb, blk = u - which * nb;
-                pool_block<D>((which ? a.k : a.q) + at + (long long)(64 * blk) * g.stride_n, g.stride_n, min(64, g.N - 64 * blk),
-                              const_cast<double*>(which ? mean_k : mean_q) + (long long)blk * D, lane, [] {});
-            }
-            if (a.cluster > 1) cluster_sync();
-            else __syncthreads();
+    const int ph = blockIdx.x / a.cluster;             // the grid is a cluster for each (image, head)
+    const int p = ph / H, h = ph - p * H;
+    const double* mean_q = a.pooled + (long long)ph * nb * D;
+    const double* mean_k = a.pooled + ((long long)a.imgs.n * H + ph) * nb * D;
+    if (a.pool) {
+        const int batch = a.imgs.batch[p];
+        const long long at = (long long)batch * g.stride_b + (long long)(g.h0 + h) * g.stride_h;
+        for (int u = rank * WARPS + warp; u < 2 * nb; u += a.cluster * WARPS) {
+            const int which = u >= nb, blk = u - which * nb;
+            pool_block<D>((which ? a.k : a.q) + at + (long long)(64 * blk) * g.stride_n, g.stride_n, min(64, g.N - 64 * blk),
+                          const_cast<double*>(which ? mean_k : mean_q) + (long long)blk * D, lane, [] {});
         }
-        for (int q0 = q_first; q0 < q_end; q0 += rows >> 2) {
-            auto load_k = [&](int ch) {                  // one group of copies, empty past the end
-                if (KCOLS * ch < nb) {
-                    double* dst = sk + (ch % KSTAGES) * (KCOLS * LDS);
-                    for (int e = threadIdx.x; e < KCOLS * (D / 2); e += WARPS * 32) {
-                        const int r = e / (D / 2), c = 2 * (e % (D / 2)), j = KCOLS * ch + r;
-                        copy16_async(dst + r * LDS + c, j < nb ? mean_k + (long long)j * D + c : a.pooled, j < nb);
-                    }
+        if (a.cluster > 1) cluster_sync();
+        else __syncthreads();
+    }
+    for (int q0 = q_first; q0 < q_end; q0 += rows >> 2) {
+        auto load_k = [&](int ch) {                  // one group of copies, empty past the end
+            if (KCOLS * ch < nb) {
+                double* dst = sk + (ch % KSTAGES) * (KCOLS * LDS);
+                for (int e = threadIdx.x; e < KCOLS * (D / 2); e += WARPS * 32) {
+                    const int r = e / (D / 2), c = 2 * (e % (D / 2)), j = KCOLS * ch + r;
+                    copy16_async(dst + r * LDS + c, j < nb ? mean_k + (long long)j * D + c : a.pooled, j < nb);
                 }
-                asm volatile("cp.async.commit_group;" ::: "memory");
-            };
-            for (int e = threadIdx.x; e < rows * (D / 2); e += WARPS * 32) {
-                const int r = e / (D / 2), c = 2 * (e % (D / 2)), i = row_block(q0, r);
-                copy16_async(sq + r * LDS + c, i < nb ? mean_q + (long long)i * D + c : a.pooled, i < nb);
             }
+            asm volatile("cp.async.commit_group;" ::: "memory");
+        };
+        for (int e = threadIdx.x; e < rows * (D / 2); e += WARPS * 32) {
+            const int r = e / (D / 2), c = 2 * (e % (D / 2)), i = row_block(q0, r);
+            copy16_async(sq + r * LDS + c, i < nb ? mean_q + (long long)i * D + c : a.pooled, i < nb);
+        }
 #pragma unroll
-            for (int ch = 0; ch < KSTAGES; ++ch) load_k(ch);
-            const int gr = lane >> 2, c4 = lane & 3;
-            for (int ch = 0; KCOLS * ch < nb; ++ch) {
-                asm volatile("cp.async.wait_group %0;" ::"n"(KSTAGES - 1) : "memory");
-                __syncthreads();
-                // two fragments of 8 x 8 side by side a warp
-                const int pairs = (min(nb - KCOLS * ch, KCOLS) + 15) >> 4;
-                for (int f = warp; f < (rows >> 3) * pairs; f += WARPS) {
-                    const int ri = (f / pairs) * 8, cj = (f % pairs) * 16;
-                    const double* aq = sq + (ri + gr) * LDS + c4;
-                    const double* bk = sk + (ch % KSTAGES) * (KCOLS * LDS) + (cj + gr) * LDS + c4;
-                    double acc[2][2] = {{0.0, 0.0}, {0.0, 0.0}};
+        for (int ch = 0; ch < KSTAGES; ++ch) load_k(ch);
+        const int gr = lane >> 2, c4 = lane & 3;
+        for (int ch = 0; KCOLS * ch < nb; ++ch) {
+            asm volatile("cp.async.wait_group %0;" ::"n"(KSTAGES - 1) : "memory");
+            __syncthreads();
+            // two fragments of 8 x 8 side by side a warp
+            const int pairs = (min(nb - KCOLS * ch, KCOLS) + 15) >> 4;
+            for (int f = warp; f < (rows >> 3) * pairs; f += WARPS) {
+                const int ri = (f / pairs) * 8, cj = (f % pairs) * 16;
+                const double* aq = sq + (ri + gr) * LDS + c4;
+                const double* bk = sk + (ch % KSTAGES) * (KCOLS * LDS) + (cj + gr) * LDS + c4;
+                double acc[2][2] = {{0.0, 0.0}, {0.0, 0.0}};
 #pragma unroll 8
-                    for (int d = 0; d < D; d += 4) {
-                        const double x = aq[d];
-                        dmma_8x8x4(acc[0][0], acc[0][1], x, bk[d]);
-                        dmma_8x8x4(acc[1][0], acc[1][1], x, bk[8 * LDS + d]);
-                    }
-                    float* o = ss + (ri + gr) * LDN + KCOLS * ch + cj + 2 * c4;
-                    *reinterpret_cast<float2*>(o) = make_float2((float)acc[0][0], (float)acc[0][1]);
-                    *reinterpret_cast<float2*>(o + 8) = make_float2((float)acc[1][0], (float)acc[1][1]);
+                for (int d = 0; d < D; d += 4) {
+                    const double x = aq[d];
+                    dmma_8x8x4(acc[0][0], acc[0][1], x, bk[d]);
+                    dmma_8x8x4(acc[1][0], acc[1][1], x, bk[8 * LDS + d]);
                 }
-                __syncthreads();
-                load_k(ch + KSTAGES);
-            }
-            for (int r = warp; r < rows; r += WARPS) {
-                const int i = row_block(q0, r);
-                const float* src = ss + r * LDN;
-                const long long row = (long long)ph * nb + i;
-                if (i < nb) {
-                    for (int j = lane; j < nb; j += 32) a.scores[row * nb + j] = src[j];
-                    auto score = [&](int j) { return src[j]; };
-                    int k;
-                    if constexpr (HK::mode == MassRule::mode) k = mass_row<IPL>(score, i, nb, g.n_text_blocks, hk.share.tau[p], hk.scale, lane);
-                    else if constexpr (HK::mode == HeadKeep::mode) k = hk.k[ph];
-                    else k = a.plan ? __ldcg(&a.plan->sparse.k_free[p]) : a.imgs.k_free[p];
-                    select_row<IPL>(score, i, nb, g.n_text_blocks, k, lane, a.bitmask32 + row * a.words32, a.words32, a.kept_idx + row * nb,
-                                    a.kept_cnt + row, [&](int x, uint32_t bits) { kept[r * IPL + x] = bits; });
-                } else if (lane < IPL) {
-                    kept[r * IPL + lane] = 0u;
-                }
+                float* o = ss + (ri + gr) * LDN + KCOLS * ch + cj + 2 * c4;
+                *reinterpret_cast<float2*>(o) = make_float2((float)acc[0][0], (float)acc[0][1]);
+                *reinterpret_cast<float2*>(o + 8) = make_float2((float)acc[1][0], (float)acc[1][1]);
             }
             __syncthreads();
-            if (a.order.cls) {
-                const int place = a.plan ? plan_place(a.plan, p, lane) : a.imgs.slot[p];
-                for (int x = warp; x < rows >> 2 && q0 + x < q_end; x += WARPS) {
-                    uint32_t m[4];
-#pragma unroll
-                    for (int b = 0; b < 4; ++b) m[b] = 32 * lane < nb ? kept[(4 * x + b) * IPL + lane] : 0u;
-                    order_quad(a.order, g, n_sparse, place, h, q0 + x, m, lane);
-                }
-                __syncthreads();
+            load_k(ch + KSTAGES);
+        }
+        for (int r = warp; r < rows; r += WARPS) {
+            const int i = row_block(q0, r);
+            const float* src = ss + r * LDN;
+            const long long row = (long long)ph * nb + i;
+            if (i < nb) {
+                for (int j = lane; j < nb; j += 32) a.scores[row * nb + j] = src[j];
+                auto score = [&](int j) { return src[j]; };
+                int k;
+                if constexpr (HK::mode == MassRule::mode) k = mass_row<IPL>(score, i, nb, g.n_text_blocks, hk.share.tau[p], hk.scale, lane);
+                else if constexpr (HK::mode == HeadKeep::mode) k = hk.k[ph];
+                else k = a.imgs.k_free[p];
+                select_row<IPL>(score, i, nb, g.n_text_blocks, k, lane, a.bitmask32 + row * a.words32, a.words32, a.kept_idx + row * nb,
+                                a.kept_cnt + row, [&](int x, uint32_t bits) { kept[r * IPL + x] = bits; });
+            } else if (lane < IPL) {
+                kept[r * IPL + lane] = 0u;
             }
+        }
+        __syncthreads();
+        if (a.order.cls) {
+            for (int x = warp; x < rows >> 2 && q0 + x < q_end; x += WARPS) {
+                uint32_t m[4];
+#pragma unroll
+                for (int b = 0; b < 4; ++b) m[b] = 32 * lane < nb ? kept[(4 * x + b) * IPL + lane] : 0u;
+                order_quad(a.order, g, a.imgs.n, a.imgs.slot[p], h, q0 + x, m, lane);
+            }
+            __syncthreads();
         }
     }
 }
@@ -225,8 +220,7 @@ int scoring_cluster(const TensorGeom& g, int images, int pairs, bool pool, bool 
 
 cudaError_t launch_scoring(const void* q, const void* k, const TensorGeom& g, const ImgList& imgs, double* pooled, float* scores,
                            uint64_t* bitmask, int32_t* kept_idx, int32_t* kept_cnt, int cluster, bool pool, const HeadKeep* heads,
-                           const MassShare* share, float mass_scale, cudaStream_t s, const DevPlan* plan, int n_cap,
-                           const QuadOrder& order) {
+                           const MassShare* share, float mass_scale, cudaStream_t s, const QuadOrder& order) {
     ScoreArgs a;
     a.q = static_cast<const uint16_t*>(q);
     a.k = static_cast<const uint16_t*>(k);
@@ -238,13 +232,11 @@ cudaError_t launch_scoring(const void* q, const void* k, const TensorGeom& g, co
     a.kept_idx = kept_idx;
     a.kept_cnt = kept_cnt;
     a.words32 = 2 * ((g.nb + 63) / 64);
-    a.plan = plan;
-    a.n_cap = plan ? n_cap : imgs.n;
     a.order = order;
     a.cluster = cluster;
     a.rows = 0;
     a.pool = pool;
-    const int pairs = a.n_cap * g.H;
+    const int pairs = imgs.n * g.H;
     if (share) {
         MassRule m;
         m.share = *share;
