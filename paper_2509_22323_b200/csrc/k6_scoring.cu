@@ -196,10 +196,18 @@ cudaError_t launch(ScoreArgs& a, const HK& hk, int pairs, cudaStream_t s) {
 // fewer quads than SCORING_FROM wait for the first masks, not for SMs (96 quads of 15 blocks 23.7 / 28.0, 192 of 29 35.3 / 37.1).
 // Steps, us, three kernels / clusters: two images of 24 heads, 1357 tokens, D = 64 43.4 / 41.5 (of two); 864 quads with per-head
 // ratios 189.3 / 184.9 (two), by mass 343 / 337 (two), a dense and a sparse image at D = 64 258.7 / 254.2 (one); one image from
-// raw projections 202.3 / 195.5 (two to four); a dense and two sparse at D = 128 518.0 / 514.0 (one).
+// raw projections 202.3 / 195.5 (two to four).
+// Beside few pairs and no dense image only text rows need no mask.  Worked on early they shorten a launch whose last round of SMs is
+// nearly full; in any other that round has room for them, and the clusters only keep the first masks back: one image by top-k,
+// ratio 0.25, 16 heads x 57 blocks (240 quads, 1.62 rounds) 67.1 / 76.8, 24 x 57 (2.43) 95.8 / 101.6, 24 x 108 (4.38) 270 / 288,
+// D = 64 24 x 106 168 / 174; but 24 x 72 (2.92) 147.5 / 131.0, 16 x 72 (1.95) 98.3 / 91.8, D = 64 24 x 72 97.3 / 91.4.
+constexpr int FEW_PAIRS = 24;
+constexpr int FULL_ROUND = 104;    // quads
 int scoring_cluster(const TensorGeom& g, int images, int pairs, bool pool, bool mass, double heavy_us) {
     const int nq = (g.nb + 3) / 4;
-    if (g.nb > 192 || pairs < 16 || images * g.H * nq < SCORING_FROM) return 0;
+    const int quads = images * g.H * nq;
+    if (g.nb > 192 || pairs < 16 || quads < SCORING_FROM) return 0;
+    if (!mass && pairs <= FEW_PAIRS && images * g.H == pairs && (quads - 1) % SM_COUNT + 1 < FULL_ROUND) return 0;
     const double mb = pool ? 256e-6 * g.nb * g.D : 0.0;                  // of Q and K, a pair
     int best = 0;
     double least = 0.95 * SM_COUNT * (7.0 + pairs * (mb / 4.5 + 1.5e-5 * g.nb * g.nb) + (mass ? 2.5 + 2e-5 * pairs * g.nb * g.nb : 0.0));

@@ -62,6 +62,27 @@ def test_clusters_equal_the_stages(D, n_text, n_image, H, ratios):
         assert torch.equal(bits(out), bits(alone)), name
 
 
+@pytest.mark.parametrize("n_blocks,H,ratios,launches", [
+    (44, 24, (0.5,), 2),               # 264 quads: the second round of 148 SMs is 0.78 full
+    (57, 24, (0.5,), 4),               # 360: the third is 0.43 full
+    (57, 16, (0.25,), 4),              # 240: 0.62
+    (72, 16, (0.25,), 2),              # 288: 0.95
+    (57, 12, (0.5, 1.0), 4),           # 360, a dense image beside, but less than 16 pairs
+    (57, 24, (0.5, 1.0), 2),           # 720, a dense image beside
+    (57, 24, (0.5, 0.5), 2),           # 720, two images: 48 pairs
+])
+def test_which_steps_take_clusters(n_blocks, H, ratios, launches):
+    """One sparse image with nothing dense beside it takes the three kernels where its last round of SMs has room."""
+    B, N, D = len(ratios), 64 * n_blocks, 128
+    q, k, v = (torch.randn((B, H, N, D), device=DEV).to(torch.bfloat16) for _ in range(3))
+    ctx, out = binding.Context(B, H, D, 512, N - 512), torch.empty_like(q)
+    n0 = ctx.launch_count()
+    ctx.rapid3_gated_step(q, k, v, out, [2] * B, ratios)
+    torch.cuda.synchronize()
+    assert ctx.last_status() == 0
+    assert ctx.launch_count() - n0 == launches
+
+
 def test_means_of_numbers_that_are_not_finite():
     """A block with an infinity or a NaN has them in its scores as sums in 64 bits give them, whichever half of a word holds it."""
     B, H, D, N = 2, 24, 64, 64 * 22
