@@ -201,9 +201,10 @@ __device__ __forceinline__ void row_maxima(const uint32_t (&r)[32], float& lo, f
 //
 // ORDERED is the build for launches whose last quads are handed out by their length (QuadOrder).
 //
-// MASKS: the sparse images' blocks come as the selection kernel's bitmask, and the code for the caller's lists is left out.  The
-// list warp's code is part of what ptxas allots registers for: 1296 quads at D = 128 541.2 -> 535.8 us, six images of 2592
-// 1114 -> 1103; 864 at D = 64 the same.
+// MASKS: the sparse images' blocks come as the selection kernel's bitmask, or there are none, and the code for the caller's lists is
+// left out.  Both builds have 96 registers and spill the same five words; by turns, whole steps, us, with that code / without:
+// 1296 quads at D = 128 530.7 / 524.7, 2592 1184.6 / 1170.0, 1584 of a 2048^2 image 1117.6 / 1110.4; all dense 1296 669.3 / 660.9,
+// 1584 2848 / 2813.  Dense launches at D = 64 keep the build with it: 840 quads 304.5 / 306.3, 288 36.8 / 37.0.
 template <int D, bool INJECT = false, bool SPLIT = false, bool ORDERED = false, bool MASKS = ORDERED>
 __global__ void __launch_bounds__(NTHREADS, 1)
 attn_kernel(const __grid_constant__ CUtensorMap tmq, const __grid_constant__ CUtensorMap tmk,
@@ -1239,8 +1240,9 @@ cudaError_t launch_attention(const CUtensorMap& tmq, const CUtensorMap& tmk, con
         return launch_kernel(g.D == 128 ? add_parts_kernel<128> : add_parts_kernel<64>, dim3(left * SOFTMAX_WARPS * (g.D / 32) / 4), dim3(128), 0, s,
                              static_cast<uint16_t*>(out), g, imgs, n_dense, plan, prm.parts);
     } else {
+        const bool masks = bitmask || (!kept_idx && g.D == 128);         // see MASKS
         return launch_kernel(order.cls ? (g.D == 128 ? attn_kernel<128, false, false, true> : attn_kernel<64, false, false, true>)
-                             : bitmask ? (g.D == 128 ? attn_kernel<128, false, false, false, true> : attn_kernel<64, false, false, false, true>)
+                             : masks ? (g.D == 128 ? attn_kernel<128, false, false, false, true> : attn_kernel<64, false, false, false, true>)
                                        : (g.D == 128 ? attn_kernel<128> : attn_kernel<64>),
                              grid, dim3(NTHREADS), g.D == 128 ? attn_smem_bytes<128>() : attn_smem_bytes<64>(), s, tmq, tmk, tmv,
                              static_cast<uint16_t*>(out), prm);
