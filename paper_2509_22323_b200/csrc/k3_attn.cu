@@ -33,6 +33,8 @@
 // (two of them and O at 128 for D = 128; three and O at 192 for D = 64, where the columns allow it).
 // Every mbarrier wait is bounded; a wait that runs out records RAPID3_ERR_TIMEOUT in the status
 // word and the thread block drains its copies, releases its TMEM and exits normally.
+#include <float.h>
+
 #include <algorithm>
 
 #include "common.cuh"
@@ -811,6 +813,8 @@ attn_kernel(const __grid_constant__ CUtensorMap tmq, const __grid_constant__ CUt
                     // the pass twice (from -inf every row "grows")
                     row_maxima(r, nm_lo, nm_hi);
                     nm_lo *= -c2; nm_hi *= -c2;
+                    // a part may begin with a block whose scores are all -inf: no NaN (-inf - -inf) from them, the next ones count
+                    if (SPLIT) { nm_lo = fminf(nm_lo, FLT_MAX); nm_hi = fminf(nm_hi, FLT_MAX); }
                     seeded = true;
                     if (SPLIT && cg == 0) { ref[0] = nm_lo; ref[8] = nm_hi; }
                 }

@@ -84,3 +84,32 @@ def test_an_image_of_a_context_with_parts_does_not_depend_on_its_launch(D, n_tex
         assert torch.equal(out.view(torch.int16), alone.view(torch.int16))
         assert torch.equal(out.view(torch.int16), dev.view(torch.int16))
         assert torch.isfinite(out).all()
+
+
+@pytest.mark.parametrize("D,n_text,n_image,H,B", SHAPES)
+@pytest.mark.parametrize("finite", ["ends", "even"])
+def test_blocks_whose_scores_are_below_all_numbers(D, n_text, n_image, H, B, finite):
+    """Finite numbers whose products with Q leave the range of single precision downwards, in whole key blocks: such a block counts
+    for nothing, wherever a part of a list begins (behind the row's first block)."""
+    N = n_text + n_image
+    nb = (N + 63) // 64
+    (q, k, v), _ = random_qkv((B, H, N, D), nb)
+    at = torch.arange(nb, device=DEV)
+    low = (at % 2 == 1) if finite == "even" else (at > 0) & (at < nb - 1)
+    q[..., 0] = 8.0
+    k[..., 0] = torch.where(low[torch.arange(N, device=DEV) // 64], torch.finfo(torch.bfloat16).min, k[..., 0])
+    ctx, out = binding.Context(B, H, D, n_text, n_image), torch.full_like(q, float("nan"))
+    ctx.rapid3_gated_step(q, k, v, out, [2] * B, [1.0] * B)
+    ratios = [0.5] * B
+    sparse = torch.full_like(q, float("nan"))
+    ctx.rapid3_gated_step(q, k, v, sparse, [2] * B, ratios)
+    torch.cuda.synchronize()
+    assert ctx.last_status() == 0
+    keep = binding.bitmask_to_dense(ctx.workspace(B)[1], nb).bool().to(DEV)
+    for b in range(B):
+        for h in range(H):
+            for o, mask in ((out, torch.ones_like(keep[b, h])), (sparse, keep[b, h])):
+                ref = attention_64(q[b, h], k[b, h], v[b, h], mask)
+                first = mask.int().argmax(-1)                      # a row's first block has numbers here: kept by all rows if it is text
+                rows = (~low[first]).repeat_interleave(64)[:N]
+                assert float((o[b, h].double() - ref).abs()[rows].max()) <= 2 ** -7 * float(v[b, h].abs().max())
