@@ -333,7 +333,9 @@ int rapid3_last_status(rapid3_ctx* ctx, int* device_status);
  * therefore run out: each thread block records RAPID3_ERR_TIMEOUT in the status word, waits
  * (bounded) for its copies in flight, lets its tensor-core work finish, releases its tensor
  * memory and returns.  Nothing waits without a limit and nothing faults; `out` is left partly
- * or wholly unwritten.  The context stays usable: after rapid3_last_status has returned (and
+ * or wholly unwritten.  In a context that works on kept blocks in parts (see rapid3_sparse_joint_attn)
+ * the groups are those of a part, stop_group counts as its last where it has fewer, and the launch
+ * that adds up the parts follows and writes nothing.  The context stays usable: after rapid3_last_status has returned (and
  * cleared) the code, ordinary calls compute as before.  Asynchronous on `stream`.
  */
 int rapid3_debug_inject_timeout(rapid3_ctx* ctx, const void* q, const void* k, const void* v, void* out,

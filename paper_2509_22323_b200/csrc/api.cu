@@ -262,7 +262,8 @@ int rapid3_create(rapid3_ctx** out, const rapid3_shape* shape) {
               cudaMemset(c->plan, 0, sizeof(DevPlan)) == cudaSuccess;
     if (ok && !c->parts.any() && attention_units(g, c->parts, (int)B, 0) > ORDER_FROM)
         ok = cudaMalloc(&c->order.cls, ORDER_LAST) == cudaSuccess;
-    if (ok && c->parts.any()) ok = cudaMalloc(&c->parts.partial, attention_partial_bytes(g, shape->B_max, c->parts)) == cudaSuccess;
+    if (ok && c->parts.any()) ok = cudaMalloc(&c->parts.partial, attention_partial_bytes(g, shape->B_max, c->parts)) == cudaSuccess &&
+                                   cudaMalloc(&c->parts.given_up, sizeof(int)) == cudaSuccess;
     if (!ok) {
         cudaGetLastError();
         rapid3_destroy(c);
@@ -288,6 +289,7 @@ int rapid3_destroy(rapid3_ctx* c) {
     cudaFree(c->status);
     cudaFree(c->plan);
     cudaFree(c->parts.partial);
+    cudaFree(c->parts.given_up);
     cudaFree(c->order.cls);
     for (void* s : c->stage) cudaFree(s);
     if (c->up_s) cudaStreamDestroy(c->up_s);
@@ -694,7 +696,7 @@ int rapid3_debug_inject_timeout(rapid3_ctx* c, const void* q, const void* k, con
         return r;
     if (reinterpret_cast<uintptr_t>(out) % 16) return RAPID3_ERR_INVALID_ARG;
     if (launch_attention(tq, tk, tv, out, c->g, l, nullptr, nullptr, nullptr, softmax_scale, c->status,
-                         static_cast<cudaStream_t>(stream), nullptr, 0, stop_group) != cudaSuccess)
+                         static_cast<cudaStream_t>(stream), nullptr, 0, stop_group, true, &c->parts, &c->launches) != cudaSuccess)
         return RAPID3_ERR_CUDA;
     c->launches += 1;
     return RAPID3_OK;

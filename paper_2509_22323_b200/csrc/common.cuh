@@ -65,6 +65,7 @@ struct TensorGeom {
 struct AttnParts {
     int dense = 1, text = 1, light = 1;
     float4* partial = nullptr;       // attention_partial_bytes()
+    int* given_up = nullptr;         // a wait of the launch has run out: its parts are not complete, and add_parts_kernel stores nothing
     __host__ __device__ bool any() const { return dense > 1 || text > 1 || light > 1; }
 };
 // Units of work of an attention launch over n_img images, n_dense of them dense.

@@ -288,12 +288,17 @@ attn_kernel(const __grid_constant__ CUtensorMap tmq, const __grid_constant__ CUt
         tc_fence_before();
     }
     if (prm.wait_first) grid_dependency_wait();
+    // The launch's own word (the status stays until the host has read it).  Thread blocks start in order, and a wait runs out only
+    // after thousands of polls, so nothing sets it before this; what read it last has ended before the selection kernel began, if
+    // that is in front.
+    if (SPLIT && blockIdx.x == 0 && tid == 0) __stcg(prm.parts.given_up, 0);
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem_base = ctl->tmem_base;
 
     auto fail = [&]() {
         atomicExch(prm.status, RAPID3_ERR_TIMEOUT);
+        if (SPLIT) atomicExch(prm.parts.given_up, 1);
         ctl->abort_flag = 1;
     };
     // bounded wait that also gives up quickly once another role has failed
@@ -595,7 +600,7 @@ attn_kernel(const __grid_constant__ CUtensorMap tmq, const __grid_constant__ CUt
                 const int n_early = i == 0 ? ctl->n_early : 0;
                 if (n_early > max(n_u - TAKE_AHEAD, 0)) mbar_arrive(bNE);
                 for (int gi = n_early; gi <= n_u; ++gi) {
-                    if (INJECT && gi == prm.stop_group) { ok = false; break; }
+                    if (INJECT && gi == min(prm.stop_group, n_u)) { ok = false; break; }
                     if (gi == max(n_u - TAKE_AHEAD, 0)) mbar_arrive(bNE);
                     // A group is issued once both ring stages it fills have been released.  The K stage's release also
                     // tells that both MMA warps are past their wait on this barrier's previous phase (group G - KS),
@@ -1015,6 +1020,7 @@ __global__ void __launch_bounds__(128) add_parts_kernel(uint16_t* __restrict__ o
     const int tok_hi = tok_lo + 8;
     if (tok_lo - (lane >> 2) >= g.N) return;             // nothing was left for rows past the end
     const int b = plan ? __ldcg(&plan->all.batch[p]) : imgs.batch[p];
+    const int given_up = __ldcg(ap.given_up);
     const float4* base = ap.partial + (size_t)store * part_f4 + (size_t)warp * PARTIAL_F4<D> * 32 + lane;
     float4 v[MAX_PARTS], x4[MAX_PARTS][4];
 #pragma unroll
@@ -1058,6 +1064,7 @@ __global__ void __launch_bounds__(128) add_parts_kernel(uint16_t* __restrict__ o
     const uint4 o_lo = quad_transpose(a_lo[0], a_lo[1], a_lo[2], a_lo[3], cg);
     const uint4 o_hi = quad_transpose(a_hi[0], a_hi[1], a_hi[2], a_hi[3], cg);
     uint16_t* o = out + (long long)b * g.stride_b + (long long)(g.h0 + h) * g.stride_h + (long long)tok_lo * g.stride_n + 8 * cg + 32 * ch;
+    if (given_up) return;                                // parts of an earlier launch, or of none, may be among these
     if (tok_lo < g.N) *reinterpret_cast<uint4*>(o) = o_lo;
     if (tok_hi < g.N) *reinterpret_cast<uint4*>(o + 8 * g.stride_n) = o_hi;
 }
@@ -1067,34 +1074,17 @@ bool g_attr_set = false;
 }  // namespace
 
 cudaError_t attention_static_init() {
-    cudaError_t e = cudaFuncSetAttribute(attn_kernel<128>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)attn_smem_bytes<128>());
-    if (e != cudaSuccess) return e;
-    e = cudaFuncSetAttribute(attn_kernel<64>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)attn_smem_bytes<64>());
-    if (e != cudaSuccess) return e;
-    e = cudaFuncSetAttribute(attn_kernel<128, false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)attn_smem_bytes<128>());
-    if (e != cudaSuccess) return e;
-    e = cudaFuncSetAttribute(attn_kernel<64, false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)attn_smem_bytes<64>());
-    if (e != cudaSuccess) return e;
-    e = cudaFuncSetAttribute(attn_kernel<128, false, false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)attn_smem_bytes<128>());
-    if (e != cudaSuccess) return e;
-    e = cudaFuncSetAttribute(attn_kernel<64, false, false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)attn_smem_bytes<64>());
-    if (e != cudaSuccess) return e;
-    e = cudaFuncSetAttribute(attn_kernel<128, false, false, false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)attn_smem_bytes<128>());
-    if (e != cudaSuccess) return e;
-    e = cudaFuncSetAttribute(attn_kernel<64, false, false, false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)attn_smem_bytes<64>());
-    if (e != cudaSuccess) return e;
-    e = cudaFuncSetAttribute(attn_kernel<128, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)attn_smem_bytes<128>());
-    if (e != cudaSuccess) return e;
-    e = cudaFuncSetAttribute(attn_kernel<64, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)attn_smem_bytes<64>());
+    const auto set = [](auto... kernels) {
+        cudaError_t e = cudaSuccess;
+        const int smem[] = {(int)attn_smem_bytes<128>(), (int)attn_smem_bytes<64>()};      // the builds come in pairs
+        int i = 0;
+        ((e = e != cudaSuccess ? e : cudaFuncSetAttribute(kernels, cudaFuncAttributeMaxDynamicSharedMemorySize, smem[i++ % 2])), ...);
+        return e;
+    };
+    const cudaError_t e = set(attn_kernel<128>, attn_kernel<64>, attn_kernel<128, false, true>, attn_kernel<64, false, true>,
+                              attn_kernel<128, false, false, true>, attn_kernel<64, false, false, true>,
+                              attn_kernel<128, false, false, false, true>, attn_kernel<64, false, false, false, true>,
+                              attn_kernel<128, true>, attn_kernel<64, true>, attn_kernel<128, true, true>, attn_kernel<64, true, true>);
     if (e != cudaSuccess) return e;
     g_attr_set = true;
     return cudaSuccess;
@@ -1222,7 +1212,7 @@ cudaError_t launch_attention(const CUtensorMap& tmq, const CUtensorMap& tmk, con
     prm.stop_group = inject_stop_group;
     const int n_img = plan ? n_cap : imgs.n, pairs = g.H * n_img, nq = (g.nb + 3) / 4, ntq = std::min(nq, (g.n_text_blocks + 3) / 4);
     int left = 0;                              // quads whose lists are worked on in parts, at most
-    if (parts && inject_stop_group < 0) {
+    if (parts) {
         const int d = parts->dense > 1 ? nq : 0, t = (parts->text > 1 ? ntq : 0) + (parts->light > 1 ? nq - ntq : 0);
         left = plan ? pairs * std::max(d, t) : g.H * (n_dense * d + (imgs.n - n_dense) * t);
         if (left > 0) prm.parts = *parts;
@@ -1231,18 +1221,20 @@ cudaError_t launch_attention(const CUtensorMap& tmq, const CUtensorMap& tmk, con
                            : attention_units(g, prm.parts, n_img, n_dense);
     // halves: up to as many thread blocks as SMs.  Where a plan may hold fewer units than the largest launch, it may halve them.
     dim3 grid(2 * units <= SM_COUNT ? 2 * units : plan ? std::max(units, SM_COUNT) : units, 1, 1);
-    if (inject_stop_group >= 0) {
-        if (g.D == 128)
-            attn_kernel<128, true><<<grid, NTHREADS, attn_smem_bytes<128>(), s>>>(tmq, tmk, tmv, static_cast<uint16_t*>(out), prm);
-        else
-            attn_kernel<64, true><<<grid, NTHREADS, attn_smem_bytes<64>(), s>>>(tmq, tmk, tmv, static_cast<uint16_t*>(out), prm);
-    } else if (left > 0) {
-        cudaError_t e = launch_kernel(g.D == 128 ? attn_kernel<128, false, true> : attn_kernel<64, false, true>, grid, dim3(NTHREADS),
-                                      g.D == 128 ? attn_smem_bytes<128>() : attn_smem_bytes<64>(), s, tmq, tmk, tmv, static_cast<uint16_t*>(out), prm);
+    if (left > 0) {
+        const auto kernel = inject_stop_group >= 0 ? (g.D == 128 ? attn_kernel<128, true, true> : attn_kernel<64, true, true>)
+                                                   : (g.D == 128 ? attn_kernel<128, false, true> : attn_kernel<64, false, true>);
+        cudaError_t e = launch_kernel(kernel, grid, dim3(NTHREADS), g.D == 128 ? attn_smem_bytes<128>() : attn_smem_bytes<64>(), s, tmq, tmk, tmv,
+                                      static_cast<uint16_t*>(out), prm);
         if (e != cudaSuccess) return e;
         *launches += 1;
         return launch_kernel(g.D == 128 ? add_parts_kernel<128> : add_parts_kernel<64>, dim3(left * SOFTMAX_WARPS * (g.D / 32) / 4), dim3(128), 0, s,
                              static_cast<uint16_t*>(out), g, imgs, n_dense, plan, prm.parts);
+    } else if (inject_stop_group >= 0) {
+        if (g.D == 128)
+            attn_kernel<128, true><<<grid, NTHREADS, attn_smem_bytes<128>(), s>>>(tmq, tmk, tmv, static_cast<uint16_t*>(out), prm);
+        else
+            attn_kernel<64, true><<<grid, NTHREADS, attn_smem_bytes<64>(), s>>>(tmq, tmk, tmv, static_cast<uint16_t*>(out), prm);
     } else {
         const bool masks = bitmask || (!kept_idx && g.D == 128);         // see MASKS
         return launch_kernel(order.cls ? (g.D == 128 ? attn_kernel<128, false, false, true> : attn_kernel<64, false, false, true>)

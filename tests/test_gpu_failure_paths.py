@@ -56,6 +56,31 @@ def test_wait_that_runs_out_sets_the_status_and_returns(D, stop_group):
         parity.compare_outputs(out[b], ref[b]["out"], f"after a timeout, img {b}")
 
 
+@pytest.mark.parametrize("D,n_blocks,stop_group", [(64, 40, 0), (64, 40, 2), (64, 40, 40), (128, 36, 0), (128, 36, 1), (128, 36, 3)])
+def test_a_wait_that_runs_out_leaves_rows_in_parts_unwritten(D, n_blocks, stop_group):
+    """A context whose attention works on lists in parts: a launch that has given up adds up neither the parts of the call before
+    nor memory that nothing has written.  The launch after it does."""
+    gen = torch.Generator(device=DEV).manual_seed(n_blocks)
+    q, k, v = (torch.randn((1, 2, 64 * n_blocks, D), generator=gen, device=DEV).to(torch.bfloat16) for _ in range(3))
+    ctx = binding.Context(1, 2, D, 64, 64 * (n_blocks - 1))
+    want = None
+    for _ in range(2):                             # on a new context, and after a call that has left its parts
+        n0, scratch = ctx.launch_count(), poison_like(q)
+        ctx.rapid3_debug_inject_timeout(q, k, v, scratch, stop_group)
+        torch.cuda.synchronize()
+        assert ctx.launch_count() - n0 == 2        # attention, sum of the parts
+        assert ctx.last_status() == ERR_TIMEOUT
+        assert (scratch.view(torch.int16) == np.int16(POISON)).all()
+        out = poison_like(q)
+        ctx.rapid3_sparse_joint_attn(q, k, v, out)
+        torch.cuda.synchronize()
+        assert ctx.last_status() == 0
+        want = out if want is None else want
+        assert torch.equal(out.view(torch.int16), want.view(torch.int16))
+    ref = (q[0].double() @ k[0].double().transpose(1, 2) * D ** -0.5).softmax(-1) @ v[0].double()
+    assert float((want[0].double() - ref).abs().max()) <= 2 ** -7 * float(v.abs().max())    # P and the result rounded to bf16
+
+
 @pytest.mark.parametrize("D", [64, 128])
 def test_a_wait_that_ran_out_does_not_delay_the_end_by_the_sequence(D):
     """512 key blocks: 256 thread blocks, two rounds of them, each over after 4096 polls and 16 more for each of the next 32
