@@ -145,3 +145,111 @@ def test_steps_in_place(D, H, n_text, n_image, ratios, packed):
         assert torch.equal(ctx.workspace(n_sparse)[0], scores), name
         assert torch.equal(bits(place), bits(apart)), name
         q.copy_(q0)
+
+
+@pytest.mark.parametrize("D,n_text,n_blocks,H", [(128, 512, 97, 8), (64, 512, 192, 16)])
+def test_masks_of_a_ratio_for_every_head(D, n_text, n_blocks, H):
+    """The masks, lists and counts of the staged selection at each head's own ratio."""
+    B, N = 4 if H == 8 else 2, 64 * n_blocks
+    q, k, v = (torch.randn((B, H, N, D), device=DEV).to(torch.bfloat16) for _ in range(3))
+    per_head = [[(0.15, 0.3, 0.6, 0.9, 1.0)[(b + h) % 5] for h in range(H)] for b in range(B)]
+    ctx, out = binding.Context(B, H, D, n_text, N - n_text), torch.empty_like(q)
+    n0 = ctx.launch_count()
+    ctx.rapid3_gated_step_heads(q, k, v, out, [2] * B, per_head)
+    assert ctx.launch_count() - n0 == 2
+    got = [t.clone() for t in ctx.workspace(B)]
+    scores = ctx.rapid3_block_scores(q, k)
+    assert torch.equal(bits(got[0]), bits(scores))
+    for ratio in (0.15, 0.3, 0.6, 0.9, 1.0):
+        ref = ctx.rapid3_select_mask(scores, [ratio] * B)
+        at = torch.tensor(per_head, device=DEV) == torch.tensor(ratio, device=DEV)
+        for a, b in zip(got[1:], ref):
+            assert torch.equal(a[at], b[at]), ratio
+    assert ctx.last_status() == 0
+
+
+STEP = (2, 24, 64, 128, 28 * 64 - 128)             # images, heads, D, text, image tokens: 336 quads, the last ones by length
+
+
+def step_inputs(seed):
+    B, H, D, n_text, n_image = STEP
+    gen = torch.Generator(device=DEV).manual_seed(seed)
+    return [torch.randn((B, H, n_text + n_image, D), generator=gen, device=DEV).to(torch.bfloat16) for _ in range(3)]
+
+
+def step_context():
+    return binding.Context(*STEP)
+
+
+def step_calls(ctx, q, k, v, out, acts_dev, ratios_dev):
+    ratios = [1.0, 0.25]
+    return {"step": lambda: ctx.rapid3_gated_step(q, k, v, out, [2, 2], ratios),
+            "heads": lambda: ctx.rapid3_gated_step_heads(q, k, v, out, [2, 2], [[r] * 24 for r in ratios]),
+            "mass": lambda: ctx.rapid3_gated_step_mass(q, k, v, out, [2, 2], ratios, 0.5),
+            "device": lambda: ctx.rapid3_gated_step_device(q, k, v, out, acts_dev, ratios_dev)}
+
+
+@pytest.mark.parametrize("kind", ["step", "heads", "mass", "device"])
+def test_replays_of_a_captured_step(kind):
+    """A step whose attention runs beside the clusters and ends by length, captured and replayed on buffers refilled in place."""
+    q, k, v = step_inputs(0)
+    out, ctx, plain = torch.empty_like(q), step_context(), step_context()
+    acts, ratios = torch.full((2,), 2, dtype=torch.int32, device=DEV), torch.tensor([1.0, 0.25], device=DEV)
+    call = step_calls(ctx, q, k, v, out, acts, ratios)[kind]
+    n0 = ctx.launch_count()
+    call()
+    assert ctx.launch_count() - n0 == (5 if kind == "device" else 2)
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        call()
+    for seed in (1, 2, 3):
+        for t, new in zip((q, k, v), step_inputs(seed)):
+            t.copy_(new)
+        for _ in range(3):                         # replays behind one another
+            out.fill_(float("nan"))
+            graph.replay()
+        want = torch.empty_like(q)
+        step_calls(plain, q, k, v, want, acts, ratios)[kind]()
+        torch.cuda.synchronize()
+        assert ctx.last_status() == 0 and plain.last_status() == 0
+        assert torch.equal(bits(out), bits(want)), seed
+        for a, b in zip(ctx.workspace(1), plain.workspace(1)):
+            assert torch.equal(a, b), seed
+
+
+@pytest.mark.parametrize("kind", ["step", "heads", "mass", "device"])
+def test_two_contexts_on_two_streams(kind):
+    """Two contexts, whose clusters and attention kernels share the GPU: the results of each alone."""
+    acts, ratios = torch.full((2,), 2, dtype=torch.int32, device=DEV), torch.tensor([1.0, 0.25], device=DEV)
+    tensors = [step_inputs(seed) for seed in (4, 5)]
+    want, outs = [torch.empty_like(t[0]) for t in tensors], [torch.empty_like(t[0]) for t in tensors]
+    alone = step_context()
+    for t, o in zip(tensors, want):
+        step_calls(alone, *t, o, acts, ratios)[kind]()
+    torch.cuda.synchronize()
+    ctxs, streams = [step_context() for _ in range(2)], [torch.cuda.Stream() for _ in range(2)]
+    calls = [step_calls(c, *t, o, acts, ratios)[kind] for c, t, o in zip(ctxs, tensors, outs)]
+    for _ in range(20):
+        for call, s in zip(calls, streams):
+            with torch.cuda.stream(s):
+                call()
+    torch.cuda.synchronize()
+    for c, o, w in zip(ctxs, outs, want):
+        assert c.last_status() == 0
+        assert torch.equal(bits(o), bits(w))
+
+
+def test_host_buffers_whose_head_groups_take_clusters():
+    """The last image of a step on host buffers goes in four groups of heads, 16 of 64 here: the step's result on device tensors."""
+    B, H, D, n_text, n_image = 2, 64, 64, 512, 56 * 64 - 1
+    q, k, v = (torch.randn((B, H, n_text + n_image, D), device=DEV).to(torch.bfloat16) for _ in range(3))
+    ctx, out, ratios = binding.Context(B, H, D, n_text, n_image), torch.empty_like(q), [1.0, 0.4]
+    ctx.rapid3_gated_step(q, k, v, out, [2, 2], ratios)
+    host = [t.cpu().pin_memory() for t in (q, k, v, torch.empty_like(q))]
+    n0 = ctx.launch_count()
+    ctx.rapid3_gated_step_host(*host, [2, 2], ratios)
+    torch.cuda.synchronize()
+    assert ctx.last_status() == 0
+    assert ctx.launch_count() - n0 == 1 + 4 * 2                # the dense image; clusters and attention of each group
+    assert torch.equal(bits(host[3]), bits(out.cpu()))
