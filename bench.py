@@ -293,13 +293,24 @@ class Prepared:
 
 
 def timed_region(pw, steps, warmup, dist=None):
-    """W warm-up steps, then K steps between one event pair (barrier + synchronize on both sides); right after, the same K steps
-    with an event pair around every attention launch (which would keep the attention from starting beside the scoring
-    pass).  Returns (ms_total, launches, (attention ms, attention launches), wall-clock window of the timed steps)."""
+    """W warm-up steps, then K steps between one event pair (barrier + synchronize on both sides).  Half of as many steps before
+    them and half after have an event pair around every attention launch (which would keep the attention from starting beside
+    the scoring pass): the GPU is as warm on both sides of the timed steps as in them.  Returns (ms_total, launches, (attention ms,
+    attention launches), wall-clock window of the timed steps)."""
     ctx = pw.ctx
+
+    def attention_steps(first, last):
+        ctx.profile(2)                 # an event pair around the attention kernel only: the roofline's duration
+        for i in range(first, last):
+            pw.step(i)
+        torch.cuda.synchronize()
+        ctx.profile(False)
+
     for i in range(warmup):
         pw.step(i)
     torch.cuda.synchronize()
+    ctx.profile_read()
+    attention_steps(0, steps // 2)
     n0 = ctx.launch_count()
     if dist is not None:
         dist.barrier()
@@ -319,14 +330,8 @@ def timed_region(pw, steps, warmup, dist=None):
     if dist is not None:
         dist.barrier()
     launches = ctx.launch_count() - n0
-    ctx.profile(2)                     # an event pair around the attention kernel only: the roofline's duration
-    ctx.profile_read()
-    for i in range(steps):
-        pw.step(i)
-    torch.cuda.synchronize()
-    attn = ctx.profile_read()["attention"]
-    ctx.profile(False)
-    return ms_total, launches, attn, (w0, w1)
+    attention_steps(steps // 2, steps)
+    return ms_total, launches, ctx.profile_read()["attention"], (w0, w1)
 
 
 def per_step_times(pw, n):
