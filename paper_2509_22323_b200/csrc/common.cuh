@@ -15,7 +15,8 @@
 constexpr int SM_COUNT = 148; // of a B200
 
 // Per-launch image list.  batch[p]: index into the B dimension of Q/K/V/O.
-// slot[p]: index into the compacted scores / mask / kept-list arrays, or -1 for a dense image.
+// slot[p]: index into the compacted scores / mask / kept-list arrays, or -1 for a dense image.  In the list of sparse images that the
+// selection and scoring_kernel get with a QuadOrder: the image's place among the sparse ones in the attention's list.
 // k_free[p]: free candidates kept per image row (select kernel).
 struct ImgList {
     int n;
@@ -96,8 +97,10 @@ __host__ __device__ inline int quad_block(const TensorGeom& g, int quad, int a) 
 // wait; the quads before them stay in that order, in which the thread blocks at work share the K and V of a few heads.
 // For launches of more than ORDER_FROM quads (two for each SM) up to ORDER_TO: whole steps of 864 quads, us, two images with a ratio for every
 // head 197.5 -> 190.2, by cumulative mass 358.2 -> 346.3, a dense one and one at 0.5 (D = 64) 262.5 -> 257.3; one image of 432
-// quads at 0.5 from raw projections 190.5 -> 182.9.  Outside these bounds the idle SMs at the end cost less than the heads'
-// first reads at once and the longer selection do (192 quads 41.2 -> 42.1; 1632 quads at D = 64 303.5 -> 313.7).
+// quads at 0.5 from raw projections 190.5 -> 182.9; 316 steps drawn at random between the bounds 1.8 % faster in the mean, the
+// worst 3.4 % slower.  Above them the idle SMs at the end cost less than the heads' first reads at once and the longer selection
+// do (1632 quads at D = 64 303.5 -> 313.7); below, steps of 180 to 221 quads gain 0.6 % in the mean (65, the worst +7.3 %) and those
+// of 222 to 296, which this line leaves out, 2.1 % (102, the worst +2.2 %).
 constexpr int ORDER_CLASSES = 32, ORDER_LAST = 448, ORDER_FROM = 296, ORDER_TO = 1000;
 struct QuadOrder {
     uint8_t* cls = nullptr;          // [ORDER_LAST] class of the quad at that place from the first of the last on; 16-byte aligned
@@ -208,17 +211,18 @@ cudaError_t launch_plan(const int32_t* action_dev, const float* ratio_dev, int B
                         DevPlan* plan, int* status, cudaStream_t s);
 // K3: attention over kept tiles.  `bitmask` (optional) is the select kernel's bitmask of the same
 // lists; when present the kernel reads it instead of walking the lists.  inject_stop_group >= 0
-// launches the failure-injection build of the kernel (see rapid3_debug_inject_timeout).
+// launches the failure-injection build of the kernel (see rapid3_debug_inject_timeout).  wait_first = false: after the selection
+// kernel, for whose masks the quads of sparse images wait themselves.  With `parts` lists may be worked on in parts, in one
+// launch more (added to *launches).
 cudaError_t launch_attention(const CUtensorMap& tmq, const CUtensorMap& tmk, const CUtensorMap& tmv,
                              void* out, const TensorGeom& g, const ImgList& imgs, const int32_t* kept_idx,
                              const int32_t* kept_cnt, const uint64_t* bitmask, float softmax_scale, int* status,
                              cudaStream_t s, const DevPlan* plan = nullptr, int n_cap = 0, int inject_stop_group = -1,
-                             bool wait_first = true,
-                             // with `parts` lists may be worked on in parts, in one launch more (added to *launches)
-                             const AttnParts* parts = nullptr, int64_t* launches = nullptr,
-                             const QuadOrder& order = QuadOrder());   // false: after the selection kernel, for whose masks the quads of sparse images wait themselves
+                             bool wait_first = true, const AttnParts* parts = nullptr, int64_t* launches = nullptr,
+                             const QuadOrder& order = QuadOrder());
 AttnParts attention_parts(const TensorGeom& g, int n_img);     // without its pointers
 size_t attention_partial_bytes(const TensorGeom& g, int n_img, const AttnParts& parts);
 // Kernel attributes on the current device; set when a context is created (scoring: also by the context-free entry).
 cudaError_t attention_static_init();
 cudaError_t scoring_static_init();
+cudaError_t scoring_cluster_static_init();

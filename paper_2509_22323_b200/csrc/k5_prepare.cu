@@ -6,12 +6,13 @@
 // token row of D channels is D / 8 lanes of 16 bytes; the row's sum of squares is reduced over
 // those lanes with shuffles, the rotation is lane-local (a lane holds four whole pairs).
 // HBM-bound: reads the raw Q and K once, writes Q and K once.
-#include "common.cuh"
+#include "scoring.cuh"
+
+using scoring::bf16_hi;
+using scoring::bf16_lo;
 
 namespace {
 
-__device__ __forceinline__ float bf16_lo(uint32_t w) { return __uint_as_float(w << 16); }
-__device__ __forceinline__ float bf16_hi(uint32_t w) { return __uint_as_float(w & 0xffff0000u); }
 __device__ __forceinline__ uint32_t pack2(float lo, float hi) {
     uint32_t d;
     asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(d) : "f"(hi), "f"(lo));

@@ -2,7 +2,7 @@
 //
 // Three kernels one after the other (k1, k2) each spread over the GPU, wait for one another's last thread block and keep every
 // SM from the attention, of which much needs no mask: quads of dense images and of text rows.  Here a pair belongs to a
-// cluster of 1 to 8 thread blocks, which meet once, between the means and the scores; the attention kernel starts beside
+// cluster of 1 to 6 thread blocks, which meet once, between the means and the scores; the attention kernel starts beside
 // them (programmatic dependent launch) on the SMs that they leave free and works on what needs no mask until they are through.
 // The cluster size is the launch's choice (scoring_cluster below): few SMs where there is other work for the rest, all of
 // them where there is not.
@@ -178,8 +178,6 @@ cudaError_t launch(ScoreArgs& a, const HK& hk, int pairs, cudaStream_t s) {
         const int nq = (a.g.nb + 3) / 4, own = 4 * ((nq + a.cluster - 1) / a.cluster);
         a.rows = std::min((own + 7) / 8 * 8, (SMEM_MAX - ring) / row / 8 * 8);
         const int smem = ring + a.rows * row;
-        cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_MAX);
-        if (e != cudaSuccess) return e;
         return launch_kernel_cluster(kernel, dim3(pairs * a.cluster), dim3(WARPS * 32), smem, s, a.cluster, a, hk);
     };
     return a.g.D == 128 ? with_kernel<128, HK>(a.g.nb, go) : with_kernel<64, HK>(a.g.nb, go);
@@ -187,12 +185,28 @@ cudaError_t launch(ScoreArgs& a, const HK& hk, int pairs, cudaStream_t s) {
 
 }  // namespace
 
+cudaError_t scoring_cluster_static_init() {
+    cudaError_t e = cudaSuccess;
+    const auto set = [&](auto kernel, int, int) {
+        return e = e != cudaSuccess ? e : cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_MAX);
+    };
+    for (int nb : {96, 192}) {
+        with_kernel<128, NoHeadKeep>(nb, set);
+        with_kernel<128, HeadKeep>(nb, set);
+        with_kernel<128, MassRule>(nb, set);
+        with_kernel<64, NoHeadKeep>(nb, set);
+        with_kernel<64, HeadKeep>(nb, set);
+        with_kernel<64, MassRule>(nb, set);
+    }
+    return e;
+}
+
 // Thread blocks of a cluster for that many (image, head) pairs, or 0 for the three kernels, which spread over the GPU what a few
 // pairs cannot.  The least SM time decides: what the pass takes of its own SMs, and what the others wait for it after the attention
 // that needs no mask (heavy_us of SM time).  The times in us: a thread block alone 21 for a MB of Q and K, the scores at half
 // of the fp64 tensor rate, 3.3 or 5 for every 24 rows (5 more by cumulative mass); the three kernels 7 (one more by mass 2.5) and
-// 4.5 TB/s.  One thread block a pair, the longest of all, only beside much other work; a second wave of clusters (45 of three fit at
-// a time) never; rows of more than 192 blocks gain nothing (24 pairs of 264: 1114 us a step, this way 1109 to 1140).  Launches of
+// 4.5 TB/s.  One thread block a pair, the longest of all, only beside much other work, and only so a second wave of them; of clusters
+// (45 of three fit at a time) no second wave; rows of more than 192 blocks gain nothing (24 pairs of 264: 1114 us a step, this way 1109 to 1140).  Launches of
 // fewer quads than SCORING_FROM wait for the first masks, not for SMs (96 quads of 15 blocks 23.7 / 28.0, 192 of 29 35.3 / 37.1).
 // Steps, us, three kernels / clusters: two images of 24 heads, 1357 tokens, D = 64 43.4 / 41.5 (of two); 864 quads with per-head
 // ratios 189.3 / 184.9 (two), by mass 343 / 337 (two), a dense and a sparse image at D = 64 258.7 / 254.2 (one); one image from
