@@ -49,6 +49,7 @@ namespace {
 constexpr int SOFTMAX_WARPS = 16;
 constexpr int PRODUCER_WARP = 16, MMA_WARP0 = 17, LIST_WARP = 19;
 constexpr int NTHREADS = 32 * (SOFTMAX_WARPS + 4);
+constexpr int SOFTMAX_REGS = 104, LIGHT_REGS = 64;     // SPLIT build: registers a thread of the softmax warps, of the others
 constexpr int TMEM_COLS = 512;
 constexpr int TILE_COLS = 256;      // TMEM columns of one Q tile
 constexpr int BLK_BYTES = 8192;     // 64 rows x 128 bytes: one 64-channel half of a 64-token block
@@ -346,7 +347,7 @@ attn_kernel(const __grid_constant__ CUtensorMap tmq, const __grid_constant__ CUt
 
     // The pool is the launch's 640 x 96: 512 x 104 + 128 x 64.  Without it this build keeps ten words of the softmax warps in
     // local memory; in the other builds it gains nothing (ordered, D = 128: fused step of 432 quads 197.0 us without, 199.8 with).
-    if (SPLIT && warp >= SOFTMAX_WARPS) reg_dec<64>();
+    if (SPLIT && warp >= SOFTMAX_WARPS) reg_dec<LIGHT_REGS>();
     if (warp == LIST_WARP) {
         // ------------------------------------------------------------ quads and their union lists
         // one lane polls: these waits are long, and the other lanes' polls would only take issue slots
@@ -750,7 +751,7 @@ attn_kernel(const __grid_constant__ CUtensorMap tmq, const __grid_constant__ CUt
         // (r_lo = lane / 4 and r_lo + 8 of the sixteen) and, of every group of eight score columns, the pair
         // 2 (lane % 4), + 1 -- 32 scores per key block.  The four threads of a quad share their rows' maximum
         // with two shuffles, and only when some row of the warp may have grown.
-        if (SPLIT) reg_inc<104>();
+        if (SPLIT) reg_inc<SOFTMAX_REGS>();
         const int t = (warp >> 2) & 1, wl = warp & 3, hf = warp >> 3;
         const int a = 2 * t + (wl >> 1);               // query block of the quad
         const uint32_t tile_bits = 3u << (2 * t), act_bit = 1u << a;
@@ -1086,6 +1087,14 @@ cudaError_t attention_static_init() {
                               attn_kernel<128, false, false, false, true>, attn_kernel<64, false, false, false, true>,
                               attn_kernel<128, true>, attn_kernel<64, true>, attn_kernel<128, true, true>, attn_kernel<64, true, true>);
     if (e != cudaSuccess) return e;
+    // the warps that take registers wait for them: a build that is launched with fewer would wait for good
+    for (const void* kernel : {(const void*)attn_kernel<128, false, true>, (const void*)attn_kernel<64, false, true>,
+                               (const void*)attn_kernel<128, true, true>, (const void*)attn_kernel<64, true, true>}) {
+        cudaFuncAttributes attr;
+        const cudaError_t r = cudaFuncGetAttributes(&attr, kernel);
+        if (r != cudaSuccess) return r;
+        if (attr.numRegs * NTHREADS < 32 * (SOFTMAX_WARPS * SOFTMAX_REGS + 4 * LIGHT_REGS)) return cudaErrorInvalidKernelImage;
+    }
     g_attr_set = true;
     return cudaSuccess;
 }
