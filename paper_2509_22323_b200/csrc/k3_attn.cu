@@ -34,6 +34,7 @@
 // Every mbarrier wait is bounded; a wait that runs out records RAPID3_ERR_TIMEOUT in the status
 // word and the thread block drains its copies, releases its TMEM and exits normally.
 #include <float.h>
+#include <stddef.h>
 
 #include <algorithm>
 
@@ -86,9 +87,15 @@ struct AttnParams {
     float scale_log2;
     QuadOrder order;               // optional: the order of the sparse images' quads without text rows
     AttnParts parts;               // SPLIT build: how many units of work the union list of a quad goes to
+    uint32_t div_all, div_text, div_light, div_pure, div_mixed, div_heads;   // divider() of the quads of a head by kind, and of the heads
     bool wait_first;               // nothing is read before the kernel in front has ended
     int stop_group;                // failure-injection build of the kernel only: the producer stops before this group
 };
+
+// x / d as a product with divider(d): exact while x d < 2^32.  Quads number below 2^24 and those of a head 256 at most; pairs and
+// heads below 2^16.  (A division takes some twenty instructions, which a thread block's first quad waits for: see the list warp.)
+__host__ __device__ constexpr uint32_t divider(uint32_t d) { return d < 2 ? 0u : 0xffffffffu / d + 1u; }
+__device__ __forceinline__ int divide(int x, uint32_t by) { return (int)__umulhi((uint32_t)x, by) + (by ? 0 : x); }
 
 template <int D>
 struct Cfg {
@@ -253,35 +260,27 @@ attn_kernel(const __grid_constant__ CUtensorMap tmq, const __grid_constant__ CUt
     const uint32_t bNE = smem_u32(&ctl->near_end), bT = smem_u32(&ctl->taken_full), bFK = smem_u32(&ctl->first_known);
 
     // ---------------------------------------------------------------- setup
-    if (warp == 0) {                                    // one barrier group per lane
-        if (lane < MAX_STAGES) {
-            mbar_init(bKF + 8 * lane, 1);
-            mbar_init(bKE + 8 * lane, 2);   // both tiles pass a stage before it is refilled
-            mbar_init(bVE + 8 * lane, 2);
-        } else if (lane < MAX_STAGES + 6) {
-            mbar_init(bSF + 8 * (lane - MAX_STAGES), 1);
-            mbar_init(bPF + 8 * (lane - MAX_STAGES), 8);      // one arrival per softmax warp of the tile
-        } else if (lane < MAX_STAGES + 8) {
-            const int t = lane - MAX_STAGES - 6;
-            mbar_init(bPV + 16 * t, 1);
-            mbar_init(bPV + 16 * t + 8, 1);
-            mbar_init(bOD + 8 * t, 1);
-            mbar_init(smem_u32(&ctl->drain[t]), 1);
-            mbar_init(bUF + 8 * t, 1);
-            mbar_init(bUE + 8 * t, QUAD_USERS);
-        } else if (lane == MAX_STAGES + 8) {
-            mbar_init(bQ, 1);
-            mbar_init(bQE, 2);
-            mbar_init(bNE, 1);
-            mbar_init(bT, 1);
-            mbar_init(bFK, 1);
-            ctl->abort_flag = 0;
-        } else if (lane == MAX_STAGES + 9) {
-            prefetch_tmap(&tmq);
-            prefetch_tmap(&tmk);
-            prefetch_tmap(&tmv);
+    // The list warp needs nothing of it until it arrives on a barrier, so it only waits for warp 0 (named barrier 1), later on.
+    if (warp == 0) {
+        constexpr uint32_t at = offsetof(Ctl, taken_full) / 8, bars = offsetof(Ctl, tmem_base) / 8 - at;
+        auto has = [&](uint32_t x, size_t member, int n) { return x + at - (uint32_t)(member / 8) < (uint32_t)n; };
+#pragma unroll
+        for (uint32_t x = lane; x < bars; x += 32) {
+            uint32_t count = 1;
+            if (has(x, offsetof(Ctl, quad_empty), 2)) count = QUAD_USERS;
+            if (has(x, offsetof(Ctl, q_empty), 1) || has(x, offsetof(Ctl, k_empty), 2 * MAX_STAGES)) count = 2;   // both tiles pass a stage before it is refilled
+            if (has(x, offsetof(Ctl, p_full), 6)) count = 8;                   // one arrival per softmax warp of the tile
+            mbar_init(smem_u32(ctl) + 8 * (at + x), count);
         }
+        if (lane == 0) ctl->abort_flag = 0;
         fence_mbar_init();
+        __syncwarp();
+        bar_arrive(1, 64);
+    }
+    if (warp == PRODUCER_WARP && lane < 3) prefetch_tmap(lane == 0 ? &tmq : lane == 1 ? &tmk : &tmv);
+    if (warp == LIST_WARP && !prm.plan) {
+        // the kernel's arguments are not in the SM's cache yet: what the first quad's index arithmetic ends with is fetched beside it
+        asm volatile("" ::"r"(prm.imgs.batch[0]), "r"(prm.imgs.slot[0]), "r"(g.pair_stride), "r"(g.h0));
     }
     if (warp == MMA_WARP0) {
         tmem_alloc(smem_u32(&ctl->tmem_base), TMEM_COLS);
@@ -293,7 +292,8 @@ attn_kernel(const __grid_constant__ CUtensorMap tmq, const __grid_constant__ CUt
     // after thousands of polls, so nothing sets it before this; what read it last has ended before the selection kernel began, if
     // that is in front.
     if (SPLIT && blockIdx.x == 0 && tid == 0) __stcg(prm.parts.given_up, 0);
-    __syncthreads();
+    if (warp == LIST_WARP) bar_arrive(0, NTHREADS);
+    else bar_sync(0, NTHREADS);
     tc_fence_after();
     const uint32_t tmem_base = ctl->tmem_base;
 
@@ -350,6 +350,11 @@ attn_kernel(const __grid_constant__ CUtensorMap tmq, const __grid_constant__ CUt
     if (SPLIT && warp >= SOFTMAX_WARPS) reg_dec<LIGHT_REGS>();
     if (warp == LIST_WARP) {
         // ------------------------------------------------------------ quads and their union lists
+        // A thread block's first quad waits for this warp, whose code the SM has to fetch first: what lies in front of the first list is
+        // short, and beside the set-up as far as it can be.  Divisions by the launch's constants as products, a member a lane
+        // instead of four in a row, no masks where every block is kept, the arguments fetched early: the first list 2.1 -> 1.3 us
+        // after the start of a thread block, the first Q's loads 1.6 -> 0.9 (steps of 288 quads at D = 64 41.7 -> 40.5 us, one dense
+        // image of 12 quads 9.7 -> 9.1).
         // one lane polls: these waits are long, and the other lanes' polls would only take issue slots
         auto wait_lane0 = [&](uint32_t bar, uint32_t parity) -> bool {
             return __shfl_sync(0xffffffffu, (int)(lane != 0 || wait(bar, parity)), 0);
@@ -360,7 +365,7 @@ attn_kernel(const __grid_constant__ CUtensorMap tmq, const __grid_constant__ CUt
         bool have_classes = false;
         for (uint32_t i = 0;; ++i) {
             Quad& u = ctl->quad[i & 1];
-            if (!wait_lane0(bUE + 8 * (i & 1), ((i >> 1) & 1) ^ 1)) break;
+            if (i > 1 && !wait_lane0(bUE + 8 * (i & 1), ((i >> 1) & 1) ^ 1)) break;
             if (L < 0) {
                 if (lane == 0) {
                     u.n_u = -1;
@@ -406,78 +411,89 @@ attn_kernel(const __grid_constant__ CUtensorMap tmq, const __grid_constant__ CUt
                         u.parts = parts;
                     }
                 }
-                if (L < heavy_dense) {
-                    p = L / (g.H * nq); L -= p * g.H * nq;
-                    h = L / nq; quad = L - h * nq;
-                } else if (L < heavy_dense + heavy_sparse) {
+                int first = 0, n = nq;                   // the quads of a head of this kind: so many from `first` on
+                uint32_t by = prm.div_all;
+                p = 0;
+                if (L >= heavy_dense) {
                     L -= heavy_dense;
-                    // those of text rows alone first: they need no mask, which may not be there yet
-                    const int ntf = SPLIT ? ntq : g.n_text_blocks >> 2, n_full = ns * g.H * ntf;
-                    const bool full = L < n_full;
-                    const int first = full ? 0 : ntf, n = full ? ntf : ntq - ntf;       // quads of a head from `first` on
-                    if (!full) L -= n_full;
-                    p = L / (g.H * n); L -= p * g.H * n; p += nd;
-                    h = L / n; quad = first + L - h * n;
-                } else {
-                    L -= heavy_dense + heavy_sparse;
-                    const int nl = nq - ntq, in_order = max(ns * g.H * nl - ORDER_LAST, 0), rest = L - in_order;
-                    if (ORDERED && rest >= 0) {
-                        // the quad at place `rest` of the order that the selection kernel has found: of sixteen classes a lane
-                        if (!have_classes) {
-                            if (!waited) grid_dependency_wait();
-                            waited = have_classes = true;
-                            const uint4 v = 16 * lane < ORDER_LAST ? __ldcg(reinterpret_cast<const uint4*>(prm.order.cls) + lane) : make_uint4(0, 0, 0, 0);
-                            classes[0] = v.x; classes[1] = v.y; classes[2] = v.z; classes[3] = v.w;
-                            const int n = ns * g.H * nl - in_order;      // quads in the order; the bytes behind them count for nothing
+                    p = nd;
+                    if (L < heavy_sparse) {
+                        // those of text rows alone first: they need no mask, which may not be there yet
+                        const int ntf = SPLIT ? ntq : g.n_text_blocks >> 2, n_full = ns * g.H * ntf;
+                        const bool full = L < n_full;
+                        first = full ? 0 : ntf;
+                        n = full ? ntf : ntq - ntf;
+                        by = SPLIT ? prm.div_text : full ? prm.div_pure : prm.div_mixed;
+                        if (!full) L -= n_full;
+                    } else {
+                        L -= heavy_sparse;
+                        first = ntq;
+                        n = nq - ntq;
+                        by = prm.div_light;
+                        const int in_order = max(ns * g.H * n - ORDER_LAST, 0), rest = L - in_order;
+                        if (ORDERED && rest >= 0) {
+                            // the quad at place `rest` of the order that the selection kernel has found: of sixteen classes a lane
+                            if (!have_classes) {
+                                if (!waited) grid_dependency_wait();
+                                waited = have_classes = true;
+                                const uint4 v = 16 * lane < ORDER_LAST ? __ldcg(reinterpret_cast<const uint4*>(prm.order.cls) + lane) : make_uint4(0, 0, 0, 0);
+                                classes[0] = v.x; classes[1] = v.y; classes[2] = v.z; classes[3] = v.w;
+                                const int places = ns * g.H * n - in_order;      // quads in the order; the bytes behind them count for nothing
 #pragma unroll
-                            for (int x = 0; x < 16; ++x)
-                                if (16 * lane + x >= n) classes[x / 4] |= 0xffu << (8 * (x % 4));
+                                for (int x = 0; x < 16; ++x)
+                                    if (16 * lane + x >= places) classes[x / 4] |= 0xffu << (8 * (x % 4));
+                            }
+                            L = in_order + order_find(classes, rest, lane);
                         }
-                        L = in_order + order_find(classes, rest, lane);
                     }
-                    p = L / (g.H * nl); L -= p * g.H * nl; p += nd;
-                    h = L / nl; quad = ntq + (L - h * nl);
                 }
+                const int pair = divide(L, by);          // (image, head) of this kind
+                quad = first + L - pair * n;
+                const int image = divide(pair, prm.div_heads);
+                h = pair - image * g.H;
+                p += image;
             }
             const int b = prm.plan ? __ldcg(&prm.plan->all.batch[p]) : prm.imgs.batch[p];
             const int slot = prm.plan ? __ldcg(&prm.plan->all.slot[p]) : prm.imgs.slot[p];
-            auto qblk = [&](int a) -> int {              // member a's query block
-                if (half >= 0 && (a >> 1) != half) return nb;           // not of this unit: like a block past the end
-                return quad_block(g, quad, a);
-            };
+            // Lanes a, a + 4, ... hold member a's query block; which members there are, one of the other half counting like one past the end.
+            const int own = quad_block(g, quad, lane & 3);
+            const bool here_own = own < nb && (half < 0 || ((lane & 3) >> 1) == half);
+            const uint32_t here = __ballot_sync(0xffffffffu, here_own) & 15u;
             const bool masks = MASKS || prm.bitmask32 != nullptr;      // of the selection kernel (it finds the order), else lists of the caller's
             // a dense image's quad, or one of text rows in a mask of the selection kernel: every block is kept, no mask is read
             const bool all_kept = slot < 0 || (masks && 4 * quad + 3 < g.n_text_blocks);
-            // the query block whose kept blocks m[a] below holds: where a list is cut into parts depends on the whole quad
-            auto mblk = [&](int a) -> int { return SPLIT && parts > 1 ? quad_block(g, quad, a) : qblk(a); };
+            // the members whose kept blocks m[a] below holds: where a list is cut into parts depends on the whole quad
+            const uint32_t listed = SPLIT && parts > 1 ? __ballot_sync(0xffffffffu, own < nb) & 15u : here;
+            if (i == 0) bar_sync(1, 64);                 // the barriers are set up
+            if (lane < 4) u.tok[lane] = (here_own ? own : nb) * 64;
+            __syncwarp();
             if (lane == 0) {
                 u.b = b;
                 u.h = g.h0 + h;
-#pragma unroll
-                for (int a = 0; a < 4; ++a) u.tok[a] = qblk(a) * 64;
                 if (i == 0) {
                     // The first quad's Q tiles do not depend on the mask, nor do key blocks known before it is read: a
                     // dense image keeps every block, and a mask of the selection kernel keeps the text blocks in every
                     // row, so the union list starts 0, 1, ....  The producer loads them while the list is built (by this
                     // lane, ahead of the masks, they kept the first list back: steps of 288 quads at D = 64 41.6 -> 40.8 us,
                     // of 24 at D = 128 23.9 -> 23.0, lists of the caller's for 324 quads 80.2 -> 78.9).
-                    const bool none = min(min(qblk(0), qblk(1)), min(qblk(2), qblk(3))) >= nb;   // the second half of a ragged last quad
-                    int n_early = (!INJECT && !none && (all_kept || masks)) ? min(min(all_kept ? nb : g.n_text_blocks, nb), KS) : 0;
+                    // (no members: the second half of a ragged last quad)
+                    int n_early = (!INJECT && here && (all_kept || masks)) ? min(min(all_kept ? nb : g.n_text_blocks, nb), KS) : 0;
                     if (SPLIT && parts > 1) n_early = part == 0 ? min(n_early, (all_kept ? nb : g.n_text_blocks) / parts) : 0;   // its part of the list is no shorter
                     ctl->n_early = n_early;
                     mbar_arrive(bFK);
                 }
             }
-            // m[a] = 32 bits of the set of key blocks that member a keeps: from the bitmask when the caller has one,
-            // else rebuilt from the kept list; every block for a dense image.
-            const int nw = (nb + 31) >> 5;
-            uint32_t m[4];
+            int n_u;
+            auto entry = [&](uint32_t f, int j) { return f | ((j + 1) * 64 > N ? ENT_TAIL : 0u) | ((uint32_t)j << ENT_BLK); };
             if (all_kept) {
-                const int n = min(max(nb - lane * 32, 0), 32);
-                const uint32_t val = n == 32 ? 0xffffffffu : ((1u << n) - 1u);
-#pragma unroll
-                for (int a = 0; a < 4; ++a) m[a] = mblk(a) < nb ? val : 0u;
+                const int first = SPLIT ? nb * part / parts : 0, last = !here ? first : SPLIT ? nb * (part + 1) / parts : nb;
+                n_u = last - first;
+                for (int j = first + lane; j < last; j += 32) u.ent[j - first] = entry(here, j);
             } else {
+                // m[a] = 32 bits of the set of key blocks that member a keeps: from the bitmask when the caller has one,
+                // else rebuilt from the kept list.
+                const int nw = (nb + 31) >> 5;
+                uint32_t m[4];
                 // Launched as a dependent of the selection kernel, the masks have to be waited for once.  They are read
                 // past the L1 (ld.global.cg): this thread block may have started before they were written, and an L1
                 // line of an earlier step must not answer.
@@ -485,9 +501,10 @@ attn_kernel(const __grid_constant__ CUtensorMap tmq, const __grid_constant__ CUt
                 waited = true;
                 if (masks) {
 #pragma unroll
-                    for (int a = 0; a < 4; ++a)
-                        m[a] = (mblk(a) < nb && lane < nw)
-                                   ? __ldcg(prm.bitmask32 + (((long long)slot * g.H + h) * nb + mblk(a)) * prm.words32 + lane) : 0u;
+                    for (int a = 0; a < 4; ++a) {
+                        const long long row = ((long long)slot * g.H + h) * nb + __shfl_sync(0xffffffffu, own, a);
+                        m[a] = ((listed >> a) & 1u) && lane < nw ? __ldcg(prm.bitmask32 + row * prm.words32 + lane) : 0u;
+                    }
                 } else {
 #pragma unroll
                     for (int a = 0; a < 4; ++a) ctl->bm[a][lane] = 0u;
@@ -498,8 +515,9 @@ attn_kernel(const __grid_constant__ CUtensorMap tmq, const __grid_constant__ CUt
                     int cnt[4], first[4], second[4];
 #pragma unroll
                     for (int a = 0; a < 4; ++a) {
-                        const bool in = mblk(a) < nb;
-                        const long long row = ((long long)slot * g.H + h) * nb + (in ? mblk(a) : 0);
+                        const bool in = (listed >> a) & 1u;
+                        const int block = __shfl_sync(0xffffffffu, own, a);
+                        const long long row = ((long long)slot * g.H + h) * nb + (in ? block : 0);
                         lst[a] = prm.kept_idx + row * nb;
                         cnt[a] = in ? __ldcg(prm.kept_cnt + row) : 0;
                         first[a] = in && lane < nb ? __ldcg(lst[a] + lane) : 0;
@@ -527,38 +545,37 @@ attn_kernel(const __grid_constant__ CUtensorMap tmq, const __grid_constant__ CUt
 #pragma unroll
                     for (int a = 0; a < 4; ++a) m[a] = ctl->bm[a][lane];
                 }
-            }
-            // the position of a key block in the ascending union list is the number of union bits below it
-            auto union_bits_below = [&](uint32_t bits, int& all) -> int {
-                int x = __popc(bits);
+                // the position of a key block in the ascending union list is the number of union bits below it
+                auto union_bits_below = [&](uint32_t bits, int& all) -> int {
+                    int x = __popc(bits);
 #pragma unroll
-                for (int o = 1; o < 32; o <<= 1) {
-                    const int v = __shfl_up_sync(0xffffffffu, x, o);
-                    if (lane >= o) x += v;
+                    for (int o = 1; o < 32; o <<= 1) {
+                        const int v = __shfl_up_sync(0xffffffffu, x, o);
+                        if (lane >= o) x += v;
+                    }
+                    all = __shfl_sync(0xffffffffu, x, 31);
+                    return x - __popc(bits);
+                };
+                if (SPLIT && parts > 1) {                    // of the quad's union, the blocks from `first` up to `last` are this part's
+                    uint32_t from = m[0] | m[1] | m[2] | m[3], to = from;
+                    const int at = union_bits_below(from, n_u), first = n_u * part / parts, last = n_u * (part + 1) / parts;
+                    for (int x = min(max(first - at, 0), 32); x > 0; --x) from &= from - 1u;
+                    for (int x = min(max(last - at, 0), 32); x > 0; --x) to &= to - 1u;
+#pragma unroll
+                    for (int a = 0; a < 4; ++a) m[a] &= (here >> a) & 1u ? from & ~to : 0u;
                 }
-                all = __shfl_sync(0xffffffffu, x, 31);
-                return x - __popc(bits);
-            };
-            int n_u;
-            if (SPLIT && parts > 1) {                    // of the quad's union, the blocks from `first` up to `last` are this part's
-                uint32_t from = m[0] | m[1] | m[2] | m[3], to = from;
-                const int at = union_bits_below(from, n_u), first = n_u * part / parts, last = n_u * (part + 1) / parts;
-                for (int x = min(max(first - at, 0), 32); x > 0; --x) from &= from - 1u;
-                for (int x = min(max(last - at, 0), 32); x > 0; --x) to &= to - 1u;
+                const uint32_t un = m[0] | m[1] | m[2] | m[3];
+                const int below = union_bits_below(un, n_u);
+                for (int w = 0; w < nw; ++w) {
+                    const uint32_t uw = __shfl_sync(0xffffffffu, un, w);
+                    const int pos = __shfl_sync(0xffffffffu, below, w) + __popc(uw & ((1u << lane) - 1u));
+                    uint32_t f = 0u;
 #pragma unroll
-                for (int a = 0; a < 4; ++a) m[a] &= qblk(a) < nb ? from & ~to : 0u;
-            }
-            const uint32_t un = m[0] | m[1] | m[2] | m[3];
-            const int below = union_bits_below(un, n_u);
-            for (int w = 0; w < nw; ++w) {
-                const uint32_t uw = __shfl_sync(0xffffffffu, un, w);
-                const int pos = __shfl_sync(0xffffffffu, below, w) + __popc(uw & ((1u << lane) - 1u));
-                uint32_t f = 0u;
-#pragma unroll
-                for (int a = 0; a < 4; ++a) f |= ((__shfl_sync(0xffffffffu, m[a], w) >> lane) & 1u) << a;
-                if (f) {
-                    const int j = 32 * w + lane;
-                    u.ent[pos] = f | ((j + 1) * 64 > N ? ENT_TAIL : 0u) | ((uint32_t)j << ENT_BLK);
+                    for (int a = 0; a < 4; ++a) f |= ((__shfl_sync(0xffffffffu, m[a], w) >> lane) & 1u) << a;
+                    if (f) {
+                        const int j = 32 * w + lane;
+                        u.ent[pos] = entry(f, j);
+                    }
                 }
             }
             if (lane == 0) u.n_u = n_u;
@@ -1218,6 +1235,15 @@ cudaError_t launch_attention(const CUtensorMap& tmq, const CUtensorMap& tmk, con
     prm.plan = plan;
     prm.order = order;
     prm.wait_first = wait_first;
+    {
+        const int quads = (g.nb + 3) / 4, text = std::min(quads, (g.n_text_blocks + 3) / 4), pure = g.n_text_blocks / 4;
+        prm.div_all = divider(quads);
+        prm.div_text = divider(text);
+        prm.div_pure = divider(pure);
+        prm.div_mixed = divider(text - pure);
+        prm.div_light = divider(quads - text);
+        prm.div_heads = divider(g.H);
+    }
     prm.stop_group = inject_stop_group;
     const int n_img = plan ? n_cap : imgs.n, pairs = g.H * n_img, nq = (g.nb + 3) / 4, ntq = std::min(nq, (g.n_text_blocks + 3) / 4);
     int left = 0;                              // quads whose lists are worked on in parts, at most
