@@ -470,7 +470,8 @@ static int gated_step_impl(rapid3_ctx* c, const void* q, const void* k, const vo
         if (launch_prepare(*prep, g, all, sparse.n, c->pooled, st) != cudaSuccess) return RAPID3_ERR_CUDA;
         c->launches += 1;
     }
-    const QuadOrder order = sparse.n > 0 ? step_order(c, g, all.n) : QuadOrder();
+    QuadOrder order = sparse.n > 0 ? step_order(c, g, all.n) : QuadOrder();
+    order.n_dense = all.n - sparse.n;
     for (int p = 0; p < all.n; ++p)                       // for the selection kernel: place in the attention's list
         if (all.slot[p] >= 0) sparse.slot[all.slot[p]] = p - (all.n - sparse.n);
     if (sparse.n > 0) {

@@ -58,7 +58,7 @@ __global__ void __launch_bounds__(WARPS * 32) select_kernel(const float* scores,
         uint32_t m[4];
 #pragma unroll
         for (int a = 0; a < 4; ++a) m[a] = 32 * lane < nb ? kept[a][lane] : 0u;
-        order_quad(order, g, n_sparse, place, ph % g.H, blockIdx.x, m, lane);
+        order_quad(order, g, plan ? __ldcg(&plan->n_dense) : order.n_dense, n_sparse, place, ph % g.H, blockIdx.x, m, lane);
     }
 }
 

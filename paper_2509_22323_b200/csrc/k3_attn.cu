@@ -430,7 +430,7 @@ attn_kernel(const __grid_constant__ CUtensorMap tmq, const __grid_constant__ CUt
                         first = ntq;
                         n = nq - ntq;
                         by = prm.div_light;
-                        const int in_order = max(ns * g.H * n - ORDER_LAST, 0), rest = L - in_order;
+                        const int in_order = order_after(ns * g.H * n, heavy_dense + heavy_sparse), rest = L - in_order;
                         if (ORDERED && rest >= 0) {
                             // the quad at place `rest` of the order that the selection kernel has found: of sixteen classes a lane
                             if (!have_classes) {

@@ -159,7 +159,7 @@ __global__ void __launch_bounds__(WARPS * 32, 1) scoring_kernel(const __grid_con
                 uint32_t m[4];
 #pragma unroll
                 for (int b = 0; b < 4; ++b) m[b] = 32 * lane < nb ? kept[(4 * x + b) * IPL + lane] : 0u;
-                order_quad(a.order, g, a.imgs.n, a.imgs.slot[p], h, q0 + x, m, lane);
+                order_quad(a.order, g, a.order.n_dense, a.imgs.n, a.imgs.slot[p], h, q0 + x, m, lane);
             }
             __syncthreads();
         }

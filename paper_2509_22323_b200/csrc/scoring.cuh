@@ -298,10 +298,10 @@ __device__ __forceinline__ int plan_place(const DevPlan* plan, int p, int lane) 
 
 // A quad's class in the attention's order (QuadOrder), by one warp: m[a] are the 32 bits of member a's mask from block 32 * lane
 // on.  `place`: the image's place among the sparse ones in the attention's list.
-__device__ __forceinline__ void order_quad(const QuadOrder& order, const TensorGeom& g, int n_sparse, int place, int h, int quad,
+__device__ __forceinline__ void order_quad(const QuadOrder& order, const TensorGeom& g, int n_dense, int n_sparse, int place, int h, int quad,
                                            const uint32_t (&m)[4], int lane) {
-    const int ntq = (g.n_text_blocks + 3) >> 2, nl = ((g.nb + 3) >> 2) - ntq;
-    const int at = (place * g.H + h) * nl + quad - ntq - max(n_sparse * g.H * nl - ORDER_LAST, 0);
+    const int nq = (g.nb + 3) >> 2, ntq = (g.n_text_blocks + 3) >> 2, nl = nq - ntq;
+    const int at = (place * g.H + h) * nl + quad - ntq - order_after(n_sparse * g.H * nl, g.H * (n_dense * nq + n_sparse * ntq));
     if (quad < ntq || at < 0) return;                      // quads with text rows, and all but the last of the others, come as they are
     // the quad's time, in quarters of a key block of two tiles: one that only one tile uses takes three quarters
     const uint32_t t0 = m[0] | m[1], t1 = m[2] | m[3];

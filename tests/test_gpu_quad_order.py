@@ -65,3 +65,13 @@ def test_masks_and_lists_give_the_same(D, n_text, n_image, H, B):
     torch.cuda.synchronize()
     assert ctx.last_status() == 0
     assert torch.equal(step.view(torch.int16), staged.view(torch.int16))
+
+
+@pytest.mark.parametrize("D,n_text,n_image,H,B", [
+    (64, 0, 17 * 64 - 3, 17, 3),   # 255 quads, the first 148 of a step without dense images come as they are
+    (128, 200, 800, 26, 2),        # 208: 130 dense or with text, of the others the first 18 come as they are
+    (64, 512, 8 * 64 + 1, 40, 2),  # 400: every SM begins with a dense quad or one with text
+    (64, 512, 60, 67, 1),          # 201: one quad in three has no text, fewer than the SMs begin with
+])
+def test_ordered_quads_behind_those_that_the_sms_begin_with(D, n_text, n_image, H, B):
+    test_ordered_quads_equal_quads_in_order(D, n_text, n_image, H, B)
