@@ -32,6 +32,25 @@ __device__ __forceinline__ void add_row(double (&acc)[8], float& finite, const u
     }
 }
 
+// The mean of `valid` rows from the lanes' sums (add_row's), to `out`.
+template <int D, bool WIDE>
+__device__ __forceinline__ void write_mean(double (&acc)[8], int valid, double* out, int lane) {
+    constexpr int TPR = D / 8;          // lanes that hold different channels
+    if constexpr (!WIDE) {
+#pragma unroll
+        for (int e = 1; e < 8; e += 2) acc[e] *= 0x1p896;
+    }
+#pragma unroll
+    for (int off = TPR; off < 32; off <<= 1)
+#pragma unroll
+        for (int e = 0; e < 8; ++e) acc[e] += __shfl_xor_sync(0xffffffffu, acc[e], off);
+    if (lane < TPR) {
+        const double inv = 1.0 / (double)valid;
+#pragma unroll
+        for (int e = 0; e < 8; e += 2) *reinterpret_cast<double2*>(out + lane * 8 + e) = make_double2(acc[e] * inv, acc[e + 1] * inv);
+    }
+}
+
 // Mean of `valid` token rows (stride elements apart) by one warp, in fp64, to `out`.  A row of D channels is D / 8 lanes of 16 bytes,
 // so a warp-wide load covers 32 / (D / 8) rows; a lane keeps fp64 sums of its 8 channels over the rows that it sees, eight
 // loads in flight, and the lanes that hold the same channels are then added with shuffles.
@@ -60,19 +79,7 @@ __device__ __forceinline__ bool pool_block_as(const uint16_t* base, long long st
     }
     if (!WIDE && __any_sync(0xffffffffu, finite != 0.f)) return false;
     loaded();
-    if constexpr (!WIDE) {
-#pragma unroll
-        for (int e = 1; e < 8; e += 2) acc[e] *= 0x1p896;
-    }
-#pragma unroll
-    for (int off = TPR; off < 32; off <<= 1)
-#pragma unroll
-        for (int e = 0; e < 8; ++e) acc[e] += __shfl_xor_sync(0xffffffffu, acc[e], off);
-    if (lane < TPR) {
-        const double inv = 1.0 / (double)valid;
-#pragma unroll
-        for (int e = 0; e < 8; e += 2) *reinterpret_cast<double2*>(out + c * 8 + e) = make_double2(acc[e] * inv, acc[e + 1] * inv);
-    }
+    write_mean<D, WIDE>(acc, valid, out, lane);
     return true;
 }
 template <int D, typename Loaded>

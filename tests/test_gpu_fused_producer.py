@@ -149,3 +149,22 @@ def test_producer_of_few_and_of_many_blocks(D, H, n_text, n_image, in_place):
         for x, y in zip(both, step(slice(b, b + 1))):
             assert torch.equal(x[b:b + 1], y)
     check_produced(Qr[1], both[0][1].view(torch.bfloat16), gain[0], rot, "Q")
+
+
+@pytest.mark.parametrize("D,H,B", [(64, 9, 2), (128, 5, 4)])
+def test_producer_of_many_blocks_without_a_table(D, H, B):
+    """Heads that do not fill the last thread block of a token block, token-major tensors, a ragged last block, no rotation: every
+    element against the oracle, and the block means' scores against those of the produced Q and K."""
+    n_text, n_image = 130, 33 * 64
+    gen = torch.Generator(device=DEV).manual_seed(H)
+    major = lambda t: t.permute(0, 2, 1, 3).contiguous().permute(0, 2, 1, 3)
+    Qr, Kr, V = [major(torch.randn((B, H, n_text + n_image, D), generator=gen, device=DEV).to(torch.bfloat16)) for _ in range(3)]
+    gain = [0.5 + torch.rand(D, generator=gen, device=DEV) for _ in range(2)]
+    q, k, out = (major(poison_like(V)) for _ in range(3))
+    ctx = binding.Context(B, H, D, n_text, n_image, strides=q.stride()[:3])
+    ctx.rapid3_gated_step_fused(Qr, Kr, V, *gain, None, EPS, q, k, out, [2] * B, [0.5] * B)
+    torch.cuda.synchronize()
+    assert ctx.last_status() == 0
+    check_produced(Qr[0], q[0], gain[0], None, "Q")
+    check_produced(Kr[B - 1], k[B - 1], gain[1], None, "K")
+    assert torch.equal(ctx.workspace(B)[0].clone(), ctx.rapid3_block_scores(q, k))
