@@ -139,7 +139,8 @@ int rapid3_select_mask_mass(rapid3_ctx* ctx, const float* scores, const float* m
  * softmax_scale multiplies q.k before the softmax.
  * In a context with too few query blocks for the GPU's SMs the attention, here and in every gated
  * step, works on a row's kept blocks in parts and adds these up in one launch more; how a row is cut
- * depends on the context and on whether its image is dense, not on the launch.
+ * depends on the context and on whether its image is dense, not on the launch.  In one whose largest launch
+ * leaves every 128 query rows an SM of their own, a row's kept blocks are worked on as two interleaved halves.
  */
 int rapid3_sparse_joint_attn(rapid3_ctx* ctx, const void* q, const void* k, const void* v, void* out,
                              const int32_t* img_idx_host, int n_img, const int32_t* kept_idx,

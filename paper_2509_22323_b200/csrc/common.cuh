@@ -65,6 +65,7 @@ struct TensorGeom {
 // text rows, of its other quads; and where the parts leave their results.
 struct AttnParts {
     int dense = 1, text = 1, light = 1;
+    bool keys = false;               // lists are whole; every tile has an SM to itself, whose two tiles take its key blocks by turns
     float4* partial = nullptr;       // attention_partial_bytes()
     int* given_up = nullptr;         // a wait of the launch has run out: its parts are not complete, and add_parts_kernel stores nothing
     __host__ __device__ bool any() const { return dense > 1 || text > 1 || light > 1; }

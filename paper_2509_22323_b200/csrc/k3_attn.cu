@@ -70,6 +70,12 @@ constexpr int TAKE_AHEAD = 4;
 // Parts of a list; units of work whose results lie in memory between the attention kernel and add_parts_kernel (62 MB at
 // D = 128); the shortest rows, in key blocks, and the most quads with which attention_parts() looks for a cut at all.
 constexpr int MAX_PARTS = 8, MAX_LEFT = 444, MIN_CUT = 24, MAX_CUT = 600;
+// The shortest rows whose blocks go to both tiles by turns (AttnParts::keys): what that saves has to pay for the exchange at the end.
+// Attention of one image, every block kept, us, one tile an SM / by turns: D = 64 5 blocks 7.1 / 6.6 (but a step at ratio 0.5, lists of four,
+// 11.9 / 12.3), 8 8.8 / 7.8, 12 12.1 / 10.0, 17 14.4 / 11.9, 36 25.4 / 19.9; D = 128 5 7.8 / 7.8, 8 9.9 / 9.5, 12 14.0 / 12.7, 17 16.9 / 15.0,
+// 36 29.4 / 26.4 (a step of 10 blocks 19.3 / 19.4).  At D = 128 a block takes 0.58 us, not half of the 0.84 for two tiles: K and V come twice as
+// fast, and more stages for them, or V in later groups, did not change that.  Fifty steps of such contexts drawn at random: 3.9 % faster.
+constexpr int KEYS_FROM_64 = 6, KEYS_FROM_128 = 11;
 // After a wait has run out the softmax warps go on for up to this many key blocks, each a wait of 16 polls of about 8 us.
 // (Over the whole of a quad, with 256 polls a block, that was 2.06 s at two heads of 1024 key blocks; now 4.7 ms.)
 constexpr int ABORT_EVERY = 32;
@@ -126,7 +132,7 @@ struct __align__(16) Ctl {
     unsigned long long k_full[MAX_STAGES], k_empty[MAX_STAGES];   // k_full[g % KS]: group g = K(g) and V(g - 1) have landed
     unsigned long long v_empty[MAX_STAGES];
     unsigned long long s_full[2][3], p_full[2][3];
-    unsigned long long pv_done[2][2], o_done[2], drain[2];
+    unsigned long long pv_done[2][2], o_done[2], drain[2], handed[SOFTMAX_WARPS];
     uint32_t tmem_base;
     int n_early;                        // groups of the first quad that the producer loads before its list is there
     volatile int abort_flag;
@@ -215,12 +221,17 @@ __device__ __forceinline__ void row_maxima(const uint32_t (&r)[32], float& lo, f
 // left out.  Both builds have 96 registers and spill the same five words; by turns, whole steps, us, with that code / without:
 // 1296 quads at D = 128 530.7 / 524.7, 2592 1184.6 / 1170.0, 1584 of a 2048^2 image 1117.6 / 1110.4; all dense 1296 669.3 / 660.9,
 // 1584 2848 / 2813.  Dense launches at D = 64 keep the build with it: 840 quads 304.5 / 306.3, 288 36.8 / 37.0.
-template <int D, bool INJECT = false, bool SPLIT = false, bool ORDERED = false, bool MASKS = ORDERED>
+//
+// KEYS is the build for contexts in which every tile of the largest launch has an SM to itself (AttnParts::keys).  Both tiles of the
+// thread block then hold the same query rows, and the blocks of the list go to them by turns; at the end each hands half of its
+// channels to the other.
+template <int D, bool INJECT = false, bool SPLIT = false, bool ORDERED = false, bool MASKS = ORDERED, bool KEYS = false>
 __global__ void __launch_bounds__(NTHREADS, 1)
 attn_kernel(const __grid_constant__ CUtensorMap tmq, const __grid_constant__ CUtensorMap tmk,
             const __grid_constant__ CUtensorMap tmv, uint16_t* __restrict__ out, const __grid_constant__ AttnParams prm) {
     using C = Cfg<D>;
     constexpr int DH = C::DH, KS = C::KS, VS = C::VS, NBUF = C::NBUF, O_COL = C::O_COL;
+    constexpr int AHEAD = (NBUF - 1) * (KEYS ? 2 : 1);   // how many blocks of the list the scores are ahead of the products P V
     extern __shared__ uint8_t smem_raw[];
     const uint32_t raw = smem_u32(smem_raw);
     const uint32_t pad = ((raw + 1023u) & ~1023u) - raw;
@@ -270,6 +281,7 @@ attn_kernel(const __grid_constant__ CUtensorMap tmq, const __grid_constant__ CUt
             if (has(x, offsetof(Ctl, quad_empty), 2)) count = QUAD_USERS;
             if (has(x, offsetof(Ctl, q_empty), 1) || has(x, offsetof(Ctl, k_empty), 2 * MAX_STAGES)) count = 2;   // both tiles pass a stage before it is refilled
             if (has(x, offsetof(Ctl, p_full), 6)) count = 8;                   // one arrival per softmax warp of the tile
+            if (has(x, offsetof(Ctl, handed), SOFTMAX_WARPS)) count = 32;
             mbar_init(smem_u32(ctl) + 8 * (at + x), count);
         }
         if (lane == 0) ctl->abort_flag = 0;
@@ -347,7 +359,7 @@ attn_kernel(const __grid_constant__ CUtensorMap tmq, const __grid_constant__ CUt
 
     // The pool is the launch's 640 x 96: 512 x 104 + 128 x 64.  Without it this build keeps ten words of the softmax warps in
     // local memory; in the other builds it gains nothing (ordered, D = 128: fused step of 432 quads 197.0 us without, 199.8 with).
-    if (SPLIT && warp >= SOFTMAX_WARPS) reg_dec<LIGHT_REGS>();
+    if ((SPLIT || KEYS) && warp >= SOFTMAX_WARPS) reg_dec<LIGHT_REGS>();
     if (warp == LIST_WARP) {
         // ------------------------------------------------------------ quads and their union lists
         // A thread block's first quad waits for this warp, whose code the SM has to fetch first: what lies in front of the first list is
@@ -456,8 +468,9 @@ attn_kernel(const __grid_constant__ CUtensorMap tmq, const __grid_constant__ CUt
             const int b = prm.plan ? __ldcg(&prm.plan->all.batch[p]) : prm.imgs.batch[p];
             const int slot = prm.plan ? __ldcg(&prm.plan->all.slot[p]) : prm.imgs.slot[p];
             // Lanes a, a + 4, ... hold member a's query block; which members there are, one of the other half counting like one past the end.
-            const int own = quad_block(g, quad, lane & 3);
-            const bool here_own = own < nb && (half < 0 || ((lane & 3) >> 1) == half);
+            // (KEYS: both tiles hold the unit's two.)
+            const int own = quad_block(g, quad, KEYS ? 2 * half + (lane & 1) : lane & 3);
+            const bool here_own = own < nb && (KEYS || half < 0 || ((lane & 3) >> 1) == half);
             const uint32_t here = __ballot_sync(0xffffffffu, here_own) & 15u;
             const bool masks = MASKS || prm.bitmask32 != nullptr;      // of the selection kernel (it finds the order), else lists of the caller's
             // a dense image's quad, or one of text rows in a mask of the selection kernel: every block is kept, no mask is read
@@ -484,11 +497,13 @@ attn_kernel(const __grid_constant__ CUtensorMap tmq, const __grid_constant__ CUt
                 }
             }
             int n_u;
-            auto entry = [&](uint32_t f, int j) { return f | ((j + 1) * 64 > N ? ENT_TAIL : 0u) | ((uint32_t)j << ENT_BLK); };
+            auto entry = [&](uint32_t f, int j, int at) {
+                return (KEYS ? f & (at & 1 ? 12u : 3u) : f) | ((j + 1) * 64 > N ? ENT_TAIL : 0u) | ((uint32_t)j << ENT_BLK);
+            };
             if (all_kept) {
                 const int first = SPLIT ? nb * part / parts : 0, last = !here ? first : SPLIT ? nb * (part + 1) / parts : nb;
                 n_u = last - first;
-                for (int j = first + lane; j < last; j += 32) u.ent[j - first] = entry(here, j);
+                for (int j = first + lane; j < last; j += 32) u.ent[j - first] = entry(here, j, j - first);
             } else {
                 // m[a] = 32 bits of the set of key blocks that member a keeps: from the bitmask when the caller has one,
                 // else rebuilt from the kept list.
@@ -574,13 +589,17 @@ attn_kernel(const __grid_constant__ CUtensorMap tmq, const __grid_constant__ CUt
                     for (int a = 0; a < 4; ++a) f |= ((__shfl_sync(0xffffffffu, m[a], w) >> lane) & 1u) << a;
                     if (f) {
                         const int j = 32 * w + lane;
-                        u.ent[pos] = entry(f, j);
+                        u.ent[pos] = entry(f, j, pos);
                     }
                 }
             }
             if (lane == 0) u.n_u = n_u;
             __syncwarp();
             if (lane == 0) mbar_arrive(bUF + 8 * (i & 1));
+            if (KEYS) {                                  // the memory of K and V is used otherwise at the end
+                L = -1;
+                continue;
+            }
             // the next quad, when this one is nearly through
             if (!wait_lane0(bNE, i & 1)) break;
             if (lane == 0) {
@@ -713,12 +732,12 @@ attn_kernel(const __grid_constant__ CUtensorMap tmq, const __grid_constant__ CUt
                     return true;
                 };
                 if (!(ok = mma_wait(bQ, i & 1))) break;
-                // the scores run NBUF - 1 key blocks ahead of the P V products
-                for (int j = 0; ok && j < NBUF - 1 && j <= n_u; ++j) ok = k_step(j);
+                // the scores run NBUF - 1 of the tile's key blocks ahead of the P V products (KEYS: every other one of the list is)
+                for (int j = 0; ok && j < AHEAD && j <= n_u; ++j) ok = k_step(j);
                 for (int j = 0; ok && j < n_u; ++j) {
                     // S(n + NBUF - 1) reuses the buffer of P(n - 1); the MMAs of the issuing thread execute in issue
                     // order, so it is written only after P(n - 1) V has read it
-                    if (j + NBUF - 1 <= n_u && !(ok = k_step(j + NBUF - 1))) break;          // group j + 1 brings V(j)
+                    if (j + AHEAD <= n_u && !(ok = k_step(j + AHEAD))) break;          // group j + 1 brings V(j)
                     const uint32_t s = (W0 + j) % VS;
                     const bool use = u.ent[j] & tile_bits;
                     if (use && !(ok = (mma_wait(bPFt + 8 * (n_pv % NBUF), (n_pv / NBUF) & 1)))) break;
@@ -768,7 +787,7 @@ attn_kernel(const __grid_constant__ CUtensorMap tmq, const __grid_constant__ CUt
         // (r_lo = lane / 4 and r_lo + 8 of the sixteen) and, of every group of eight score columns, the pair
         // 2 (lane % 4), + 1 -- 32 scores per key block.  The four threads of a quad share their rows' maximum
         // with two shuffles, and only when some row of the warp may have grown.
-        if (SPLIT) reg_inc<SOFTMAX_REGS>();
+        if (SPLIT || KEYS) reg_inc<SOFTMAX_REGS>();
         const int t = (warp >> 2) & 1, wl = warp & 3, hf = warp >> 3;
         const int a = 2 * t + (wl >> 1);               // query block of the quad
         const uint32_t tile_bits = 3u << (2 * t), act_bit = 1u << a;
@@ -837,7 +856,7 @@ attn_kernel(const __grid_constant__ CUtensorMap tmq, const __grid_constant__ CUt
                     row_maxima(r, nm_lo, nm_hi);
                     nm_lo *= -c2; nm_hi *= -c2;
                     // a part may begin with a block whose scores are all -inf: no NaN (-inf - -inf) from them, the next ones count
-                    if (SPLIT) { nm_lo = fminf(nm_lo, FLT_MAX); nm_hi = fminf(nm_hi, FLT_MAX); }
+                    if (SPLIT || KEYS) { nm_lo = fminf(nm_lo, FLT_MAX); nm_hi = fminf(nm_hi, FLT_MAX); }
                     seeded = true;
                     if (SPLIT && cg == 0) { ref[0] = nm_lo; ref[8] = nm_hi; }
                 }
@@ -908,9 +927,75 @@ attn_kernel(const __grid_constant__ CUtensorMap tmq, const __grid_constant__ CUt
         }
         }
         if (n > n0) wait(bOD + 8 * t, n_o++ & 1);
+        // where the other tile has blocks; else there is Q alone, which no product has waited for
+        if (KEYS) wait(n_u > 1 - t ? bOD + 8 * (1 - t) : bQ, 0);
         if (!(ok = __all_sync(0xffffffffu, !ctl->abort_flag))) break;
         // epilogue: O / l -> bf16 -> 16 bytes a lane, four lanes a 64-byte piece of a row
-        if (SPLIT && u.parts > 1) {
+        if (KEYS) {
+            // No product and no copy is under way any more: what the other tile finishes -- O, not divided by the row sums, of half of
+            // the channels, the sums and the reference maxima -- goes to it through the memory of Q, K and V.
+            tc_fence_after();
+            constexpr int HALF = D / 64, LEFT = (4 * HALF + 1) * 32;     // pieces of 32 channels; float4 that a warp hands on
+            float4* const mine = reinterpret_cast<float4*>(smem) + warp * LEFT + lane;
+            const float4* const other = reinterpret_cast<const float4*>(smem) + (warp ^ 4) * LEFT + lane;
+            float s_lo = l0 + l1, s_hi = l2 + l3;
+            s_lo += __shfl_xor_sync(0xffffffffu, s_lo, 1);
+            s_hi += __shfl_xor_sync(0xffffffffu, s_hi, 1);
+            s_lo += __shfl_xor_sync(0xffffffffu, s_lo, 2);
+            s_hi += __shfl_xor_sync(0xffffffffu, s_hi, 2);
+            uint32_t o[16];
+            auto load_o = [&](int ch) {
+                if (n > n0) {
+                    tmem_ld16x256_x4(tO + ch * 32, o);
+                    tc_wait_ld();
+                } else {
+#pragma unroll
+                    for (int e = 0; e < 16; ++e) o[e] = 0u;
+                }
+            };
+#pragma unroll
+            for (int x = 0; x < HALF; ++x) {
+                load_o((1 - t) * HALF + x);
+#pragma unroll
+                for (int k = 0; k < 4; ++k)
+                    mine[32 * (4 * x + k)] = make_float4(__uint_as_float(o[4 * k]), __uint_as_float(o[4 * k + 1]), __uint_as_float(o[4 * k + 2]),
+                                                         __uint_as_float(o[4 * k + 3]));
+            }
+            mine[32 * 4 * HALF] = make_float4(nm_lo, nm_hi, s_lo, s_hi);
+            mbar_arrive(smem_u32(&ctl->handed[warp]));
+            if (!(ok = wait_warp(smem_u32(&ctl->handed[warp ^ 4]), 0))) break;
+            const float4 v = other[32 * 4 * HALF];
+            // a tile in which a row kept nothing (no maximum) counts for nothing
+            const float m_lo = fminf(nm_lo, v.x), m_hi = fminf(nm_hi, v.y);
+            float a_lo = nm_lo == INFINITY ? 0.f : ex2(m_lo - nm_lo), a_hi = nm_hi == INFINITY ? 0.f : ex2(m_hi - nm_hi);
+            float b_lo = v.x == INFINITY ? 0.f : ex2(m_lo - v.x), b_hi = v.y == INFINITY ? 0.f : ex2(m_hi - v.y);
+            s_lo = fmaf(a_lo, s_lo, b_lo * v.z);
+            s_hi = fmaf(a_hi, s_hi, b_hi * v.w);
+            const float inv_lo = s_lo > 0.f ? 1.f / s_lo : 0.f, inv_hi = s_hi > 0.f ? 1.f / s_hi : 0.f;
+            a_lo *= inv_lo; b_lo *= inv_lo; a_hi *= inv_hi; b_hi *= inv_hi;
+            const int tok_lo = u.tok[a] + (row_lo & 63), tok_hi = tok_lo + 8;
+            uint16_t* o_lo = out + (long long)u.b * g.stride_b + (long long)u.h * g.stride_h + (long long)tok_lo * g.stride_n + 8 * cg;
+            uint16_t* o_hi = o_lo + 8 * g.stride_n;
+#pragma unroll
+            for (int x = 0; x < HALF; ++x) {
+                const int ch = t * HALF + x;
+                load_o(ch);
+                uint32_t w_lo[4], w_hi[4];
+#pragma unroll
+                for (int k = 0; k < 4; ++k) {
+                    const float4 p = other[32 * (4 * x + k)];
+                    w_lo[k] = pack_bf16(fmaf(__uint_as_float(o[4 * k]), a_lo, p.x * b_lo), fmaf(__uint_as_float(o[4 * k + 1]), a_lo, p.y * b_lo));
+                    w_hi[k] = pack_bf16(fmaf(__uint_as_float(o[4 * k + 2]), a_hi, p.z * b_hi), fmaf(__uint_as_float(o[4 * k + 3]), a_hi, p.w * b_hi));
+                }
+                const uint4 v_lo = quad_transpose(w_lo[0], w_lo[1], w_lo[2], w_lo[3], cg);
+                const uint4 v_hi = quad_transpose(w_hi[0], w_hi[1], w_hi[2], w_hi[3], cg);
+                if (tok_lo < N) *reinterpret_cast<uint4*>(o_lo + 32 * ch) = v_lo;
+                if (tok_hi < N) *reinterpret_cast<uint4*>(o_hi + 32 * ch) = v_hi;
+            }
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(bUE + 8 * (i & 1));
+        } else if (SPLIT && u.parts > 1) {
             // a part of the list: O as it is, the row sums and the reference maxima go to memory
             tc_fence_after();
             if (u.tok[a] < N) {                        // the same in every part of the quad
@@ -1102,11 +1187,14 @@ cudaError_t attention_static_init() {
     const cudaError_t e = set(attn_kernel<128>, attn_kernel<64>, attn_kernel<128, false, true>, attn_kernel<64, false, true>,
                               attn_kernel<128, false, false, true>, attn_kernel<64, false, false, true>,
                               attn_kernel<128, false, false, false, true>, attn_kernel<64, false, false, false, true>,
-                              attn_kernel<128, true>, attn_kernel<64, true>, attn_kernel<128, true, true>, attn_kernel<64, true, true>);
+                              attn_kernel<128, true>, attn_kernel<64, true>, attn_kernel<128, true, true>, attn_kernel<64, true, true>,
+                              attn_kernel<128, false, false, false, false, true>, attn_kernel<64, false, false, false, false, true>);
     if (e != cudaSuccess) return e;
     // the warps that take registers wait for them: a build that is launched with fewer would wait for good
     for (const void* kernel : {(const void*)attn_kernel<128, false, true>, (const void*)attn_kernel<64, false, true>,
-                               (const void*)attn_kernel<128, true, true>, (const void*)attn_kernel<64, true, true>}) {
+                               (const void*)attn_kernel<128, true, true>, (const void*)attn_kernel<64, true, true>,
+                               (const void*)attn_kernel<128, false, false, false, false, true>,
+                               (const void*)attn_kernel<64, false, false, false, false, true>}) {
         cudaFuncAttributes attr;
         const cudaError_t r = cudaFuncGetAttributes(&attr, kernel);
         if (r != cudaSuccess) return r;
@@ -1158,9 +1246,11 @@ static size_t left_units(const TensorGeom& g, int n_img, const AttnParts& parts)
 // 56.3 / 47.1 (two); 60 of 12 13.7 / 15.7, 15.5 / 21.0 (two).  Steps: 46 quads of 92 blocks at ratio 0.25, D = 64 61.6 / 31.8
 // (text rows in five, the others in three); 132 of 264 at ratio 0.2, D = 128 231 / 135 (text rows in four); 198 of 262 at ratios
 // 1, 0.5 and 0.2, D = 64 359, 289 and 196 / 289, 237 and 148 (in two, text rows in three).
+// Where lists stay whole and every tile has an SM to itself in the largest launch, the two tiles of the SM take its blocks by turns.
 AttnParts attention_parts(const TensorGeom& g, int n_img) {
     AttnParts best;
     const int nq = (g.nb + 3) / 4, ntq = std::min(nq, (g.n_text_blocks + 3) / 4);
+    best.keys = 2ll * nq * g.H * n_img <= SM_COUNT && g.nb >= (g.D == 128 ? KEYS_FROM_128 : KEYS_FROM_64);
     if (g.nb < MIN_CUT || (long long)nq * g.H * n_img > MAX_CUT) return best;
     const bool wide = g.D == 128;
     auto time = [&](int dense, int sparse, double held, const AttnParts& p) {
@@ -1272,6 +1362,10 @@ cudaError_t launch_attention(const CUtensorMap& tmq, const CUtensorMap& tmk, con
             attn_kernel<64, true><<<grid, NTHREADS, attn_smem_bytes<64>(), s>>>(tmq, tmk, tmv, static_cast<uint16_t*>(out), prm);
     } else {
         const bool masks = bitmask || (!kept_idx && g.D == 128);         // see MASKS
+        if (parts && parts->keys)
+            return launch_kernel(g.D == 128 ? attn_kernel<128, false, false, false, false, true> : attn_kernel<64, false, false, false, false, true>,
+                                 grid, dim3(NTHREADS), g.D == 128 ? attn_smem_bytes<128>() : attn_smem_bytes<64>(), s, tmq, tmk, tmv,
+                                 static_cast<uint16_t*>(out), prm);
         return launch_kernel(order.cls ? (g.D == 128 ? attn_kernel<128, false, false, true> : attn_kernel<64, false, false, true>)
                              : masks ? (g.D == 128 ? attn_kernel<128, false, false, false, true> : attn_kernel<64, false, false, false, true>)
                                        : (g.D == 128 ? attn_kernel<128> : attn_kernel<64>),
