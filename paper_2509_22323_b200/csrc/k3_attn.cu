@@ -73,9 +73,9 @@ constexpr int MAX_PARTS = 8, MAX_LEFT = 444, MIN_CUT = 24, MAX_CUT = 600;
 // The shortest rows whose blocks go to both tiles by turns (AttnParts::keys): what that saves has to pay for the exchange at the end.
 // Attention of one image, every block kept, us, one tile an SM / by turns: D = 64 5 blocks 7.1 / 6.6 (but a step at ratio 0.5, lists of four,
 // 11.9 / 12.3), 8 8.8 / 7.8, 12 12.1 / 10.0, 17 14.4 / 11.9, 36 25.4 / 19.9; D = 128 5 7.8 / 7.8, 8 9.9 / 9.5, 12 14.0 / 12.7, 17 16.9 / 15.0,
-// 36 29.4 / 26.4 (a step of 10 blocks 19.3 / 19.4).  At D = 128 a block takes 0.58 us, not half of the 0.84 for two tiles: K and V come twice as
+// 36 29.4 / 26.4 (steps of 6 blocks 15.3 / 15.7, of 8 to 10 1 to 5 % faster).  At D = 128 a block takes 0.58 us, not half of the 0.84 for two tiles: K and V come twice as
 // fast, and more stages for them, or V in later groups, did not change that.  Fifty steps of such contexts drawn at random: 3.9 % faster.
-constexpr int KEYS_FROM_64 = 6, KEYS_FROM_128 = 11;
+constexpr int KEYS_FROM_64 = 6, KEYS_FROM_128 = 8;
 // After a wait has run out the softmax warps go on for up to this many key blocks, each a wait of 16 polls of about 8 us.
 // (Over the whole of a quad, with 256 polls a block, that was 2.06 s at two heads of 1024 key blocks; now 4.7 ms.)
 constexpr int ABORT_EVERY = 32;

@@ -13,7 +13,7 @@ SHAPES = [  # D, text and image tokens, heads, images
     (64, 0, 5 * 64 + 1, 1, 1),       # the shortest rows, one token in the last block
     (64, 77, 13 * 64, 3, 2),         # a quad of three rows, 61 tokens in the last block
     (64, 130, 22 * 64 + 5, 12, 1),   # 72 quads
-    (128, 64, 10 * 64, 2, 3),        # the shortest rows
+    (128, 64, 7 * 64, 2, 3),         # the shortest rows
     (128, 200, 19 * 64 + 1, 6, 2),   # 72 quads, one token in the last block
 ]
 
