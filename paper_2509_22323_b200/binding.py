@@ -6,6 +6,7 @@ missing or a call fails, an exception is raised.
 """
 from __future__ import annotations
 
+import array
 import ctypes
 import os
 from typing import Optional, Sequence
@@ -102,7 +103,12 @@ def _i32(xs: Optional[Sequence[int]]):
 
 
 def _f32(xs: Sequence[float]):
-    return (ctypes.c_float * len(xs))(*[float(x) for x in xs])
+    # number by number through ctypes, 192 ratios took 27 us of a call (7.8 so)
+    try:
+        a = array.array("f", xs)
+    except TypeError:                              # what only float() takes
+        a = array.array("f", [float(x) for x in xs])
+    return (ctypes.c_float * len(a)).from_buffer(a)
 
 
 def _stream() -> int:
@@ -221,7 +227,7 @@ class Context:
                                 softmax_scale: Optional[float] = None):
         """keep_ratio: [B][H], one ratio per image and head."""
         scale = softmax_scale if softmax_scale is not None else self.D ** -0.5
-        flat = [float(r) for row in keep_ratio for r in row]
+        flat = [r for row in keep_ratio for r in row]
         assert len(flat) == len(actions) * self.H
         _check(self.lib.rapid3_gated_step_heads(self.handle, _ptr(q), _ptr(k), _ptr(v), _ptr(out), _i32(actions),
                                                 _f32(flat), len(actions), scale, _stream()),
