@@ -160,7 +160,7 @@ bool apart(const rapid3_ctx* c, const void* q, const void* out) {
 // Whether a step over n_img attending images hands its last quads out by their length, and where that is kept.
 QuadOrder step_order(const rapid3_ctx* c, const TensorGeom& g, int n_img) {
     const int quads = attention_units(g, AttnParts(), n_img, 0);
-    return quads > ORDER_FROM && quads <= ORDER_TO ? c->order : QuadOrder();      // without pointers where the context has none
+    return quads > ORDER_FROM ? c->order : QuadOrder();      // without pointers where the context has none
 }
 
 // SM time, in us, of a step's attention that needs no mask: quads of dense images, of text rows alone in sparse ones.

@@ -97,13 +97,13 @@ __host__ __device__ inline int quad_block(const TensorGeom& g, int quad, int a) 
 // class by class.  In the order of images and heads the last quads of a launch may be long ones, for which the other SMs
 // wait; the quads before them stay in that order, in which the thread blocks at work share the K and V of a few heads.  So do those that
 // an SM begins with: all of them start at once, and without the order they start 1 us sooner (40 steps of 297 to 1000 quads 0.4 %).
-// For launches of more than ORDER_FROM quads up to ORDER_TO: whole steps of 864 quads, us, two images with a ratio for every
-// head 197.5 -> 190.2, by cumulative mass 358.2 -> 346.3, a dense one and one at 0.5 (D = 64) 262.5 -> 257.3; one image of 432
-// quads at 0.5 from raw projections 190.5 -> 182.9; two images of 288 quads at D = 64 39.6 -> 38.6.  Steps drawn at random, in the mean and the
-// worst: 297 to 1000 quads -1.8 % and +3.4 % (316), 201 to 296 -2.1 % and +2.5 % (60).  Above them the idle SMs at the end cost less than the
-// heads' first reads at once and the longer selection do (1632 quads at D = 64 303.5 -> 313.7); below, few SMs have a second quad: 149 to
-// 200 go both ways (168 33.3 -> 31.4 and 33.7 -> 34.3, 192 66.9 -> 63.6 and 43.0 -> 43.8).
-constexpr int ORDER_CLASSES = 32, ORDER_LAST = 448, ORDER_FROM = 200, ORDER_TO = 1000;
+// One quad for nearly every SM is enough, its last: of 448, 288, 192, 160, 144, 128, 112, 96 and 64 quads 128 were the best in launches above and
+// below 1000 quads (36 and 40 steps drawn at random: -1.6 and -0.6 % against 448, which loses what the quads of a head share in the L2 and is
+// longer to search).  For launches of more than ORDER_FROM quads, us against quads in order: two images of 288 quads at D = 64 39.6 -> 38.5,
+// 864 quads with a ratio for every head 197.5 -> 183, by cumulative mass 358.2 -> 341, one image of 432 at 0.5 from raw projections 8 less, 1584
+// of one 16896-token image 1124 -> 1115; steps drawn at random in the mean and the worst: 149 to 200 quads -1.4 % and +0.7 % (30), more -0.7 %
+// and +1.7 % (30) against 448 from 201 to 1000 quads, which was 1.8 % better than quads in order.  With a quad an SM nothing is handed out.
+constexpr int ORDER_CLASSES = 32, ORDER_LAST = 128, ORDER_FROM = SM_COUNT;
 // Of `light` quads without text rows, behind `heavy` others, how many stay where they are.
 __host__ __device__ inline int order_after(int light, int heavy) {
     const int begun = heavy < SM_COUNT ? SM_COUNT - heavy : 0, first = light - ORDER_LAST;
@@ -111,7 +111,7 @@ __host__ __device__ inline int order_after(int light, int heavy) {
 }
 struct QuadOrder {
     int n_dense = 0;                 // dense images of the launch, where the host knows
-    uint8_t* cls = nullptr;          // [ORDER_LAST] class of the quad at that place from the first of the last on; 16-byte aligned
+    uint8_t* cls = nullptr;          // [ORDER_LAST] class of the quad at that place from the first of the last on; 4-byte aligned
 };
 
 // Programmatic dependent launch: every kernel of a step is launched so that it may start while the kernel before it in the stream

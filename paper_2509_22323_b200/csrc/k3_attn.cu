@@ -165,14 +165,10 @@ __device__ __forceinline__ uint4 quad_transpose(uint32_t w0, uint32_t w1, uint32
     return b1 ? make_uint4(r0, r1, q0, q1) : make_uint4(p0, p1, r0, r1);
 }
 
-// Place of the `rest`-th quad in the order of the classes; a lane holds those of quads 16 lane .. 16 lane + 15, 0xff: no quad.
-__device__ __forceinline__ int order_find(const uint32_t (&cls)[4], int rest, int lane) {
-    auto below = [&](uint32_t c) {                       // of the lane's quads, those of a class below c
-        int n = 0;
-#pragma unroll
-        for (int x = 0; x < 4; ++x) n += __popc(__vcmpltu4(cls[x], c * 0x01010101u)) >> 3;
-        return n;
-    };
+// Place of the `rest`-th quad in the order of the classes; a lane holds those of quads 4 lane .. 4 lane + 3, 0xff: no quad.
+__device__ __forceinline__ int order_find(uint32_t cls, int rest, int lane) {
+    static_assert(ORDER_LAST == 4 * 32, "a lane holds four classes");
+    auto below = [&](uint32_t c) { return __popc(__vcmpltu4(cls, c * 0x01010101u)) >> 3; };   // of the lane's quads, those of a class below c
     uint32_t c = 0u;                                     // the quad's class: the last with no more than `rest` quads below it
 #pragma unroll
     for (uint32_t bit = ORDER_CLASSES / 2; bit > 0; bit >>= 1)
@@ -186,8 +182,8 @@ __device__ __forceinline__ int order_find(const uint32_t (&cls)[4], int rest, in
     }
     int skip = rest - (int)__reduce_add_sync(0xffffffffu, (uint32_t)lower) - (before - own), at = -1;
 #pragma unroll
-    for (int x = 0; x < 16; ++x)
-        if (((cls[x / 4] >> (8 * (x % 4))) & 0xffu) == c && skip-- == 0) at = 16 * lane + x;
+    for (int x = 0; x < 4; ++x)
+        if (((cls >> (8 * x)) & 0xffu) == c && skip-- == 0) at = 4 * lane + x;
     return (int)__reduce_max_sync(0xffffffffu, at);      // the other lanes have -1
 }
 
@@ -373,7 +369,7 @@ attn_kernel(const __grid_constant__ CUtensorMap tmq, const __grid_constant__ CUt
         };
         int L = blockIdx.x;
         bool waited = false;                             // for the selection kernel, see below
-        uint32_t classes[4];                             // of sixteen quads in the order, once `have_classes`
+        uint32_t classes = 0;                            // of four quads in the order, once `have_classes`
         bool have_classes = false;
         for (uint32_t i = 0;; ++i) {
             Quad& u = ctl->quad[i & 1];
@@ -444,16 +440,13 @@ attn_kernel(const __grid_constant__ CUtensorMap tmq, const __grid_constant__ CUt
                         by = prm.div_light;
                         const int in_order = order_after(ns * g.H * n, heavy_dense + heavy_sparse), rest = L - in_order;
                         if (ORDERED && rest >= 0) {
-                            // the quad at place `rest` of the order that the selection kernel has found: of sixteen classes a lane
+                            // the quad at place `rest` of the order that the selection kernel has found: of four classes a lane
                             if (!have_classes) {
                                 if (!waited) grid_dependency_wait();
                                 waited = have_classes = true;
-                                const uint4 v = 16 * lane < ORDER_LAST ? __ldcg(reinterpret_cast<const uint4*>(prm.order.cls) + lane) : make_uint4(0, 0, 0, 0);
-                                classes[0] = v.x; classes[1] = v.y; classes[2] = v.z; classes[3] = v.w;
-                                const int places = ns * g.H * n - in_order;      // quads in the order; the bytes behind them count for nothing
-#pragma unroll
-                                for (int x = 0; x < 16; ++x)
-                                    if (16 * lane + x >= places) classes[x / 4] |= 0xffu << (8 * (x % 4));
+                                classes = __ldcg(reinterpret_cast<const uint32_t*>(prm.order.cls) + lane);
+                                const int left = ns * g.H * n - in_order - 4 * lane;     // of the lane's, the bytes behind those count for nothing
+                                if (left < 4) classes |= left > 0 ? 0xffffffffu << (8 * left) : 0xffffffffu;
                             }
                             L = in_order + order_find(classes, rest, lane);
                         }
