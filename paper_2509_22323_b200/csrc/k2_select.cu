@@ -121,64 +121,49 @@ cudaError_t launch_select_mask_heads(const float* scores, const TensorGeom& g, c
 // entry point does on the CPU, for callers whose sampled actions never leave the GPU.
 namespace {
 
-// One thread decides; the loads, which would cost it a round trip each, and the stores are the whole block's.
+// A thread an image: it counts the images in front of its own in both lists.  Bound by the round trip of the loads.
 __global__ void __launch_bounds__(RAPID3_MAX_IMG) plan_kernel(const int32_t* action, const float* ratio, int B, int n_free_img,
                                                               DevPlan* __restrict__ plan, int* __restrict__ status) {
-    __shared__ DevPlan out;
-    __shared__ int act[RAPID3_MAX_IMG];
-    __shared__ float rat[RAPID3_MAX_IMG], ratio_of[RAPID3_MAX_IMG];
-    constexpr int WORDS = sizeof(DevPlan) / sizeof(int);
-    static_assert(sizeof(DevPlan) % sizeof(int) == 0, "copied word by word");
+    __shared__ float of[RAPID3_MAX_IMG];              // an attending image's ratio, 0 for the others
+    const int b = threadIdx.x;
     grid_dependency_wait();                           // first kernel of a call
     grid_dependency_launch();
-    for (int x = threadIdx.x; x < WORDS; x += RAPID3_MAX_IMG) reinterpret_cast<int*>(&out)[x] = 0;
-    if (threadIdx.x < B) {
-        act[threadIdx.x] = __ldcg(action + threadIdx.x);
-        rat[threadIdx.x] = __ldcg(ratio + threadIdx.x);
+    float r = 0.f;
+    if (b < B) {
+        const int a = __ldcg(action + b);
+        const float want = __ldcg(ratio + b);
+        const bool known = a == RAPID3_ACT_SKIP || a == RAPID3_ACT_REUSE || a == RAPID3_ACT_ATTEND;
+        const bool valid = want > 0.f && want <= 1.f;
+        // an unknown action is treated as a skip, an image with a ratio outside (0, 1] is not processed
+        if (!known || (a == RAPID3_ACT_ATTEND && !valid)) atomicExch(status, RAPID3_ERR_INVALID_ARG);
+        if (a == RAPID3_ACT_ATTEND && valid) r = want;
     }
+    of[b] = r;
     __syncthreads();
-    if (threadIdx.x == 0) {
-        ImgList& sp = out.sparse;
-        ImgList& al = out.all;
-        int n_dense = 0;
-        for (int b = 0; b < B; ++b) {
-            const int a = act[b];
-            if (a != RAPID3_ACT_SKIP && a != RAPID3_ACT_REUSE && a != RAPID3_ACT_ATTEND) {
-                atomicExch(status, RAPID3_ERR_INVALID_ARG);   // unknown action: treated as a skip
-                continue;
-            }
-            if (a != RAPID3_ACT_ATTEND) continue;
-            const float r = rat[b];
-            if (!(r > 0.f) || !(r <= 1.f)) {
-                atomicExch(status, RAPID3_ERR_INVALID_ARG);   // ratio outside (0, 1]: image not processed
-                continue;
-            }
-            int slot = -1;
-            if (r < 1.f) {
-                slot = sp.n++;
-                sp.batch[slot] = b;
-                sp.slot[slot] = slot;
-                double x = ceil((double)r * (double)n_free_img - 1e-6);
-                x = x < 0.0 ? 0.0 : (x > (double)n_free_img ? (double)n_free_img : x);
-                sp.k_free[slot] = (int)x;
-            } else {
-                ++n_dense;
-            }
-            int pos = al.n++;
-            while (pos > 0 && ratio_of[pos - 1] < r) {        // insertion sort, descending ratio, stable
-                al.batch[pos] = al.batch[pos - 1];
-                al.slot[pos] = al.slot[pos - 1];
-                ratio_of[pos] = ratio_of[pos - 1];
-                --pos;
-            }
-            al.batch[pos] = b;
-            al.slot[pos] = slot;
-            ratio_of[pos] = r;
+    int n_all = 0, n_sparse = 0, pos = 0, slot = 0;   // sparse images in batch order; all by descending ratio, equal ones in batch order
+    for (int o = 0; o < B; ++o) {
+        const float x = of[o];
+        const bool sparse = x > 0.f && x < 1.f;
+        n_all += x > 0.f;
+        n_sparse += sparse;
+        slot += sparse && o < b;
+        pos += x > r || (x == r && o < b);
+    }
+    if (r > 0.f) {
+        if (r < 1.f) {
+            const double x = ceil((double)r * (double)n_free_img - 1e-6);
+            plan->sparse.batch[slot] = b;
+            plan->sparse.slot[slot] = slot;
+            plan->sparse.k_free[slot] = (int)(x < 0.0 ? 0.0 : (x > (double)n_free_img ? (double)n_free_img : x));
         }
-        out.n_dense = n_dense;
+        plan->all.batch[pos] = b;
+        plan->all.slot[pos] = r < 1.f ? slot : -1;
     }
-    __syncthreads();
-    for (int x = threadIdx.x; x < WORDS; x += RAPID3_MAX_IMG) reinterpret_cast<int*>(plan)[x] = reinterpret_cast<const int*>(&out)[x];
+    if (b == 0) {
+        plan->sparse.n = n_sparse;
+        plan->all.n = n_all;
+        plan->n_dense = n_all - n_sparse;
+    }
 }
 
 }  // namespace

@@ -110,3 +110,26 @@ def test_device_actions_change_between_graph_replays():
                 parity.compare_outputs(out[b], ref[b]["out"], f"graph replay {acts} img {b}")
             else:
                 assert (out[b].view(torch.int16) == np.int16(POISON)).all()
+
+
+@pytest.mark.parametrize("B", [1, 31, 33, 64])
+def test_plans_of_many_images(B):
+    """Equal ratios, dense and sparse images in any order, in one and in two warps of images: the step with decisions on the host, and the
+    images' masks where it puts them."""
+    H, D, n_text, n_image = 2, 64, 64, 6 * 64 - 1
+    gen = torch.Generator().manual_seed(B)
+    q, k, v = (torch.randn((B, H, n_text + n_image, D), generator=gen).to(torch.bfloat16).to(DEV) for _ in range(3))
+    host_ctx, dev_ctx = (binding.Context(B, H, D, n_text, n_image) for _ in range(2))
+    for _ in range(4):
+        acts = torch.randint(0, 3, (B,), generator=gen, dtype=torch.int32)
+        acts[int(torch.randint(0, B, (1,), generator=gen))] = 2
+        ratios = torch.tensor([1.0, 0.3, 0.6, 0.3])[torch.randint(0, 4, (B,), generator=gen)]
+        want, got = torch.full_like(q, float("nan")), torch.full_like(q, float("nan"))
+        host_ctx.rapid3_gated_step(q, k, v, want, acts.tolist(), ratios.tolist())
+        dev_ctx.rapid3_gated_step_device(q, k, v, got, acts.to(DEV), ratios.to(DEV))
+        torch.cuda.synchronize()
+        assert host_ctx.last_status() == 0 and dev_ctx.last_status() == 0
+        assert torch.equal(want.view(torch.int16), got.view(torch.int16))
+        n_sparse = int(((acts == 2) & (ratios < 1.0)).sum())
+        for a, b in zip(host_ctx.workspace(n_sparse), dev_ctx.workspace(n_sparse)) if n_sparse else ():
+            assert torch.equal(a, b)
