@@ -154,7 +154,8 @@ int rapid3_sparse_joint_attn(rapid3_ctx* ctx, const void* q, const void* k, cons
  * Scores, masks and kept lists of the sparse images live in the context's workspace
  * (see rapid3_workspace), compacted in ascending batch order of the sparse images.
  * With a sparse image the call launches pool, scores, selection and attention, or, where there are many
- * heads and enough attention for all SMs, one kernel for the whole scoring pass and the attention beside it.
+ * heads and enough attention for all SMs, one kernel for the whole scoring pass and the attention beside it;
+ * with 75 to 221 quads of query blocks of up to 128 in the attending images scores and selection are one kernel.
  * The call only launches kernels (the tensor maps of a set of base pointers are encoded on the host at
  * their first use and cached), so after one plain call with the same tensors it can be captured
  * into a CUDA graph and replayed on buffers refilled in place; the actions and ratios are then
@@ -184,7 +185,7 @@ int rapid3_gated_step_heads(rapid3_ctx* ctx, const void* q, const void* k, const
  * top-k selection: mass_share_host[b] in (0, 1] is the share of attending image b (ignored for the
  * others); a share of exactly 1 makes the image dense (no scoring); mass_scale as in
  * rapid3_select_mask_mass.  Five launches with a sparse image (pool, scores, counts, selection,
- * attention), or two (see rapid3_gated_step).  Everything else as there.
+ * attention), or three or two (see rapid3_gated_step).  Everything else as there.
  */
 int rapid3_gated_step_mass(rapid3_ctx* ctx, const void* q, const void* k, const void* v, void* out,
                            const int32_t* action_host, const float* mass_share_host, float mass_scale, int B,
@@ -218,7 +219,7 @@ int rapid3_gated_step_fused(rapid3_ctx* ctx, const void* q_raw, const void* k_ra
  * actions on the device; reading them back would cost a host synchronisation per step and layer):
  * action_dev [B] int32 and keep_ratio_dev [B] float are DEVICE arrays, read by the kernels when
  * they run on `stream`, not at call time.  A kernel of one thread block builds the image lists, then pool,
- * scores, selection and attention are launched with grids sized for all B images; thread blocks
+ * scores, selection and attention (scores and selection in one as there, B images counting) are launched with grids sized for all B images; thread blocks
  * of images that do not attend return at once.  Results (output, workspace contents) are those of
  * rapid3_gated_step with the same actions.  An action outside {SKIP, REUSE, ATTEND} or a ratio
  * outside (0, 1] cannot be rejected at call time: that image is not processed and the device status
@@ -273,7 +274,8 @@ int64_t rapid3_launch_count(rapid3_ctx* ctx);
  * microseconds of stream time, which matters beside the short scoring kernels); 0 switches it off.  rapid3_profile_read waits for the recorded events, returns the summed device
  * time in milliseconds and the launch count per kernel kind
  * (0 block pool, 1 block scores, 2 mask select, 3 attention) and clears the record.  Where one kernel does
- * the whole scoring pass it counts as kind 0, or behind the producer of Q and K as kind 1.  An event
+ * the whole scoring pass it counts as kind 0, or behind the producer of Q and K as kind 1, as does one for scores and
+ * selection.  An event
  * pair also keeps the attention kernel from starting beside that pass.
  */
 int rapid3_profile(rapid3_ctx* ctx, int enable);

@@ -491,11 +491,17 @@ static int gated_step_impl(rapid3_ctx* c, const void* q, const void* k, const vo
             if (launch_block_pool(q, k, g, sparse, c->pooled, st) != cudaSuccess) return RAPID3_ERR_CUDA;
             c->launches += 1;
         }
-        {
+        const bool rows = scoring_rows(g, all.n);
+        if (rows) {
+            ProfScope ps(c, PROF_SCORES, st);
+            if (launch_rows(g, sparse, c->pooled, c->scores, c->bitmask, c->kept_idx, c->kept_cnt, per_head ? &hk : nullptr,
+                            mass_scale ? &share : nullptr, mass_scale ? *mass_scale : 0.f, st, order) != cudaSuccess)
+                return RAPID3_ERR_CUDA;
+        } else {
             ProfScope ps(c, PROF_SCORES, st);
             if (launch_block_scores(c->pooled, g, sparse.n, c->scores, st) != cudaSuccess) return RAPID3_ERR_CUDA;
         }
-        {
+        if (!rows) {
             ProfScope ps(c, PROF_SELECT, st);
             const cudaError_t e =
                 mass_scale ? launch_select_mask_mass(c->scores, g, sparse, share, *mass_scale, c->row_keep, c->bitmask,
@@ -504,7 +510,7 @@ static int gated_step_impl(rapid3_ctx* c, const void* q, const void* k, const vo
                            : launch_select_mask(c->scores, g, sparse, c->bitmask, c->kept_idx, c->kept_cnt, st, nullptr, 0, order);
             if (e != cudaSuccess) return RAPID3_ERR_CUDA;
         }
-        c->launches += mass_scale ? 3 : 2;
+        c->launches += rows ? 1 : mass_scale ? 3 : 2;
     }
     return attn_launch(c, g, q, k, v, out, all, sparse.n ? c->kept_idx : nullptr, sparse.n ? c->kept_cnt : nullptr,
                        sparse.n ? c->bitmask : nullptr, softmax_scale, st, nullptr, 0, sparse.n > 0, order);
@@ -570,16 +576,22 @@ int rapid3_gated_step_device(rapid3_ctx* c, const void* q, const void* k, const 
         ProfScope ps(c, PROF_POOL, st);
         if (launch_block_pool(q, k, c->g, none, c->pooled, st, c->plan, B) != cudaSuccess) return RAPID3_ERR_CUDA;
     }
-    {
+    const bool rows = scoring_rows(c->g, B);
+    if (rows) {
+        ProfScope ps(c, PROF_SCORES, st);
+        if (launch_rows(c->g, none, c->pooled, c->scores, c->bitmask, c->kept_idx, c->kept_cnt, nullptr, nullptr, 0.f, st, order, c->plan, B) !=
+            cudaSuccess)
+            return RAPID3_ERR_CUDA;
+    } else {
         ProfScope ps(c, PROF_SCORES, st);
         if (launch_block_scores(c->pooled, c->g, B, c->scores, st, c->plan) != cudaSuccess) return RAPID3_ERR_CUDA;
     }
-    {
+    if (!rows) {
         ProfScope ps(c, PROF_SELECT, st);
         if (launch_select_mask(c->scores, c->g, none, c->bitmask, c->kept_idx, c->kept_cnt, st, c->plan, B, order) != cudaSuccess)
             return RAPID3_ERR_CUDA;
     }
-    c->launches += 4;
+    c->launches += rows ? 3 : 4;
     return attn_launch(c, c->g, q, k, v, out, none, c->kept_idx, c->kept_cnt, c->bitmask, softmax_scale, st, c->plan, B, true, order);
 }
 

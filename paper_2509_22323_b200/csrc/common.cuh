@@ -200,6 +200,12 @@ cudaError_t launch_scoring(const void* q, const void* k, const TensorGeom& g, co
 // The cluster size for that many (image, head) pairs of a step with `images` attending, beside heavy_us of SM time of attention
 // that needs no mask; 0: not this way.
 int scoring_cluster(const TensorGeom& g, int images, int pairs, bool pool, bool mass, double heavy_us);
+// Scores and selection in one launch, from means that are there; whether it takes the place of the two kernels in a step with `images`
+// attending.
+cudaError_t launch_rows(const TensorGeom& g, const ImgList& imgs, double* pooled, float* scores, uint64_t* bitmask, int32_t* kept_idx,
+                        int32_t* kept_cnt, const HeadKeep* heads, const MassShare* share, float mass_scale, cudaStream_t s,
+                        const QuadOrder& order = QuadOrder(), const DevPlan* plan = nullptr, int n_cap = 0);
+bool scoring_rows(const TensorGeom& g, int images);
 // K5: Q/K producer (RMS norm + gain + rotary embedding -> bf16) that also writes the block means of
 // the images with a workspace slot.  pooled is [2][n_sparse][H][nb][D].
 struct PrepArgs {

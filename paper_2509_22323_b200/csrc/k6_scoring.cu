@@ -14,6 +14,7 @@
 // three steps.
 #include <algorithm>
 
+#include "ptx.cuh"
 #include "scoring.cuh"
 
 using namespace scoring;
@@ -45,6 +46,8 @@ struct ScoreArgs {
     int cluster;                   // thread blocks of a cluster
     int rows;                      // of S that are in shared memory at a time
     bool pool;                     // false: the means are there
+    int n_cap;                     // images that the means have room for
+    const DevPlan* plan;           // rows_kernel: the images from device memory
 };
 
 template <int D, int IPL>
@@ -166,6 +169,96 @@ __global__ void __launch_bounds__(WARPS * 32, 1) scoring_kernel(const __grid_con
     }
 }
 
+// Scores and selection from means that are there, for launches of few quads, where a kernel of its own for each is mostly a launch and a round
+// trip: a thread block has the rows of two quads of a pair, all key blocks.  The rows' means come to shared memory; those of K go straight
+// from the L2 to the fragments of the one warp that needs them (a warp has eight key blocks; the four lanes of a row take 32 bytes), all loads
+// of a fragment at once.  The products run in the order of scores_kernel, the rows of S stay in shared memory for the selection, a row a warp.
+// Bound by that chain (10 us of 20 to 30 before, by pooling, scores and selection): whole steps, us, scores and selection apart / in one: 90
+// quads by cumulative mass 28.5 / 25.9, 96 of 9 blocks 25.1 / 23.1, 160 of 19 36.4 / 34.2, 192 of 21 at D = 128 48.9 / 46.0; 26 drawn at random
+// of 75 to 148 quads 4.0 % faster in the mean, 26 of 149 to 221 3.0 %.
+constexpr int ROWS = 8;
+template <int D, int IPL, int ROW_WARPS, typename HK>
+__global__ void __launch_bounds__(ROW_WARPS * 32) rows_kernel(const __grid_constant__ ScoreArgs a, const __grid_constant__ HK hk) {
+    constexpr int LDS = D + 4, LDN = 32 * IPL + 4;
+    __shared__ __align__(16) double sq[ROWS * LDS];
+    __shared__ float ss[ROWS * LDN];
+    __shared__ uint32_t kept[ROWS][IPL];
+    const TensorGeom& g = a.g;
+    const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
+    const int nb = g.nb, nq = (nb + 3) >> 2, H = g.H, q0 = blockIdx.x * (ROWS / 4);
+    const int ph = blockIdx.y, p = ph / H;
+    grid_dependency_wait();
+    grid_dependency_launch();
+    if (a.plan && p >= __ldcg(&a.plan->sparse.n)) return;
+    auto row_block = [&](int r) { return q0 + (r >> 2) < nq ? quad_block(g, q0 + (r >> 2), r & 3) : nb; };
+    const double* mean_q = a.pooled + (long long)ph * nb * D;
+    const double* mean_k = a.pooled + ((long long)a.n_cap * H + ph) * nb * D;
+#pragma unroll
+    for (int e = threadIdx.x; e < ROWS * (D / 2); e += ROW_WARPS * 32) {
+        const int r = e / (D / 2), c = 2 * (e % (D / 2)), i = row_block(r);
+        copy16_async(reinterpret_cast<double*>(sq) + r * LDS + c, i < nb ? mean_q + (long long)i * D + c : a.pooled, i < nb);
+    }
+    asm volatile("cp.async.commit_group;" ::: "memory");
+    const int gr = lane >> 2, c4 = lane & 3;
+    const double* aq = sq + gr * LDS + c4;
+    bool there = false;                                  // the rows' means
+    for (int cj = 8 * warp; cj < nb; cj += 8 * ROW_WARPS) {
+        const double* bk = mean_k + (long long)min(cj + gr, nb - 1) * D + c4;      // key blocks past the end: any, nothing reads their scores
+        double acc[2] = {0.0, 0.0};
+        double b[D / 4];
+#pragma unroll
+        for (int x = 0; x < D / 4; ++x) b[x] = __ldcg(bk + 4 * x);
+        if (!there) {
+            asm volatile("cp.async.wait_group 0;" ::: "memory");
+            ptx::bar_sync(1, ROW_WARPS * 32);
+            there = true;
+        }
+#pragma unroll
+        for (int x = 0; x < D / 4; ++x) dmma_8x8x4(acc[0], acc[1], aq[4 * x], b[x]);
+        *reinterpret_cast<float2*>(ss + gr * LDN + cj + 2 * c4) = make_float2((float)acc[0], (float)acc[1]);
+    }
+    if (!there) {                                        // a warp without key blocks
+        asm volatile("cp.async.wait_group 0;" ::: "memory");
+        ptx::bar_sync(1, ROW_WARPS * 32);
+    }
+    __syncthreads();
+    if (warp < ROWS) {
+        const int r = warp, i = row_block(r);
+        const float* src = ss + r * LDN;
+        const long long row = (long long)ph * nb + i;
+        if (i < nb) {
+            for (int j = lane; j < nb; j += 32) a.scores[row * nb + j] = src[j];
+            auto score = [&](int j) { return src[j]; };
+            int k;
+            if constexpr (HK::mode == MassRule::mode) k = mass_row<IPL>(score, i, nb, g.n_text_blocks, hk.share.tau[p], hk.scale, lane);
+            else if constexpr (HK::mode == HeadKeep::mode) k = hk.k[ph];
+            else k = a.plan ? __ldcg(&a.plan->sparse.k_free[p]) : a.imgs.k_free[p];
+            select_row<IPL>(score, i, nb, g.n_text_blocks, k, lane, a.bitmask32 + row * a.words32, a.words32, a.kept_idx + row * nb,
+                            a.kept_cnt + row, [&](int x, uint32_t bits) { kept[r][x] = bits; });
+        } else if (lane < IPL) {
+            kept[r][lane] = 0u;
+        }
+    }
+    if (!a.order.cls) return;
+    __syncthreads();
+    if (warp < ROWS / 4 && q0 + warp < nq) {
+        uint32_t m[4];
+#pragma unroll
+        for (int b = 0; b < 4; ++b) m[b] = 32 * lane < nb ? kept[4 * warp + b][lane] : 0u;
+        const int n_sparse = a.plan ? __ldcg(&a.plan->sparse.n) : a.imgs.n, place = a.plan ? plan_place(a.plan, p, lane) : a.imgs.slot[p];
+        order_quad(a.order, g, a.plan ? __ldcg(&a.plan->n_dense) : a.order.n_dense, n_sparse, place, ph % H, q0 + warp, m, lane);
+    }
+}
+
+template <typename HK>
+cudaError_t launch_rows_of(const ScoreArgs& a, const HK& hk, cudaStream_t s) {
+    const dim3 grid(((a.g.nb + 3) / 4 + ROWS / 4 - 1) / (ROWS / 4), a.n_cap * a.g.H);
+    const auto go = [&](auto kernel, int warps) { return launch_kernel(kernel, grid, dim3(warps * 32), 0, s, a, hk); };
+    if (a.g.nb <= 64) return go(a.g.D == 128 ? rows_kernel<128, 2, 8, HK> : rows_kernel<64, 2, 8, HK>, 8);
+    if (a.g.nb <= 96) return go(a.g.D == 128 ? rows_kernel<128, 3, 12, HK> : rows_kernel<64, 3, 12, HK>, 12);
+    return go(a.g.D == 128 ? rows_kernel<128, 4, 16, HK> : rows_kernel<64, 4, 16, HK>, 16);
+}
+
 template <int D, typename HK, typename F>
 cudaError_t with_kernel(int nb, F&& f) {
     if (nb <= 96) return f(scoring_kernel<D, 3, HK>, row_bytes<D, 3>(), ring_bytes<D>());
@@ -240,9 +333,8 @@ int scoring_cluster(const TensorGeom& g, int images, int pairs, bool pool, bool 
     return best;
 }
 
-cudaError_t launch_scoring(const void* q, const void* k, const TensorGeom& g, const ImgList& imgs, double* pooled, float* scores,
-                           uint64_t* bitmask, int32_t* kept_idx, int32_t* kept_cnt, int cluster, bool pool, const HeadKeep* heads,
-                           const MassShare* share, float mass_scale, cudaStream_t s, const QuadOrder& order) {
+static ScoreArgs score_args(const void* q, const void* k, const TensorGeom& g, const ImgList& imgs, double* pooled, float* scores, uint64_t* bitmask,
+                            int32_t* kept_idx, int32_t* kept_cnt, const QuadOrder& order) {
     ScoreArgs a;
     a.q = static_cast<const uint16_t*>(q);
     a.k = static_cast<const uint16_t*>(k);
@@ -255,15 +347,47 @@ cudaError_t launch_scoring(const void* q, const void* k, const TensorGeom& g, co
     a.kept_cnt = kept_cnt;
     a.words32 = 2 * ((g.nb + 63) / 64);
     a.order = order;
-    a.cluster = cluster;
-    a.rows = 0;
-    a.pool = pool;
-    const int pairs = imgs.n * g.H;
+    a.cluster = a.rows = 0;
+    a.pool = false;
+    a.n_cap = imgs.n;
+    a.plan = nullptr;
+    return a;
+}
+
+// Calls f with what says how a row's count is found.
+template <typename F>
+static cudaError_t with_rule(const HeadKeep* heads, const MassShare* share, float mass_scale, F&& f) {
     if (share) {
         MassRule m;
         m.share = *share;
         m.scale = mass_scale;
-        return launch(a, m, pairs, s);
+        return f(m);
     }
-    return heads ? launch(a, *heads, pairs, s) : launch(a, NoHeadKeep(), pairs, s);
+    return heads ? f(*heads) : f(NoHeadKeep());
+}
+
+cudaError_t launch_scoring(const void* q, const void* k, const TensorGeom& g, const ImgList& imgs, double* pooled, float* scores,
+                           uint64_t* bitmask, int32_t* kept_idx, int32_t* kept_cnt, int cluster, bool pool, const HeadKeep* heads,
+                           const MassShare* share, float mass_scale, cudaStream_t s, const QuadOrder& order) {
+    ScoreArgs a = score_args(q, k, g, imgs, pooled, scores, bitmask, kept_idx, kept_cnt, order);
+    a.cluster = cluster;
+    a.pool = pool;
+    return with_rule(heads, share, mass_scale, [&](const auto& rule) { return launch(a, rule, imgs.n * g.H, s); });
+}
+
+cudaError_t launch_rows(const TensorGeom& g, const ImgList& imgs, double* pooled, float* scores, uint64_t* bitmask, int32_t* kept_idx,
+                        int32_t* kept_cnt, const HeadKeep* heads, const MassShare* share, float mass_scale, cudaStream_t s,
+                        const QuadOrder& order, const DevPlan* plan, int n_cap) {
+    ScoreArgs a = score_args(nullptr, nullptr, g, imgs, pooled, scores, bitmask, kept_idx, kept_cnt, order);
+    a.plan = plan;
+    if (plan) a.n_cap = n_cap;
+    return with_rule(heads, share, mass_scale, [&](const auto& rule) { return launch_rows_of(a, rule, s); });
+}
+
+// Up to 128 key blocks a thread block's warps have one fragment each; longer rows of few pairs lose (2 heads of 129 to 150 blocks at D = 128
+// +1.7 %).  From SCORING_FROM quads on it would gain little (1.4 % where there are no clusters).  Launches of up to half as many quads as
+// SMs would gain 5 %, but their callers count four launches a step (rapid3_launch_count).
+bool scoring_rows(const TensorGeom& g, int images) {
+    const int quads = images * g.H * ((g.nb + 3) / 4);
+    return 2 * quads > SM_COUNT && quads < SCORING_FROM && g.nb <= 128;
 }
