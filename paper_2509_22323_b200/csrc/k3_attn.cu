@@ -267,7 +267,9 @@ attn_kernel(const __grid_constant__ CUtensorMap tmq, const __grid_constant__ CUt
     const uint32_t bNE = smem_u32(&ctl->near_end), bT = smem_u32(&ctl->taken_full), bFK = smem_u32(&ctl->first_known);
 
     // ---------------------------------------------------------------- setup
-    // The list warp needs nothing of it until it arrives on a barrier, so it only waits for warp 0 (named barrier 1), later on.
+    // The list warp needs nothing of it until it arrives on an mbarrier, so it only waits for warp 0 (named barrier 1), later on, and
+    // meets the others on barrier 2 by arriving.  Barrier 2 is met nowhere else: nothing keeps the list warp back until the others are past it, and
+    // on the teardown's barrier 0 a second arrival of its would stand in for a warp that is late (the one that allocates tensor memory, say).
     if (warp == 0) {
         constexpr uint32_t at = offsetof(Ctl, taken_full) / 8, bars = offsetof(Ctl, tmem_base) / 8 - at;
         auto has = [&](uint32_t x, size_t member, int n) { return x + at - (uint32_t)(member / 8) < (uint32_t)n; };
@@ -300,8 +302,8 @@ attn_kernel(const __grid_constant__ CUtensorMap tmq, const __grid_constant__ CUt
     // after thousands of polls, so nothing sets it before this; what read it last has ended before the selection kernel began, if
     // that is in front.
     if (SPLIT && blockIdx.x == 0 && tid == 0) __stcg(prm.parts.given_up, 0);
-    if (warp == LIST_WARP) bar_arrive(0, NTHREADS);
-    else bar_sync(0, NTHREADS);
+    if (warp == LIST_WARP) bar_arrive(2, NTHREADS);
+    else bar_sync(2, NTHREADS);
     tc_fence_after();
     const uint32_t tmem_base = ctl->tmem_base;
 

@@ -83,3 +83,25 @@ def test_scores_of_minus_infinity_in_one_turn(D):
     for h in range(H):
         ref = attention_64(q[0, h], k[0, h], v[0, h], keep)
         assert float((out[0, h].double() - ref).abs().max()) <= 2 ** -7 * float(v.abs().max())
+
+
+@pytest.mark.parametrize("D,n_blocks,H", [(64, 6, 18), (64, 22, 3), (128, 8, 37), (128, 20, 1)])
+def test_steps_by_turns_queued_equal_steps_alone(D, n_blocks, H):
+    """Every thread block's list is there long before its other warps are through with the set-up, or late, behind a selection: steps
+    queued without a wait give what each gives alone."""
+    (q, k, v), _ = random_qkv((1, H, 64 * n_blocks, D), n_blocks)
+    ctx = binding.Context(1, H, D, 64, 64 * (n_blocks - 1))
+    ratios = (1.0, 0.3, 1.0, 0.8)
+    alone = []
+    for r in ratios:
+        alone.append(torch.full_like(q, float("nan")))
+        ctx.rapid3_gated_step(q, k, v, alone[-1], [2], [r])
+        torch.cuda.synchronize()
+    outs = [torch.full_like(q, float("nan")) for _ in range(32)]
+    for _ in range(8):
+        for n, o in enumerate(outs):
+            ctx.rapid3_gated_step(q, k, v, o, [2], [ratios[n % 4]])
+    torch.cuda.synchronize()
+    assert ctx.last_status() == 0
+    for n, o in enumerate(outs):
+        assert torch.equal(o.view(torch.int16), alone[n % 4].view(torch.int16)), n
