@@ -338,7 +338,8 @@ int rapid3_last_status(rapid3_ctx* ctx, int* device_status);
  * memory and returns.  Nothing waits without a limit and nothing faults; `out` is left partly
  * or wholly unwritten.  In a context that works on kept blocks in parts (see rapid3_sparse_joint_attn)
  * the groups are those of a part, stop_group counts as its last where it has fewer, and the launch
- * that adds up the parts follows and writes nothing.  The context stays usable: after rapid3_last_status has returned (and
+ * that adds up the parts follows and writes nothing; in one that works on them as two interleaved halves
+ * nothing is written either.  The context stays usable: after rapid3_last_status has returned (and
  * cleared) the code, ordinary calls compute as before.  Asynchronous on `stream`.
  */
 int rapid3_debug_inject_timeout(rapid3_ctx* ctx, const void* q, const void* k, const void* v, void* out,

@@ -1183,13 +1183,16 @@ cudaError_t attention_static_init() {
                               attn_kernel<128, false, false, true>, attn_kernel<64, false, false, true>,
                               attn_kernel<128, false, false, false, true>, attn_kernel<64, false, false, false, true>,
                               attn_kernel<128, true>, attn_kernel<64, true>, attn_kernel<128, true, true>, attn_kernel<64, true, true>,
-                              attn_kernel<128, false, false, false, false, true>, attn_kernel<64, false, false, false, false, true>);
+                              attn_kernel<128, false, false, false, false, true>, attn_kernel<64, false, false, false, false, true>,
+                              attn_kernel<128, true, false, false, false, true>, attn_kernel<64, true, false, false, false, true>);
     if (e != cudaSuccess) return e;
     // the warps that take registers wait for them: a build that is launched with fewer would wait for good
     for (const void* kernel : {(const void*)attn_kernel<128, false, true>, (const void*)attn_kernel<64, false, true>,
                                (const void*)attn_kernel<128, true, true>, (const void*)attn_kernel<64, true, true>,
                                (const void*)attn_kernel<128, false, false, false, false, true>,
-                               (const void*)attn_kernel<64, false, false, false, false, true>}) {
+                               (const void*)attn_kernel<64, false, false, false, false, true>,
+                               (const void*)attn_kernel<128, true, false, false, false, true>,
+                               (const void*)attn_kernel<64, true, false, false, false, true>}) {
         cudaFuncAttributes attr;
         const cudaError_t r = cudaFuncGetAttributes(&attr, kernel);
         if (r != cudaSuccess) return r;
@@ -1351,10 +1354,10 @@ cudaError_t launch_attention(const CUtensorMap& tmq, const CUtensorMap& tmk, con
         return launch_kernel(g.D == 128 ? add_parts_kernel<128> : add_parts_kernel<64>, dim3(left * SOFTMAX_WARPS * (g.D / 32) / 4), dim3(128), 0, s,
                              static_cast<uint16_t*>(out), g, imgs, n_dense, plan, prm.parts);
     } else if (inject_stop_group >= 0) {
-        if (g.D == 128)
-            attn_kernel<128, true><<<grid, NTHREADS, attn_smem_bytes<128>(), s>>>(tmq, tmk, tmv, static_cast<uint16_t*>(out), prm);
-        else
-            attn_kernel<64, true><<<grid, NTHREADS, attn_smem_bytes<64>(), s>>>(tmq, tmk, tmv, static_cast<uint16_t*>(out), prm);
+        const bool keys = parts && parts->keys;
+        const auto kernel = g.D == 128 ? (keys ? attn_kernel<128, true, false, false, false, true> : attn_kernel<128, true>)
+                                       : (keys ? attn_kernel<64, true, false, false, false, true> : attn_kernel<64, true>);
+        kernel<<<grid, NTHREADS, g.D == 128 ? attn_smem_bytes<128>() : attn_smem_bytes<64>(), s>>>(tmq, tmk, tmv, static_cast<uint16_t*>(out), prm);
     } else {
         const bool masks = bitmask || (!kept_idx && g.D == 128);         // see MASKS
         if (parts && parts->keys)

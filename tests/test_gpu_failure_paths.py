@@ -81,6 +81,36 @@ def test_a_wait_that_runs_out_leaves_rows_in_parts_unwritten(D, n_blocks, stop_g
     assert float((want[0].double() - ref).abs().max()) <= 2 ** -7 * float(v.abs().max())    # P and the result rounded to bf16
 
 
+@pytest.mark.parametrize("D,n_blocks,H,stop_group", [(64, 6, 3, 0), (64, 6, 3, 5), (64, 21, 2, 1), (64, 21, 2, 20), (64, 21, 2, 21),
+                                                     (128, 8, 3, 0), (128, 19, 2, 2), (128, 19, 2, 18), (128, 19, 2, 19)])
+def test_a_wait_that_runs_out_by_turns(D, n_blocks, H, stop_group):
+    """A context whose tiles take the key blocks by turns: the copies stop before the first block, or so late that one of the two tiles has
+    all of its own.  Neither waits for good for what the other would hand it, nothing is written, and the steps after it are whole."""
+    gen = torch.Generator(device=DEV).manual_seed(n_blocks)
+    q, k, v = (torch.randn((1, H, 64 * n_blocks, D), generator=gen, device=DEV).to(torch.bfloat16) for _ in range(3))
+    ctx = binding.Context(1, H, D, 64, 64 * (n_blocks - 1))
+    want = {}
+    for ratio in (1.0, 0.5):
+        want[ratio] = poison_like(q)
+        ctx.rapid3_gated_step(q, k, v, want[ratio], [2], [ratio])
+    for _ in range(2):
+        n0, scratch = ctx.launch_count(), poison_like(q)
+        ctx.rapid3_debug_inject_timeout(q, k, v, scratch, stop_group)
+        torch.cuda.synchronize()
+        assert ctx.launch_count() - n0 == 1
+        assert ctx.last_status() == ERR_TIMEOUT
+        assert ctx.last_status() == 0
+        assert (scratch.view(torch.int16) == np.int16(POISON)).all()
+        for ratio in (1.0, 0.5):
+            out = poison_like(q)
+            ctx.rapid3_gated_step(q, k, v, out, [2], [ratio])
+            torch.cuda.synchronize()
+            assert ctx.last_status() == 0
+            assert torch.equal(out.view(torch.int16), want[ratio].view(torch.int16))
+    ref = (q[0].double() @ k[0].double().transpose(1, 2) * D ** -0.5).softmax(-1) @ v[0].double()
+    assert float((want[1.0][0].double() - ref).abs().max()) <= 2 ** -7 * float(v.abs().max())    # P and the result rounded to bf16
+
+
 @pytest.mark.parametrize("D", [64, 128])
 def test_a_wait_that_ran_out_does_not_delay_the_end_by_the_sequence(D):
     """512 key blocks: 256 thread blocks, two rounds of them, each over after 4096 polls and 16 more for each of the next 32
