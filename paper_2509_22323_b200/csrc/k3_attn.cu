@@ -103,6 +103,13 @@ struct AttnParams {
 __host__ __device__ constexpr uint32_t divider(uint32_t d) { return d < 2 ? 0u : 0xffffffffu / d + 1u; }
 __device__ __forceinline__ int divide(int x, uint32_t by) { return (int)__umulhi((uint32_t)x, by) + (by ? 0 : x); }
 
+// Reference maximum, times -c2, of a row all of whose scores so far are -inf, where O and l may be added to others' (parts, blocks by turns).
+constexpr float LOWEST = FLT_MAX;
+// 1 / row sum: 0 for a row that keeps nothing, not a number for one that keeps blocks and has no score above -inf in any: softmax's 0 / 0.
+__device__ __forceinline__ float one_over(float sum, float nm) {
+    return sum > 0.f ? 1.f / sum : nm == LOWEST ? __int_as_float(0x7fffffff) : 0.f;
+}
+
 template <int D>
 struct Cfg {
     static constexpr int DH = D / 64;                       // 64-channel halves per row
@@ -851,7 +858,7 @@ attn_kernel(const __grid_constant__ CUtensorMap tmq, const __grid_constant__ CUt
                     row_maxima(r, nm_lo, nm_hi);
                     nm_lo *= -c2; nm_hi *= -c2;
                     // a part may begin with a block whose scores are all -inf: no NaN (-inf - -inf) from them, the next ones count
-                    if (SPLIT || KEYS) { nm_lo = fminf(nm_lo, FLT_MAX); nm_hi = fminf(nm_hi, FLT_MAX); }
+                    if (SPLIT || KEYS) { nm_lo = fminf(nm_lo, LOWEST); nm_hi = fminf(nm_hi, LOWEST); }
                     seeded = true;
                     if (SPLIT && cg == 0) { ref[0] = nm_lo; ref[8] = nm_hi; }
                 }
@@ -966,7 +973,7 @@ attn_kernel(const __grid_constant__ CUtensorMap tmq, const __grid_constant__ CUt
             float b_lo = v.x == INFINITY ? 0.f : ex2(m_lo - v.x), b_hi = v.y == INFINITY ? 0.f : ex2(m_hi - v.y);
             s_lo = fmaf(a_lo, s_lo, b_lo * v.z);
             s_hi = fmaf(a_hi, s_hi, b_hi * v.w);
-            const float inv_lo = s_lo > 0.f ? 1.f / s_lo : 0.f, inv_hi = s_hi > 0.f ? 1.f / s_hi : 0.f;
+            const float inv_lo = one_over(s_lo, m_lo), inv_hi = one_over(s_hi, m_hi);
             a_lo *= inv_lo; b_lo *= inv_lo; a_hi *= inv_hi; b_hi *= inv_hi;
             const int tok_lo = u.tok[a] + (row_lo & 63), tok_hi = tok_lo + 8;
             uint16_t* o_lo = out + (long long)u.b * g.stride_b + (long long)u.h * g.stride_h + (long long)tok_lo * g.stride_n + 8 * cg;
@@ -1029,7 +1036,8 @@ attn_kernel(const __grid_constant__ CUtensorMap tmq, const __grid_constant__ CUt
             s_hi += __shfl_xor_sync(0xffffffffu, s_hi, 1);
             s_lo += __shfl_xor_sync(0xffffffffu, s_lo, 2);
             s_hi += __shfl_xor_sync(0xffffffffu, s_hi, 2);
-            const float inv_lo = s_lo > 0.f ? 1.f / s_lo : 0.f, inv_hi = s_hi > 0.f ? 1.f / s_hi : 0.f;
+            // (in builds without LOWEST the O of a row of scores of -inf is not a number as it is)
+            const float inv_lo = one_over(s_lo, SPLIT ? nm_lo : 0.f), inv_hi = one_over(s_hi, SPLIT ? nm_hi : 0.f);
             const int tok_lo = u.tok[a] + (row_lo & 63), tok_hi = tok_lo + 8;
             uint16_t* o_lo = out + (long long)u.b * g.stride_b + (long long)u.h * g.stride_h + (long long)tok_lo * g.stride_n + 8 * cg;
             uint16_t* o_hi = o_lo + 8 * g.stride_n;
@@ -1152,7 +1160,7 @@ __global__ void __launch_bounds__(128) add_parts_kernel(uint16_t* __restrict__ o
                 f[4 * k + 2] = fmaf(w_hi, x4[i][k].z, f[4 * k + 2]); f[4 * k + 3] = fmaf(w_hi, x4[i][k].w, f[4 * k + 3]);
             }
         }
-    const float inv_lo = s_lo > 0.f ? 1.f / s_lo : 0.f, inv_hi = s_hi > 0.f ? 1.f / s_hi : 0.f;
+    const float inv_lo = one_over(s_lo, m_lo), inv_hi = one_over(s_hi, m_hi);
     uint32_t a_lo[4], a_hi[4];
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
