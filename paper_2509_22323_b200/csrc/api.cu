@@ -269,7 +269,8 @@ int rapid3_create(rapid3_ctx** out, const rapid3_shape* shape) {
         rapid3_destroy(c);
         return RAPID3_ERR_WORKSPACE;
     }
-    if (attention_static_init() != cudaSuccess || scoring_static_init() != cudaSuccess || scoring_cluster_static_init() != cudaSuccess) {
+    if (attention_static_init() != cudaSuccess || scoring_static_init() != cudaSuccess || scoring_cluster_static_init() != cudaSuccess ||
+        prepare_static_init() != cudaSuccess) {
         cudaGetLastError();
         rapid3_destroy(c);
         return RAPID3_ERR_CUDA;

@@ -218,6 +218,7 @@ struct PrepArgs {
     const float* rot;     // [N][D/2][2] (cos, sin) or nullptr
     float eps;
 };
+cudaError_t prepare_static_init();
 cudaError_t launch_prepare(const PrepArgs& a, const TensorGeom& g, const ImgList& imgs, int n_sparse, double* pooled,
                            cudaStream_t s);
 // Builds the plan from device-resident actions and keep ratios (one thread block; B <= RAPID3_MAX_IMG).

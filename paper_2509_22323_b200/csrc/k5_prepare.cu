@@ -8,6 +8,8 @@
 // Reads the raw Q and K once, writes Q and K once: 4.5 to 5 TB/s of that where all SMs are busy for long (three images of 4608 tokens,
 // 24 heads, D = 128 77 -> 69 us, one of 16896 95 -> 76), issue slots (118 instructions for 256 numbers, 56 % of the
 // slots) and the chain of a warp's rows in smaller launches (one of 4608 33.1 -> 23.2 us, two of 4429 at D = 64 29.0 -> 23.0).
+#include <algorithm>
+
 #include "ptx.cuh"
 #include "scoring.cuh"
 
@@ -132,7 +134,22 @@ __global__ void __launch_bounds__(32 * WARPS, INFL > 4 ? 8 / WARPS : 24 / WARPS)
     scoring::write_mean<D, true>(acc, valid, mean, lane);
 }
 
+// Shared memory, beside the table, that a thread block of a launch of few asks for: so much that no more of them fit an SM than the launch needs.
+// They may be let in while add_parts_kernel of the call before still holds most SMs (two of its thread blocks fit one), and would pile up on those with
+// room: 2 heads of 24 to 32 blocks at D = 128, whole steps from raw projections, us, without / with 31.0 to 33.2 / 26.8 to 29.3; one head of 36 32.4 / 27.9;
+// 96 steps of 1 to 6 heads of 20 to 58 blocks 3 % faster in the mean.
+int spread_smem_bytes(int D, int blocks) {
+    const int sm_bytes = 228 << 10, per_sm = (blocks + SM_COUNT - 1) / SM_COUNT;
+    return std::max(0, sm_bytes / (per_sm + 1) - 256 * D);              // 256 D: the table; each thread block takes 1 KB more
+}
+
 }  // namespace
+
+cudaError_t prepare_static_init() {
+    const cudaError_t e = cudaFuncSetAttribute(prepare_kernel<128, 8, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, spread_smem_bytes(128, 1));
+    if (e != cudaSuccess) return e;
+    return cudaFuncSetAttribute(prepare_kernel<64, 8, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, spread_smem_bytes(64, 1));
+}
 
 cudaError_t launch_prepare(const PrepArgs& a, const TensorGeom& g, const ImgList& imgs, int n_sparse, double* pooled,
                            cudaStream_t s) {
@@ -143,7 +160,8 @@ cudaError_t launch_prepare(const PrepArgs& a, const TensorGeom& g, const ImgList
     const bool few = (g.nb + 3) / 4 * 2ll * g.H * imgs.n <= 2 * SM_COUNT;
     const int warps = few ? 2 : 4;
     const dim3 grid(g.nb, (2 * g.H + warps - 1) / warps, imgs.n);
-    return launch_kernel(few ? (g.D == 128 ? prepare_kernel<128, 8, 2> : prepare_kernel<64, 8, 2>)
-                             : (g.D == 128 ? prepare_kernel<128, 4, 4> : prepare_kernel<64, 4, 4>), grid, dim3(32 * warps), 0, s, qr, kr, qo, ko, a.q_gain,
-                         a.k_gain, a.rot, a.eps, g, imgs, n_sparse, pooled);
+    const auto kernel = few ? (g.D == 128 ? prepare_kernel<128, 8, 2> : prepare_kernel<64, 8, 2>)
+                            : (g.D == 128 ? prepare_kernel<128, 4, 4> : prepare_kernel<64, 4, 4>);
+    return launch_kernel(kernel, grid, dim3(32 * warps), few ? spread_smem_bytes(g.D, (int)(grid.x * grid.y * grid.z)) : 0, s, qr, kr, qo, ko,
+                         a.q_gain, a.k_gain, a.rot, a.eps, g, imgs, n_sparse, pooled);
 }
