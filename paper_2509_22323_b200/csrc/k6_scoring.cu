@@ -181,7 +181,8 @@ template <int D, int IPL, int ROW_WARPS, typename HK>
 __global__ void __launch_bounds__(ROW_WARPS * 32) rows_kernel(const __grid_constant__ ScoreArgs a, const __grid_constant__ HK hk) {
     constexpr int LDS = D + 4, LDN = 32 * IPL + 4;
     __shared__ __align__(16) double sq[ROWS * LDS];
-    __shared__ float ss[ROWS * LDN];
+    __shared__ __align__(8) float ss[ROWS * LDN];        // stored two at a time
+    static_assert(LDN % 2 == 0, "a row's pairs lie on 8 bytes");
     __shared__ uint32_t kept[ROWS][IPL];
     const TensorGeom& g = a.g;
     const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
