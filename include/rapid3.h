@@ -264,7 +264,9 @@ int rapid3_cache_step(const void* x, void* o, void* delta, const int32_t* action
 int rapid3_workspace(rapid3_ctx* ctx, float** scores, uint64_t** bitmask, int32_t** kept_idx,
                      int32_t** kept_cnt);
 
-/* Number of kernels this context has launched so far (all entry points). */
+/* Number of kernels this context has launched so far (all entry points).  How many a call takes is part of the interface and is
+ * said at each entry point: callers count them.  A step with a sparse image and up to 74 quads takes the four (five by mass) that
+ * rapid3_gated_step names first, although scores and selection in one would be faster there too. */
 int64_t rapid3_launch_count(rapid3_ctx* ctx);
 
 /*

@@ -387,7 +387,7 @@ cudaError_t launch_rows(const TensorGeom& g, const ImgList& imgs, double* pooled
 
 // Up to 128 key blocks a thread block's warps have one fragment each; longer rows of few pairs lose (2 heads of 129 to 150 blocks at D = 128
 // +1.7 %).  From SCORING_FROM quads on it would gain little (1.4 % where there are no clusters).  Launches of up to half as many quads as
-// SMs would gain 5 %, but their callers count four launches a step (rapid3_launch_count).
+// SMs would gain 5 %: this line is no measured one, rapid3.h promises the launches of such steps one by one (rapid3_launch_count).
 bool scoring_rows(const TensorGeom& g, int images) {
     const int quads = images * g.H * ((g.nb + 3) / 4);
     return 2 * quads > SM_COUNT && quads < SCORING_FROM && g.nb <= 128;
