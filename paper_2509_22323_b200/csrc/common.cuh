@@ -99,10 +99,11 @@ __host__ __device__ inline int quad_block(const TensorGeom& g, int quad, int a) 
 // an SM begins with: all of them start at once, and without the order they start 1 us sooner (40 steps of 297 to 1000 quads 0.4 %).
 // One quad for nearly every SM is enough, its last: of 448, 288, 192, 160, 144, 128, 112, 96 and 64 quads 128 were the best in launches above and
 // below 1000 quads (36 and 40 steps drawn at random: -1.6 and -0.6 % against 448, which loses what the quads of a head share in the L2 and is
-// longer to search).  For launches of more than ORDER_FROM quads, us against quads in order: two images of 288 quads at D = 64 39.6 -> 38.5,
-// 864 quads with a ratio for every head 197.5 -> 183, by cumulative mass 358.2 -> 341, one image of 432 at 0.5 from raw projections 8 less, 1584
-// of one 16896-token image 1124 -> 1115; steps drawn at random in the mean and the worst: 149 to 200 quads -1.4 % and +0.7 % (30), more -0.7 %
-// and +1.7 % (30) against 448 from 201 to 1000 quads, which was 1.8 % better than quads in order.  With a quad an SM nothing is handed out.
+// longer to search).  For launches of more than ORDER_FROM quads, us, in order / so, by turns: two images of 288 quads at D = 64 39.7 / 38.5,
+// 864 quads with a ratio for every head 193.9 / 180.6, by cumulative mass 354.5 / 335.0, one image of 432 at 0.5 from raw projections 195.3 / 189.5, 1584
+// quads of one 16896-token image 1100 / 1104 (no difference shown); steps drawn at random, in the mean and the worst that differed by more than its own
+// runs: 149 to 221 quads -0.8 % and +6.6 % (18; the worst 160 quads of rows of 5 blocks), 222 to 296 -3.7 % and +0.9 % (18), more -1.3 % (24).  With a
+// quad an SM nothing is handed out.
 constexpr int ORDER_CLASSES = 32, ORDER_LAST = 128, ORDER_FROM = SM_COUNT;
 // Of `light` quads without text rows, behind `heavy` others, how many stay where they are.
 __host__ __device__ inline int order_after(int light, int heavy) {

@@ -74,7 +74,8 @@ constexpr int MAX_PARTS = 8, MAX_LEFT = 444, MIN_CUT = 24, MAX_CUT = 600;
 // Attention of one image, every block kept, us, one tile an SM / by turns: D = 64 5 blocks 7.1 / 6.6 (but a step at ratio 0.5, lists of four,
 // 11.9 / 12.3), 8 8.8 / 7.8, 12 12.1 / 10.0, 17 14.4 / 11.9, 36 25.4 / 19.9; D = 128 5 7.8 / 7.8, 8 9.9 / 9.5, 12 14.0 / 12.7, 17 16.9 / 15.0,
 // 36 29.4 / 26.4 (steps of 6 blocks 15.3 / 15.7, of 8 to 10 1 to 5 % faster).  At D = 128 a block takes 0.58 us, not half of the 0.84 for two tiles: K and V come twice as
-// fast, and more stages for them, or V in later groups, did not change that.  Fifty steps of such contexts drawn at random: 3.9 % faster.
+// fast, and more stages for them, or V in later groups, did not change that.  Forty steps of contexts of up to 74 quads drawn at random: 3.9 %
+// faster in the mean, at worst 2.0 % slower (18 quads of 9 blocks at D = 128); ratios of 0.1 to 0.75 in 110 steps: at worst 1.7 % slower (rows of 6 blocks).
 constexpr int KEYS_FROM_64 = 6, KEYS_FROM_128 = 8;
 // After a wait has run out the softmax warps go on for up to this many key blocks, each a wait of 16 polls of about 8 us.
 // (Over the whole of a quad, with 256 polls a block, that was 2.06 s at two heads of 1024 key blocks; now 4.7 ms.)
@@ -1252,7 +1253,9 @@ static size_t left_units(const TensorGeom& g, int n_img, const AttnParts& parts)
 // 56.3 / 47.1 (two); 60 of 12 13.7 / 15.7, 15.5 / 21.0 (two).  Steps: 46 quads of 92 blocks at ratio 0.25, D = 64 61.6 / 31.8
 // (text rows in five, the others in three); 132 of 264 at ratio 0.2, D = 128 231 / 135 (text rows in four); 198 of 262 at ratios
 // 1, 0.5 and 0.2, D = 64 359, 289 and 196 / 289, 237 and 148 (in two, text rows in three).
-// Where lists stay whole and every tile has an SM to itself in the largest launch, the two tiles of the SM take its blocks by turns.
+// Where lists stay whole and every tile has an SM to itself in the largest launch, the two tiles of the SM take its blocks by turns.  The model has
+// the times of a tile alone for such lists, not the 0.42 and 0.60 us a block that they take by turns: with these it would leave whole the lists of 0.7 % of
+// the contexts drawn at random that it cuts now (54 quads of 36 blocks, D = 64).
 AttnParts attention_parts(const TensorGeom& g, int n_img) {
     AttnParts best;
     const int nq = (g.nb + 3) / 4, ntq = std::min(nq, (g.n_text_blocks + 3) / 4);

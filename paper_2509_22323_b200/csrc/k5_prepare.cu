@@ -5,9 +5,9 @@
 // Layout of the work as in the pooling kernel: one warp per (Q|K, image, head, 64-token block), a
 // token row of D channels is D / 8 lanes of 16 bytes; the row's sum of squares is reduced over
 // those lanes with shuffles, the rotation is lane-local (a lane holds four whole pairs).
-// Reads the raw Q and K once, writes Q and K once: 4.5 to 5 TB/s of that where all SMs are busy for long (three images of 4608 tokens,
-// 24 heads, D = 128 77 -> 69 us, one of 16896 95 -> 76), issue slots (118 instructions for 256 numbers, 56 % of the
-// slots) and the chain of a warp's rows in smaller launches (one of 4608 33.1 -> 23.2 us, two of 4429 at D = 64 29.0 -> 23.0).
+// Reads the raw Q and K once, writes Q and K once: 4.4 to 4.7 TB/s of that in launches of 24 heads, bound by issue slots (118 instructions for 256
+// numbers, 56 % of the slots) and the chain of a warp's rows.  The kernel alone, us, before its warps shared a table / since (one run of ncu, caches
+// as they are): D = 128 one image of 4608 tokens 28.6 / 26.1, three 79.9 / 71.8, one of 16896 100.8 / 90.7; D = 64 two of 4480 29.4 / 23.8.
 #include <algorithm>
 
 #include "ptx.cuh"
@@ -26,7 +26,7 @@ namespace {
 // conversion unit, which has room (a third of its rate), where bits would cost issue slots.
 // INFL rows are in flight a lane, each replaced by the one INFL further on as soon as it is taken.  Four of them and 24 warps an SM
 // were the best for large launches (two 27.3, 16 warps 38.5, 32 warps with fewer registers 29 us for one image of 4608 tokens; thread blocks of 8 warps
-// 26.0, of 4 23.3); eight where the thread blocks have an SM to themselves or nearly so and the time is the chain of their loads
+// 26.0, of 4 23.3, by events in one run); eight where the thread blocks have an SM to themselves or nearly so and the time is the chain of their loads
 // (steps of one image from raw projections: 2 heads x 36 blocks at D = 64 26.6 -> 25.5 us, 12 heads x 10 blocks at D = 128 29.0 -> 27.4).
 template <int D, int INFL, int WARPS>
 __global__ void __launch_bounds__(32 * WARPS, INFL > 4 ? 8 / WARPS : 24 / WARPS) prepare_kernel(const uint16_t* q_raw,
